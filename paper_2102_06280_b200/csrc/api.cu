@@ -399,21 +399,23 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, 
         sel = h->side;
         forked = true;
     }
+    // Tensor-core rounds: the dW GEMMs take the step of the workers that take no part, so they wait for the selection.
+    const bool stepped = batch_idx && (h->flags & DBW_GEMM_BF16) && mix_active_usable(h);
     if (ev) cuda(cudaEventRecord(ev[2], sel));
-    note(launch_select(h, t, b, kept, T_worker, T_nbr, T_round, true, sel));
+    note(launch_select(h, t, b, kept, T_worker, T_nbr, T_round, true, sel, stepped));
     if (ev) cuda(cudaEventRecord(ev[3], sel));
+    if (forked) cuda(cudaEventRecord(h->ev_join, sel));
     if (ev) cuda(cudaEventRecord(ev[0], s));
+    const StepArgs step{lr, lr_per_worker, X_out, h->ev_join};
     if (batch_idx && first == DBW_OK)
-        note((h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, h->d_G, loss, s)
+        note((h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, h->d_G, loss, s, stepped ? &step : nullptr)
                                         : launch_grad_fp32(h, X, batch_idx, h->d_G, loss, s));
     if (ev) cuda(cudaEventRecord(ev[1], s));
-    if (forked) {  // whatever failed above, the side stream is joined back: it never dangles, a capture stays valid
-        cuda(cudaEventRecord(h->ev_join, sel));
-        cuda(cudaStreamWaitEvent(s, h->ev_join, 0));
-    }
+    // whatever failed above, the side stream is joined back: it never dangles, a capture stays valid
+    if (forked) cuda(cudaStreamWaitEvent(s, h->ev_join, 0));
     if (first != DBW_OK) return first;
     if (ev) cuda(cudaEventRecord(ev[4], s));
-    note(launch_mix(h, X, G, lr, lr_per_worker, X_out, s));
+    note(stepped ? launch_mix_active(h, X, G, lr, lr_per_worker, X_out, s) : launch_mix(h, X, G, lr, lr_per_worker, X_out, s));
     if (ev) cuda(cudaEventRecord(ev[5], s));
     return first;
 }

@@ -77,6 +77,18 @@ __device__ __forceinline__ int checked(int idx, int limit, uint32_t* status) {
     return idx;
 }
 
+// Which workers take part in a round (they keep a neighbour or are kept by one), as the selection kernel leaves it on
+// the device.  The rows of the others are mixed with nothing: x' = x - lr g is all that happens to them.
+struct ActiveRows {
+    int* list = nullptr;   // [N] the participants in ascending order
+    int* pos = nullptr;    // [N] position of a participant in the list, -1 for the others
+    int* slot = nullptr;   // [N][plan.stride] the mixing plan's entries of the participants as list positions
+    int* count = nullptr;  // [1]
+};
+// Up to this many participants the dW GEMMs take the others' step and the mix works on the participants alone; above it
+// the round is mixed as a whole.  (Half: x and g of the participants then fit the panel buffer of all rows.)
+__host__ __device__ inline int active_limit(int N) { return N / 2; }
+
 struct BF16State;  // tensor-core gradient path (grad_bf16.cu)
 struct TcMixState;  // tensor-core mix (mix_tc.cu)
 struct SpMixState;  // tensor-core mix with 2:4 structured sparsity (mix_sp.cu)
@@ -107,6 +119,7 @@ struct dbw_handle {
     uint32_t* d_waited = nullptr;    // [N] scratch flags of the selection kernel (kept zero between calls)
     uint32_t* d_ticket = nullptr;    // [1] block ticket of the selection kernel (kept zero between calls)
     double* d_Tnbr_ws = nullptr;     // [N]
+    dbw::ActiveRows active;          // participants of the round (tensor-core rounds only, allocated with that path)
 
     const double* t_edge = nullptr;  // optional per-link arrival times (caller-owned, DEVICE, aligned with col)
 
@@ -164,7 +177,7 @@ namespace dbw {
 
 // select.cu
 int launch_select(dbw_handle* h, const double* t, const int32_t* b, uint8_t* kept, double* T_worker,
-                  double* T_nbr, double* T_round, bool build_plan, cudaStream_t s);
+                  double* T_nbr, double* T_round, bool build_plan, cudaStream_t s, bool list_active = false);
 int launch_plan_from_kept(dbw_handle* h, const uint8_t* kept, const int32_t* b, cudaStream_t s);
 
 // mix.cu
@@ -178,6 +191,9 @@ __device__ __forceinline__ uint2 pack_bf16x4_rn(float a, float b, float c, float
     return make_uint2(lo, hi);
 }
 bool mix_panel_fits(const dbw_handle* h);
+// The mix of a round whose dW GEMMs may already have taken the step x' = x - lr g of every worker that takes no part.
+bool mix_active_usable(const dbw_handle* h);
+int launch_mix_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, cudaStream_t s);
 int mix_kernel_kind(const dbw_handle* h);
 
 // mix_staged.cu
@@ -231,7 +247,14 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
 // grad_bf16.cu
 int grad_bf16_alloc(dbw_handle* h);
 void grad_bf16_free(dbw_handle* h);
-int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss,
-                     cudaStream_t s);
+// The SGD step of the workers that take no part in the round, taken in the epilogue of the dW GEMMs.
+struct StepArgs {
+    float lr;
+    const float* lr_pw;
+    float* X_out;
+    cudaEvent_t selected;  // the selection (and with it the list of participants) is complete after this event
+};
+int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss, cudaStream_t s,
+                     const StepArgs* step = nullptr);
 
 }  // namespace dbw

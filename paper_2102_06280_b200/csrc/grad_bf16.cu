@@ -69,7 +69,7 @@ constexpr int TILE_BYTES = BM * BK * 2;  // 16 KiB per 128-row operand tile
 constexpr int GEMM_THREADS = 320;  // TMA warp, MMA warp, eight epilogue warps (two per accumulator lane quarter)
 constexpr int EPI_WARPS = 8;
 constexpr size_t gemm_smem(int stages, int bn) {
-    return (size_t)stages * (TILE_BYTES + bn * BK * 2) + 8 * 32 * 36 * 4 /*epilogue staging*/ + 1024 /*align slack*/ + 256 /*barriers*/;
+    return (size_t)stages * (TILE_BYTES + bn * BK * 2) + 1024 /*align slack*/ + 256 /*barriers*/;
 }
 // kind::f16, D = f32, A = B = bf16, M = 128, N = bn; bits 15 / 16 select MN-major A / B operands
 __host__ __device__ constexpr uint32_t idesc_for(int bn, bool a_mn, bool b_mn) {
@@ -77,35 +77,31 @@ __host__ __device__ constexpr uint32_t idesc_for(int bn, bool a_mn, bool b_mn) {
            ((uint32_t)(BM >> 4) << 24);
 }
 
-enum { EPI_FWD = 0, EPI_DA = 1, EPI_DW = 2 };
+enum { EPI_FWD = 0, EPI_DA = 1 };
 
 struct TcArgs {
     int M, N, K, epi;
     bf16* out;  long long out_z;  int out_pitch;    // [M][N] bf16 (EPI_FWD, EPI_DA)
-    float* outf; long long outf_z; long long outf_pitch;  // [M][N] fp32 (EPI_DW)
     const float* bias; long long bias_z;            // fp32 [N] (EPI_FWD)
     const bf16* mask; long long mask_z; int mask_pitch;   // bf16 [M][N]: keep where > 0 (EPI_DA)
     uint32_t* status;
 };
 
-constexpr int STAGING_FLOATS = EPI_WARPS * 32 * 36;  // per epilogue warp a 32 x 32 fp32 block, rows 36 words apart
-
-// Persistent, warp-specialised GEMM: one CTA per SM walks the tiles (n fastest, then m, then worker).
+// Persistent, warp-specialised GEMM of the forward and dA steps: one CTA per SM walks the tiles (n fastest, then m, then worker).
 // Warp 0 streams operand tiles by TMA through a STAGES-deep ring, warp 1 issues the MMAs into one of
 // ACC accumulator buffers in tensor memory, warps 2-9 drain a finished buffer through the epilogue
 // while the next tile's loads and MMAs are already running.
-template <int STAGES, int BN, int ACC, bool AMN, bool BMN>
+template <int STAGES, int BN, int ACC, bool BMN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs g, int tiles_m,
                int tiles_n, int n_tiles) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int TILE_B_BYTES = BN * BK * 2;
-    constexpr uint32_t IDESC = idesc_for(BN, AMN, BMN);
+    constexpr uint32_t IDESC = idesc_for(BN, false, BMN);
     uint8_t* tilesA = smem;
     uint8_t* tilesB = smem + STAGES * TILE_BYTES;
-    float* staging = reinterpret_cast<float*>(smem + STAGES * (TILE_BYTES + TILE_B_BYTES));
-    uint64_t* full = reinterpret_cast<uint64_t*>(staging + STAGING_FLOATS);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * (TILE_BYTES + TILE_B_BYTES));
     uint64_t* empty = full + STAGES;
     uint64_t* acc_full = empty + STAGES;
     uint64_t* acc_empty = acc_full + ACC;
@@ -151,18 +147,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         break;
                     }
                     mbar_expect_tx(&full[s], TILE_BYTES + TILE_B_BYTES);
-                    if (!AMN) {
-                        tma_load_3d(tilesA + s * TILE_BYTES, &tmA, kb * BK, m0, z, &full[s]);
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < BM / 64; ++c)  // MN-major: 64 x 64 chunks, coordinates (mn, k row, worker)
-                            tma_load_3d(tilesA + s * TILE_BYTES + c * 8192, &tmA, m0 + c * 64, kb * BK, z, &full[s]);
-                    }
+                    tma_load_3d(tilesA + s * TILE_BYTES, &tmA, kb * BK, m0, z, &full[s]);
                     if (!BMN) {
                         tma_load_3d(tilesB + s * TILE_B_BYTES, &tmB, kb * BK, n0, z, &full[s]);
                     } else {
 #pragma unroll
-                        for (int c = 0; c < BN / 64; ++c)
+                        for (int c = 0; c < BN / 64; ++c)  // MN-major: 64 x 64 chunks, coordinates (mn, k row, worker)
                             tma_load_3d(tilesB + s * TILE_B_BYTES + c * 8192, &tmB, n0 + c * 64, kb * BK, z, &full[s]);
                     }
                 }
@@ -189,10 +179,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     }
                     tc_fence_after();
                     const uint32_t sa = smem_u32(tilesA + s * TILE_BYTES), sb = smem_u32(tilesB + s * TILE_B_BYTES);
-                    const uint64_t da = AMN ? mnmajor_desc(sa) : kmajor_sw128_desc(sa);
+                    const uint64_t da = kmajor_sw128_desc(sa);
                     const uint64_t db = BMN ? mnmajor_desc(sb) : kmajor_sw128_desc(sb);
                     // 16 further along K: 32 bytes inside the swizzle atom (K-major) or 16 rows of 128 bytes (MN-major)
-                    constexpr uint64_t ka = (AMN ? UMMA_K * 128 : UMMA_K * 2) / 16, kbs = (BMN ? UMMA_K * 128 : UMMA_K * 2) / 16;
+                    constexpr uint64_t ka = UMMA_K * 2 / 16, kbs = (BMN ? UMMA_K * 128 : UMMA_K * 2) / 16;
 #pragma unroll
                     for (int k = 0; k < BK / UMMA_K; ++k)
                         tc_mma_bf16(d_tmem, da + (uint64_t)k * ka, db + (uint64_t)k * kbs, IDESC, (kb > 0 || k > 0) ? 1u : 0u);
@@ -210,7 +200,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // one half of the tile's columns (two warps share a lane quarter) ----
         const int q = warp & 3;
         const int half = (warp - 2) >> 2;
-        float* stg = staging + (warp - 2) * (32 * 36);
         int lt = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++lt) {
             const int n0 = (tile % tiles_n) * BN, m0 = ((tile / tiles_n) % tiles_m) * BM, z = tile / (tiles_n * tiles_m);
@@ -225,26 +214,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (nb >= g.N) break;  // warp-uniform
                 uint32_t r[32];
                 tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + c * 32), r);
-                if (g.epi == EPI_DW) {
-                    // Each lane holds one row of a 32 x 32 fp32 block.  It goes through shared memory
-                    // (rows 36 words apart keep both 128-bit phases conflict-free) so that a warp
-                    // stores four full 128-byte lines per instruction.
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4)
-                        *reinterpret_cast<uint4*>(stg + lane * 36 + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
-                    __syncwarp();
-                    const int f4 = lane & 7;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int row = 4 * i + (lane >> 3);
-                        const int mm = m0 + q * 32 + row;
-                        const float4 val = *reinterpret_cast<const float4*>(stg + row * 36 + 4 * f4);
-                        if (mm < g.M && nb + 4 * f4 < g.N)
-                            *reinterpret_cast<float4*>(g.outf + (size_t)z * g.outf_z + (size_t)mm * g.outf_pitch + nb + 4 * f4) = val;
-                    }
-                    __syncwarp();
-                    continue;
-                }
                 float v[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
@@ -289,9 +258,236 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
 }
 
+// ----------------------------------------------------------------------------- dW, and the step of workers that mix with nobody
+// dW_l = dZ_{l+1}^T A_l in fp32, straight into G: HBM-bound (the reduction runs over the mini-batch only, 4 bytes leave per
+// weight for every 2 B multiply-adds).  Inside a round the epilogue does more for a worker that takes no part (it keeps nobody
+// and nobody keeps it: seven to nine of ten workers in an average round of the threshold rule): its new weights are
+// x' = x - lr dW whatever the others do, so they are written here with their bf16 copy, 10 bytes a weight, and neither a
+// gradient nor a row of the mix is needed for them (4 bytes here and 14 in the mix otherwise).
+//
+// Each of the eight epilogue warps owns 32 rows (its tensor-memory lane quarter) x half of the tile's columns, in blocks of
+// 64 columns, and works on its own: a block of x arrives by cp.async while other warps finish theirs, is stepped in place (a
+// lane per row; 16-byte pieces XOR-swizzled by row, conflict-free both ways), and leaves row by row, 256 bytes of x' and 128
+// of the copy at a time.
+// 128 workers x (1024 x 3072 + 1024 x 1024), batch 256, both launches: nobody steps 452 us; everybody steps 1030 us = 5.6 TB/s
+// of what must move (a streaming kernel with these row pieces reaches 5.4 - 6.0).  Measured against it: blocks of 128 columns
+// leave room for two operand stages instead of three (515 / 1156 us); 32 columns twice buffered 453 / 1176 us (128-byte and
+// 64-byte pieces: 4.9 TB/s in the streaming kernel too); 64 columns twice buffered with two stages 535 / 1213 us.
+constexpr int DW_CW = 64;  // columns of a warp's block
+__host__ __device__ constexpr int dw_stages(int bn) { return bn == 256 ? 3 : 5; }
+constexpr size_t dw_smem(int bn) {
+    return (size_t)dw_stages(bn) * (TILE_BYTES + bn * BK * 2) + EPI_WARPS * 32 * DW_CW * 4 + 1024 /*align slack*/ + 256 /*barriers*/;
+}
+
+struct DwArgs {
+    int M, N, K;                       // out, in, mini-batch
+    float* G; const float* X; float* Xout; bf16* copy;  // W_l inside the rows [worker][ld]; copy nullable (bf16 copy of the stepped weights)
+    long long ld;
+    const int* active_pos;             // worker -> position among the participants (-1: takes the step here); null: dW for everybody
+    const int* active_count; int step_limit;  // with more participants than this nobody steps here
+    float lr; const float* lr_pw;
+    uint32_t* status;
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+template <int BN>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+gemm_dw_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ DwArgs g, int tiles_m, int tiles_n,
+               int n_tiles) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    constexpr int STAGES = dw_stages(BN), TILE_B_BYTES = BN * BK * 2;
+    constexpr uint32_t IDESC = idesc_for(BN, true, true);
+    constexpr int PER = BN / 2 / DW_CW;           // blocks of a tile per warp
+    constexpr int LPR = DW_CW / 4, RPI = 32 / LPR;   // lanes per row and rows per instruction when a warp walks its block row by row
+    uint8_t* tilesA = smem;
+    uint8_t* tilesB = tilesA + STAGES * TILE_BYTES;
+    uint8_t* blocks = tilesB + STAGES * TILE_B_BYTES;  // one of 32 x BW floats per epilogue warp
+    uint64_t* full = reinterpret_cast<uint64_t*>(blocks + EPI_WARPS * 32 * DW_CW * 4);
+    uint64_t* empty = full + STAGES;
+    uint64_t* acc_full = empty + STAGES;
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* drain = acc_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile uint32_t* abort = tmem_slot + 1;  // set by the first wait that runs out; every later wait returns at once
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int num_kb = (g.K + BK - 1) / BK;
+    if (threadIdx.x == 0) {
+        *abort = 0u;
+        mbar_init(drain, 1);
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], EPI_WARPS);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * BN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    auto coords = [&](int tile, int& n0, int& m0, int& z) {
+        n0 = (tile % tiles_n) * BN;
+        m0 = ((tile / tiles_n) % tiles_m) * BM;
+        z = tile / (tiles_n * tiles_m);
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool live = true;
+            for (int tile = blockIdx.x; tile < n_tiles && live; tile += gridDim.x) {
+                int n0, m0, z;
+                coords(tile, n0, m0, z);
+                for (int kb = 0; kb < num_kb; ++kb, ++it) {
+                    const int s = it % STAGES;
+                    if (it >= STAGES && !mbar_wait(&empty[s], ((it / STAGES) - 1) & 1, abort, g.status)) {
+                        live = false;
+                        break;
+                    }
+                    mbar_expect_tx(&full[s], TILE_BYTES + TILE_B_BYTES);
+#pragma unroll
+                    for (int c = 0; c < BM / 64; ++c)  // MN-major: 64 x 64 chunks, coordinates (mn, k row, worker)
+                        tma_load_3d(tilesA + s * TILE_BYTES + c * 8192, &tmA, m0 + c * 64, kb * BK, z, &full[s]);
+#pragma unroll
+                    for (int c = 0; c < BN / 64; ++c)
+                        tma_load_3d(tilesB + s * TILE_B_BYTES + c * 8192, &tmB, n0 + c * 64, kb * BK, z, &full[s]);
+                }
+            }
+            for (int j = it > STAGES ? it - STAGES : 0; j < it; ++j) mbar_wait_quiet<false>(&full[j % STAGES], (j / STAGES) & 1, 1u << 20);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int it = 0, lt = 0;
+            bool live = true;
+            for (int tile = blockIdx.x; tile < n_tiles && live; tile += gridDim.x, ++lt) {
+                const int buf = lt & 1;
+                if (lt >= 2) {  // the epilogue must have drained this buffer's previous tile
+                    if (!mbar_wait(&acc_empty[buf], ((lt / 2) - 1) & 1, abort, g.status)) break;
+                    tc_fence_after();
+                }
+                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
+                for (int kb = 0; kb < num_kb; ++kb, ++it) {
+                    const int s = it % STAGES;
+                    if (!mbar_wait(&full[s], (it / STAGES) & 1, abort, g.status)) {
+                        live = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t da = mnmajor_desc(smem_u32(tilesA + s * TILE_BYTES)), db = mnmajor_desc(smem_u32(tilesB + s * TILE_B_BYTES));
+                    constexpr uint64_t step = UMMA_K * 128 / 16;  // 16 K rows of 128 bytes
+#pragma unroll
+                    for (int k = 0; k < BK / UMMA_K; ++k)
+                        tc_mma_bf16(d_tmem, da + (uint64_t)k * step, db + (uint64_t)k * step, IDESC, (kb > 0 || k > 0) ? 1u : 0u);
+                    tc_commit(&empty[s]);
+                }
+                if (live) tc_commit(&acc_full[buf]);
+            }
+            if (*abort) {  // shutdown after an expired wait: the MMAs issued so far are complete before tensor memory is freed
+                tc_commit(drain);
+                mbar_wait_quiet<false>(drain, 0, 1u << 20);
+            }
+        }
+    } else {
+        const int q = warp & 3, half = (warp - 2) >> 2;
+        float4* block = reinterpret_cast<float4*>(blocks + (warp - 2) * 32 * DW_CW * 4);
+        const int r_in = lane / LPR, c_in = lane % LPR;  // this lane's row (of RPI) and 16-byte piece when a block is walked by rows
+        auto piece = [&](int r, int c) -> float4& { return block[r * LPR + (c ^ (r & 7))]; };
+        const bool steps = g.active_pos && __ldg(g.active_count) <= g.step_limit;
+        auto stepping = [&](int tile) { return steps && tile < n_tiles && __ldg(g.active_pos + tile / (tiles_n * tiles_m)) < 0; };
+        auto load_x = [&](int tile, int j) {  // x of the warp's block j of a tile, asynchronously
+            if (!stepping(tile)) return;
+            int n0, m0, z;
+            coords(tile, n0, m0, z);
+            const int n = n0 + (half * PER + j) * DW_CW + 4 * c_in, rows = min(32, g.M - m0 - q * 32);
+            const float* x = g.X + (size_t)z * g.ld + (size_t)(m0 + q * 32) * g.N + n;
+            if (n < g.N)
+#pragma unroll 8
+                for (int r = r_in; r < rows; r += RPI) cp_async16(&piece(r, c_in), x + (size_t)r * g.N);
+        };
+        load_x(blockIdx.x, 0);
+        int lt = 0;
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++lt) {
+            int n0, m0, z;
+            coords(tile, n0, m0, z);
+            const int buf = lt & 1;
+            const bool step = stepping(tile);
+            const float nlr = step ? -(g.lr_pw ? __ldg(g.lr_pw + z) : g.lr) : 0.f;
+            const bool ready = mbar_wait(&acc_full[buf], (lt / 2) & 1, abort, g.status);
+            if (!__all_sync(0xffffffffu, ready)) break;  // a wait ran out: leave together (the tensor-memory loads below are warp-collective)
+            tc_fence_after();
+            const int rows = min(32, g.M - m0 - q * 32);
+#pragma unroll 1
+            for (int j = 0; j < PER; ++j) {
+                if (step) asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+                uint32_t acc[DW_CW / 32][32];
+#pragma unroll
+                for (int c = 0; c < DW_CW / 32; ++c) tc_ld32_issue(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * BN + (half * PER + j) * DW_CW + c * 32), acc[c]);
+                tc_ld_wait();
+#pragma unroll
+                for (int c = 0; c < DW_CW / 32; ++c) {
+                    uint32_t (&r)[32] = acc[c];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        float4 v = make_float4(__uint_as_float(r[4 * e]), __uint_as_float(r[4 * e + 1]), __uint_as_float(r[4 * e + 2]), __uint_as_float(r[4 * e + 3]));
+                        float4& at = piece(lane, 8 * c + e);
+                        if (step) {
+                            const float4 x = at;
+                            v = make_float4(fmaf(nlr, v.x, x.x), fmaf(nlr, v.y, x.y), fmaf(nlr, v.z, x.z), fmaf(nlr, v.w, x.w));
+                        }
+                        at = v;
+                    }
+                }
+                if (j == PER - 1) {  // this warp's reads of the accumulator are complete: hand it back to the MMA warp
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[buf]);
+                }
+                __syncwarp();
+                const int n = n0 + (half * PER + j) * DW_CW + 4 * c_in;
+                const size_t at = (size_t)z * g.ld + (size_t)(m0 + q * 32) * g.N + n;
+                float* out = (step ? g.Xout : g.G) + at;
+                bf16* copy = step && g.copy ? g.copy + at : nullptr;
+                if (n < g.N) {
+#pragma unroll 8
+                    for (int r = r_in; r < rows; r += RPI) {
+                        const float4 v = piece(r, c_in);
+                        *reinterpret_cast<float4*>(out + (size_t)r * g.N) = v;
+                        if (copy) *reinterpret_cast<uint2*>(copy + (size_t)r * g.N) = pack_bf16x4_rn(v.x, v.y, v.z, v.w);
+                    }
+                }
+                __syncwarp();
+                if (j + 1 < PER)
+                    load_x(tile, j + 1);
+                else
+                    load_x(tile + gridDim.x, 0);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(2 * BN) : "memory");
+    }
+}
+
 // ----------------------------------------------------------------------------- casts and gathers
 // fp32 [rows][cols] (row pitch src_pitch) -> bf16 [rows][cols] (row pitch cols).  Rows may be
-// indirect (row_idx: mini-batch gather).  cols % 8 == 0.  Every thread converts 16 consecutive floats
+// indirect (row_idx: mini-batch gather, then the labels too).  cols % 8 == 0.  Every thread converts 16 consecutive floats
 // of one row: four 128-bit loads, two 128-bit stores.
 __device__ __forceinline__ uint4 pack8(const float* v) {
     return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
@@ -300,7 +496,7 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
 __global__ void __launch_bounds__(256)
 cast_tile_kernel(int rows, int cols, const float* __restrict__ src, long long src_z, long long src_pitch,
                  const int32_t* __restrict__ row_idx, int idx_z, int idx_limit, bf16* __restrict__ dst, long long dst_z,
-                 uint32_t* status) {
+                 const int32_t* __restrict__ labels, int C, int32_t* __restrict__ ylab, uint32_t* status) {
     const int z = blockIdx.z;
     const int t = threadIdx.x;
     const int r = blockIdx.y * 64 + (t >> 2);
@@ -314,6 +510,14 @@ cast_tile_kernel(int rows, int cols, const float* __restrict__ src, long long sr
             s = s < 0 ? 0 : idx_limit - 1;
         }
         sr = s;
+        if (c0 == 0) {  // the row's label; one outside [0, C) is clamped and reported
+            int y = labels[(size_t)z * idx_limit + s];
+            if (y < 0 || y >= C) {
+                atomicOr(status, DBW_STATUS_BAD_INDEX);
+                y = y < 0 ? 0 : C - 1;
+            }
+            ylab[(size_t)z * idx_z + r] = y;
+        }
     }
     const float* p = src + (size_t)z * src_z + sr * src_pitch + c0;
     bf16* d = dst + (size_t)z * dst_z + (size_t)r * cols + c0;
@@ -326,23 +530,6 @@ cast_tile_kernel(int rows, int cols, const float* __restrict__ src, long long sr
     }
     *reinterpret_cast<uint4*>(d) = pack8(v);
     if (c0 + 8 < cols) *reinterpret_cast<uint4*>(d + 8) = pack8(v + 8);
-}
-
-// Labels of the mini-batch; a label outside [0, C) is clamped and reported (the batch index is
-// reported by the feature gather).
-__global__ void gather_labels_kernel(int B, int S, int C, const int32_t* __restrict__ labels, const int32_t* __restrict__ batch_idx,
-                                     int32_t* __restrict__ ylab, uint32_t* status) {
-    const int i = blockIdx.x;
-    for (int s = threadIdx.x; s < B; s += blockDim.x) {
-        int src = batch_idx[(size_t)i * B + s];
-        src = src < 0 ? 0 : (src >= S ? S - 1 : src);
-        int y = labels[(size_t)i * S + src];
-        if (y < 0 || y >= C) {
-            atomicOr(status, DBW_STATUS_BAD_INDEX);
-            y = y < 0 ? 0 : C - 1;
-        }
-        ylab[(size_t)i * B + s] = y;
-    }
 }
 
 // db[o] = sum over the batch of dZ[s][o] (dZ bf16 [B][out], out even).  A block of 256 threads owns 128
@@ -780,7 +967,7 @@ int tile_bn(int N, int M, int workers, int sm_count) {
     return wide_tiles >= sm_count ? 256 : 128;
 }
 
-template <bool AMN, bool BMN>
+template <bool BMN>
 int run_tc_major(const dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b, const TcArgs& g, int workers, cudaStream_t s) {
     const int bn = tile_bn(g.N, g.M, workers, h->sm_count);
     const int tiles_n = (g.N + bn - 1) / bn, tiles_m = (g.M + BM - 1) / BM;
@@ -788,15 +975,15 @@ int run_tc_major(const dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b
     const int grid = n_tiles < h->sm_count ? n_tiles : h->sm_count;
     static PerDeviceOnce once;
     const int rc = once.run(h->device, []() -> int {
-        DBW_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<4, 128, 2, AMN, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4, 128)));
-        DBW_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<3, 256, 2, AMN, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(3, 256)));
+        DBW_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<4, 128, 2, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4, 128)));
+        DBW_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<3, 256, 2, BMN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(3, 256)));
         return DBW_OK;
     });
     if (rc) return rc;
     if (bn == 128)
-        gemm_tc_kernel<4, 128, 2, AMN, BMN><<<grid, GEMM_THREADS, gemm_smem(4, 128), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+        gemm_tc_kernel<4, 128, 2, BMN><<<grid, GEMM_THREADS, gemm_smem(4, 128), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
     else
-        gemm_tc_kernel<3, 256, 2, AMN, BMN><<<grid, GEMM_THREADS, gemm_smem(3, 256), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+        gemm_tc_kernel<3, 256, 2, BMN><<<grid, GEMM_THREADS, gemm_smem(3, 256), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
     DBW_LAUNCHED();
     return DBW_OK;
 }
@@ -813,15 +1000,43 @@ cudaEvent_t gemm_event(dbw_handle* h) {
 }
 
 int run_tc(dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b, const TcArgs& g, int workers, cudaStream_t s,
-           bool a_mn = false, bool b_mn = false) {
+           bool b_mn = false) {
     const bool timed = h->profiling && h->prof_gemm_used < 2 * 16 * 4096;
     if (timed) {
         cudaEvent_t e = gemm_event(h);
         if (e) DBW_CUDA(cudaEventRecord(e, s));
     }
-    const int rc = (a_mn && b_mn) ? run_tc_major<true, true>(h, a, b, g, workers, s)
-                   : b_mn         ? run_tc_major<false, true>(h, a, b, g, workers, s)
-                                  : run_tc_major<false, false>(h, a, b, g, workers, s);
+    const int rc = b_mn ? run_tc_major<true>(h, a, b, g, workers, s) : run_tc_major<false>(h, a, b, g, workers, s);
+    if (timed) {
+        cudaEvent_t e = gemm_event(h);
+        if (e) DBW_CUDA(cudaEventRecord(e, s));
+    }
+    return rc;
+}
+
+template <int BN>
+int launch_dw(const dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b, const DwArgs& g, cudaStream_t s) {
+    const int tiles_n = (g.N + BN - 1) / BN, tiles_m = (g.M + BM - 1) / BM;
+    const int n_tiles = tiles_n * tiles_m * h->N;
+    const int grid = n_tiles < h->sm_count ? n_tiles : h->sm_count;
+    static PerDeviceOnce once;
+    const int rc = once.run(h->device, []() -> int {
+        DBW_CUDA(cudaFuncSetAttribute(gemm_dw_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dw_smem(BN)));
+        return DBW_OK;
+    });
+    if (rc) return rc;
+    gemm_dw_kernel<BN><<<grid, GEMM_THREADS, dw_smem(BN), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+    DBW_LAUNCHED();
+    return DBW_OK;
+}
+
+int run_dw(dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b, const DwArgs& g, cudaStream_t s) {
+    const bool timed = h->profiling && h->prof_gemm_used < 2 * 16 * 4096;
+    if (timed) {
+        cudaEvent_t e = gemm_event(h);
+        if (e) DBW_CUDA(cudaEventRecord(e, s));
+    }
+    const int rc = tile_bn(g.N, g.M, h->N, h->sm_count) == 256 ? launch_dw<256>(h, a, b, g, s) : launch_dw<128>(h, a, b, g, s);
     if (timed) {
         cudaEvent_t e = gemm_event(h);
         if (e) DBW_CUDA(cudaEventRecord(e, s));
@@ -854,6 +1069,8 @@ int grad_bf16_alloc(dbw_handle* h) {
     for (int l = 0; l <= L - 2 && ok; ++l) st->Wh[l] = shadow + m.w_off[l];
     ok = ok && balloc(st, &st->dwp, (size_t)4 * N * m.dims[L] * m.dims[L - 1]);
     ok = ok && balloc(st, &st->dzL, NB * m.dims[L]) && balloc(st, &st->loss_s, NB) && balloc(st, &st->ylab, NB);
+    ok = ok && balloc(st, &h->active.list, N) && balloc(st, &h->active.pos, N) && balloc(st, &h->active.slot, (size_t)N * h->plan.stride) &&
+         balloc(st, &h->active.count, 1);
     if (!ok) return DBW_ERR_CUDA;
     for (int l = 0; l <= L - 2; ++l) {
         ok = ok && make_operand_map(&st->fwdA[l], st->A[l], m.dims[l], B, N);
@@ -877,12 +1094,14 @@ int grad_bf16_alloc(dbw_handle* h) {
 void grad_bf16_free(dbw_handle* h) {
     if (!h->bf16) return;
     h->d_shadow = nullptr;
+    h->active = ActiveRows{};
     for (void* p : h->bf16->owned) cudaFree(p);
     delete h->bf16;
     h->bf16 = nullptr;
 }
 
-int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss, cudaStream_t s) {
+int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss, cudaStream_t s,
+                     const StepArgs* step) {
     const dbw_model_desc& m = h->model;
     BF16State* st = h->bf16;
     const int L = m.n_layers, B = m.batch, N = h->N, C = m.dims[L];
@@ -893,15 +1112,13 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     for (int l = 0; l <= L - 2 && !have_shadow; ++l) {
         const int in = m.dims[l], out = m.dims[l + 1];
         cast_tile_kernel<<<dim3((in + 63) / 64, (out + 63) / 64, N), 256, 0, s>>>(
-            out, in, X + m.w_off[l], h->ld, in, nullptr, 0, 0, st->Wh[l], h->ld, h->d_status);
+            out, in, X + m.w_off[l], h->ld, in, nullptr, 0, 0, st->Wh[l], h->ld, nullptr, 0, nullptr, h->d_status);
         DBW_LAUNCHED();
     }
-    // mini-batch gather: A_0 in bf16
+    // mini-batch gather: A_0 in bf16, and the labels
     cast_tile_kernel<<<dim3((m.dims[0] + 63) / 64, (B + 63) / 64, N), 256, 0, s>>>(
         B, m.dims[0], h->feat, (long long)h->S * m.dims[0], m.dims[0], batch_idx, B, h->S, st->A[0], (long long)B * m.dims[0],
-        h->d_status);
-    DBW_LAUNCHED();
-    gather_labels_kernel<<<N, 128, 0, s>>>(B, h->S, C, h->labels, batch_idx, st->ylab, h->d_status);
+        h->labels, C, st->ylab, h->d_status);
     DBW_LAUNCHED();
     // forward through the tensor-core layers
     for (int l = 0; l <= L - 2; ++l) {
@@ -944,22 +1161,29 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         head_backward_kernel<32, 1><<<dim3((K + 63) / 64, N, parts), 64, (size_t)B * 32 * 4, s>>>(
             B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
     DBW_LAUNCHED();
-    // backward through the tensor-core layers
+    // backward through the tensor-core layers; dA_l before dW_l, which may replace the bf16 copy of W_l
+    if (step) DBW_CUDA(cudaStreamWaitEvent(s, step->selected, 0));
     for (int l = L - 2; l >= 0; --l) {
         const int in = m.dims[l], out = m.dims[l + 1];
-        TcArgs w{};
-        w.M = out; w.N = in; w.K = B; w.epi = EPI_DW;
-        w.outf = G + m.w_off[l]; w.outf_z = h->ld; w.outf_pitch = in;
-        w.status = h->d_status;
-        if ((rc = run_tc(h, st->dwA[l], st->dwB[l], w, N, s, true, true))) return rc;
         if (l >= 1) {
             TcArgs a{};
             a.M = B; a.N = in; a.K = out; a.epi = EPI_DA;
             a.out = st->dZ[l]; a.out_z = (long long)B * in; a.out_pitch = in;
             a.mask = st->A[l]; a.mask_z = (long long)B * in; a.mask_pitch = in;
             a.status = h->d_status;
-            if ((rc = run_tc(h, st->daA[l], st->daB[l], a, N, s, false, true))) return rc;
+            if ((rc = run_tc(h, st->daA[l], st->daB[l], a, N, s, true))) return rc;
         }
+        DwArgs w{};
+        w.M = out; w.N = in; w.K = B;
+        w.G = G + m.w_off[l]; w.ld = h->ld;
+        w.status = h->d_status;
+        if (step) {
+            w.X = X + m.w_off[l]; w.Xout = step->X_out + m.w_off[l];
+            w.copy = h->track_params ? st->Wh[l] : nullptr;
+            w.active_pos = h->active.pos; w.active_count = h->active.count; w.step_limit = active_limit(N);
+            w.lr = step->lr; w.lr_pw = step->lr_pw;
+        }
+        if ((rc = run_dw(h, st->dwA[l], st->dwB[l], w, s))) return rc;
     }
     // the reductions over the batch that only the mix needs: bias gradients, last layer's dW and db, losses
     TailArgs t{};

@@ -8,6 +8,9 @@
 // fully staged before any of it is written and panels are disjoint, so X' may overwrite X.
 // G == nullptr in any of the kernels means G = 0 (a consensus-only round): nothing of G is read, 8 bytes
 // per element.
+#include <algorithm>
+#include <utility>
+
 #include "common.cuh"
 #include "round_dev.cuh"
 
@@ -23,8 +26,9 @@ template <int GS>
 __global__ void __launch_bounds__(kMixThreads, 3)
 mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ G, float lr,
                  const float* __restrict__ lr_pw, float* Xout, uint16_t* __restrict__ shadow, MixPlan plan,
-                 int mix_then_correct, int n_panels) {
+                 int mix_then_correct, int n_panels, const int* active_count) {
     extern __shared__ float4 sm[];  // [N][GS]
+    if (active_count && *active_count <= active_limit(N)) return;  // mix_active_kernel's round
     for (int panel = blockIdx.x; panel < n_panels; panel += gridDim.x) {
         mix_panel_body<GS, kMixThreads>(panel, sm, N, ld, X, G, lr, lr_pw, Xout, shadow, plan, mix_then_correct);
         __syncthreads();
@@ -72,6 +76,127 @@ mix_direct_kernel(int N, long long ld, const float* __restrict__ X, const float*
     }
 }
 
+// The mix of a tensor-core round in which at most half of the workers take part.  The dW GEMMs have then finished the
+// weights of the others (x' = x - lr g in their epilogue); what is left is the participants' weights and every worker's
+// biases and last layer.  A panel inside a weight block stages and mixes the participants' rows only, and because those
+// are few in most rounds of the threshold rule (a tenth to a third of the workers on average), several neighbouring
+// panels are staged together, up to half of the buffer with x and the other half with g: copied asynchronously, every
+// load of the panels is in flight at once whatever the registers hold.  A panel that reaches outside the weight blocks
+// is mixed as by mix_panel_kernel, without the stores that are already done.
+// With more participants the round is mix_panel_kernel's: both are launched, and the one whose round it is not leaves at
+// once (about 2 us; as one kernel for both cases the registers of either spilled: 2.01 ms instead of 1.74 for 128 workers
+// x 4.2 million columns with all 8 neighbours kept).
+struct WeightBlocks {
+    int n;                                             // in ascending column order
+    long long lo[DBW_MAX_LAYERS], hi[DBW_MAX_LAYERS];  // column ranges whose non-participants are finished
+    int p0[DBW_MAX_LAYERS], p1[DBW_MAX_LAYERS];        // panels that lie inside them
+    int outside;                                       // panels that do not
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// Bytes behind the staged rows: for every staged row its offset, worker and panel base, and every worker's list position.
+inline size_t active_smem(int N, int gs) { return (size_t)N * gs * 16 + (size_t)N * 14; }
+
+template <int GS>
+__global__ void __launch_bounds__(kMixThreads, 3)
+mix_active_kernel(int N, long long ld, const float* X, const float* __restrict__ G, float lr, const float* __restrict__ lr_pw,
+                  float* Xout, uint16_t* __restrict__ shadow, MixPlan plan, int mix_then_correct, int max_merge,
+                  ActiveRows active, const __grid_constant__ WeightBlocks blocks) {
+    extern __shared__ float4 sm[];  // [N][GS] staged rows, then by staged row v:
+    const int n_act = *active.count;
+    const int half = active_limit(N);
+    if (n_act > half) return;  // mix_panel_kernel's round
+    long long* off = reinterpret_cast<long long*>(sm + (size_t)N * GS);  // its float offset from the panels' first column of row 0
+    uint16_t* worker = reinterpret_cast<uint16_t*>(off + N);             // its worker
+    uint16_t* first = worker + N;                                        // the first staged row of its panel
+    int16_t* pos = reinterpret_cast<int16_t*>(first + N);                // worker -> position among the participants, -1
+    const int merge = n_act > 0 ? min(half / n_act, max_merge) : 1;
+    for (int e = threadIdx.x; e < N; e += kMixThreads) {
+        pos[e] = (int16_t)active.pos[e];
+        if (e < merge * n_act) {
+            const int sub = e / n_act, r = checked(active.list[e - sub * n_act], N, plan.status);
+            off[e] = (long long)r * ld + (long long)sub * (4 * GS);
+            worker[e] = (uint16_t)r;
+            first[e] = (uint16_t)(sub * n_act);
+        }
+    }
+    __syncthreads();
+    constexpr int kGroups = kMixThreads / GS;
+    const int q = threadIdx.x % GS, gid = threadIdx.x / GS;
+    // the panels outside the weight blocks, all rows: the longest work items first
+    int item = blockIdx.x;
+    for (; item < blocks.outside; item += gridDim.x) {
+        int panel = item;
+#pragma unroll
+        for (int l = 0; l < DBW_MAX_LAYERS - 1; ++l)
+            if (l < blocks.n && panel >= blocks.p0[l]) panel += blocks.p1[l] - blocks.p0[l];
+        bool done = false;
+        const long long c = ((long long)panel * GS + q) * 4;
+#pragma unroll
+        for (int l = 0; l < DBW_MAX_LAYERS - 1; ++l) done = done || (l < blocks.n && c >= blocks.lo[l] && c < blocks.hi[l]);
+        mix_panel_body<GS, kMixThreads>(panel, sm, N, ld, X, G, lr, lr_pw, Xout, shadow, plan, mix_then_correct,
+                                        [&](int i) { return !done || pos[i] >= 0; });
+        __syncthreads();
+    }
+    if (n_act == 0) return;
+    // the merged panels of every block
+#pragma unroll 1
+    for (;; item += gridDim.x) {
+        int rest = item - blocks.outside, panel = 0, merged = 0;
+#pragma unroll
+        for (int l = 0; l < DBW_MAX_LAYERS - 1; ++l) {
+            if (l < blocks.n && merged == 0) {
+                const int groups = (blocks.p1[l] - blocks.p0[l] + merge - 1) / merge;
+                if (rest < groups) {
+                    panel = blocks.p0[l] + rest * merge;
+                    merged = min(merge, blocks.p1[l] - panel);
+                }
+                rest -= groups;
+            }
+        }
+        if (merged == 0) break;
+        const int V = merged * n_act;
+        const long long c = ((long long)panel * GS + q) * 4;
+        for (int v = gid; v < V; v += kGroups) {
+            cp_async16(&sm[v * GS + q], X + off[v] + c);
+            cp_async16(&sm[(half + v) * GS + q], G + off[v] + c);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (!mix_then_correct)
+            for (int v = gid; v < V; v += kGroups)  // this thread's own copies
+                sm[v * GS + q] = fma4(-(lr_pw ? lr_pw[worker[v]] : lr), sm[(half + v) * GS + q], sm[v * GS + q]);
+        __syncthreads();
+        for (int v = gid; v < V; v += kGroups) {
+            const int i = worker[v];
+            const float4* rows = sm + (int)first[v] * GS + q;
+            const float ws = plan.w_self[i];
+            const float4 self = sm[v * GS + q];
+            float4 acc = make_float4(ws * self.x, ws * self.y, ws * self.z, ws * self.w);
+            const int cnt = plan.cnt[i];
+            const int4* pj = reinterpret_cast<const int4*>(active.slot + (size_t)i * plan.stride);
+            const float4* pw = reinterpret_cast<const float4*>(plan.w + (size_t)i * plan.stride);
+            for (int k = 0; k < cnt; k += 4) {  // list padding is (own row, weight 0)
+                int4 j = __ldg(pj + (k >> 2));
+                const float4 w = __ldg(pw + (k >> 2));
+                j.x = checked(j.x, n_act, plan.status); j.y = checked(j.y, n_act, plan.status);
+                j.z = checked(j.z, n_act, plan.status); j.w = checked(j.w, n_act, plan.status);
+                acc = fma4(w.x, rows[j.x * GS], acc);
+                acc = fma4(w.y, rows[j.y * GS], acc);
+                acc = fma4(w.z, rows[j.z * GS], acc);
+                acc = fma4(w.w, rows[j.w * GS], acc);
+            }
+            if (mix_then_correct) acc = fma4(-(lr_pw ? lr_pw[i] : lr), sm[(half + v) * GS + q], acc);
+            const long long at = off[v] + c;
+            *reinterpret_cast<float4*>(Xout + at) = acc;
+            if (shadow) *reinterpret_cast<uint2*>(shadow + at) = pack_bf16x4_rn(acc.x, acc.y, acc.z, acc.w);
+        }
+        __syncthreads();
+    }
+}
+
 int auto_group_size(const dbw_handle* h) {
     if (h->mix_panel_cols < 0) return 0;  // direct kernel forced
     if (h->mix_panel_cols >= 1 && h->mix_panel_cols <= 3) return 0;  // staged / tensor-core kernels forced (handled by the caller)
@@ -88,7 +213,7 @@ int auto_group_size(const dbw_handle* h) {
 
 template <int GS>
 int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
-                 uint16_t* shadow, cudaStream_t s) {
+                 uint16_t* shadow, cudaStream_t s, const int* active_count = nullptr) {
     const size_t smem = (size_t)h->N * GS * 16;
     static PerDeviceOnce once;
     const int rc = once.run(h->device, [h]() -> int {
@@ -103,7 +228,47 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
     const int grid = n_panels < per_sm * h->sm_count ? n_panels : per_sm * h->sm_count;
     mix_panel_kernel<GS><<<grid, kMixThreads, smem, s>>>(h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
                                                         (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0,
-                                                        n_panels);
+                                                        n_panels, active_count);
+    DBW_LAUNCHED();
+    return DBW_OK;
+}
+
+template <int GS>
+int launch_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow,
+                  cudaStream_t s) {
+    const size_t smem = active_smem(h->N, GS);
+    int rc = launch_panel<GS>(h, X, G, lr, lr_pw, X_out, shadow, s, h->active.count);
+    if (rc) return rc;
+    static PerDeviceOnce once;
+    rc = once.run(h->device, [h]() -> int {
+        DBW_CUDA(cudaFuncSetAttribute(mix_active_kernel<GS>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin));
+        return DBW_OK;
+    });
+    if (rc) return rc;
+    int per_sm = 0;
+    DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_active_kernel<GS>, kMixThreads, smem));
+    if (per_sm < 1) return DBW_ERR_BAD_SHAPE;
+    const int n_panels = (int)((h->ld + 4 * GS - 1) / (4 * GS));
+    WeightBlocks blocks{};
+    const dbw_model_desc& m = h->model;
+    blocks.n = m.n_layers - 1;
+    std::pair<long long, long long> range[DBW_MAX_LAYERS];
+    for (int l = 0; l < blocks.n; ++l) range[l] = {m.w_off[l], m.w_off[l] + (long long)m.dims[l] * m.dims[l + 1]};
+    std::sort(range, range + blocks.n);
+    blocks.outside = n_panels;
+    for (int l = 0; l < blocks.n; ++l) {
+        blocks.lo[l] = range[l].first;
+        blocks.hi[l] = range[l].second;
+        blocks.p0[l] = (int)((blocks.lo[l] + 4 * GS - 1) / (4 * GS));
+        blocks.p1[l] = std::max(blocks.p0[l], (int)(blocks.hi[l] / (4 * GS)));
+        blocks.outside -= blocks.p1[l] - blocks.p0[l];
+    }
+    const int slots = per_sm * h->sm_count;
+    // panels staged together: at least two groups for every resident block, so that the blocks stay evenly loaded
+    const int max_merge = std::min(32, std::max(1, n_panels / (2 * slots)));
+    mix_active_kernel<GS><<<n_panels < slots ? n_panels : slots, kMixThreads, smem, s>>>(
+        h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, max_merge,
+        h->active, blocks);
     DBW_LAUNCHED();
     return DBW_OK;
 }
@@ -136,6 +301,28 @@ bool mix_panel_fits(const dbw_handle* h) {
     return use_tc(h) ? mix_tc_in_place_ok(h) : (use_staged(h) || auto_group_size(h) != 0);
 }
 int mix_kernel_kind(const dbw_handle* h) { return use_sp(h) ? 4 : use_tc(h) ? 3 : use_staged(h) ? 2 : (auto_group_size(h) != 0 ? 1 : 0); }
+
+// With tensor-core layers and a panel of all workers in shared memory the dW GEMMs can take the step of the workers that
+// take no part in the round, whose weights then cross HBM once (read x, write x' and its bf16 copy: 10 bytes an element)
+// instead of as a gradient written, read back with x and mixed with nothing (18 bytes).
+bool mix_active_usable(const dbw_handle* h) {
+    return h->active.list && h->has_model && h->model.n_layers >= 2 && mix_kernel_kind(h) == 1 &&
+           active_smem(h->N, auto_group_size(h)) <= (size_t)h->smem_optin;
+}
+
+int launch_mix_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, cudaStream_t s) {
+    uint16_t* shadow = (h->track_params && h->d_shadow) ? h->d_shadow : nullptr;
+    h->shadow_valid = shadow != nullptr;
+    h->shadow_of = X_out;
+    switch (auto_group_size(h)) {
+        case 64: return launch_active<64>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        case 32: return launch_active<32>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        case 16: return launch_active<16>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        case 8: return launch_active<8>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        case 4: return launch_active<4>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        default: return DBW_ERR_BAD_SHAPE;
+    }
+}
 
 int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
                cudaStream_t s) {

@@ -587,10 +587,14 @@ __device__ __forceinline__ float4 fma4(float w, float4 v, float4 a) {
 // set): the panel of X (and G) is staged in shared memory sm [N][GS] as x - lr*g (or x), then every output
 // row is the weighted sum of staged rows in plan order (self first, then the kept neighbours in CSR order).
 // The caller puts a block barrier after it before the next panel.  G == nullptr: G = 0.
-template <int GS, int THREADS, bool NC = true>
+// `mine(i)`: whether row i is wanted here, as a staged row and as an output (all of them by default).
+struct AllRows {
+    __device__ __forceinline__ bool operator()(int) const { return true; }
+};
+template <int GS, int THREADS, bool NC = true, class Mine = AllRows>
 __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, long long ld, const float* X, const float* G,
                                                float lr, const float* __restrict__ lr_pw, float* Xout, uint16_t* __restrict__ shadow,
-                                               const MixPlan& plan, int mix_then_correct) {
+                                               const MixPlan& plan, int mix_then_correct, Mine mine = Mine()) {
     const int tid = threadIdx.x;
     const int q = tid % GS;
     const int gid = tid / GS;
@@ -603,7 +607,7 @@ __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, lon
         const int r = idx / GS;
         const long long c = col0 + 4 * (idx % GS);
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < ld) {
+        if (c < ld && mine(r)) {
             v = ldg4(X + (size_t)r * ld + c);
             if (G && !mix_then_correct) {
                 const float4 g = load_g<NC>(reinterpret_cast<const float4*>(G + (size_t)r * ld + c));
@@ -633,7 +637,7 @@ __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, lon
             acc = fma4(w.z, sm[j.z * GS + q], acc);
             acc = fma4(w.w, sm[j.w * GS + q], acc);
         }
-        if (c < ld) {
+        if (c < ld && mine(i)) {
             if (G && mix_then_correct) {
                 const float4 g = load_g<NC>(reinterpret_cast<const float4*>(G + (size_t)i * ld + c));
                 acc = fma4(-(lr_pw ? lr_pw[i] : lr), g, acc);

@@ -11,6 +11,39 @@ constexpr int kWarpsPerBlock = 4;
 
 using namespace dev;
 
+// The participants of the round in ascending order, by the block that has seen every worker's selection (before the
+// "waited for" flags are cleared).  All threads of the block call it.
+__device__ __forceinline__ void list_active_rows(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ b, const uint32_t* waited,
+                                                 const MixPlan& plan, const ActiveRows& active) {
+    __shared__ int per_warp[kWarpsPerBlock];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int listed = 0;
+    for (int base = 0; base < N; base += kWarpsPerBlock * 32) {
+        const int w = base + threadIdx.x;
+        bool part = false;
+        if (w < N) part = rowptr[w + 1] - rowptr[w] - max(b[w], 0) >= 1 || __ldcg(&waited[w]) != 0u;
+        const unsigned m = __ballot_sync(0xffffffffu, part);
+        if (lane == 0) per_warp[warp] = __popc(m);
+        __syncthreads();
+        int before = listed;
+#pragma unroll
+        for (int k = 0; k < kWarpsPerBlock; ++k) {
+            if (k < warp) before += per_warp[k];
+            listed += per_warp[k];
+        }
+        const int at = before + __popc(m & ((1u << lane) - 1u));
+        if (w < N) active.pos[w] = part ? at : -1;
+        if (part) active.list[at] = w;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *active.count = listed;
+    if (listed > active_limit(N)) return;
+    for (int e = threadIdx.x; e < listed * plan.stride; e += kWarpsPerBlock * 32) {
+        const size_t at = (size_t)active.list[e / plan.stride] * plan.stride + e % plan.stride;
+        active.slot[at] = active.pos[checked(__ldcg(&plan.idx[at]), N, plan.status)];
+    }
+}
+
 // Selection: one warp per worker (dev::select_worker); the last block to finish computes the per-worker and
 // per-round times, which need to know who is waited for by whom.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
@@ -19,7 +52,7 @@ select_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restri
               uint8_t* __restrict__ kept,
               double* __restrict__ T_nbr_ws, double* T_nbr_out, double* T_worker, double* T_round,
               uint32_t* waited, uint32_t* ticket, uint32_t* status, MixPlan plan, int build_plan,
-              int uniform) {
+              int uniform, ActiveRows active) {
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     if (i < N) select_worker(i, lane, rowptr, col, t, t_edge, b, kept, T_nbr_ws, waited, status, plan, build_plan, uniform);
@@ -33,6 +66,7 @@ select_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restri
     __syncthreads();
     if (!is_last) return;
     __threadfence();
+    if (active.list) list_active_rows(N, rowptr, b, waited, plan, active);
     double tr = round_times_part(N, rowptr, t, b, T_nbr_ws, T_nbr_out, T_worker, waited, status);
     tr = warp_max(tr);
     if (lane == 0) red[threadIdx.x >> 5] = tr;
@@ -85,11 +119,12 @@ plan_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict
 }  // namespace
 
 int launch_select(dbw_handle* h, const double* t, const int32_t* b, uint8_t* kept, double* T_worker,
-                  double* T_nbr, double* T_round, bool build_plan, cudaStream_t s) {
+                  double* T_nbr, double* T_round, bool build_plan, cudaStream_t s, bool list_active) {
     const int blocks = (h->N + kWarpsPerBlock - 1) / kWarpsPerBlock;
     select_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(
         h->N, h->d_rowptr, h->d_col, t, h->t_edge, b, kept, h->d_Tnbr_ws, T_nbr, T_worker, T_round, h->d_waited,
-        h->d_ticket, h->d_status, h->plan, build_plan ? 1 : 0, (h->flags & DBW_WEIGHT_UNIFORM) ? 1 : 0);
+        h->d_ticket, h->d_status, h->plan, build_plan ? 1 : 0, (h->flags & DBW_WEIGHT_UNIFORM) ? 1 : 0,
+        list_active ? h->active : ActiveRows{});
     DBW_LAUNCHED();
     return DBW_OK;
 }
@@ -158,7 +193,7 @@ extern "C" int dbw_select_static(int32_t N, const int32_t* rowptr, const int32_t
     dbw::MixPlan no_plan{};
     no_plan.n = N;  // only the bounds-checked build looks at it: this entry point's CSR is not validated on the host
     dbw::select_kernel<<<blocks, dbw::kWarpsPerBlock * 32, 0, s>>>(N, rowptr, col, t, nullptr, b, kept, tnbr, T_nbr, T_worker,
-                                                                   T_round, waited, ticket, status, no_plan, 0, 0);
+                                                                   T_round, waited, ticket, status, no_plan, 0, 0, dbw::ActiveRows{});
     DBW_LAUNCHED();
     if (status_out) DBW_CUDA(cudaMemcpyAsync(status_out, status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
     return DBW_OK;

@@ -664,3 +664,58 @@ def test_selection_with_per_link_times_bit_exact(name):
         assert np.array_equal(kept0, orc.select_fastest(rowptr, col, t, b))
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("dims,batch,n", [([72, 200, 136, 10], 40, 10),      # 128-wide dW tiles, ragged on every side
+                                          ([328, 264, 10], 24, 40),          # 256-wide dW tiles, ragged
+                                          ([256, 128, 64, 10], 64, 150)])    # whole tiles; panels of fewer columns
+@pytest.mark.parametrize("order", ["local_then_mix", "mix_then_correct"])
+def test_round_with_few_participants_gives_the_bits_of_its_steps(dims, batch, n, order):
+    """In a tensor-core round the dW GEMMs take the SGD step of the workers that take no part and the mix works on the
+    others.  From no participant to all of them, around the count at which the round is mixed as a whole, in place and
+    not, with and without parameter tracking, the round gives the bits of its steps called one by one (dbw_grad,
+    dbw_select, dbw_mix), which the oracle tests pin."""
+    p = _dbw()
+    rowptr, col = wl.ring(n)
+    deg = np.diff(rowptr)
+    flags = p.GEMM_BF16 | (p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m, flags=flags)
+    rng = np.random.default_rng(5)
+    S = 2 * batch
+    feat = dev(rng.standard_normal((n, S, dims[0]), dtype=np.float32))
+    labels = dev(rng.integers(0, dims[-1], size=(n, S)).astype(np.int32))
+    h.set_dataset(feat, labels, S)
+    X0 = np.zeros((n, m.ld), dtype=np.float32)
+    X0[:] = m.pack(0.1 * rng.standard_normal((n, m.d)).astype(np.float32))
+    idx = dev(rng.integers(0, S, size=(n, batch)).astype(np.int32))
+    lr_pw = dev(rng.uniform(0.01, 0.1, size=n).astype(np.float32))
+    kept, kept2 = (torch.zeros(len(col), dtype=torch.uint8, device="cuda") for _ in range(2))
+    G = torch.zeros(n, m.ld, device="cuda")
+    for k in (0, 2, n // 2, n // 2 + 1, n):
+        inside = np.arange(n) < k
+        t = dev(np.where(inside, 1.0, 9.0) + rng.random(n))
+        mates = np.array([inside[col[rowptr[i]:rowptr[i + 1]]].sum() for i in range(n)])
+        b = dev(np.where(inside, deg - mates, deg).astype(np.int32))
+        X = dev(X0)
+        h.set_param_tracking(False)
+        ref = torch.empty_like(X)
+        h.grad(X, idx, G)
+        h.select(t, b, kept)
+        h.mix(X, G, kept, b, 0.05, ref, lr_per_worker=lr_pw)
+        for track in (False, True):
+            h.set_param_tracking(track)
+            out = torch.full_like(X, float("nan"))
+            h.round(X, t, b, 0.05, out, kept2, batch_idx=idx, lr_per_worker=lr_pw)
+            assert torch.equal(out, ref) and torch.equal(kept, kept2), (k, track)
+            Y = X.clone()
+            h.round(Y, t, b, 0.05, Y, kept2, batch_idx=idx, lr_per_worker=lr_pw)
+            assert torch.equal(Y, ref), (k, track)
+        # the tracked bf16 copy is that of a cast after the fact: the next gradients agree
+        G2 = torch.zeros_like(G)
+        h.grad(Y, idx, G2)
+        h.set_param_tracking(False)
+        h.grad(Y, idx, G)
+        assert torch.equal(G, G2), k
+    assert h.status() == 0
+    h.close()
