@@ -140,6 +140,7 @@ struct dbw_handle {
     float* d_act[DBW_MAX_LAYERS + 1] = {};  // fp32 path: A_0 (gathered batch) .. A_L (logits), [N][B][dims[l]]
     float* d_dz[DBW_MAX_LAYERS + 1] = {};   // fp32 path: dZ_l for l = 1..L, [N][B][dims[l]]
     int32_t* d_ylab = nullptr;              // [N][B] gathered labels
+    float* d_head_part = nullptr;           // fp32 path, batches of several parts: [parts][N][fp32_head_partial]
     float* d_G = nullptr;                   // [N][ld] gradient workspace of dbw_round (lazy)
     dbw::BF16State* bf16 = nullptr;
     // bf16 shadow of the parameter matrix, [N][ld], same layout as X (tensor-core path only).  The
@@ -229,15 +230,26 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
 int launch_update_backups(dbw_handle* h, const double* t, int32_t* b_out, double* theta_out, cudaStream_t s);
 
 // grad_fp32.cu
-// fp32 gradient path: shared memory of the last layer's backward step (the worker's dZ and its row offsets),
-// and whether the last layer can take the small-output path (at most 32 classes, 16-byte rows).
-inline size_t fp32_head_smem_bytes(int B, int C) { return (size_t)((B * C + 1) & ~1) * 4 + (size_t)B * 8; }
+// fp32 gradient path: the last layer's backward step works on parts of at most kHeadPart samples (a worker's dZ of a part,
+// its row offsets and losses lie in shared memory); more than one part leave partial sums that are added in a fixed order.
+// Bound by the latency of a block's serial passes, so the part length sets the time: 256 samples give ten workers x batch 1024
+// x 256 features 80 blocks and 45 us (with the whole batch in one block the layer fell back to GEMMs, a loss kernel of a block
+// per worker and a column sum: 230 us).
+constexpr int kHeadPart = 256;
+__host__ __device__ inline int fp32_head_parts(int B) { return (B + kHeadPart - 1) / kHeadPart; }
+inline size_t fp32_head_smem_bytes(int B, int C) {
+    const int s = B < kHeadPart ? B : kHeadPart;
+    return (size_t)((s * C + 1) & ~1) * 4 + (size_t)s * 12;
+}
+// floats of one worker's partial sums: dW, db, the bias gradient of the layer before, the loss
+__host__ __device__ inline long long fp32_head_partial(int in, int C) { return (long long)C * in + (C + in + 1 + 3) / 4 * 4; }
+// Whether the last layer can take the small-output path (at most 32 classes, 16-byte rows).
 inline bool fp32_head_usable(const dbw_handle* h) {
     const dbw_model_desc& m = h->model;
     const int L = m.n_layers;
     if (L < 1) return false;
     return m.dims[L] <= 32 && (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 &&
-           ((uintptr_t)h->feat & 15) == 0 && fp32_head_smem_bytes(m.batch, m.dims[L]) <= 32768;
+           ((uintptr_t)h->feat & 15) == 0;
 }
 int grad_fp32_alloc(dbw_handle* h);
 void grad_fp32_free(dbw_handle* h);

@@ -45,7 +45,8 @@ __global__ void bias_grad_kernel(int B, int out_dim, const float* __restrict__ d
 // 4 x 4 layout of gemm_simt_kernel needs the same four wavefronts for 16.  Global loads and stores are
 // 128-bit along the operand's unit-stride dimension.  Every output element is summed over k in ascending
 // order, exactly as in gemm_simt_kernel: the two give the same bits.
-template <int WM, int RM>
+// SUMS: the blocks of the first columns also add every row of A over k (g.rowsum): the bias gradient of a dW GEMM.
+template <int WM, int RM, bool SUMS>
 __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
     constexpr int BM = 2 * RM * WM, BN = 64, TK = 16, THREADS = 32 * WM;
     constexpr int PA = BM * TK / 4 / THREADS, PB = BN * TK / 4 / THREADS;  // float4 per thread and k-step
@@ -58,6 +59,8 @@ __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
     const int mw = warp * 2 * RM + (lane >> 4) * RM, nw = (lane & 15) * 4;
     const bool a_k_fast = g.sAk == 1, b_k_fast = g.sBk == 1;
     float acc[RM][4] = {};
+    const bool sums = SUMS && n0 == 0 && tid < BM;
+    float rowsum = 0.f;
     float4 pa[PA], pb[PB];
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     auto fetch = [&](int k0) {
@@ -123,8 +126,13 @@ __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
+        if (SUMS && sums) {
+#pragma unroll
+            for (int kk = 0; kk < TK; ++kk) rowsum += As[kk][tid];  // zero past the end
+        }
         __syncthreads();
     }
+    if (SUMS && sums && m0 + tid < g.M) g.rowsum[(size_t)z * g.sRz + m0 + tid] = rowsum;
     float* C = g.C + (size_t)z * g.sCz;
     const float* bias = g.bias ? g.bias + (size_t)z * g.sBiasz : nullptr;
     const float* mask = g.mask ? g.mask + (size_t)z * g.sMz : nullptr;
@@ -183,12 +191,39 @@ template <int CP>
 __global__ void __launch_bounds__(256)
 last_layer_backward_kernel(int B, int in, int C, HeadRows rows, const float* __restrict__ dz, const float* __restrict__ loss_s,
                            const float* __restrict__ X, float* __restrict__ G, long long ld, long long w_off, long long b_off,
-                           float* __restrict__ loss, float* __restrict__ dz_prev, long long b_off_prev, uint32_t* status) {
+                           float* __restrict__ loss, float* __restrict__ dz_prev, long long b_off_prev, float* __restrict__ partial, uint32_t* status) {
     extern __shared__ __align__(16) float head_smem[];
     const int i = blockIdx.y, k_lo = blockIdx.x * kHeadChunk4;
     const int k_hi = min(in >> 2, k_lo + kHeadChunk4);
-    head_backward_part<CP, true>(i, k_lo, k_hi, B, in, C, rows, dz, loss_s, X + (size_t)i * ld + w_off, G + (size_t)i * ld + w_off,
-                                 G + (size_t)i * ld + b_off, loss, dz_prev, G + (size_t)i * ld + b_off_prev, head_smem, status);
+    const int s_lo = blockIdx.z * kHeadPart, s_hi = min(B, s_lo + kHeadPart);
+    float *Gw = G + (size_t)i * ld + w_off, *Gb = G + (size_t)i * ld + b_off, *Gp = G + (size_t)i * ld + b_off_prev, *li = loss ? loss + i : nullptr;
+    float scale = 1.0f / (float)B;
+    if (gridDim.z > 1) {
+        Gw = partial + ((size_t)blockIdx.z * gridDim.y + i) * fp32_head_partial(in, C);
+        Gb = Gw + (size_t)C * in;
+        Gp = Gb + C;
+        li = Gp + in;
+        scale = 1.f;
+    }
+    head_backward_part<CP, true>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, C, rows, dz, loss_s, X + (size_t)i * ld + w_off, Gw, Gb, li, dz_prev, Gp,
+                                 head_smem, status);
+}
+
+__global__ void __launch_bounds__(256)
+last_layer_add_parts_kernel(int parts, int N, int B, int in, int C, const float* __restrict__ partial, float* __restrict__ G, long long ld, long long w_off,
+                            long long b_off, long long b_off_prev, float* __restrict__ loss) {
+    const int i = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
+    float* Gi = G + (size_t)i * ld;
+    if (e <= C * in + C + in) head_add_parts(i, e, parts, N, B, in, C, partial, Gi + w_off, Gi + b_off, b_off_prev >= 0 ? Gi + b_off_prev : nullptr, loss ? loss + i : nullptr);
+}
+
+template <int WM, int RM>
+void launch_gemm_vec(const GemmArgs& g, int batch, cudaStream_t s) {
+    const dim3 grid((g.N + 63) / 64, (g.M + 2 * RM * WM - 1) / (2 * RM * WM), batch);
+    if (g.rowsum)
+        gemm_vec_kernel<WM, RM, true><<<grid, 32 * WM, 0, s>>>(g);
+    else
+        gemm_vec_kernel<WM, RM, false><<<grid, 32 * WM, 0, s>>>(g);
 }
 
 int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
@@ -198,11 +233,11 @@ int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
         const long long t64 = (long long)((g.N + 63) / 64) * ((g.M + 63) / 64) * batch;
         const long long t32 = (long long)((g.N + 63) / 64) * ((g.M + 31) / 32) * batch;
         if (t64 >= 2LL * sm_count)
-            gemm_vec_kernel<4, 8><<<dim3((g.N + 63) / 64, (g.M + 63) / 64, batch), 128, 0, s>>>(g);
+            launch_gemm_vec<4, 8>(g, batch, s);
         else if (t32 >= sm_count)
-            gemm_vec_kernel<4, 4><<<dim3((g.N + 63) / 64, (g.M + 31) / 32, batch), 128, 0, s>>>(g);
+            launch_gemm_vec<4, 4>(g, batch, s);
         else
-            gemm_vec_kernel<2, 4><<<dim3((g.N + 63) / 64, (g.M + 15) / 16, batch), 64, 0, s>>>(g);
+            launch_gemm_vec<2, 4>(g, batch, s);
         DBW_LAUNCHED();
         return DBW_OK;
     }
@@ -232,6 +267,9 @@ int grad_fp32_alloc(dbw_handle* h) {
         if (l >= 1) DBW_CUDA(cudaMalloc(&h->d_dz[l], NB * m.dims[l] * sizeof(float)));
     }
     DBW_CUDA(cudaMalloc(&h->d_ylab, NB * sizeof(int32_t)));
+    const int parts = fp32_head_parts(m.batch);
+    if (parts > 1 && m.dims[m.n_layers] <= 32)
+        DBW_CUDA(cudaMalloc(&h->d_head_part, (size_t)parts * h->N * fp32_head_partial(m.dims[m.n_layers - 1], m.dims[m.n_layers]) * sizeof(float)));
     return DBW_OK;
 }
 
@@ -243,6 +281,8 @@ void grad_fp32_free(dbw_handle* h) {
     }
     if (h->d_ylab) cudaFree(h->d_ylab);
     h->d_ylab = nullptr;
+    if (h->d_head_part) cudaFree(h->d_head_part);
+    h->d_head_part = nullptr;
 }
 
 int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss,
@@ -280,22 +320,29 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         }
         float* loss_s = h->d_act[L];  // [N][B] of the logits' buffer: the logits themselves are never stored
         float* dz_prev = L > 1 ? h->d_dz[L - 1] : nullptr;
-        const dim3 bgrid(((in >> 2) + kHeadChunk4 - 1) / kHeadChunk4, N);
+        const int parts = fp32_head_parts(B);
+        const dim3 bgrid(((in >> 2) + kHeadChunk4 - 1) / kHeadChunk4, N, parts);
+        const long long b_prev = L > 1 ? m.b_off[L - 2] : -1;
         const size_t smem = fp32_head_smem_bytes(B, C);
         if (C <= 16) {
             last_layer_forward_kernel<16><<<(N * B + 7) / 8, 256, 0, s>>>(N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                           h->d_dz[L], loss_s, h->d_status);
             DBW_LAUNCHED();
             last_layer_backward_kernel<16><<<bgrid, 256, smem, s>>>(B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
-                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? m.b_off[L - 2] : 0, h->d_status);
+                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
         } else {
             last_layer_forward_kernel<32><<<(N * B + 7) / 8, 256, 0, s>>>(N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                           h->d_dz[L], loss_s, h->d_status);
             DBW_LAUNCHED();
             last_layer_backward_kernel<32><<<bgrid, 256, smem, s>>>(B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
-                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? m.b_off[L - 2] : 0, h->d_status);
+                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
         }
         DBW_LAUNCHED();
+        if (parts > 1) {
+            last_layer_add_parts_kernel<<<dim3((C * in + C + in + 256) / 256, N), 256, 0, s>>>(parts, N, B, in, C, h->d_head_part, G, h->ld, m.w_off[L - 1],
+                                                                                            m.b_off[L - 1], b_prev, loss);
+            DBW_LAUNCHED();
+        }
     } else {
         softmax_ce_kernel<<<N, 256, 0, s>>>(B, m.dims[L], h->d_act[L], h->d_ylab, h->d_dz[L], loss, G, h->ld, m.b_off[L - 1]);
         DBW_LAUNCHED();
@@ -308,8 +355,13 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.B = h->d_act[l]; g.sBz = (long long)B * in; g.sBn = 1; g.sBk = in;
         g.C = G + m.w_off[l]; g.sCz = h->ld; g.sCm = in;
         g.M = out; g.N = in; g.K = B;
+        const bool needs_db = l < L - 1 && !(head && l == L - 2), db_here = needs_db && gemm_vec_ok(g);
+        if (db_here) {  // the sums of dZ's columns come with the GEMM that reads them
+            g.rowsum = G + m.b_off[l];
+            g.sRz = h->ld;
+        }
         if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
-        if (l < L - 1 && !(head && l == L - 2)) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
+        if (needs_db && !db_here) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
             bias_grad_kernel<<<dim3((out + 127) / 128, N), 128, 0, s>>>(B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
             DBW_LAUNCHED();
         }

@@ -54,6 +54,8 @@ struct GemmArgs {
     long long sMz, sMm;
     int M, N, K;
     int relu;
+    float* rowsum;  // nullable (gemm_vec_kernel only): sum over k of A(m, k), in ascending k
+    long long sRz;
 };
 
 
@@ -347,29 +349,38 @@ __device__ __forceinline__ void head_forward_sample(int i, int s, int B, int in,
 //   dW[c][f] = sum_s dZ[s][c] a[s][f]: each lane adds its samples in ascending order, a butterfly adds the lanes;
 //   with dz_prev also dZ of the layer before, (sum_c dZ[s][c] W[c][f]) [a[s][f] > 0], classes in ascending order,
 //   and that layer's bias gradient (the sum of its dZ over the samples) into Gb_prev.
-// The block that owns the first features also adds the bias gradient and the worker's mean loss, in sample
-// order.  smem: B * C floats + B 64-bit offsets.  Ends with a block barrier (shared memory free again).
+// The block that owns the first features also adds the bias gradient and the worker's loss, in sample order.
+// Only samples [s_lo, s_hi): all of them, with `scale` = 1 / B for the mean loss, or one part of a large batch, whose sums
+// go to partial buffers (scale 1) and are added by head_add_parts.
+// smem: (s_hi - s_lo) * C floats + as many 64-bit offsets + as many floats.  Ends with a block barrier (shared memory free again).
 constexpr int kHeadChunk4 = 32;
 template <int CP, bool NC>
-__device__ __forceinline__ void head_backward_part(int i, int k_lo, int k_hi, int B, int in, int C, const HeadRows& rows,
+__device__ __forceinline__ void head_backward_part(int i, int s_lo, int s_hi, float scale, int k_lo, int k_hi, int B, int in, int C, const HeadRows& rows,
                                                    const float* dz, const float* loss_s, const float* W, float* Gw, float* Gb,
                                                    float* loss, float* dz_prev, float* Gb_prev, float* smem, uint32_t* status) {
+    const int S = s_hi - s_lo;
     float* dzs = smem;
-    long long* rowoff = reinterpret_cast<long long*>(smem + ((B * C + 1) & ~1));
-    for (int e = threadIdx.x; e < B * C; e += blockDim.x) dzs[e] = dz[(size_t)i * B * C + e];
+    long long* rowoff = reinterpret_cast<long long*>(smem + ((S * C + 1) & ~1));
+    float* losses = reinterpret_cast<float*>(rowoff + S);
+    for (int e = threadIdx.x; e < S * C; e += blockDim.x) dzs[e] = dz[((size_t)i * B + s_lo) * C + e];
     const float* base = rows.act ? rows.act : rows.feat;
-    for (int s = threadIdx.x; s < B; s += blockDim.x) rowoff[s] = head_row<NC>(rows, i, s, B, in, C, status, nullptr) - base;
+    for (int s = threadIdx.x; s < S; s += blockDim.x) {
+        rowoff[s] = head_row<NC>(rows, i, s_lo + s, B, in, C, status, nullptr) - base;
+        if (k_lo == 0) losses[s] = loss_s[(size_t)i * B + s_lo + s];
+    }
     __syncthreads();
     if (k_lo == 0) {
         if ((int)threadIdx.x < C) {
             float t = 0.f;
-            for (int s = 0; s < B; ++s) t += dzs[s * C + threadIdx.x];
+#pragma unroll 8
+            for (int s = 0; s < S; ++s) t += dzs[s * C + threadIdx.x];
             Gb[threadIdx.x] = t;
         }
         if (threadIdx.x == 32 && loss) {
             float t = 0.f;
-            for (int s = 0; s < B; ++s) t += loss_s[(size_t)i * B + s];
-            loss[i] = t * (1.0f / (float)B);
+#pragma unroll 8
+            for (int s = 0; s < S; ++s) t += losses[s];
+            *loss = t * scale;
         }
     }
     const int lane = threadIdx.x & 31, slice = lane & 7;
@@ -379,7 +390,7 @@ __device__ __forceinline__ void head_backward_part(int i, int k_lo, int k_hi, in
 #pragma unroll
         for (int c = 0; c < CP; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-        for (int s = slice; s < B; s += 8) {
+        for (int s = slice; s < S; s += 8) {
             const float4 a = *(reinterpret_cast<const float4*>(base + rowoff[s]) + k);
 #pragma unroll
             for (int c = 0; c < CP; ++c) {
@@ -408,7 +419,7 @@ __device__ __forceinline__ void head_backward_part(int i, int k_lo, int k_hi, in
                 if (c < C) acc[c] = load_g<NC>(reinterpret_cast<const float4*>(W + (size_t)c * in) + k);
             float4 db = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-            for (int s = slice; s < B; s += 8) {
+            for (int s = slice; s < S; s += 8) {
                 const float4 a = *(reinterpret_cast<const float4*>(base + rowoff[s]) + k);
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -421,7 +432,7 @@ __device__ __forceinline__ void head_backward_part(int i, int k_lo, int k_hi, in
                 }
                 v.x = a.x > 0.f ? v.x : 0.f; v.y = a.y > 0.f ? v.y : 0.f;
                 v.z = a.z > 0.f ? v.z : 0.f; v.w = a.w > 0.f ? v.w : 0.f;
-                reinterpret_cast<float4*>(dz_prev + ((size_t)i * B + s) * in)[k] = v;
+                reinterpret_cast<float4*>(dz_prev + ((size_t)i * B + s_lo + s) * in)[k] = v;
                 db.x += v.x; db.y += v.y; db.z += v.z; db.w += v.w;
             }
             // bias gradient of the layer before: this lane's samples in ascending order, then the eight lanes
@@ -436,6 +447,18 @@ __device__ __forceinline__ void head_backward_part(int i, int k_lo, int k_hi, in
         }
     }
     __syncthreads();
+}
+
+// Sum e of worker i's last-layer results from the parts of a large batch, in part order.
+__device__ __forceinline__ void head_add_parts(int i, int e, int parts, int N, int B, int in, int C, const float* partial, float* Gw, float* Gb,
+                                               float* Gb_prev, float* loss) {
+    const long long Q = fp32_head_partial(in, C);
+    float t = 0.f;
+    for (int p = 0; p < parts; ++p) t += partial[((size_t)p * N + i) * Q + e];
+    if (e < C * in) Gw[e] = t;
+    else if (e < C * in + C) Gb[e - C * in] = t;
+    else if (e < C * in + C + in) { if (Gb_prev) Gb_prev[e - C * in - C] = t; }
+    else if (loss) *loss = t * (1.0f / (float)B);
 }
 
 // ------------------------------------------------------------------ selection, weights, times

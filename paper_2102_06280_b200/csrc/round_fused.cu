@@ -69,6 +69,7 @@ struct FusedArgs {
     const float* lr_pw;
     float* loss;
     signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];
+    float* head_part;
     int head;  // the last layer takes the small-output steps (at most 32 classes)
 };
 
@@ -168,18 +169,37 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         // ---- last layer backward: dW_L, db_L, the loss, dZ_{L-1} ----
         const int in = a.dims[L - 1], in4 = in >> 2;
         const int chunks = (in4 + kHeadChunk4 - 1) / kHeadChunk4;
-        for (int item = blockIdx.x; item < N * chunks; item += gridDim.x) {
-            const int i = item / chunks, k_lo = (item % chunks) * kHeadChunk4;
-            const int k_hi = min(in4, k_lo + kHeadChunk4);
+        const int parts = fp32_head_parts(B);
+        const long long b_prev = L > 1 ? a.b_off[L - 2] : 0;
+        for (int item = blockIdx.x; item < N * chunks * parts; item += gridDim.x) {
+            const int i = item / chunks % N, part = item / (chunks * N), k_lo = (item % chunks) * kHeadChunk4;
+            const int k_hi = min(in4, k_lo + kHeadChunk4), s_lo = part * kHeadPart, s_hi = min(B, s_lo + kHeadPart);
             const float* Xi = a.X + (size_t)i * a.ld;
             float* Gi = a.G + (size_t)i * a.ld;
+            float *Gw = Gi + a.w_off[L - 1], *Gb = Gi + a.b_off[L - 1], *Gp = Gi + b_prev, *li = a.loss ? a.loss + i : nullptr;
+            float scale = 1.0f / (float)B;
+            if (parts > 1) {
+                Gw = a.head_part + ((size_t)part * N + i) * fp32_head_partial(in, a.C);
+                Gb = Gw + (size_t)a.C * in;
+                Gp = Gb + a.C;
+                li = Gp + in;
+                scale = 1.f;
+            }
             float* dz_prev = L > 1 ? a.dz[L - 1] : nullptr;
             if (a.C <= 16)
-                head_backward_part<16, false>(i, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gi + a.w_off[L - 1],
-                                              Gi + a.b_off[L - 1], a.loss, dz_prev, Gi + (L > 1 ? a.b_off[L - 2] : 0), smem, a.status);
+                head_backward_part<16, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gw, Gb, li, dz_prev, Gp, smem, a.status);
             else
-                head_backward_part<32, false>(i, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gi + a.w_off[L - 1],
-                                              Gi + a.b_off[L - 1], a.loss, dz_prev, Gi + (L > 1 ? a.b_off[L - 2] : 0), smem, a.status);
+                head_backward_part<32, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gw, Gb, li, dz_prev, Gp, smem, a.status);
+        }
+        if (parts > 1) {
+            grid.sync();
+            const int sums = a.C * in + a.C + in + 1;
+            for (int e = blockIdx.x * kThreads + tid; e < N * sums; e += gridDim.x * kThreads) {
+                const int i = e / sums;
+                float* Gi = a.G + (size_t)i * a.ld;
+                head_add_parts(i, e % sums, parts, N, B, in, a.C, a.head_part, Gi + a.w_off[L - 1], Gi + a.b_off[L - 1], L > 1 ? Gi + b_prev : nullptr,
+                               a.loss ? a.loss + i : nullptr);
+            }
         }
         grid.sync();
     } else {
@@ -299,7 +319,7 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     }
     a.ld = h->ld;
     a.X = X; a.Xout = X_out; a.G = h->d_G;
-    a.feat = h->feat; a.labels = h->labels; a.batch_idx = batch_idx; a.ylab = h->d_ylab;
+    a.feat = h->feat; a.labels = h->labels; a.batch_idx = batch_idx; a.ylab = h->d_ylab; a.head_part = h->d_head_part;
     a.rowptr = h->d_rowptr; a.col = h->d_col; a.t = t; a.t_edge = h->t_edge; a.b = b; a.kept = kept;
     a.T_nbr_ws = h->d_Tnbr_ws; a.T_nbr = T_nbr; a.T_worker = T_worker; a.T_round = T_round;
     a.waited = h->d_waited; a.status = h->d_status;

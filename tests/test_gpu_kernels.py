@@ -719,3 +719,43 @@ def test_round_with_few_participants_gives_the_bits_of_its_steps(dims, batch, n,
         assert torch.equal(G, G2), k
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("dims,batch,n", [([32, 10], 257, 3),           # two parts of the batch, the second of one sample
+                                          ([40, 24, 32], 256, 3),       # one part, the most classes: the largest staging
+                                          ([64, 48, 36, 10], 520, 4)])  # three parts; a bias gradient out of a dW GEMM
+def test_fp32_last_layer_in_parts_of_the_batch(dims, batch, n):
+    """The last layer's backward step splits a large batch into parts whose sums are added in a fixed order.  Gradients and
+    losses against the oracle (hidden units are far on one side of zero, so no ReLU decision is a matter of rounding), and
+    the single-launch round against the step-by-step one, bit for bit."""
+    p = _dbw()
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    rng = np.random.default_rng(2)
+    S = batch + 40
+    feat = rng.random((n, S, dims[0]), dtype=np.float32)
+    labels = rng.integers(0, dims[-1], size=(n, S)).astype(np.int32)
+    X = m.pack((0.05 * rng.standard_normal((n, m.d))).astype(np.float32))
+    for l in range(len(dims) - 2):
+        X[:, m.b_off[l]: m.b_off[l] + dims[l + 1]] = np.where(np.arange(dims[l + 1]) % 3 == 0, -9.0, 9.0) * 0.5 ** l
+    idx = np.stack([rng.permutation(S)[:batch] for _ in range(n)]).astype(np.int32)
+    h.set_dataset(dev(feat), dev(labels), S)
+    G, loss = torch.zeros(n, m.ld, device="cuda"), torch.zeros(n, device="cuda")
+    h.grad(dev(X), dev(idx), G, loss)
+    got = m.unpack(G.cpu().numpy())
+    for i in range(n):
+        g, l = orc.mlp_grad(m.unpack(X[i:i + 1])[0], dims, feat[i][idx[i]], labels[i][idx[i]])
+        assert np.abs(got[i] - g).max() <= 1e-5 * np.abs(g).max()
+        assert abs(float(loss[i]) - l) <= 1e-5 * max(abs(l), 1.0)
+    t, b = dev(1.0 + rng.random(n)), torch.ones(n, dtype=torch.int32, device="cuda")
+    outs = []
+    for fused in (True, False):
+        h.set_fused_round(fused)
+        assert h.round_is_fused() == fused
+        Y, kept = dev(X), torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+        h.round(Y, t, b, 0.05, Y, kept, batch_idx=dev(idx), loss=loss)
+        outs.append((Y, loss.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    assert h.status() == 0
+    h.close()
