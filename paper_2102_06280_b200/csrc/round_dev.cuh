@@ -578,19 +578,35 @@ __device__ __forceinline__ double round_times_part(int N, const int32_t* __restr
                                                    const int32_t* __restrict__ b, const double* T_nbr_ws, double* T_nbr_out,
                                                    double* T_worker, uint32_t* waited, uint32_t* status) {
     double tr = 0.0;
-    for (int w = threadIdx.x; w < N; w += blockDim.x) {
-        const int deg = rowptr[w + 1] - rowptr[w];
-        int bw = b[w];
-        bw = bw < 0 ? 0 : (bw > deg ? deg : bw);
-        const int p = deg - bw;
-        const bool part = p >= 1 || __ldcg(&waited[w]) != 0u;
-        const double tw = order_time(t[w], status);
-        const double tn = __ldcg(&T_nbr_ws[w]);
-        if (T_nbr_out) T_nbr_out[w] = tn;
-        const double twk = p >= 1 ? fmax(tw, tn) : (part ? tw : 0.0);
-        if (T_worker) T_worker[w] = twk;
-        if (part) tr = fmax(tr, twk);  // T(k) = max of T_j over the participating workers
-        waited[w] = 0u;
+    constexpr int U = 4;  // workers per thread and pass: their loads are issued together
+    for (int w0 = threadIdx.x; w0 < N; w0 += U * blockDim.x) {
+        int deg[U], bw[U];
+        uint32_t wait[U];
+        double tv[U], tn[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int w = w0 + u * (int)blockDim.x;
+            if (w < N) {
+                deg[u] = rowptr[w + 1] - rowptr[w];
+                bw[u] = b[w];
+                wait[u] = __ldcg(&waited[w]);
+                tv[u] = t[w];
+                tn[u] = __ldcg(&T_nbr_ws[w]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int w = w0 + u * (int)blockDim.x;
+            if (w >= N) break;
+            const int p = deg[u] - (bw[u] < 0 ? 0 : (bw[u] > deg[u] ? deg[u] : bw[u]));
+            const bool part = p >= 1 || wait[u] != 0u;
+            const double tw = order_time(tv[u], status);
+            if (T_nbr_out) T_nbr_out[w] = tn[u];
+            const double twk = p >= 1 ? fmax(tw, tn[u]) : (part ? tw : 0.0);
+            if (T_worker) T_worker[w] = twk;
+            if (part) tr = fmax(tr, twk);  // T(k) = max of T_j over the participating workers
+            waited[w] = 0u;
+        }
     }
     return tr;
 }

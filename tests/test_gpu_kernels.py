@@ -759,3 +759,29 @@ def test_fp32_last_layer_in_parts_of_the_batch(dims, batch, n):
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 127, 512, 513, 4097, 6016, 6100])  # strides of the loads, the last size with its times in shared memory
+def test_threshold_rule_and_times_at_the_edges_of_the_worker_count(n):
+    p = _dbw()
+    rowptr, col = wl.ring(n) if n >= 3 else wl.path(n)
+    h = p.Dbw(rowptr, col, d=4)
+    ref = orc.Dtur(rowptr, col) if n > 1 else None
+    rng = np.random.default_rng(n)
+    b, kept = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.zeros(max(len(col), 1), dtype=torch.uint8, device="cuda")
+    Tw, Tn, Tr, theta = (torch.zeros(k, dtype=torch.float64, device="cuda") for k in (n, n, 1, 1))
+    for k in range(3):
+        t = 1.0 + np.round(rng.exponential(1.0, size=n), 2)      # with ties
+        h.update_backups(dev(t), b, theta)
+        h.select(dev(t), b, kept, Tw, Tn, Tr)
+        if n == 1:
+            assert int(b[0]) == 0 and float(Tr[0]) == 0.0
+            continue
+        rb, rt = ref.update_backups(t)
+        assert np.array_equal(b.cpu().numpy(), rb) and float(theta[0]) == rt
+        rk = orc.select_fastest(rowptr, col, t, rb)
+        assert np.array_equal(kept.cpu().numpy(), np.asarray(rk, dtype=np.uint8))
+        rTn, rTw, rTr = orc.round_times(rowptr, col, t, rb, rk)
+        assert np.array_equal(Tn.cpu().numpy(), rTn) and np.array_equal(Tw.cpu().numpy(), rTw) and float(Tr[0]) == rTr
+    assert h.status() == 0
+    h.close()
