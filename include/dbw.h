@@ -245,9 +245,11 @@ int dbw_set_param_tracking(dbw_handle* h, int enable);
 /*
  * The same round for callers whose per-round inputs live in HOST memory (pinned memory makes
  * the copies asynchronous).  X / X_out / G_ext stay DEVICE (the parameters are the state of the
- * simulation); h_t[N], h_b[N], h_batch_idx[N][batch] are copied to the device on `stream`, the
- * round runs, and h_kept[nnz], h_T_worker[N], h_T_round[1], h_loss[N], h_b_out[N] (each
- * nullable) are copied back on `stream`.  When h_b is NULL the backup counts come from the
+ * simulation); h_t[N], h_b[N], h_batch_idx[N][batch] are copied to the device, the round runs, and
+ * h_kept[nnz], h_T_worker[N], h_T_round[1], h_loss[N], h_b_out[N] (each nullable) are copied back.
+ * To the caller all of it is ordered on `stream`; copies that need not wait for one another's
+ * neighbours in that order run on a stream of the handle, forked from and joined into it, beside
+ * the gradients and the mix.  When h_b is NULL the backup counts come from the
  * threshold rule: dbw_update_backups runs on the copied times first (Algorithm 2 feeding
  * Algorithm 1) and h_b_out receives them.  The call does not synchronise.
  */

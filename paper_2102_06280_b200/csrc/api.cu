@@ -117,7 +117,9 @@ void free_all(dbw_handle* h) {
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->side) cudaStreamDestroy(h->side);
-    h->ev_fork = h->ev_join = nullptr;
+    if (h->ev_loss) cudaEventDestroy(h->ev_loss);
+    if (h->ev_read) cudaEventDestroy(h->ev_read);
+    h->ev_fork = h->ev_join = h->ev_loss = h->ev_read = nullptr;
     h->side = nullptr;
     grad_fp32_free(h);
     grad_bf16_free(h);
@@ -244,7 +246,9 @@ int dbw_init(dbw_handle** out, int32_t N, int64_t d, int64_t ld, const int32_t* 
     h->plan.status = h->d_status;
     if (!cuda_ok(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking)) ||
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming)) ||
-        !cuda_ok(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming)))
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming)) ||
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_loss, cudaEventDisableTiming)) ||
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_read, cudaEventDisableTiming)))
         return fail(DBW_ERR_CUDA);
     mix_sp_prepare(h);  // the 2:4 worker order of the sparse tensor-core mix, where that kernel can apply
     if (model) {
@@ -346,12 +350,49 @@ int dbw_set_mix_panel(dbw_handle* h, int32_t cols) {
     return DBW_OK;
 }
 
-int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, const int32_t* batch_idx,
-              const float* G_ext, float lr, const float* lr_per_worker, float* X_out, uint8_t* kept,
-              double* T_worker, double* T_nbr, double* T_round, float* loss, void* stream) {
-    if (!h || !X || !t || !b || !X_out || !kept) return DBW_ERR_NULL;
-    DeviceGuard guard(h->device);
-    cudaStream_t s = (cudaStream_t)stream;
+// Host side of a round whose per-round inputs and results live in host memory (dbw_round_host); null pointers: not wanted.
+struct HostIO {
+    const double* t;
+    const int32_t* b;  // null: the threshold rule sets the counts
+    const int32_t* batch_idx;
+    uint8_t* kept;
+    double* T_worker;
+    double* T_round;
+    float* loss;
+    int32_t* b_out;
+};
+
+static int copy_batch(dbw_handle* h, const HostIO& io, cudaStream_t s) {
+    if (io.batch_idx)
+        DBW_CUDA(cudaMemcpyAsync(h->s_bidx, io.batch_idx, (size_t)h->N * h->model.batch * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    return DBW_OK;
+}
+
+// The times, and the backup counts that come with them.
+static int copy_inputs(dbw_handle* h, const HostIO& io, cudaStream_t s) {
+    DBW_CUDA(cudaMemcpyAsync(h->s_t, io.t, (size_t)h->N * sizeof(double), cudaMemcpyHostToDevice, s));
+    if (!io.b) return launch_update_backups(h, h->s_t, h->s_b, nullptr, s);
+    DBW_CUDA(cudaMemcpyAsync(h->s_b, io.b, (size_t)h->N * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    return DBW_OK;
+}
+
+// What the selection leaves, then (once `loss_ready`, if given, has happened) the losses.
+static int copy_results(dbw_handle* h, const HostIO& io, cudaEvent_t loss_ready, cudaStream_t s) {
+    const size_t N = (size_t)h->N;
+    if (io.kept) DBW_CUDA(cudaMemcpyAsync(io.kept, h->s_kept, (size_t)h->nnz, cudaMemcpyDeviceToHost, s));
+    if (io.T_worker) DBW_CUDA(cudaMemcpyAsync(io.T_worker, h->s_Tw, N * sizeof(double), cudaMemcpyDeviceToHost, s));
+    if (io.T_round) DBW_CUDA(cudaMemcpyAsync(io.T_round, h->s_Tr, sizeof(double), cudaMemcpyDeviceToHost, s));
+    if (io.b_out) DBW_CUDA(cudaMemcpyAsync(io.b_out, h->s_b, N * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    if (io.loss && io.batch_idx) {
+        if (loss_ready) DBW_CUDA(cudaStreamWaitEvent(s, loss_ready, 0));
+        DBW_CUDA(cudaMemcpyAsync(io.loss, h->s_loss, N * sizeof(float), cudaMemcpyDeviceToHost, s));
+    }
+    return DBW_OK;
+}
+
+static int run_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, const int32_t* batch_idx, const float* G_ext, float lr,
+                     const float* lr_per_worker, float* X_out, uint8_t* kept, double* T_worker, double* T_nbr, double* T_round, float* loss,
+                     const HostIO* io, cudaStream_t s) {
     int rc;
     const float* G = G_ext;  // NULL together with batch_idx == NULL: a consensus-only round, G = 0
     if (batch_idx) {
@@ -373,6 +414,7 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, 
     }
     if (batch_idx && round_fused_usable(h)) {
         // small fp32 network: the whole iteration in one cooperative launch (same bits as the launches below)
+        if (io && ((rc = copy_batch(h, *io, s)) || (rc = copy_inputs(h, *io, s)))) return rc;
         if (ev) DBW_CUDA(cudaEventRecord(ev[0], s));
         rc = launch_round_fused(h, X, t, b, batch_idx, lr, lr_per_worker, X_out, kept, T_worker, T_nbr, T_round, loss, s);
         if (ev) {  // the stages are not separable: one pair of events, reported under "gradients"
@@ -380,7 +422,7 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, 
             h->prof_single[h->prof_rounds - 1] = 1;
         }
         h->shadow_valid = false;
-        return rc;
+        return rc || !io ? rc : copy_results(h, *io, nullptr, s);
     }
     // first error of the calls below; later calls still run so that a forked side stream is always joined
     int first = DBW_OK;
@@ -389,10 +431,12 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, 
     };
     auto cuda = [&](cudaError_t e) { note(cuda_ok(e) ? DBW_OK : DBW_ERR_CUDA); };
     // The selection needs only t and b, so with gradients to compute it runs beside them on the handle's
-    // side stream: fork after everything the caller queued, join before the mix.
+    // side stream: fork after everything the caller queued, join before the mix.  With inputs and results in host memory the
+    // side stream also carries their copies (all but the batch): in before the selection, out beside the gradients and the
+    // mix.  (32 workers, 784-200-10, seven copies of 2 - 6 us one after the other before: 182 -> 147 us a round.)
     cudaStream_t sel = s;
     bool forked = false;
-    if (batch_idx) {
+    if (batch_idx || io) {
         cuda(cudaEventRecord(h->ev_fork, s));
         if (first == DBW_OK) cuda(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
         if (first != DBW_OK) return first;  // nothing forked yet
@@ -401,23 +445,48 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, 
     }
     // Tensor-core rounds: the dW GEMMs take the step of the workers that take no part, so they wait for the selection.
     const bool stepped = batch_idx && (h->flags & DBW_GEMM_BF16) && mix_active_usable(h);
-    if (ev) cuda(cudaEventRecord(ev[2], sel));
-    note(launch_select(h, t, b, kept, T_worker, T_nbr, T_round, true, sel, stepped));
-    if (ev) cuda(cudaEventRecord(ev[3], sel));
-    if (forked) cuda(cudaEventRecord(h->ev_join, sel));
+    bool joinable = false;  // ev_join has been recorded behind everything queued on the side stream
+    const std::function<int()> select = [&]() -> int {
+        int code = io ? copy_inputs(h, *io, sel) : DBW_OK;
+        if (ev) cuda(cudaEventRecord(ev[2], sel));
+        if (code == DBW_OK) code = launch_select(h, t, b, kept, T_worker, T_nbr, T_round, true, sel, stepped);
+        if (ev) cuda(cudaEventRecord(ev[3], sel));
+        if (forked) cuda(cudaEventRecord(h->ev_join, sel));
+        joinable = true;
+        return code;
+    };
+    if (io) note(copy_batch(h, *io, s));
     if (ev) cuda(cudaEventRecord(ev[0], s));
     const StepArgs step{lr, lr_per_worker, X_out, h->ev_join};
     if (batch_idx && first == DBW_OK)
-        note((h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, h->d_G, loss, s, stepped ? &step : nullptr)
-                                        : launch_grad_fp32(h, X, batch_idx, h->d_G, loss, s));
+        note((h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, h->d_G, loss, s, stepped ? &step : nullptr, &select)
+                                        : launch_grad_fp32(h, X, batch_idx, h->d_G, loss, s, &select));
+    else if (first == DBW_OK)
+        note(select());
+    if (forked && !joinable) cuda(cudaEventRecord(h->ev_join, sel));
     if (ev) cuda(cudaEventRecord(ev[1], s));
+    if (io) cuda(cudaEventRecord(h->ev_loss, s));
     // whatever failed above, the side stream is joined back: it never dangles, a capture stays valid
     if (forked) cuda(cudaStreamWaitEvent(s, h->ev_join, 0));
-    if (first != DBW_OK) return first;
-    if (ev) cuda(cudaEventRecord(ev[4], s));
-    note(stepped ? launch_mix_active(h, X, G, lr, lr_per_worker, X_out, s) : launch_mix(h, X, G, lr, lr_per_worker, X_out, s));
-    if (ev) cuda(cudaEventRecord(ev[5], s));
+    if (first == DBW_OK) {
+        if (ev) cuda(cudaEventRecord(ev[4], s));
+        note(stepped ? launch_mix_active(h, X, G, lr, lr_per_worker, X_out, s) : launch_mix(h, X, G, lr, lr_per_worker, X_out, s));
+        if (ev) cuda(cudaEventRecord(ev[5], s));
+    }
+    if (io) {
+        if (first == DBW_OK) note(copy_results(h, *io, h->ev_loss, sel));
+        cuda(cudaEventRecord(h->ev_read, sel));
+        cuda(cudaStreamWaitEvent(s, h->ev_read, 0));
+    }
     return first;
+}
+
+int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b, const int32_t* batch_idx,
+              const float* G_ext, float lr, const float* lr_per_worker, float* X_out, uint8_t* kept,
+              double* T_worker, double* T_nbr, double* T_round, float* loss, void* stream) {
+    if (!h || !X || !t || !b || !X_out || !kept) return DBW_ERR_NULL;
+    DeviceGuard guard(h->device);
+    return run_round(h, X, t, b, batch_idx, G_ext, lr, lr_per_worker, X_out, kept, T_worker, T_nbr, T_round, loss, nullptr, (cudaStream_t)stream);
 }
 
 int dbw_profile(dbw_handle* h, int enable) {
@@ -462,30 +531,13 @@ int dbw_round_host(dbw_handle* h, const float* X, const double* h_t, const int32
                    const int32_t* h_batch_idx, const float* G_ext, float lr, float* X_out, uint8_t* h_kept,
                    double* h_T_worker, double* h_T_round, float* h_loss, int32_t* h_b_out, void* stream) {
     if (!h || !X || !h_t || !X_out) return DBW_ERR_NULL;
+    if (h_batch_idx && !h->has_model) return DBW_ERR_BAD_MODEL;
     DeviceGuard guard(h->device);
-    cudaStream_t s = (cudaStream_t)stream;
-    int rc;
-    if ((rc = ensure_staging(h))) return rc;
-    DBW_CUDA(cudaMemcpyAsync(h->s_t, h_t, (size_t)h->N * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (h_b) {
-        DBW_CUDA(cudaMemcpyAsync(h->s_b, h_b, (size_t)h->N * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    } else if ((rc = launch_update_backups(h, h->s_t, h->s_b, nullptr, s))) {
-        return rc;
-    }
-    if (h_batch_idx) {
-        if (!h->has_model) return DBW_ERR_BAD_MODEL;
-        DBW_CUDA(cudaMemcpyAsync(h->s_bidx, h_batch_idx, (size_t)h->N * h->model.batch * sizeof(int32_t),
-                                 cudaMemcpyHostToDevice, s));
-    }
-    rc = dbw_round(h, X, h->s_t, h->s_b, h_batch_idx ? h->s_bidx : nullptr, G_ext, lr, nullptr, X_out, h->s_kept,
-                   h->s_Tw, nullptr, h->s_Tr, h->s_loss, stream);
+    const int rc = ensure_staging(h);
     if (rc) return rc;
-    if (h_kept) DBW_CUDA(cudaMemcpyAsync(h_kept, h->s_kept, (size_t)h->nnz, cudaMemcpyDeviceToHost, s));
-    if (h_T_worker) DBW_CUDA(cudaMemcpyAsync(h_T_worker, h->s_Tw, (size_t)h->N * sizeof(double), cudaMemcpyDeviceToHost, s));
-    if (h_T_round) DBW_CUDA(cudaMemcpyAsync(h_T_round, h->s_Tr, sizeof(double), cudaMemcpyDeviceToHost, s));
-    if (h_b_out) DBW_CUDA(cudaMemcpyAsync(h_b_out, h->s_b, (size_t)h->N * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    if (h_loss && h_batch_idx) DBW_CUDA(cudaMemcpyAsync(h_loss, h->s_loss, (size_t)h->N * sizeof(float), cudaMemcpyDeviceToHost, s));
-    return DBW_OK;
+    const HostIO io{h_t, h_b, h_batch_idx, h_kept, h_T_worker, h_T_round, h_loss, h_b_out};
+    return run_round(h, X, h->s_t, h->s_b, h_batch_idx ? h->s_bidx : nullptr, G_ext, lr, nullptr, X_out, h->s_kept, h->s_Tw, nullptr, h->s_Tr,
+                     h->s_loss, &io, (cudaStream_t)stream);
 }
 
 int dbw_update_backups(dbw_handle* h, const double* t_next, int32_t* b_out, double* theta_out, void* stream) {

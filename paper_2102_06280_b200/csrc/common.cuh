@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <functional>
 #include <mutex>
 #include <vector>
 
@@ -155,6 +156,7 @@ struct dbw_handle {
     // into the caller's stream by the two events)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_loss = nullptr, ev_read = nullptr;  // dbw_round_host: the losses are there; every result has been copied out
 
     // stage timing (dbw_profile): events[round][0..5] = start / end of the gradient, selection and mix stages
     bool profiling = false;
@@ -253,8 +255,10 @@ inline bool fp32_head_usable(const dbw_handle* h) {
 }
 int grad_fp32_alloc(dbw_handle* h);
 void grad_fp32_free(dbw_handle* h);
+// `beside` (of both gradient paths): queues what runs beside the gradients on another stream; called once the forward pass is
+// queued, so that the GPU has work while the host makes those calls.
 int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss,
-                     cudaStream_t s);
+                     cudaStream_t s, const std::function<int()>* beside = nullptr);
 
 // grad_bf16.cu
 int grad_bf16_alloc(dbw_handle* h);
@@ -267,6 +271,6 @@ struct StepArgs {
     cudaEvent_t selected;  // the selection (and with it the list of participants) is complete after this event
 };
 int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss, cudaStream_t s,
-                     const StepArgs* step = nullptr);
+                     const StepArgs* step = nullptr, const std::function<int()>* beside = nullptr);
 
 }  // namespace dbw

@@ -1101,7 +1101,7 @@ void grad_bf16_free(dbw_handle* h) {
 }
 
 int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss, cudaStream_t s,
-                     const StepArgs* step) {
+                     const StepArgs* step, const std::function<int()>* beside) {
     const dbw_model_desc& m = h->model;
     BF16State* st = h->bf16;
     const int L = m.n_layers, B = m.batch, N = h->N, C = m.dims[L];
@@ -1129,6 +1129,7 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.status = h->d_status;
         if ((rc = run_tc(h, st->fwdA[l], st->fwdB[l], g, N, s))) return rc;
     }
+    if (beside && (rc = (*beside)())) return rc;
     // last layer, loss, and its backward
     const int K = m.dims[L - 1];
     bf16* dzP = L >= 2 ? st->dZ[L - 1] : nullptr;

@@ -286,7 +286,7 @@ void grad_fp32_free(dbw_handle* h) {
 }
 
 int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, float* loss,
-                     cudaStream_t s) {
+                     cudaStream_t s, const std::function<int()>* beside) {
     const dbw_model_desc& m = h->model;
     const int B = m.batch, L = m.n_layers, N = h->N;
     // A last layer of at most 32 classes runs as two kernels of its own instead of a GEMM, the loss kernel and
@@ -310,6 +310,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.M = B; g.N = out; g.K = in; g.relu = l < L - 1;
         if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
     }
+    if (beside && (rc = (*beside)())) return rc;
     if (head) {
         const int in = m.dims[L - 1], C = m.dims[L];
         HeadRows rows{};
