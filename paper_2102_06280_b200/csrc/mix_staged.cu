@@ -1,7 +1,8 @@
 // Mix kernel for many workers and many terms per output: one persistent CTA per
 // SM, warp-specialised, with the NEXT column panel prefetched into tensor memory.
 //
-// With N of the order of 1000 a 32-column panel of all rows (N x 128 B) plus the neighbour lists
+// With N of the order of 1000 a 32-column panel of all rows (N x 128 B; beyond 1024 rows 16 columns, beyond 2048 eight) plus
+// the neighbour lists
 // fill shared memory, so there is no room for a second panel buffer, and with about 30 terms per
 // output the gather out of shared memory takes longer than the HBM stream.  To overlap the two,
 // eight producer warps stream the next panel of X and G from HBM (128-bit loads, x - lr*g formed
@@ -10,7 +11,7 @@
 // trips, so it wants every warp the SM can hold).  When both are done the producers move the parked
 // panel from tensor memory into shared memory (tcgen05.ld + 128-bit shared stores) and the roles
 // repeat.  The neighbour lists (16-bit entries built once per launch from the mixing plan: a bare row
-// index with uniform weights, a 10-bit index and a 6-bit weight code with the Metropolis weights) stay
+// index with uniform weights, an index and a weight code with the Metropolis weights) stay
 // in shared memory for the whole launch.  HBM traffic is the algorithmic 12 bytes per element; a panel
 // is fully staged before any of it is written and panels are disjoint, so X' may overwrite X.
 #include "common.cuh"
@@ -22,11 +23,21 @@ namespace {
 constexpr int kProdWarps = 8, kConsWarps = 24;
 constexpr int kThreads = (kProdWarps + kConsWarps) * 32;  // 1024
 constexpr int kTmemCols = 256;                            // 128 lanes x 256 columns x 4 B = one 1024 x 32 panel
-constexpr int kMaxN = 1024;
-constexpr int kZeroCode = 63;  // weight code of list padding (weighted lists): weight 0
+constexpr int kMaxN = 4096;
+// Columns of a panel: the widest whose panel of all rows fits the 128 KB of tensor memory and shared memory it is given.
+__host__ __device__ constexpr int staged_width(int N) { return N <= 1024 ? 32 : N <= 2048 ? 16 : 8; }
+// Bits of a list entry that hold the row index; with weighted lists the rest of its 16 bits is the weight code.
+__host__ __device__ constexpr int index_bits(int W) { return W == 32 ? 10 : W == 16 ? 11 : 12; }
+__host__ __device__ constexpr int zero_code(int W) { return (1 << (16 - index_bits(W))) - 1; }  // code of list padding: weight 0
+// Uniform 32-column lists hold the own row as a row's first entry (one padding read in two less: 1268 us against 1312 for 1024
+// workers x 262,144 columns, 32 neighbours); weighted and narrower ones do not (weighted: 1430 us against 1470).
+__host__ __device__ constexpr int listed_self(int W, bool weighted) { return W == 32 && !weighted ? 1 : 0; }
+__host__ __device__ constexpr int list_entries(int W, bool weighted, int maxdeg) {
+    return maxdeg + listed_self(W, weighted) < 4 ? 4 : (maxdeg + listed_self(W, weighted) + 3) / 4 * 4;
+}
 
-// 1 / (1 + m) for the weight codes m = 0 .. 62 of the weighted lists (Assumption 1: the weight worker i puts on a kept
-// neighbour j is 1 / (1 + max(p_i, p_j))), the same fp32 quotient the mixing plan holds; code 63 is weight 0.
+// 1 / (1 + m) for the weight codes m of the weighted lists (Assumption 1: the weight worker i puts on a kept neighbour j is
+// 1 / (1 + max(p_i, p_j))), the same fp32 quotient the mixing plan holds.
 __constant__ float c_weight[64] = {
     1.0f / 1,  1.0f / 2,  1.0f / 3,  1.0f / 4,  1.0f / 5,  1.0f / 6,  1.0f / 7,  1.0f / 8,  1.0f / 9,  1.0f / 10, 1.0f / 11,
     1.0f / 12, 1.0f / 13, 1.0f / 14, 1.0f / 15, 1.0f / 16, 1.0f / 17, 1.0f / 18, 1.0f / 19, 1.0f / 20, 1.0f / 21, 1.0f / 22,
@@ -58,15 +69,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float4 (&v)[4]) {
 }
 
 __device__ __forceinline__ float4 ldg4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+// The same with the whole 128-byte line asked of L2: the blocks of the neighbouring panels read the rest of it.
+__device__ __forceinline__ float4 ldg4_line(const float* p) {
+    float4 v;
+    asm("ld.global.nc.L2::128B.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ void add4(float4& a, const float4 v) {
     a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
 }
 __device__ __forceinline__ void fma4(float4& a, const float w, const float4 v) {
     a.x = fmaf(w, v.x, a.x); a.y = fmaf(w, v.y, a.y); a.z = fmaf(w, v.z, a.z); a.w = fmaf(w, v.w, a.w);
 }
+__device__ __forceinline__ float4 mul4(const float4 v, const float w) { return make_float4(w * v.x, w * v.y, w * v.z, w * v.w); }
 
 struct StagedArgs {
-    int N, n_panels, mix_then_correct, plan_row;  // plan_row: 16-bit entries per neighbour-list row (multiple of 8)
+    int N, n_panels, mix_then_correct, list_row;  // list_row: 16-bit entries per neighbour-list row (multiple of 4)
     long long ld;
     const float* X;
     const float* G;
@@ -77,21 +95,28 @@ struct StagedArgs {
     MixPlan plan;
 };
 
-// Shared memory: panel float4 [N + 1][8] (row N is all zero: the target of list padding), then the
-// neighbour lists uint16 [N][plan_row + 8] (the 16-byte skew keeps four consecutive rows in distinct
-// banks), then the per-row scale float [N], then the list lengths in blocks of 8, uint8 [N].
+// Shared memory: panel float4 [N + 1][W / 4] (row N is all zero: the target of list padding), then the neighbour lists
+// uint16 [N][list_row], then the per-row scale float [N], then the list lengths in blocks of 4, uint8 [N].
 // WEIGHTED = false: uniform weights, a list entry is a bare 16-bit row index and the sum is scaled once per row.
-// WEIGHTED = true: a list entry is a 10-bit row index and a 6-bit weight code; padding is (own row, weight 0).
-template <bool WEIGHTED>
+// WEIGHTED = true: a list entry is a row index and a weight code; padding is (own row, weight 0).
+// LPR lanes share an output row.  With weights and 128-byte rows there are four, each lane with two 16-byte pieces: two rows to
+// a quarter-warp phase of a 128-bit shared load, the odd groups of lanes reading the second half first so that the two never
+// share a bank.  A list or weight read then serves eight rows instead of four (1430 us against 1632 for 1024 workers x 262,144
+// columns, 32 neighbours).  Without weight reads eight lanes of one piece are better (1268 us against 1291).
+template <bool WEIGHTED, int W>
 __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
+    constexpr int SLOTS = W / 4, PIECES = W == 32 && WEIGHTED ? 2 : 1, LPR = SLOTS / PIECES, RPW = 32 / LPR;  // RPW: output rows per warp
+    constexpr bool SELF = listed_self(W, WEIGHTED) != 0;
+    constexpr uint32_t kIdx = WEIGHTED ? (1u << index_bits(W)) - 1 : 0xffffu;
+    constexpr int kCodeShift = index_bits(W), ZERO = zero_code(W);
     extern __shared__ float4 smem4[];
     float4* panel = smem4;
     const int N = a.N;
-    const int prow = a.plan_row + 8;  // uint16 per list row
-    uint16_t* lists = reinterpret_cast<uint16_t*>(panel + (size_t)(N + 1) * 8);
-    float* scale = reinterpret_cast<float*>(lists + (size_t)N * prow);
+    const int lrow = a.list_row;
+    uint16_t* lists = reinterpret_cast<uint16_t*>(panel + (size_t)(N + 1) * SLOTS);
+    float* scale = reinterpret_cast<float*>(lists + (size_t)N * lrow);
     uint8_t* nblk = reinterpret_cast<uint8_t*>(scale + N);
-    float* wtab = reinterpret_cast<float*>(nblk + (N + 15) / 16 * 16);  // copy of c_weight (weighted lists)
+    float* wtab = reinterpret_cast<float*>(nblk + (N + 15) / 16 * 16);  // weights by code (weighted lists)
     __shared__ uint32_t tmem_slot;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -100,64 +125,64 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // neighbour lists, scales and the zero row: once per launch
-    for (int e = tid; e < N * (prow / 8); e += kThreads) {
-        const int i = e / (prow / 8), k0 = (e % (prow / 8)) * 8;
+    for (int e = tid; e < N * (lrow / 4); e += kThreads) {
+        const int i = e / (lrow / 4), k0 = (e % (lrow / 4)) * 4;
         const int cnt = a.plan.cnt[i];
-        uint32_t w[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const int k = k0 + 2 * h;
-            auto entry = [&](int kk) -> uint32_t {
-                if (!WEIGHTED) return kk < cnt ? (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) : (uint32_t)N;
-                if (kk >= cnt) return (uint32_t)i | ((uint32_t)kZeroCode << 10);
-                // the plan's weight is 1 / (1 + m): recover m (exact for m <= 62) and keep it as the code
-                const int m = __float2int_rn(1.0f / a.plan.w[(size_t)i * a.plan.stride + kk]) - 1;
-                return (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) | ((uint32_t)min(max(m, 0), kZeroCode - 1) << 10);
-            };
-            w[h] = entry(k) | (entry(k + 1) << 16);
-        }
-        *reinterpret_cast<uint4*>(lists + (size_t)i * prow + k0) = make_uint4(w[0], w[1], w[2], w[3]);
+        auto entry = [&](int k) -> uint32_t {
+            if (SELF && k == 0) return (uint32_t)i;
+            const int kk = k - (SELF ? 1 : 0);
+            if (!WEIGHTED) return kk < cnt ? (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) : (uint32_t)N;
+            if (kk >= cnt) return (uint32_t)i | ((uint32_t)ZERO << kCodeShift);
+            // the plan's weight is 1 / (1 + m): recover m (exact for m <= 62) and keep it as the code
+            const int m = __float2int_rn(1.0f / a.plan.w[(size_t)i * a.plan.stride + kk]) - 1;
+            return (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) | ((uint32_t)min(max(m, 0), ZERO - 1) << kCodeShift);
+        };
+        *reinterpret_cast<uint2*>(lists + (size_t)i * lrow + k0) =
+            make_uint2(entry(k0) | (entry(k0 + 1) << 16), entry(k0 + 2) | (entry(k0 + 3) << 16));
     }
     for (int i = tid; i < N; i += kThreads) {
         scale[i] = a.plan.w_self[i];
-        nblk[i] = (uint8_t)((a.plan.cnt[i] + 7) / 8);
+        nblk[i] = (uint8_t)max((a.plan.cnt[i] + (SELF ? 1 : 0) + 3) / 4, 1);  // a row without kept neighbours gathers one block
     }
-    if (WEIGHTED && tid < 64) wtab[tid] = c_weight[tid];
-    if (tid < 8) panel[(size_t)N * 8 + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (WEIGHTED && tid <= ZERO) wtab[tid] = tid == ZERO ? 0.f : c_weight[tid];
+    if (tid < SLOTS) panel[(size_t)N * SLOTS + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_slot;
 
-    const int n_its = (N + 31) / 32;  // a producer warp stages 4 rows per iteration, the eight warps 32
+    constexpr int RPS = 32 / SLOTS;                      // rows a producer warp stages per instruction
+    constexpr int IT_ROWS = kProdWarps * RPS;            // rows the producer warps stage per iteration: N needs at most 32
+    const int n_its = (N + IT_ROWS - 1) / IT_ROWS;
     const bool producer = warp < kProdWarps;
-    // producer coordinates: row (within an iteration) and 16-byte slot of the 128-byte row segment
-    const int p_row = warp * 4 + (lane >> 3), slot = lane & 7;
+    // producer coordinates: row (within an iteration) and 16-byte slot of the row segment
+    const int p_row = warp * RPS + lane / SLOTS, slot = lane % SLOTS;
     const uint32_t p_taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 128);
-    // consumer coordinates: 64 groups of 8 lanes, each group owns rows grp, grp + 64, ...
-    const int grp = (warp - kProdWarps) * 4 + (lane >> 3);
+    // consumer coordinates: groups of LPR lanes, each owns rows grp, grp + kRowsPar, ...
+    constexpr int kRowsPar = kConsWarps * RPW;
+    const int grp = (warp - kProdWarps) * RPW + lane / LPR;
 
     auto stage = [&](int pn) {  // HBM -> registers -> tensor memory
-        const long long c = (long long)pn * 32 + 4 * slot;
+        const long long c = (long long)pn * W + 4 * slot;
         const bool c_ok = c < a.ld;
         for (int bt = 0; bt < n_its; bt += 4) {
             float4 x[4], g[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int r = (bt + u) * 32 + p_row;
+                const int r = (bt + u) * IT_ROWS + p_row;
                 const bool ok = c_ok && r < N;
-                x[u] = ok ? ldg4(a.X + (size_t)r * a.ld + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                x[u] = ok ? (W < 32 ? ldg4_line(a.X + (size_t)r * a.ld + c) : ldg4(a.X + (size_t)r * a.ld + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
             if (a.G && !a.mix_then_correct) {  // G == nullptr: consensus-only round, G = 0
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int r = (bt + u) * 32 + p_row;
+                    const int r = (bt + u) * IT_ROWS + p_row;
                     const bool ok = c_ok && r < N;
-                    g[u] = ok ? ldg4(a.G + (size_t)r * a.ld + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    g[u] = ok ? (W < 32 ? ldg4_line(a.G + (size_t)r * a.ld + c) : ldg4(a.G + (size_t)r * a.ld + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    const int r = (bt + u) * 32 + p_row;
+                    const int r = (bt + u) * IT_ROWS + p_row;
                     const float nlr = -((a.lr_pw && r < N) ? a.lr_pw[r] : a.lr);
                     x[u].x = fmaf(nlr, g[u].x, x[u].x);
                     x[u].y = fmaf(nlr, g[u].y, x[u].y);
@@ -175,102 +200,103 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
             tmem_ld16(p_taddr + (uint32_t)(4 * bt), x);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int r = (bt + u) * 32 + p_row;
-                if (r < N) panel[(size_t)r * 8 + slot] = x[u];
+                const int r = (bt + u) * IT_ROWS + p_row;
+                if (r < N) panel[(size_t)r * SLOTS + slot] = x[u];
             }
         }
     };
     auto gather = [&](int pn) {  // every output row of the panel out of shared memory
-        const long long c = (long long)pn * 32 + 4 * slot;
-        // Flattened loop over (row, list block) with the NEXT block's indices (of this row, or of the
-        // group's next row together with that row's own segment) fetched before the current block's
-        // eight rows are gathered, so that no shared-memory round trip sits between two gathers.
+        // this lane's pieces of a row: 16-byte slots piece[0], piece[1]
+        int piece[PIECES];
+        piece[0] = lane % LPR;
+        if (PIECES == 2) {
+            const int odd = (lane / LPR) & 1;
+            piece[PIECES - 1] = piece[0] + LPR * (1 - odd);
+            piece[0] += LPR * odd;
+        }
+        // Flattened loop over (row, list block) with the NEXT block's entries fetched before the current block's rows are
+        // gathered, so that no shared-memory round trip sits between two gathers.
         int i = grp;
         if (i >= N) return;
-        const uint4* lp = reinterpret_cast<const uint4*>(lists + (size_t)i * prow);
-        int nb = max((int)nblk[i], 1), kb = 0;  // a row without kept neighbours gathers one all-padding block
-        uint4 u = lp[0];
-        auto first = [&](int row) {  // uniform: the own row, scaled with the sum at the end; weighted: own weight x own row
-            float4 v = panel[(size_t)row * 8 + slot];
-            if (WEIGHTED) {
-                const float ws = scale[row];
-                v.x *= ws; v.y *= ws; v.z *= ws; v.w *= ws;
+        const uint2* lp = reinterpret_cast<const uint2*>(lists + (size_t)i * lrow);
+        int nb = nblk[i], kb = 0;
+        uint2 u = lp[0];
+        float4 acc[PIECES];
+        auto first = [&](int row, float4 (&q)[PIECES]) {  // uniform: the own row, scaled with the sum at the end; weighted: own weight x own row
+#pragma unroll
+            for (int h = 0; h < PIECES; ++h) {
+                if (SELF) {
+                    q[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
+                    q[h] = panel[(size_t)row * SLOTS + piece[h]];
+                    if (WEIGHTED) q[h] = mul4(q[h], scale[row]);
+                }
             }
-            return v;
         };
-        float4 acc = first(i);
+        first(i, acc);
         while (true) {
             const bool last = kb + 1 >= nb;
-            const int i2 = i + kConsWarps * 4;
+            const int i2 = i + kRowsPar;
             const bool more = !last || i2 < N;
-            const uint4* lp2 = last ? reinterpret_cast<const uint4*>(lists + (size_t)i2 * prow) : lp;
-            uint4 un = u;
-            float4 acc2 = acc;
+            const uint2* lp2 = last ? reinterpret_cast<const uint2*>(lists + (size_t)i2 * lrow) : lp;
+            uint2 un = u;
             if (more) un = lp2[last ? 0 : kb + 1];
-            if (last && i2 < N) acc2 = first(i2);
-            constexpr uint32_t kIdx = WEIGHTED ? 0x3ffu : 0xffffu;
-            const float4 v0 = panel[(size_t)(u.x & kIdx) * 8 + slot], v1 = panel[(size_t)((u.x >> 16) & kIdx) * 8 + slot];
-            const float4 v2 = panel[(size_t)(u.y & kIdx) * 8 + slot], v3 = panel[(size_t)((u.y >> 16) & kIdx) * 8 + slot];
-            const float4 v4 = panel[(size_t)(u.z & kIdx) * 8 + slot], v5 = panel[(size_t)((u.z >> 16) & kIdx) * 8 + slot];
-            const float4 v6 = panel[(size_t)(u.w & kIdx) * 8 + slot], v7 = panel[(size_t)((u.w >> 16) & kIdx) * 8 + slot];
-            if (!WEIGHTED) {
-                add4(acc, v0); add4(acc, v1); add4(acc, v2); add4(acc, v3);
-                add4(acc, v4); add4(acc, v5); add4(acc, v6); add4(acc, v7);
-            } else {  // weights out of a 64-entry table in shared memory (one wavefront for the warp's four codes), list order
-                fma4(acc, wtab[(u.x >> 10) & 63u], v0); fma4(acc, wtab[u.x >> 26], v1);
-                fma4(acc, wtab[(u.y >> 10) & 63u], v2); fma4(acc, wtab[u.y >> 26], v3);
-                fma4(acc, wtab[(u.z >> 10) & 63u], v4); fma4(acc, wtab[u.z >> 26], v5);
-                fma4(acc, wtab[(u.w >> 10) & 63u], v6); fma4(acc, wtab[u.w >> 26], v7);
+            const uint32_t e[4] = {u.x & 0xffffu, u.x >> 16, u.y & 0xffffu, u.y >> 16};
+            float4 v[4][PIECES];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int h = 0; h < PIECES; ++h) v[k][h] = panel[(size_t)(e[k] & kIdx) * SLOTS + piece[h]];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (!WEIGHTED) {
+#pragma unroll
+                    for (int h = 0; h < PIECES; ++h) add4(acc[h], v[k][h]);
+                } else {  // weights out of a table in shared memory, list order
+                    const float w = wtab[e[k] >> kCodeShift];
+#pragma unroll
+                    for (int h = 0; h < PIECES; ++h) fma4(acc[h], w, v[k][h]);
+                }
             }
             u = un;
             if (!last) {
                 ++kb;
                 continue;
             }
-            if (!WEIGHTED) {
-                const float w = scale[i];
-                acc.x *= w; acc.y *= w; acc.z *= w; acc.w *= w;
-            }
-            if (c < a.ld) {
-                if (a.G && a.mix_then_correct) {
-                    const float4 gi = ldg4(a.G + (size_t)i * a.ld + c);
-                    const float nlr = -(a.lr_pw ? a.lr_pw[i] : a.lr);
-                    acc.x = fmaf(nlr, gi.x, acc.x); acc.y = fmaf(nlr, gi.y, acc.y);
-                    acc.z = fmaf(nlr, gi.z, acc.z); acc.w = fmaf(nlr, gi.w, acc.w);
+#pragma unroll
+            for (int h = 0; h < PIECES; ++h) {
+                const long long c = (long long)pn * W + 4 * piece[h];
+                float4 o = WEIGHTED ? acc[h] : mul4(acc[h], scale[i]);
+                if (c < a.ld) {
+                    if (a.G && a.mix_then_correct) {
+                        const float4 gi = ldg4(a.G + (size_t)i * a.ld + c);
+                        const float nlr = -(a.lr_pw ? a.lr_pw[i] : a.lr);
+                        o.x = fmaf(nlr, gi.x, o.x); o.y = fmaf(nlr, gi.y, o.y);
+                        o.z = fmaf(nlr, gi.z, o.z); o.w = fmaf(nlr, gi.w, o.w);
+                    }
+                    *reinterpret_cast<float4*>(a.Xout + (size_t)i * a.ld + c) = o;
+                    if (a.shadow) *reinterpret_cast<uint2*>(a.shadow + (size_t)i * a.ld + c) = pack_bf16x4_rn(o.x, o.y, o.z, o.w);
                 }
-                *reinterpret_cast<float4*>(a.Xout + (size_t)i * a.ld + c) = acc;
-                if (a.shadow) *reinterpret_cast<uint2*>(a.shadow + (size_t)i * a.ld + c) = pack_bf16x4_rn(acc.x, acc.y, acc.z, acc.w);
             }
             if (i2 >= N) break;
             i = i2;
             lp = lp2;
-            nb = max((int)nblk[i], 1);
+            nb = nblk[i];
             kb = 0;
-            acc = acc2;
+            first(i, acc);
         }
     };
 
-    int pn = blockIdx.x;
-    if (pn < a.n_panels) {
+    for (int pn = blockIdx.x, prev = -1; prev >= 0 || pn < a.n_panels; prev = pn < a.n_panels ? pn : -1, pn += gridDim.x) {
         if (producer) {
-            stage(pn);
-            unpark();
+            if (pn < a.n_panels) stage(pn);
+        } else if (prev >= 0) {
+            gather(prev);
         }
-        __syncthreads();
-        while (true) {
-            const int next = pn + gridDim.x;
-            const bool more = next < a.n_panels;
-            if (producer) {
-                if (more) stage(next);
-            } else {
-                gather(pn);
-            }
-            __syncthreads();  // panel pn consumed, panel `next` parked
-            if (!more) break;
-            if (producer) unpark();
-            __syncthreads();  // panel `next` in shared memory
-            pn = next;
-        }
+        __syncthreads();  // the previous panel consumed, the next one parked
+        if (pn >= a.n_panels) break;
+        if (producer) unpark();
+        __syncthreads();  // the next panel in shared memory
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -280,22 +306,36 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
     }
 }
 
-size_t staged_smem(const dbw_handle* h, int plan_row) {
+size_t staged_smem(const dbw_handle* h) {
     const size_t N = (size_t)h->N;
-    return (N + 1) * 128 + N * (size_t)(plan_row + 8) * 2 + N * 4 + ((N + 15) / 16) * 16 + 256;
+    const int W = staged_width(h->N);
+    return (N + 1) * (size_t)(W * 4) + N * (size_t)list_entries(W, !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg) * 2 + N * 4 + ((N + 15) / 16) * 16 + 256;
+}
+
+template <bool WEIGHTED, int W>
+int launch_staged(const dbw_handle* h, StagedArgs& a, cudaStream_t s) {
+    static PerDeviceOnce once;
+    const int rc = once.run(h->device, [h]() -> int {
+        DBW_CUDA(cudaFuncSetAttribute(mix_staged_kernel<WEIGHTED, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 256));
+        return DBW_OK;
+    });
+    if (rc) return rc;
+    a.n_panels = (int)((h->ld + W - 1) / W);
+    const int grid = a.n_panels < h->sm_count ? a.n_panels : h->sm_count;
+    mix_staged_kernel<WEIGHTED, W><<<grid, kThreads, staged_smem(h), s>>>(a);
+    DBW_LAUNCHED();
+    return DBW_OK;
 }
 
 }  // namespace
 
-// Usable when every worker's panel row fits the tensor-memory staging area and the shared memory holds
-// panel and lists; with uniform weights a list entry is a bare 16-bit index (one scale per row), with
-// the Metropolis weights it carries a 6-bit weight code next to a 10-bit index (degrees up to 62).
+// Usable when a panel of all rows and the lists fit; with uniform weights a list entry is a bare 16-bit index (one scale per
+// row), with the Metropolis weights it carries a weight code next to the index (degrees up to 62, 30 or 14).
 bool mix_staged_usable(const dbw_handle* h) {
     if (h->N > kMaxN || h->N < 64) return false;
-    if (!(h->flags & DBW_WEIGHT_UNIFORM) && h->maxdeg > kZeroCode - 1) return false;
-    const int plan_row = (h->maxdeg + 7) / 8 * 8;
-    if (plan_row > 248) return false;
-    return staged_smem(h, plan_row) + 256 <= (size_t)h->smem_optin;
+    if (!(h->flags & DBW_WEIGHT_UNIFORM) && h->maxdeg > zero_code(staged_width(h->N)) - 1) return false;
+    if (list_entries(staged_width(h->N), !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg) > 4 * 255) return false;  // lengths are counted in blocks of 4, in a byte
+    return staged_smem(h) + 256 <= (size_t)h->smem_optin;
 }
 
 int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
@@ -303,25 +343,16 @@ int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, c
     StagedArgs a{};
     a.N = h->N;
     a.ld = h->ld;
-    a.n_panels = (int)((h->ld + 31) / 32);
     a.mix_then_correct = (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0;
-    a.plan_row = (h->maxdeg + 7) / 8 * 8;
+    const int W = staged_width(h->N);
+    a.list_row = list_entries(W, !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg);
     a.X = X; a.G = G; a.lr = lr; a.lr_pw = lr_pw; a.Xout = X_out; a.shadow = shadow; a.plan = h->plan;
-    const size_t smem = staged_smem(h, a.plan_row);
-    static PerDeviceOnce once;
-    const int rc = once.run(h->device, [h]() -> int {
-        DBW_CUDA(cudaFuncSetAttribute(mix_staged_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 256));
-        DBW_CUDA(cudaFuncSetAttribute(mix_staged_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 256));
-        return DBW_OK;
-    });
-    if (rc) return rc;
-    const int grid = a.n_panels < h->sm_count ? a.n_panels : h->sm_count;
-    if (h->flags & DBW_WEIGHT_UNIFORM)
-        mix_staged_kernel<false><<<grid, kThreads, smem, s>>>(a);
-    else
-        mix_staged_kernel<true><<<grid, kThreads, smem, s>>>(a);
-    DBW_LAUNCHED();
-    return DBW_OK;
+    const bool uniform = (h->flags & DBW_WEIGHT_UNIFORM) != 0;
+    switch (W) {
+        case 32: return uniform ? launch_staged<false, 32>(h, a, s) : launch_staged<true, 32>(h, a, s);
+        case 16: return uniform ? launch_staged<false, 16>(h, a, s) : launch_staged<true, 16>(h, a, s);
+        default: return uniform ? launch_staged<false, 8>(h, a, s) : launch_staged<true, 8>(h, a, s);
+    }
 }
 
 }  // namespace dbw

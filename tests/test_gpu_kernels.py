@@ -785,3 +785,36 @@ def test_threshold_rule_and_times_at_the_edges_of_the_worker_count(n):
         assert np.array_equal(Tn.cpu().numpy(), rTn) and np.array_equal(Tw.cpu().numpy(), rTw) and float(Tr[0]) == rTr
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("n,deg", [(960, 32), (1024, 6), (1025, 30), (2048, 8), (2049, 14), (4096, 8)])
+@pytest.mark.parametrize("rule,order", [("uniform", "local_then_mix"), ("metropolis", "mix_then_correct"), ("metropolis", "local_then_mix")])
+def test_staged_kernel_at_the_edges_of_its_panel_widths(n, deg, rule, order):
+    """Panels of 32, 16 and 8 columns by the worker count, the largest degrees whose weight codes and lists still fit, rows
+    that keep nobody, a ragged last panel, in place: against the oracle, and with the paper's weights bit for bit against the
+    kernel that gathers through L2."""
+    p = _dbw()
+    d = 1036
+    rowptr, col = wl.random_regular(n, deg, 3)
+    flags = (p.WEIGHT_UNIFORM if rule == "uniform" else 0) | (p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    h = p.Dbw(rowptr, col, d=d, flags=flags)
+    h.set_mix_panel(1)
+    assert h.mix_kernel() == "mix_staged_kernel" and h.mix_in_place_ok()
+    rng = np.random.default_rng(4)
+    X, G = (rng.standard_normal((n, d), dtype=np.float32) for _ in range(2))
+    b = rng.integers(0, deg + 1, size=n)
+    b[:40] = 0
+    t = 1.0 + rng.exponential(1.0, size=n)
+    kept = orc.select_fastest(rowptr, col, t, b)
+    ws, we = orc.mixing_weights(rowptr, col, b, kept, rule)
+    args = (dev(G), dev(kept), dev(b.astype(np.int32)), 0.05)
+    Y = dev(X)
+    h.mix(Y, *args, Y)
+    assert row_rel_err(Y.cpu().numpy(), orc.mix_update(rowptr, col, X, G, ws, we, 0.05, order)) <= 1e-5
+    if rule == "metropolis":
+        h.set_mix_panel(-1)
+        Z = torch.empty_like(Y)
+        h.mix(dev(X), *args, Z)
+        assert torch.equal(Y, Z)
+    assert h.status() == 0
+    h.close()
