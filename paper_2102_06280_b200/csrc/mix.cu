@@ -281,16 +281,20 @@ constexpr bool kSparseByDefault = false;
 // (128-byte segment) panel with two CTAs per SM.  Beyond 1024 workers its own panels are narrower too (16 columns, from 2049
 // workers 8): measured with 8 neighbours, 1300 workers x 131,072 columns 659 us against 847 (16-column panel kernel), 2048
 // workers 968 / 1669, 3000 x 65,536 907 / 1303.  The panel kernel stays better where two of its CTAs share an SM and the
-// matrix is a fraction of L2 (1100 x 4096: 31 us against 35; x 8192: 51 / 50), and the L2 kernel takes over where no panel
-// of all rows fits (4096 x 65,536: 1533 us against 1715 staged).
+// matrix is a fraction of L2 (1100 x 4096: 31 us against 35; x 8192: 51 / 50).  Where no panel of all rows leaves the panel
+// kernel any room, the L2 kernel stays when few neighbours are read or the matrix does not stream from HBM (4096 workers, 2
+// neighbours: 837 us against 1016, 4 neighbours 1046 / 1016, 8 neighbours 1541 / 1348; 16,384 columns 396 / 371).
 static bool use_staged(const dbw_handle* h) {
     if (!mix_staged_usable(h)) return false;
     if (h->mix_panel_cols == 1) return true;
+    if (h->mix_panel_cols != 0) return false;
     const int gs = auto_group_size(h);
-    if (h->mix_panel_cols != 0 || gs >= 8 || gs == 0) return false;
+    const size_t matrix = (size_t)h->N * h->ld * sizeof(float);
+    if (gs >= 8) return false;
+    if (gs == 0) return h->nnz >= 6 * h->N && matrix > ((size_t)256 << 20);
     if (h->N <= 1024) return true;
     const bool two_ctas = (size_t)h->N * gs * 16 <= (size_t)h->smem_optin / 2 - 1024;
-    return !two_ctas || (size_t)h->N * h->ld * sizeof(float) > ((size_t)32 << 20);
+    return !two_ctas || matrix > ((size_t)32 << 20);
 }
 
 // The tensor-core kernel (dense 0/1 selection product) when asked for and applicable.

@@ -20,8 +20,9 @@ namespace dbw {
 
 namespace {
 
-constexpr int kProdWarps = 8, kConsWarps = 24;
-constexpr int kThreads = (kProdWarps + kConsWarps) * 32;  // 1024
+constexpr int kWarps = 32, kThreads = kWarps * 32;
+// Producer warps; the others are consumers.  Eight-column panels have little to gather and 32-byte row segments to fetch.
+__host__ __device__ constexpr int producer_warps(int W) { return W == 8 ? 16 : 8; }
 constexpr int kTmemCols = 256;                            // 128 lanes x 256 columns x 4 B = one 1024 x 32 panel
 constexpr int kMaxN = 4096;
 // Columns of a panel: the widest whose panel of all rows fits the 128 KB of tensor memory and shared memory it is given.
@@ -29,12 +30,8 @@ __host__ __device__ constexpr int staged_width(int N) { return N <= 1024 ? 32 : 
 // Bits of a list entry that hold the row index; with weighted lists the rest of its 16 bits is the weight code.
 __host__ __device__ constexpr int index_bits(int W) { return W == 32 ? 10 : W == 16 ? 11 : 12; }
 __host__ __device__ constexpr int zero_code(int W) { return (1 << (16 - index_bits(W))) - 1; }  // code of list padding: weight 0
-// Uniform 32-column lists hold the own row as a row's first entry (one padding read in two less: 1268 us against 1312 for 1024
-// workers x 262,144 columns, 32 neighbours); weighted and narrower ones do not (weighted: 1430 us against 1470).
-__host__ __device__ constexpr int listed_self(int W, bool weighted) { return W == 32 && !weighted ? 1 : 0; }
-__host__ __device__ constexpr int list_entries(int W, bool weighted, int maxdeg) {
-    return maxdeg + listed_self(W, weighted) < 4 ? 4 : (maxdeg + listed_self(W, weighted) + 3) / 4 * 4;
-}
+// 16-bit entries of a row's neighbour list: blocks of four.
+__host__ __device__ constexpr int list_entries(int maxdeg) { return maxdeg < 4 ? 4 : (maxdeg + 3) / 4 * 4; }
 
 // 1 / (1 + m) for the weight codes m of the weighted lists (Assumption 1: the weight worker i puts on a kept neighbour j is
 // 1 / (1 + max(p_i, p_j))), the same fp32 quotient the mixing plan holds.
@@ -96,27 +93,31 @@ struct StagedArgs {
 };
 
 // Shared memory: panel float4 [N + 1][W / 4] (row N is all zero: the target of list padding), then the neighbour lists
-// uint16 [N][list_row], then the per-row scale float [N], then the list lengths in blocks of 4, uint8 [N].
+// uint16 [N][list_row], 64 weights, and LOCAL: every row's own weight or scale, float [N], and list length in blocks of 4,
+// uint8 [N].  What a block leaves of the SM's 256 KB is L1, whose lines the loads on their way need, so those two stay in global
+// memory where they would make it the smallest (kRoomyBytes): 4096 workers, 65,536 columns, 8 neighbours 1348 us with 197 KB of
+// shared memory, 1709 with 217.  Where there is room they are better local: 3000 workers 878 us against 931.
+constexpr size_t kRoomyBytes = 195 * 1024;
 // WEIGHTED = false: uniform weights, a list entry is a bare 16-bit row index and the sum is scaled once per row.
 // WEIGHTED = true: a list entry is a row index and a weight code; padding is (own row, weight 0).
 // LPR lanes share an output row.  With weights and 128-byte rows there are four, each lane with two 16-byte pieces: two rows to
 // a quarter-warp phase of a 128-bit shared load, the odd groups of lanes reading the second half first so that the two never
-// share a bank.  A list or weight read then serves eight rows instead of four (1430 us against 1632 for 1024 workers x 262,144
-// columns, 32 neighbours).  Without weight reads eight lanes of one piece are better (1268 us against 1291).
-template <bool WEIGHTED, int W>
+// share a bank.  A list or weight read then serves eight rows instead of four (1418 us against 1632 for 1024 workers x 262,144
+// columns, 32 neighbours).  Without weight reads eight lanes of one piece are better (1254 us against 1288).
+template <bool WEIGHTED, int W, bool LOCAL>
 __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
     constexpr int SLOTS = W / 4, PIECES = W == 32 && WEIGHTED ? 2 : 1, LPR = SLOTS / PIECES, RPW = 32 / LPR;  // RPW: output rows per warp
-    constexpr bool SELF = listed_self(W, WEIGHTED) != 0;
     constexpr uint32_t kIdx = WEIGHTED ? (1u << index_bits(W)) - 1 : 0xffffu;
+    constexpr int kProdWarps = producer_warps(W), kConsWarps = kWarps - kProdWarps;
     constexpr int kCodeShift = index_bits(W), ZERO = zero_code(W);
     extern __shared__ float4 smem4[];
     float4* panel = smem4;
     const int N = a.N;
     const int lrow = a.list_row;
     uint16_t* lists = reinterpret_cast<uint16_t*>(panel + (size_t)(N + 1) * SLOTS);
-    float* scale = reinterpret_cast<float*>(lists + (size_t)N * lrow);
+    float* wtab = reinterpret_cast<float*>(lists + (size_t)N * lrow);  // weights by code (weighted lists)
+    float* scale = wtab + 64;
     uint8_t* nblk = reinterpret_cast<uint8_t*>(scale + N);
-    float* wtab = reinterpret_cast<float*>(nblk + (N + 15) / 16 * 16);  // weights by code (weighted lists)
     __shared__ uint32_t tmem_slot;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -129,20 +130,18 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
         const int i = e / (lrow / 4), k0 = (e % (lrow / 4)) * 4;
         const int cnt = a.plan.cnt[i];
         auto entry = [&](int k) -> uint32_t {
-            if (SELF && k == 0) return (uint32_t)i;
-            const int kk = k - (SELF ? 1 : 0);
-            if (!WEIGHTED) return kk < cnt ? (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) : (uint32_t)N;
-            if (kk >= cnt) return (uint32_t)i | ((uint32_t)ZERO << kCodeShift);
+            if (!WEIGHTED) return k < cnt ? (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + k], N, a.plan.status) : (uint32_t)N;
+            if (k >= cnt) return (uint32_t)i | ((uint32_t)ZERO << kCodeShift);
             // the plan's weight is 1 / (1 + m): recover m (exact for m <= 62) and keep it as the code
-            const int m = __float2int_rn(1.0f / a.plan.w[(size_t)i * a.plan.stride + kk]) - 1;
-            return (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + kk], N, a.plan.status) | ((uint32_t)min(max(m, 0), ZERO - 1) << kCodeShift);
+            const int m = __float2int_rn(1.0f / a.plan.w[(size_t)i * a.plan.stride + k]) - 1;
+            return (uint32_t)checked(a.plan.idx[(size_t)i * a.plan.stride + k], N, a.plan.status) | ((uint32_t)min(max(m, 0), ZERO - 1) << kCodeShift);
         };
         *reinterpret_cast<uint2*>(lists + (size_t)i * lrow + k0) =
             make_uint2(entry(k0) | (entry(k0 + 1) << 16), entry(k0 + 2) | (entry(k0 + 3) << 16));
     }
-    for (int i = tid; i < N; i += kThreads) {
+    for (int i = tid; LOCAL && i < N; i += kThreads) {
         scale[i] = a.plan.w_self[i];
-        nblk[i] = (uint8_t)max((a.plan.cnt[i] + (SELF ? 1 : 0) + 3) / 4, 1);  // a row without kept neighbours gathers one block
+        nblk[i] = (uint8_t)max((a.plan.cnt[i] + 3) / 4, 1);
     }
     if (WEIGHTED && tid <= ZERO) wtab[tid] = tid == ZERO ? 0.f : c_weight[tid];
     if (tid < SLOTS) panel[(size_t)N * SLOTS + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -157,7 +156,7 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
     const bool producer = warp < kProdWarps;
     // producer coordinates: row (within an iteration) and 16-byte slot of the row segment
     const int p_row = warp * RPS + lane / SLOTS, slot = lane % SLOTS;
-    const uint32_t p_taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * 128);
+    const uint32_t p_taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * (kTmemCols / (kProdWarps / 4)));
     // consumer coordinates: groups of LPR lanes, each owns rows grp, grp + kRowsPar, ...
     constexpr int kRowsPar = kConsWarps * RPW;
     const int grp = (warp - kProdWarps) * RPW + lane / LPR;
@@ -219,18 +218,17 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
         int i = grp;
         if (i >= N) return;
         const uint2* lp = reinterpret_cast<const uint2*>(lists + (size_t)i * lrow);
-        int nb = nblk[i], kb = 0;
+        auto blocks_of = [&](int row) -> int { return LOCAL ? nblk[row] : max((__ldg(a.plan.cnt + row) + 3) / 4, 1); };
+        auto self_weight = [&](int row) { return LOCAL ? scale[row] : __ldg(a.plan.w_self + row); };
+        int nb = blocks_of(i), kb = 0;  // a row without kept neighbours gathers one block
+        float ws = self_weight(i);
         uint2 u = lp[0];
         float4 acc[PIECES];
         auto first = [&](int row, float4 (&q)[PIECES]) {  // uniform: the own row, scaled with the sum at the end; weighted: own weight x own row
 #pragma unroll
             for (int h = 0; h < PIECES; ++h) {
-                if (SELF) {
-                    q[h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                } else {
-                    q[h] = panel[(size_t)row * SLOTS + piece[h]];
-                    if (WEIGHTED) q[h] = mul4(q[h], scale[row]);
-                }
+                q[h] = panel[(size_t)row * SLOTS + piece[h]];
+                if (WEIGHTED) q[h] = mul4(q[h], ws);
             }
         };
         first(i, acc);
@@ -266,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
 #pragma unroll
             for (int h = 0; h < PIECES; ++h) {
                 const long long c = (long long)pn * W + 4 * piece[h];
-                float4 o = WEIGHTED ? acc[h] : mul4(acc[h], scale[i]);
+                float4 o = WEIGHTED ? acc[h] : mul4(acc[h], ws);
                 if (c < a.ld) {
                     if (a.G && a.mix_then_correct) {
                         const float4 gi = ldg4(a.G + (size_t)i * a.ld + c);
@@ -281,7 +279,8 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
             if (i2 >= N) break;
             i = i2;
             lp = lp2;
-            nb = nblk[i];
+            nb = blocks_of(i);
+            ws = self_weight(i);
             kb = 0;
             first(i, acc);
         }
@@ -306,25 +305,32 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
     }
 }
 
-size_t staged_smem(const dbw_handle* h) {
+size_t staged_smem(const dbw_handle* h, bool local) {
     const size_t N = (size_t)h->N;
-    const int W = staged_width(h->N);
-    return (N + 1) * (size_t)(W * 4) + N * (size_t)list_entries(W, !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg) * 2 + N * 4 + ((N + 15) / 16) * 16 + 256;
+    return (N + 1) * (size_t)(staged_width(h->N) * 4) + N * (size_t)list_entries(h->maxdeg) * 2 + 256 + (local ? (N * 5 + 15) / 16 * 16 : 0);
 }
+bool staged_local(const dbw_handle* h) { return staged_smem(h, true) <= kRoomyBytes && list_entries(h->maxdeg) <= 4 * 255; }
 
-template <bool WEIGHTED, int W>
+template <bool WEIGHTED, int W, bool LOCAL>
 int launch_staged(const dbw_handle* h, StagedArgs& a, cudaStream_t s) {
     static PerDeviceOnce once;
     const int rc = once.run(h->device, [h]() -> int {
-        DBW_CUDA(cudaFuncSetAttribute(mix_staged_kernel<WEIGHTED, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 256));
+        DBW_CUDA(cudaFuncSetAttribute(mix_staged_kernel<WEIGHTED, W, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin - 256));
         return DBW_OK;
     });
     if (rc) return rc;
     a.n_panels = (int)((h->ld + W - 1) / W);
     const int grid = a.n_panels < h->sm_count ? a.n_panels : h->sm_count;
-    mix_staged_kernel<WEIGHTED, W><<<grid, kThreads, staged_smem(h), s>>>(a);
+    mix_staged_kernel<WEIGHTED, W, LOCAL><<<grid, kThreads, staged_smem(h, LOCAL), s>>>(a);
     DBW_LAUNCHED();
     return DBW_OK;
+}
+
+template <int W>
+int launch_staged_width(const dbw_handle* h, StagedArgs& a, cudaStream_t s) {
+    const bool uniform = (h->flags & DBW_WEIGHT_UNIFORM) != 0;
+    if (staged_local(h)) return uniform ? launch_staged<false, W, true>(h, a, s) : launch_staged<true, W, true>(h, a, s);
+    return uniform ? launch_staged<false, W, false>(h, a, s) : launch_staged<true, W, false>(h, a, s);
 }
 
 }  // namespace
@@ -334,8 +340,7 @@ int launch_staged(const dbw_handle* h, StagedArgs& a, cudaStream_t s) {
 bool mix_staged_usable(const dbw_handle* h) {
     if (h->N > kMaxN || h->N < 64) return false;
     if (!(h->flags & DBW_WEIGHT_UNIFORM) && h->maxdeg > zero_code(staged_width(h->N)) - 1) return false;
-    if (list_entries(staged_width(h->N), !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg) > 4 * 255) return false;  // lengths are counted in blocks of 4, in a byte
-    return staged_smem(h) + 256 <= (size_t)h->smem_optin;
+    return staged_smem(h, false) + 256 <= (size_t)h->smem_optin;
 }
 
 int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
@@ -345,13 +350,12 @@ int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, c
     a.ld = h->ld;
     a.mix_then_correct = (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0;
     const int W = staged_width(h->N);
-    a.list_row = list_entries(W, !(h->flags & DBW_WEIGHT_UNIFORM), h->maxdeg);
+    a.list_row = list_entries(h->maxdeg);
     a.X = X; a.G = G; a.lr = lr; a.lr_pw = lr_pw; a.Xout = X_out; a.shadow = shadow; a.plan = h->plan;
-    const bool uniform = (h->flags & DBW_WEIGHT_UNIFORM) != 0;
     switch (W) {
-        case 32: return uniform ? launch_staged<false, 32>(h, a, s) : launch_staged<true, 32>(h, a, s);
-        case 16: return uniform ? launch_staged<false, 16>(h, a, s) : launch_staged<true, 16>(h, a, s);
-        default: return uniform ? launch_staged<false, 8>(h, a, s) : launch_staged<true, 8>(h, a, s);
+        case 32: return launch_staged_width<32>(h, a, s);
+        case 16: return launch_staged_width<16>(h, a, s);
+        default: return launch_staged_width<8>(h, a, s);
     }
 }
 
