@@ -186,6 +186,8 @@ int launch_plan_from_kept(dbw_handle* h, const uint8_t* kept, const int32_t* b, 
 // mix.cu
 int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
                cudaStream_t s);
+// Asks L2 for the line of `p`: nothing waits for it and no register is held; a later load then comes from L2.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // device helper shared by the mix kernels: four floats -> four bf16 (round to nearest even)
 __device__ __forceinline__ uint2 pack_bf16x4_rn(float a, float b, float c, float d) {
     uint32_t lo, hi;

@@ -346,7 +346,12 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     if (use_sp(h)) return launch_mix_sp(h, X, G, lr, lr_pw, X_out, shadow, s);
     if (use_tc(h)) return launch_mix_tc(h, X, G, lr, lr_pw, X_out, shadow, s);
     if (use_staged(h)) return launch_mix_staged(h, X, G, lr, lr_pw, X_out, shadow, s);
-    switch (auto_group_size(h)) {
+    int gs = auto_group_size(h);
+    // 64 instead of 128 columns: twice the panels spread more evenly over the blocks, and the row segments are still two lines
+    // (96 workers x 300,007 columns, 5.3 or 10.6 panels a block: 111 -> 104 us in Eq. 3's order, 114 -> 108 in Algorithm 1's;
+    // 128 x 2,000,000, 35 or 70 panels a block: 757 and 760)
+    if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) gs = 16;
+    switch (gs) {
         case 64: return launch_panel<64>(h, X, G, lr, lr_pw, X_out, shadow, s);
         case 32: return launch_panel<32>(h, X, G, lr, lr_pw, X_out, shadow, s);
         case 16: return launch_panel<16>(h, X, G, lr, lr_pw, X_out, shadow, s);
