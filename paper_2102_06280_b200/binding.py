@@ -153,14 +153,25 @@ def _ptr(t) -> Optional[int]:
     """Address of a torch tensor / numpy array (None stays NULL)."""
     if t is None:
         return None
-    if isinstance(t, np.ndarray):
+    try:
+        return t.data_ptr()
+    except AttributeError:
         return t.ctypes.data
-    return t.data_ptr()
+
+
+_raw_stream = None
 
 
 def _stream() -> int:
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    """The current stream of the current device.  A call of the library is queued in 3 - 5 us, of which building a
+    torch.cuda.Stream object takes one or two, so the handle is asked of torch directly where it offers that."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()  # initialises CUDA
+        raw, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        _raw_stream = (lambda: raw(dev())) if raw and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+    return _raw_stream()
 
 
 class Dbw:
@@ -179,7 +190,8 @@ class Dbw:
         self.device = device
         self._h = _P()
         self._keep = None
-        _check(lib().dbw_init(C.byref(self._h), self.N, self.d, self.ld, rowptr.ctypes.data, col.ctypes.data,
+        self._lib = lib()
+        _check(self._lib.dbw_init(C.byref(self._h), self.N, self.d, self.ld, rowptr.ctypes.data, col.ctypes.data,
                               C.byref(model.desc) if model else None, flags, device), "dbw_init")
 
     def close(self):
@@ -195,91 +207,91 @@ class Dbw:
 
     def set_dataset(self, feat, labels, S: int):
         self._keep = (feat, labels)
-        _check(lib().dbw_set_dataset(self._h, _ptr(feat), _ptr(labels), int(S)), "dbw_set_dataset")
+        _check(self._lib.dbw_set_dataset(self._h, _ptr(feat), _ptr(labels), int(S)), "dbw_set_dataset")
 
     def set_edge_times(self, t_edge):
         self._keep_edge = t_edge
-        _check(lib().dbw_set_edge_times(self._h, _ptr(t_edge)), "dbw_set_edge_times")
+        _check(self._lib.dbw_set_edge_times(self._h, _ptr(t_edge)), "dbw_set_edge_times")
 
     def select(self, t, b, kept, T_worker=None, T_nbr=None, T_round=None):
-        _check(lib().dbw_select(self._h, _ptr(t), _ptr(b), _ptr(kept), _ptr(T_worker), _ptr(T_nbr), _ptr(T_round),
+        _check(self._lib.dbw_select(self._h, _ptr(t), _ptr(b), _ptr(kept), _ptr(T_worker), _ptr(T_nbr), _ptr(T_round),
                                 _stream()), "dbw_select")
 
     def grad(self, X, batch_idx, G, loss=None):
-        _check(lib().dbw_grad(self._h, _ptr(X), _ptr(batch_idx), _ptr(G), _ptr(loss), _stream()), "dbw_grad")
+        _check(self._lib.dbw_grad(self._h, _ptr(X), _ptr(batch_idx), _ptr(G), _ptr(loss), _stream()), "dbw_grad")
 
     def mix(self, X, G, kept, b, lr: float, X_out, lr_per_worker=None):
-        _check(lib().dbw_mix(self._h, _ptr(X), _ptr(G), _ptr(kept), _ptr(b), float(lr), _ptr(lr_per_worker),
+        _check(self._lib.dbw_mix(self._h, _ptr(X), _ptr(G), _ptr(kept), _ptr(b), float(lr), _ptr(lr_per_worker),
                              _ptr(X_out), _stream()), "dbw_mix")
 
     def mix_in_place_ok(self) -> bool:
-        return bool(lib().dbw_mix_in_place_ok(self._h))
+        return bool(self._lib.dbw_mix_in_place_ok(self._h))
 
     def set_param_tracking(self, enable: bool):
-        _check(lib().dbw_set_param_tracking(self._h, int(bool(enable))), "dbw_set_param_tracking")
+        _check(self._lib.dbw_set_param_tracking(self._h, int(bool(enable))), "dbw_set_param_tracking")
 
     def set_fused_round(self, enable):
         """True / False, or None for the library's own choice."""
-        _check(lib().dbw_set_fused_round(self._h, -1 if enable is None else int(bool(enable))), "dbw_set_fused_round")
+        _check(self._lib.dbw_set_fused_round(self._h, -1 if enable is None else int(bool(enable))), "dbw_set_fused_round")
 
     def round_is_fused(self) -> bool:
-        return bool(_check(lib().dbw_round_is_fused(self._h), "dbw_round_is_fused"))
+        return bool(_check(self._lib.dbw_round_is_fused(self._h), "dbw_round_is_fused"))
 
     def mix_kernel(self) -> str:
-        return ("mix_direct_kernel", "mix_panel_kernel", "mix_staged_kernel", "mix_tc_kernel", "mix_sp_kernel")[_check(lib().dbw_mix_kernel(self._h), "dbw_mix_kernel")]
+        return ("mix_direct_kernel", "mix_panel_kernel", "mix_staged_kernel", "mix_tc_kernel", "mix_sp_kernel")[_check(self._lib.dbw_mix_kernel(self._h), "dbw_mix_kernel")]
 
     def set_mix_panel(self, cols: int):
-        _check(lib().dbw_set_mix_panel(self._h, int(cols)), "dbw_set_mix_panel")
+        _check(self._lib.dbw_set_mix_panel(self._h, int(cols)), "dbw_set_mix_panel")
 
     def round(self, X, t, b, lr: float, X_out, kept, batch_idx=None, G_ext=None, lr_per_worker=None,
               T_worker=None, T_nbr=None, T_round=None, loss=None):
-        _check(lib().dbw_round(self._h, _ptr(X), _ptr(t), _ptr(b), _ptr(batch_idx), _ptr(G_ext), float(lr),
+        _check(self._lib.dbw_round(self._h, _ptr(X), _ptr(t), _ptr(b), _ptr(batch_idx), _ptr(G_ext), float(lr),
                                _ptr(lr_per_worker), _ptr(X_out), _ptr(kept), _ptr(T_worker), _ptr(T_nbr),
                                _ptr(T_round), _ptr(loss), _stream()), "dbw_round")
 
     def round_host(self, X, h_t, h_b, lr: float, X_out, h_batch_idx=None, G_ext=None, h_kept=None,
                    h_T_worker=None, h_T_round=None, h_loss=None, h_b_out=None):
-        _check(lib().dbw_round_host(self._h, _ptr(X), _ptr(h_t), _ptr(h_b), _ptr(h_batch_idx), _ptr(G_ext),
+        _check(self._lib.dbw_round_host(self._h, _ptr(X), _ptr(h_t), _ptr(h_b), _ptr(h_batch_idx), _ptr(G_ext),
                                     float(lr), _ptr(X_out), _ptr(h_kept), _ptr(h_T_worker), _ptr(h_T_round),
                                     _ptr(h_loss), _ptr(h_b_out), _stream()), "dbw_round_host")
 
     def update_backups(self, t_next, b_out, theta_out=None):
-        _check(lib().dbw_update_backups(self._h, _ptr(t_next), _ptr(b_out), _ptr(theta_out), _stream()),
+        _check(self._lib.dbw_update_backups(self._h, _ptr(t_next), _ptr(b_out), _ptr(theta_out), _stream()),
                "dbw_update_backups")
 
     def reset_backups(self):
-        _check(lib().dbw_reset_backups(self._h, _stream()), "dbw_reset_backups")
+        _check(self._lib.dbw_reset_backups(self._h, _stream()), "dbw_reset_backups")
 
     def state_export(self) -> bytes:
         size = C.c_size_t(0)
-        _check(lib().dbw_state_export(self._h, None, C.byref(size), _stream()), "dbw_state_export")
+        _check(self._lib.dbw_state_export(self._h, None, C.byref(size), _stream()), "dbw_state_export")
         buf = C.create_string_buffer(size.value)
-        _check(lib().dbw_state_export(self._h, buf, C.byref(size), _stream()), "dbw_state_export")
+        _check(self._lib.dbw_state_export(self._h, buf, C.byref(size), _stream()), "dbw_state_export")
         return buf.raw[: size.value]
 
     def state_import(self, blob: bytes):
-        _check(lib().dbw_state_import(self._h, blob, len(blob), _stream()), "dbw_state_import")
+        _check(self._lib.dbw_state_import(self._h, blob, len(blob), _stream()), "dbw_state_import")
 
     def profile(self, enable: bool):
-        _check(lib().dbw_profile(self._h, int(bool(enable))), "dbw_profile")
+        _check(self._lib.dbw_profile(self._h, int(bool(enable))), "dbw_profile")
 
     def profile_read(self):
         """({'grad': ms, 'select': ms, 'mix': ms, 'gemm': ms}, rounds) accumulated since the last read
         ('gemm' = the tensor-core GEMM launches inside the gradient stage)."""
         ms = (C.c_double * 4)(0.0, 0.0, 0.0, 0.0)
         n = C.c_int32(0)
-        _check(lib().dbw_profile_read(self._h, ms, C.byref(n)), "dbw_profile_read")
+        _check(self._lib.dbw_profile_read(self._h, ms, C.byref(n)), "dbw_profile_read")
         return {"grad": ms[0], "select": ms[1], "mix": ms[2], "gemm": ms[3]}, int(n.value)
 
     def debug_wait_probe(self, polls: int, out):
-        _check(lib().dbw_debug_wait_probe(self._h, int(polls), _ptr(out), _stream()), "dbw_debug_wait_probe")
+        _check(self._lib.dbw_debug_wait_probe(self._h, int(polls), _ptr(out), _stream()), "dbw_debug_wait_probe")
 
     def status(self) -> int:
-        return _check(lib().dbw_status(self._h), "dbw_status")
+        return _check(self._lib.dbw_status(self._h), "dbw_status")
 
     def links(self) -> np.ndarray:
         out = np.zeros((max(self.N - 1, 0), 2), dtype=np.int32)
-        _check(lib().dbw_get_links(self._h, out.ctypes.data), "dbw_get_links")
+        _check(self._lib.dbw_get_links(self._h, out.ctypes.data), "dbw_get_links")
         return out
 
 

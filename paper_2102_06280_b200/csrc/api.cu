@@ -19,11 +19,15 @@ namespace {
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct DeviceGuard {
-    int prev = -1;
+    int prev = -1;  // the device to go back to, if it was another one
     bool ok = true;
     explicit DeviceGuard(int dev) {
-        ok = cuda_ok(cudaGetDevice(&prev));
-        if (ok && prev != dev) ok = cuda_ok(cudaSetDevice(dev));
+        int cur = -1;
+        ok = cuda_ok(cudaGetDevice(&cur));
+        if (ok && cur != dev) {
+            prev = cur;
+            ok = cuda_ok(cudaSetDevice(dev));
+        }
     }
     ~DeviceGuard() {
         if (prev >= 0) cudaSetDevice(prev);
