@@ -31,6 +31,7 @@ update_backups_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* 
                       const int32_t* __restrict__ links, int32_t* covered, int32_t* epoch,
                       const double* __restrict__ t, int32_t* __restrict__ b_out, double* theta_out,
                       uint32_t* status) {
+    dependent_begin();
     extern __shared__ double times[];
     const int D = N - 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -184,13 +185,13 @@ update_backups_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* 
 
 int launch_update_backups(dbw_handle* h, const double* t, int32_t* b_out, double* theta_out, cudaStream_t s) {
     if (h->N <= kPer * kThreads / 8)
-        update_backups_kernel<true, 8><<<1, kThreads, (size_t)h->N * sizeof(double), s>>>(h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered,
+        launch(update_backups_kernel<true, 8>, 1, kThreads, (size_t)h->N * sizeof(double), s, h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered,
                                                                                          h->d_epoch, t, b_out, theta_out, h->d_status);
     else if (h->N <= kMaxStaged)
-        update_backups_kernel<true, 1><<<1, kThreads, (size_t)h->N * sizeof(double), s>>>(h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered,
+        launch(update_backups_kernel<true, 1>, 1, kThreads, (size_t)h->N * sizeof(double), s, h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered,
                                                                                       h->d_epoch, t, b_out, theta_out, h->d_status);
     else
-        update_backups_kernel<false, 1><<<1, kThreads, 0, s>>>(h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered, h->d_epoch, t, b_out,
+        launch(update_backups_kernel<false, 1>, 1, kThreads, 0, s, h->N, h->d_rowptr, h->d_col, h->d_links, h->d_covered, h->d_epoch, t, b_out,
                                                             theta_out, h->d_status);
     DBW_LAUNCHED();
     return DBW_OK;

@@ -95,6 +95,7 @@ template <int STAGES, int BN, int ACC, bool BMN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs g, int tiles_m,
                int tiles_n, int n_tiles) {
+    dependent_begin();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int TILE_B_BYTES = BN * BK * 2;
@@ -297,6 +298,7 @@ template <int BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_dw_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ DwArgs g, int tiles_m, int tiles_n,
                int n_tiles) {
+    dependent_begin();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int STAGES = dw_stages(BN), TILE_B_BYTES = BN * BK * 2;
@@ -497,6 +499,7 @@ __global__ void __launch_bounds__(256)
 cast_tile_kernel(int rows, int cols, const float* __restrict__ src, long long src_z, long long src_pitch,
                  const int32_t* __restrict__ row_idx, int idx_z, int idx_limit, bf16* __restrict__ dst, long long dst_z,
                  const int32_t* __restrict__ labels, int C, int32_t* __restrict__ ylab, uint32_t* status) {
+    dependent_begin();
     const int z = blockIdx.z;
     const int t = threadIdx.x;
     const int r = blockIdx.y * 64 + (t >> 2);
@@ -570,6 +573,7 @@ template <int CP, int HS>
 __global__ void __launch_bounds__(128)
 head_forward_kernel(int B, int K, int C, const bf16* __restrict__ A, const float* __restrict__ X, long long ld, long long w_off,
                     long long b_off, const int32_t* __restrict__ ylab, float* __restrict__ dzL, float* __restrict__ loss_s) {
+    dependent_begin();
     const int i = blockIdx.y;
     const int s0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * HS;
     const int lane = threadIdx.x & 31;
@@ -652,6 +656,7 @@ __global__ void __launch_bounds__(256, 2)
 head_forward_staged_kernel(int N, int B, int K, int C, const bf16* __restrict__ A, const float* __restrict__ X, long long ld,
                            long long w_off, long long b_off, const int32_t* __restrict__ ylab, float* __restrict__ dzL,
                            float* __restrict__ loss_s) {
+    dependent_begin();
     extern __shared__ float4 sw4[];  // [C][K]
     const float* sw = reinterpret_cast<const float*>(sw4);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -765,6 +770,7 @@ __global__ void __launch_bounds__(64)
 head_backward_kernel(int B, int K, int C, const bf16* __restrict__ A, const float* __restrict__ X, long long ld,
                      long long w_off, const float* __restrict__ dzL, float* __restrict__ G, float* __restrict__ dwp,
                      bf16* __restrict__ dzP) {
+    dependent_begin();
     // blockIdx.z splits the batch (in chunks of 8 samples) so that enough blocks are in flight; with
     // more than one part the dW partial sums go to dwp [part][worker][C][K] and grad_tail_kernel
     // adds them in a fixed order.
@@ -890,6 +896,7 @@ struct TailArgs {
 };
 
 __global__ void __launch_bounds__(256) grad_tail_kernel(TailArgs a) {
+    dependent_begin();
     __shared__ float2 part[4][64];
     const int bx = blockIdx.x, i = blockIdx.y;
     for (int t = 0; t < a.n_bias; ++t)
@@ -981,9 +988,9 @@ int run_tc_major(const dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b
     });
     if (rc) return rc;
     if (bn == 128)
-        gemm_tc_kernel<4, 128, 2, BMN><<<grid, GEMM_THREADS, gemm_smem(4, 128), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+        launch(gemm_tc_kernel<4, 128, 2, BMN>, grid, GEMM_THREADS, gemm_smem(4, 128), s, a, b, g, tiles_m, tiles_n, n_tiles);
     else
-        gemm_tc_kernel<3, 256, 2, BMN><<<grid, GEMM_THREADS, gemm_smem(3, 256), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+        launch(gemm_tc_kernel<3, 256, 2, BMN>, grid, GEMM_THREADS, gemm_smem(3, 256), s, a, b, g, tiles_m, tiles_n, n_tiles);
     DBW_LAUNCHED();
     return DBW_OK;
 }
@@ -1025,7 +1032,7 @@ int launch_dw(const dbw_handle* h, const CUtensorMap& a, const CUtensorMap& b, c
         return DBW_OK;
     });
     if (rc) return rc;
-    gemm_dw_kernel<BN><<<grid, GEMM_THREADS, dw_smem(BN), s>>>(a, b, g, tiles_m, tiles_n, n_tiles);
+    launch(gemm_dw_kernel<BN>, grid, GEMM_THREADS, dw_smem(BN), s, a, b, g, tiles_m, tiles_n, n_tiles);
     DBW_LAUNCHED();
     return DBW_OK;
 }
@@ -1111,13 +1118,11 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     const bool have_shadow = h->track_params && h->shadow_valid && h->shadow_of == X;
     for (int l = 0; l <= L - 2 && !have_shadow; ++l) {
         const int in = m.dims[l], out = m.dims[l + 1];
-        cast_tile_kernel<<<dim3((in + 63) / 64, (out + 63) / 64, N), 256, 0, s>>>(
-            out, in, X + m.w_off[l], h->ld, in, nullptr, 0, 0, st->Wh[l], h->ld, nullptr, 0, nullptr, h->d_status);
+        launch(cast_tile_kernel, dim3((in + 63) / 64, (out + 63) / 64, N), 256, 0, s, out, in, X + m.w_off[l], h->ld, in, nullptr, 0, 0, st->Wh[l], h->ld, nullptr, 0, nullptr, h->d_status);
         DBW_LAUNCHED();
     }
     // mini-batch gather: A_0 in bf16, and the labels
-    cast_tile_kernel<<<dim3((m.dims[0] + 63) / 64, (B + 63) / 64, N), 256, 0, s>>>(
-        B, m.dims[0], h->feat, (long long)h->S * m.dims[0], m.dims[0], batch_idx, B, h->S, st->A[0], (long long)B * m.dims[0],
+    launch(cast_tile_kernel, dim3((m.dims[0] + 63) / 64, (B + 63) / 64, N), 256, 0, s, B, m.dims[0], h->feat, (long long)h->S * m.dims[0], m.dims[0], batch_idx, B, h->S, st->A[0], (long long)B * m.dims[0],
         h->labels, C, st->ylab, h->d_status);
     DBW_LAUNCHED();
     // forward through the tensor-core layers
@@ -1138,29 +1143,26 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         const int items = N * ((B + 31) / 32);
         const int grid = std::min(items, 2 * h->sm_count);
         if (C <= 12)  // ten classes: a quarter fewer accumulators than with the 16-class instance
-            head_forward_staged_kernel<12, 4><<<grid, 256, w_bytes, s>>>(N, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
+            launch(head_forward_staged_kernel<12, 4>, grid, 256, w_bytes, s, N, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                          st->ylab, st->dzL, st->loss_s);
         else
-            head_forward_staged_kernel<16, 4><<<grid, 256, w_bytes, s>>>(N, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
+            launch(head_forward_staged_kernel<16, 4>, grid, 256, w_bytes, s, N, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                          st->ylab, st->dzL, st->loss_s);
     } else if (C <= 16) {
-        head_forward_kernel<16, 2><<<dim3((B + 7) / 8, N), 128, 0, s>>>(B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1],
+        launch(head_forward_kernel<16, 2>, dim3((B + 7) / 8, N), 128, 0, s, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1],
                                                                        m.b_off[L - 1], st->ylab, st->dzL, st->loss_s);
     } else {
-        head_forward_kernel<32, 2><<<dim3((B + 7) / 8, N), 128, 0, s>>>(B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1],
+        launch(head_forward_kernel<32, 2>, dim3((B + 7) / 8, N), 128, 0, s, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1],
                                                                        m.b_off[L - 1], st->ylab, st->dzL, st->loss_s);
     }
     DBW_LAUNCHED();
     const int parts = B >= 64 ? 4 : 1;
     if (C <= 12)  // ten classes: a quarter fewer multiply-adds than with the 16-class instance
-        head_backward_kernel<12, 2><<<dim3((K + 127) / 128, N, parts), 64, (size_t)B * 12 * 4, s>>>(
-            B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
+        launch(head_backward_kernel<12, 2>, dim3((K + 127) / 128, N, parts), 64, (size_t)B * 12 * 4, s, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
     else if (C <= 16)
-        head_backward_kernel<16, 2><<<dim3((K + 127) / 128, N, parts), 64, (size_t)B * 16 * 4, s>>>(
-            B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
+        launch(head_backward_kernel<16, 2>, dim3((K + 127) / 128, N, parts), 64, (size_t)B * 16 * 4, s, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
     else
-        head_backward_kernel<32, 1><<<dim3((K + 63) / 64, N, parts), 64, (size_t)B * 32 * 4, s>>>(
-            B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
+        launch(head_backward_kernel<32, 1>, dim3((K + 63) / 64, N, parts), 64, (size_t)B * 32 * 4, s, B, K, C, st->A[L - 1], X, h->ld, m.w_off[L - 1], st->dzL, G, st->dwp, dzP);
     DBW_LAUNCHED();
     // backward through the tensor-core layers; dA_l before dW_l, which may replace the bf16 copy of W_l
     if (step) DBW_CUDA(cudaStreamWaitEvent(s, step->selected, 0));
@@ -1203,7 +1205,7 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     t.B = B; t.K = K; t.C = C; t.parts = parts; t.workers = N;
     t.dwp = st->dwp; t.dzL = st->dzL; t.loss_s = st->loss_s; t.loss = loss;
     t.G = G; t.ld = h->ld; t.w_off_last = m.w_off[L - 1]; t.b_off_last = m.b_off[L - 1];
-    grad_tail_kernel<<<dim3(next + 1, N), 256, 0, s>>>(t);
+    launch(grad_tail_kernel, dim3(next + 1, N), 256, 0, s, t);
     DBW_LAUNCHED();
     return DBW_OK;
 }

@@ -14,11 +14,13 @@ using namespace dev;
 __global__ void gather_batch_kernel(int B, int S, int in_dim, int C, const float* __restrict__ feat,
                                     const int32_t* __restrict__ labels, const int32_t* __restrict__ batch_idx,
                                     float* __restrict__ A0, int32_t* __restrict__ ylab, uint32_t* status) {
+    dependent_begin();
     gather_row(blockIdx.x, blockIdx.y, B, S, in_dim, C, feat, labels, batch_idx, A0, ylab, status);
 }
 
 template <int R, int TK>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
+    dependent_begin();
     constexpr int T = 16 * R;
     __shared__ __align__(16) float As[TK][T + 4];
     __shared__ __align__(16) float Bs[TK][T + 4];
@@ -28,12 +30,14 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
 __global__ void __launch_bounds__(256)
 softmax_ce_kernel(int B, int C, const float* __restrict__ logits, const int32_t* __restrict__ ylab,
                   float* dz, float* __restrict__ loss, float* __restrict__ G, long long ld, long long b_off) {
+    dependent_begin();
     __shared__ float sl[8];
     softmax_ce_worker(blockIdx.x, B, C, logits, ylab, dz, loss, G, ld, b_off, sl);
 }
 
 __global__ void bias_grad_kernel(int B, int out_dim, const float* __restrict__ dz, float* __restrict__ G,
                                  long long ld, long long b_off) {
+    dependent_begin();
     bias_grad_col(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, B, out_dim, dz, G, ld, b_off);
 }
 
@@ -48,6 +52,7 @@ __global__ void bias_grad_kernel(int B, int out_dim, const float* __restrict__ d
 // SUMS: the blocks of the first columns also add every row of A over k (g.rowsum): the bias gradient of a dW GEMM.
 template <int WM, int RM, bool SUMS>
 __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
+    dependent_begin();
     constexpr int BM = 2 * RM * WM, BN = 64, TK = 16, THREADS = 32 * WM;
     constexpr int PA = BM * TK / 4 / THREADS, PB = BN * TK / 4 / THREADS;  // float4 per thread and k-step
     __shared__ __align__(16) float As[TK][BM + 4];
@@ -181,6 +186,7 @@ template <int CP>
 __global__ void __launch_bounds__(256)
 last_layer_forward_kernel(int N, int B, int in, int C, HeadRows rows, const float* __restrict__ X, long long ld, long long w_off,
                           long long b_off, float* __restrict__ dz, float* __restrict__ loss_s, uint32_t* status) {
+    dependent_begin();
     const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (item >= N * B) return;
     const int i = item / B;
@@ -192,6 +198,7 @@ __global__ void __launch_bounds__(256)
 last_layer_backward_kernel(int B, int in, int C, HeadRows rows, const float* __restrict__ dz, const float* __restrict__ loss_s,
                            const float* __restrict__ X, float* __restrict__ G, long long ld, long long w_off, long long b_off,
                            float* __restrict__ loss, float* __restrict__ dz_prev, long long b_off_prev, float* __restrict__ partial, uint32_t* status) {
+    dependent_begin();
     extern __shared__ __align__(16) float head_smem[];
     const int i = blockIdx.y, k_lo = blockIdx.x * kHeadChunk4;
     const int k_hi = min(in >> 2, k_lo + kHeadChunk4);
@@ -212,6 +219,7 @@ last_layer_backward_kernel(int B, int in, int C, HeadRows rows, const float* __r
 __global__ void __launch_bounds__(256)
 last_layer_add_parts_kernel(int parts, int N, int B, int in, int C, const float* __restrict__ partial, float* __restrict__ G, long long ld, long long w_off,
                             long long b_off, long long b_off_prev, float* __restrict__ loss) {
+    dependent_begin();
     const int i = blockIdx.y, e = blockIdx.x * 256 + threadIdx.x;
     float* Gi = G + (size_t)i * ld;
     if (e <= C * in + C + in) head_add_parts(i, e, parts, N, B, in, C, partial, Gi + w_off, Gi + b_off, b_off_prev >= 0 ? Gi + b_off_prev : nullptr, loss ? loss + i : nullptr);
@@ -221,9 +229,9 @@ template <int WM, int RM>
 void launch_gemm_vec(const GemmArgs& g, int batch, cudaStream_t s) {
     const dim3 grid((g.N + 63) / 64, (g.M + 2 * RM * WM - 1) / (2 * RM * WM), batch);
     if (g.rowsum)
-        gemm_vec_kernel<WM, RM, true><<<grid, 32 * WM, 0, s>>>(g);
+        launch<false>(gemm_vec_kernel<WM, RM, true>, grid, 32 * WM, 0, s, g);
     else
-        gemm_vec_kernel<WM, RM, false><<<grid, 32 * WM, 0, s>>>(g);
+        launch<false>(gemm_vec_kernel<WM, RM, false>, grid, 32 * WM, 0, s, g);
 }
 
 int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
@@ -244,14 +252,14 @@ int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
     const long long big = (long long)((g.N + 63) / 64) * ((g.M + 63) / 64) * batch;
     if (big >= 4LL * sm_count) {
         dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, batch);
-        gemm_simt_kernel<4, 16><<<grid, 256, 0, s>>>(g);
+        launch<false>(gemm_simt_kernel<4, 16>, grid, 256, 0, s, g);
     } else {
         dim3 grid((g.N + 31) / 32, (g.M + 31) / 32, batch);
         const long long ctas = (long long)grid.x * grid.y * grid.z;
         if (g.K >= 128 && ctas < 2LL * sm_count)  // few CTAs, long reduction
-            gemm_simt_kernel<2, 64><<<grid, 256, 0, s>>>(g);
+            launch<false>(gemm_simt_kernel<2, 64>, grid, 256, 0, s, g);
         else
-            gemm_simt_kernel<2, 16><<<grid, 256, 0, s>>>(g);
+            launch<false>(gemm_simt_kernel<2, 16>, grid, 256, 0, s, g);
     }
     DBW_LAUNCHED();
     return DBW_OK;
@@ -294,7 +302,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     const bool head = fp32_head_usable(h) && (((uintptr_t)X | (uintptr_t)G) & 15) == 0;
     const int Lg = head ? L - 1 : L;  // layers that run as GEMMs
     if (Lg > 0 || !head) {
-        gather_batch_kernel<<<dim3(B, N), 128, 0, s>>>(B, h->S, m.dims[0], m.dims[L], h->feat, h->labels, batch_idx,
+        launch(gather_batch_kernel, dim3(B, N), 128, 0, s, B, h->S, m.dims[0], m.dims[L], h->feat, h->labels, batch_idx,
                                                        h->d_act[0], h->d_ylab, h->d_status);
         DBW_LAUNCHED();
     }
@@ -326,26 +334,26 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         const long long b_prev = L > 1 ? m.b_off[L - 2] : -1;
         const size_t smem = fp32_head_smem_bytes(B, C);
         if (C <= 16) {
-            last_layer_forward_kernel<16><<<(N * B + 7) / 8, 256, 0, s>>>(N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
+            launch<false>(last_layer_forward_kernel<16>, (N * B + 7) / 8, 256, 0, s, N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                           h->d_dz[L], loss_s, h->d_status);
             DBW_LAUNCHED();
-            last_layer_backward_kernel<16><<<bgrid, 256, smem, s>>>(B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
+            launch<false>(last_layer_backward_kernel<16>, bgrid, 256, smem, s, B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
                                                                     m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
         } else {
-            last_layer_forward_kernel<32><<<(N * B + 7) / 8, 256, 0, s>>>(N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
+            launch<false>(last_layer_forward_kernel<32>, (N * B + 7) / 8, 256, 0, s, N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
                                                                           h->d_dz[L], loss_s, h->d_status);
             DBW_LAUNCHED();
-            last_layer_backward_kernel<32><<<bgrid, 256, smem, s>>>(B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
+            launch<false>(last_layer_backward_kernel<32>, bgrid, 256, smem, s, B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
                                                                     m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
         }
         DBW_LAUNCHED();
         if (parts > 1) {
-            last_layer_add_parts_kernel<<<dim3((C * in + C + in + 256) / 256, N), 256, 0, s>>>(parts, N, B, in, C, h->d_head_part, G, h->ld, m.w_off[L - 1],
+            launch(last_layer_add_parts_kernel, dim3((C * in + C + in + 256) / 256, N), 256, 0, s, parts, N, B, in, C, h->d_head_part, G, h->ld, m.w_off[L - 1],
                                                                                             m.b_off[L - 1], b_prev, loss);
             DBW_LAUNCHED();
         }
     } else {
-        softmax_ce_kernel<<<N, 256, 0, s>>>(B, m.dims[L], h->d_act[L], h->d_ylab, h->d_dz[L], loss, G, h->ld, m.b_off[L - 1]);
+        launch<false>(softmax_ce_kernel, N, 256, 0, s, B, m.dims[L], h->d_act[L], h->d_ylab, h->d_dz[L], loss, G, h->ld, m.b_off[L - 1]);
         DBW_LAUNCHED();
     }
     // backward
@@ -363,7 +371,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         }
         if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
         if (needs_db && !db_here) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
-            bias_grad_kernel<<<dim3((out + 127) / 128, N), 128, 0, s>>>(B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
+            launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
             DBW_LAUNCHED();
         }
         if (l > 0) {  // dZ_{l}[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]

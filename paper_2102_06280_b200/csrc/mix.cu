@@ -27,6 +27,7 @@ __global__ void __launch_bounds__(kMixThreads, 3)
 mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ G, float lr,
                  const float* __restrict__ lr_pw, float* Xout, uint16_t* __restrict__ shadow, MixPlan plan,
                  int mix_then_correct, int n_panels, const int* active_count) {
+    dependent_begin();
     extern __shared__ float4 sm[];  // [N][GS]
     if (active_count && *active_count <= active_limit(N)) return;  // mix_active_kernel's round
     for (int panel = blockIdx.x; panel < n_panels; panel += gridDim.x) {
@@ -45,6 +46,7 @@ __global__ void __launch_bounds__(256)
 mix_direct_kernel(int N, long long ld, const float* __restrict__ X, const float* __restrict__ G, float lr,
                   const float* __restrict__ lr_pw, float* __restrict__ Xout, uint16_t* __restrict__ shadow,
                   MixPlan plan, int mix_then_correct, int panel_cols, long long n_items) {
+    dependent_begin();
     for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int i = (int)(item % N);
         const long long c = (item / N) * panel_cols + 4 * (long long)threadIdx.x;
@@ -105,6 +107,7 @@ __global__ void __launch_bounds__(kMixThreads, 3)
 mix_active_kernel(int N, long long ld, const float* X, const float* __restrict__ G, float lr, const float* __restrict__ lr_pw,
                   float* Xout, uint16_t* __restrict__ shadow, MixPlan plan, int mix_then_correct, int max_merge,
                   ActiveRows active, const __grid_constant__ WeightBlocks blocks) {
+    dependent_begin();
     extern __shared__ float4 sm[];  // [N][GS] staged rows, then by staged row v:
     const int n_act = *active.count;
     const int half = active_limit(N);
@@ -226,7 +229,7 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
     if (per_sm < 1) return DBW_ERR_BAD_SHAPE;
     const int n_panels = (int)((h->ld + 4 * GS - 1) / (4 * GS));
     const int grid = n_panels < per_sm * h->sm_count ? n_panels : per_sm * h->sm_count;
-    mix_panel_kernel<GS><<<grid, kMixThreads, smem, s>>>(h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
+    launch(mix_panel_kernel<GS>, grid, kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
                                                         (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0,
                                                         n_panels, active_count);
     DBW_LAUNCHED();
@@ -266,8 +269,7 @@ int launch_active(dbw_handle* h, const float* X, const float* G, float lr, const
     const int slots = per_sm * h->sm_count;
     // panels staged together: at least two groups for every resident block, so that the blocks stay evenly loaded
     const int max_merge = std::min(32, std::max(1, n_panels / (2 * slots)));
-    mix_active_kernel<GS><<<n_panels < slots ? n_panels : slots, kMixThreads, smem, s>>>(
-        h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, max_merge,
+    launch(mix_active_kernel<GS>, n_panels < slots ? n_panels : slots, kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, max_merge,
         h->active, blocks);
     DBW_LAUNCHED();
     return DBW_OK;
@@ -368,7 +370,7 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     const long long n_items = ((h->ld + panel_cols - 1) / panel_cols) * h->N;
     long long blocks = (long long)h->sm_count * (2048 / (panel_cols / 4) > 16 ? 16 : 2048 / (panel_cols / 4));
     if (blocks > n_items) blocks = n_items;
-    mix_direct_kernel<<<(int)blocks, panel_cols / 4, 0, s>>>(h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
+    launch(mix_direct_kernel, (int)blocks, panel_cols / 4, 0, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
                                                            (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, panel_cols, n_items);
     DBW_LAUNCHED();
     return DBW_OK;

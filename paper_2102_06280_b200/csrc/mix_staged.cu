@@ -106,6 +106,7 @@ constexpr size_t kRoomyBytes = 195 * 1024;
 // columns, 32 neighbours).  Without weight reads eight lanes of one piece are better (1254 us against 1288).
 template <bool WEIGHTED, int W, bool LOCAL>
 __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
+    dependent_begin();
     constexpr int SLOTS = W / 4, PIECES = W == 32 && WEIGHTED ? 2 : 1, LPR = SLOTS / PIECES, RPW = 32 / LPR;  // RPW: output rows per warp
     constexpr uint32_t kIdx = WEIGHTED ? (1u << index_bits(W)) - 1 : 0xffffu;
     constexpr int kProdWarps = producer_warps(W), kConsWarps = kWarps - kProdWarps;
@@ -321,7 +322,7 @@ int launch_staged(const dbw_handle* h, StagedArgs& a, cudaStream_t s) {
     if (rc) return rc;
     a.n_panels = (int)((h->ld + W - 1) / W);
     const int grid = a.n_panels < h->sm_count ? a.n_panels : h->sm_count;
-    mix_staged_kernel<WEIGHTED, W, LOCAL><<<grid, kThreads, staged_smem(h, LOCAL), s>>>(a);
+    launch<false>(mix_staged_kernel<WEIGHTED, W, LOCAL>, grid, kThreads, staged_smem(h, LOCAL), s, a);
     DBW_LAUNCHED();
     return DBW_OK;
 }

@@ -661,8 +661,8 @@ __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, lon
     // ---- every output row of the panel ----
     const long long c = col0 + 4 * q;
     for (int i = gid; i < N; i += kGroups) {
-        float4 gi = make_float4(0.f, 0.f, 0.f, 0.f);  // on its way while the row is summed
-        if (G && mix_then_correct && c < ld && mine(i)) gi = load_g<NC>(reinterpret_cast<const float4*>(G + (size_t)i * ld + c));
+        float4 gi = make_float4(0.f, 0.f, 0.f, 0.f);  // on its way while the row is summed (the single launch has no registers for it)
+        if (NC && G && mix_then_correct && c < ld && mine(i)) gi = load_g<NC>(reinterpret_cast<const float4*>(G + (size_t)i * ld + c));
         const float ws = plan.w_self[i];
         const float4 self = sm[i * GS + q];
         float4 acc = make_float4(ws * self.x, ws * self.y, ws * self.z, ws * self.w);
@@ -680,7 +680,10 @@ __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, lon
             acc = fma4(w.w, sm[j.w * GS + q], acc);
         }
         if (c < ld && mine(i)) {
-            if (G && mix_then_correct) acc = fma4(-(lr_pw ? lr_pw[i] : lr), gi, acc);
+            if (G && mix_then_correct) {
+                if (!NC) gi = load_g<NC>(reinterpret_cast<const float4*>(G + (size_t)i * ld + c));
+                acc = fma4(-(lr_pw ? lr_pw[i] : lr), gi, acc);
+            }
             *reinterpret_cast<float4*>(Xout + (size_t)i * ld + c) = acc;
             if (shadow) *reinterpret_cast<uint2*>(shadow + (size_t)i * ld + c) = pack_bf16x4_rn(acc.x, acc.y, acc.z, acc.w);
         }

@@ -55,6 +55,7 @@ select_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restri
               double* __restrict__ T_nbr_ws, double* T_nbr_out, double* T_worker, double* T_round,
               uint32_t* waited, uint32_t* ticket, uint32_t* status, MixPlan plan, int build_plan,
               int uniform, ActiveRows active) {
+    dependent_begin();
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     if (i < N) select_worker(i, lane, rowptr, col, t, t_edge, b, kept, T_nbr_ws, waited, status, plan, build_plan, uniform);
@@ -88,6 +89,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 plan_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
             const uint8_t* __restrict__ kept, const int32_t* __restrict__ b, uint32_t* status, MixPlan plan,
             int uniform) {
+    dependent_begin();
     const int lane = threadIdx.x & 31;
     const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
     if (i >= N) return;
@@ -123,8 +125,7 @@ plan_kernel(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict
 int launch_select(dbw_handle* h, const double* t, const int32_t* b, uint8_t* kept, double* T_worker,
                   double* T_nbr, double* T_round, bool build_plan, cudaStream_t s, bool list_active) {
     const int blocks = (h->N + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    select_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(
-        h->N, h->d_rowptr, h->d_col, t, h->t_edge, b, kept, h->d_Tnbr_ws, T_nbr, T_worker, T_round, h->d_waited,
+    launch(select_kernel, blocks, kWarpsPerBlock * 32, 0, s, h->N, h->d_rowptr, h->d_col, t, h->t_edge, b, kept, h->d_Tnbr_ws, T_nbr, T_worker, T_round, h->d_waited,
         h->d_ticket, h->d_status, h->plan, build_plan ? 1 : 0, (h->flags & DBW_WEIGHT_UNIFORM) ? 1 : 0,
         list_active ? h->active : ActiveRows{});
     DBW_LAUNCHED();
@@ -133,7 +134,7 @@ int launch_select(dbw_handle* h, const double* t, const int32_t* b, uint8_t* kep
 
 int launch_plan_from_kept(dbw_handle* h, const uint8_t* kept, const int32_t* b, cudaStream_t s) {
     const int blocks = (h->N + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    plan_kernel<<<blocks, kWarpsPerBlock * 32, 0, s>>>(h->N, h->d_rowptr, h->d_col, kept, b, h->d_status,
+    launch(plan_kernel, blocks, kWarpsPerBlock * 32, 0, s, h->N, h->d_rowptr, h->d_col, kept, b, h->d_status,
                                                        h->plan, (h->flags & DBW_WEIGHT_UNIFORM) ? 1 : 0);
     DBW_LAUNCHED();
     return DBW_OK;
@@ -194,7 +195,7 @@ extern "C" int dbw_select_static(int32_t N, const int32_t* rowptr, const int32_t
     const int blocks = (N + dbw::kWarpsPerBlock - 1) / dbw::kWarpsPerBlock;
     dbw::MixPlan no_plan{};
     no_plan.n = N;  // only the bounds-checked build looks at it: this entry point's CSR is not validated on the host
-    dbw::select_kernel<<<blocks, dbw::kWarpsPerBlock * 32, 0, s>>>(N, rowptr, col, t, nullptr, b, kept, tnbr, T_nbr, T_worker,
+    dbw::launch(dbw::select_kernel, blocks, dbw::kWarpsPerBlock * 32, 0, s, N, rowptr, col, t, nullptr, b, kept, tnbr, T_nbr, T_worker,
                                                                    T_round, waited, ticket, status, no_plan, 0, 0, dbw::ActiveRows{});
     DBW_LAUNCHED();
     if (status_out) DBW_CUDA(cudaMemcpyAsync(status_out, status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
