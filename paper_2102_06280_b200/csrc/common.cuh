@@ -151,6 +151,7 @@ struct dbw_handle {
 
     dbw::MixPlan plan;
     int mix_panel_cols = 0;  // 0 = automatic
+    int panel_per_sm[5] = {}, active_per_sm[5] = {};  // blocks per SM of the panel mix kernels, by panel width; 0 = not asked yet
     dbw::TcMixState* mix_tc = nullptr;  // selection matrix and tensor map of the tensor-core mix (lazy)
     dbw::SpMixState* mix_sp = nullptr;  // 2:4 order, compressed selection matrix and tensor maps of the sparse tensor-core mix (dbw_init)
 
@@ -280,6 +281,9 @@ inline bool fp32_head_usable(const dbw_handle* h) {
     return m.dims[L] <= 32 && (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 &&
            ((uintptr_t)h->feat & 15) == 0;
 }
+// Slices over k of an fp32 GEMM of `batch` problems M x N x K (GemmArgs::slice), the same for the per-step kernels and the
+// single launch, which sum in this order.
+int fp32_gemm_slice(int M, int N, int K, int batch, bool is_dw, int sm_count);
 int grad_fp32_alloc(dbw_handle* h);
 void grad_fp32_free(dbw_handle* h);
 // `beside` (of both gradient paths): queues what runs beside the gradients on another stream; called once the forward pass is

@@ -36,9 +36,9 @@ softmax_ce_kernel(int B, int C, const float* __restrict__ logits, const int32_t*
 }
 
 __global__ void bias_grad_kernel(int B, int out_dim, const float* __restrict__ dz, float* __restrict__ G,
-                                 long long ld, long long b_off) {
+                                 long long ld, long long b_off, int slice) {
     dependent_begin();
-    bias_grad_col(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, B, out_dim, dz, G, ld, b_off);
+    bias_grad_col(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, B, out_dim, dz, G, ld, b_off, slice);
 }
 
 // The GEMM for operands whose unit-stride dimension allows 128-bit accesses (every layer whose width and
@@ -170,11 +170,196 @@ __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
     }
 }
 
+// The same for few tiles (fewer than the chip has schedulers).  Too few warps to hide latency behind, so a warp owns a tile of
+// 64 x 32 outputs, 8 x 8 per thread (below that shared-memory reads bound it: a 128-bit read takes four cycles of a pipe that
+// the SM's four schedulers share), with a ring of its own (three steps of eight k, asynchronous copies, no block barriers), and
+// the kSlices warps of a block share one tile: each sums its slice of k in ascending order and the slices are added in order.
+// Operands are staged as they lie in memory: one with its unit stride along k (AK / BK) as rows of eight k, of which a thread
+// reads four at once (neighbouring lanes on neighbouring rows: distinct banks), one with its unit stride along the output as
+// eight rows.  (32 workers, 64 x 200 x 784: 29.8 us against 38.5; 10 workers, 256 x 256 x 1024: 46 against 60; with more tiles
+// the block-tile kernel is better: 10 workers, 1024 x 256 x 256: 41.5 against 45.5.)
+constexpr int kTileM = 64, kTileN = 32, kSlices = 4, kStepK = 8, kSteps = 3;
+
+// One operand of a warp's tile: R outputs, T of them per thread, LANES threads along it; KF: unit stride along k.
+template <int R, int T, int LANES, bool KF>
+struct GemmOperand {
+    static constexpr int kPitch = KF ? kStepK : R + 4;
+    static constexpr int kFloats = KF ? R * kPitch : kStepK * kPitch;
+    static __device__ __forceinline__ int index(int t, int i) { return KF ? t + i * LANES : 4 * t + (i / 4) * (4 * LANES) + i % 4; }
+    // outputs past the edge are copies of the last ones (never stored); k past the slice is zero
+    static __device__ __forceinline__ void stage(float* sm, const float* src, long long stride, int row0, int rows, int k0, int k_end, int lane) {
+#pragma unroll
+        for (int u = 0; u < R * kStepK / 128; ++u) {
+            const int e = lane + 32 * u;
+            const int r = KF ? e / 2 : 4 * (e % (R / 4)), k = KF ? 4 * (e % 2) : e / (R / 4);
+            const float* from = KF ? src + (long long)min(row0 + r, rows - 1) * stride + (k0 + k) : src + (long long)(k0 + k) * stride + min(row0 + r, rows - 4);
+            const int valid = KF ? max(0, min(4, k_end - k0 - k)) * 4 : (k0 + k < k_end ? 16 : 0);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(sm + (KF ? r * kPitch + k : k * kPitch + r))),
+                         "l"(valid ? from : src), "r"(valid)
+                         : "memory");
+        }
+    }
+    float v[4][T];  // the thread's outputs' values at k = kq .. kq + 3
+    __device__ __forceinline__ void load(const float* sm, int t, int kq) {
+        if (KF) {
+#pragma unroll
+            for (int i = 0; i < T; ++i) {
+                const float4 x = *reinterpret_cast<const float4*>(sm + index(t, i) * kPitch + kq);
+                v[0][i] = x.x; v[1][i] = x.y; v[2][i] = x.z; v[3][i] = x.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < T; i += 4) {
+                    const float4 x = *reinterpret_cast<const float4*>(sm + (kq + k) * kPitch + index(t, i));
+                    v[k][i] = x.x; v[k][i + 1] = x.y; v[k][i + 2] = x.z; v[k][i + 3] = x.w;
+                }
+        }
+    }
+};
+
+template <bool SUMS, bool AK, bool BK>
+__global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __grid_constant__ GemmArgs g) {
+    dependent_begin();
+    constexpr int TM = 8, TN = 8, TX = kTileN / TN, TY = kTileM / TM;
+    typedef GemmOperand<kTileM, TM, TY, AK> OpA;
+    typedef GemmOperand<kTileN, TN, TX, BK> OpB;
+    constexpr int kRing = kSteps * (OpA::kFloats + OpB::kFloats), kExchange = TM * TN * 32 + 64;
+    constexpr int kPerWarp = (kRing > kExchange ? kRing : kExchange + 3) / 4 * 4;
+    __shared__ __align__(16) float sm[kSlices][kPerWarp];
+    const int z = blockIdx.z, lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+    const int m0 = blockIdx.y * kTileM, n0 = blockIdx.x * kTileN;
+    const int ty = lane / TX, tx = lane % TX;
+    const float* A = g.A + (size_t)z * g.sAz;
+    const float* B = g.B + (size_t)z * g.sBz;
+    const int k_lo = part * g.slice, k_hi = min(g.K, k_lo + g.slice);
+    const int steps = (k_hi - k_lo + kStepK - 1) / kStepK;
+    float* ring = sm[part];
+    auto fetch = [&](int step, int slot) {
+        if (step < steps) {
+            float* st = ring + slot * (OpA::kFloats + OpB::kFloats);
+            OpA::stage(st, A, AK ? g.sAm : g.sAk, m0, g.M, k_lo + step * kStepK, k_hi, lane);
+            OpB::stage(st + OpA::kFloats, B, BK ? g.sBn : g.sBk, n0, g.N, k_lo + step * kStepK, k_hi, lane);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int s = 0; s < kSteps - 1; ++s) fetch(s, s);
+    float acc[TM][TN] = {};
+    float rows[2] = {0.f, 0.f};
+    const bool sums = SUMS && n0 == 0;
+    int slot = 0;
+#pragma unroll 1
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kSteps - 2) : "memory");
+        __syncwarp();  // this step's copies have landed for every lane, and every lane is done with the step before
+        fetch(step + kSteps - 1, slot == 0 ? kSteps - 1 : slot - 1);
+        const float* a_sm = ring + slot * (OpA::kFloats + OpB::kFloats);
+        const float* b_sm = a_sm + OpA::kFloats;
+        slot = slot == kSteps - 1 ? 0 : slot + 1;
+#pragma unroll
+        for (int kq = 0; kq < kStepK; kq += 4) {
+            OpA a;
+            OpB b;
+            a.load(a_sm, ty, kq);
+            b.load(b_sm, tx, kq);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.v[k][i], b.v[k][j], acc[i][j]);
+        }
+        if (SUMS && !AK && sums) {
+#pragma unroll
+            for (int k = 0; k < kStepK; ++k) {  // zero past the end
+                rows[0] += a_sm[k * OpA::kPitch + lane];
+                rows[1] += a_sm[k * OpA::kPitch + lane + 32];
+            }
+        }
+    }
+    constexpr int IPW = TM / kSlices;  // rows of a thread's outputs that its warp finishes
+    {  // the slices through shared memory: warp p adds up the outputs i = p IPW .. of every lane
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        float4* ex = reinterpret_cast<float4*>(ring);
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; j += 4) ex[(i * (TN / 4) + j / 4) * 32 + lane] = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+        if (sums) {
+            ring[TM * TN * 32 + lane] = rows[0];
+            ring[TM * TN * 32 + 32 + lane] = rows[1];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < IPW; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; j += 4) {
+                const int at = ((part * IPW + i) * (TN / 4) + j / 4) * 32 + lane;
+                float4 t = reinterpret_cast<const float4*>(sm[0])[at];
+#pragma unroll
+                for (int p = 1; p < kSlices; ++p) {
+                    const float4 x = reinterpret_cast<const float4*>(sm[p])[at];
+                    t.x += x.x; t.y += x.y; t.z += x.z; t.w += x.w;
+                }
+                acc[i][j] = t.x; acc[i][j + 1] = t.y; acc[i][j + 2] = t.z; acc[i][j + 3] = t.w;
+            }
+        if (sums && part == 0) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int p = 1; p < kSlices; ++p) rows[h] += sm[p][TM * TN * 32 + 32 * h + lane];
+        }
+    }
+    if (sums && part == 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (m0 + lane + 32 * h < g.M) g.rowsum[(size_t)z * g.sRz + m0 + lane + 32 * h] = rows[h];
+    }
+    float* C = g.C + (size_t)z * g.sCz;
+    const float* bias = g.bias ? g.bias + (size_t)z * g.sBiasz : nullptr;
+    const float* mask = g.mask ? g.mask + (size_t)z * g.sMz : nullptr;
+#pragma unroll
+    for (int i = 0; i < IPW; ++i) {
+        const int m = m0 + OpA::index(ty, part * IPW + i);
+        if (m >= g.M) continue;
+        float* c = C + (size_t)m * g.sCm;
+        const float* mk = mask ? mask + (size_t)m * g.sMm : nullptr;
+        if (BK) {
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+                const int n = n0 + OpB::index(tx, j);
+                if (n >= g.N) continue;
+                float v = acc[i][j];
+                if (bias) v += __ldg(bias + n);
+                if (g.relu) v = fmaxf(v, 0.f);
+                if (mk && !(__ldg(mk + n) > 0.f)) v = 0.f;
+                c[n] = v;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < TN; j += 4) {
+                const int n = n0 + OpB::index(tx, j);
+                if (n >= g.N) continue;  // N is a multiple of four: the four columns are inside or outside together
+                float4 v = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+                if (mk) {
+                    const float4 x = __ldg(reinterpret_cast<const float4*>(mk + n));
+                    v.x = x.x > 0.f ? v.x : 0.f; v.y = x.y > 0.f ? v.y : 0.f; v.z = x.z > 0.f ? v.z : 0.f; v.w = x.w > 0.f ? v.w : 0.f;
+                }
+                *reinterpret_cast<float4*>(c + n) = v;
+            }
+        }
+    }
+}
+
 // 128-bit accesses are possible: unit stride along k or along the output dimension, everything else a multiple of four floats
 bool gemm_vec_ok(const GemmArgs& g) {
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
     const bool a_ok = (g.sAk == 1 && g.K % 4 == 0 && g.sAm % 4 == 0) || (g.sAm == 1 && g.M % 4 == 0 && g.sAk % 4 == 0);
     const bool b_ok = (g.sBk == 1 && g.K % 4 == 0 && g.sBn % 4 == 0) || (g.sBn == 1 && g.N % 4 == 0 && g.sBk % 4 == 0);
+    if (g.sAk != 1 && g.sBk == 1) return false;  // no GEMM of the path has this pair of layouts
     const bool c_ok = g.N % 4 == 0 && g.sCm % 4 == 0 && g.sCz % 4 == 0 && al(g.C);
     const bool m_ok = !g.mask || (g.sMm % 4 == 0 && g.sMz % 4 == 0 && al(g.mask));
     return a_ok && b_ok && c_ok && m_ok && g.sAz % 4 == 0 && g.sBz % 4 == 0 && al(g.A) && al(g.B);
@@ -234,7 +419,25 @@ void launch_gemm_vec(const GemmArgs& g, int batch, cudaStream_t s) {
         launch<false>(gemm_vec_kernel<WM, RM, false>, grid, 32 * WM, 0, s, g);
 }
 
-int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
+void launch_gemm_slice(const GemmArgs& g, int batch, cudaStream_t s) {
+    const dim3 grid((g.N + kTileN - 1) / kTileN, (g.M + kTileM - 1) / kTileM, batch);
+    if (g.sAk != 1 && g.rowsum)
+        launch<false>(gemm_slice_kernel<true, false, false>, grid, kSlices * 32, 0, s, g);
+    else if (g.sAk != 1)
+        launch<false>(gemm_slice_kernel<false, false, false>, grid, kSlices * 32, 0, s, g);
+    else if (g.sBk != 1)
+        launch<false>(gemm_slice_kernel<false, true, false>, grid, kSlices * 32, 0, s, g);
+    else
+        launch<false>(gemm_slice_kernel<false, true, true>, grid, kSlices * 32, 0, s, g);
+}
+
+int run_gemm(GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
+    g.slice = fp32_gemm_slice(g.M, g.N, g.K, batch, g.sAk != 1, sm_count);
+    if (gemm_vec_ok(g) && g.slice < g.K) {
+        launch_gemm_slice(g, batch, s);
+        DBW_LAUNCHED();
+        return DBW_OK;
+    }
     if (gemm_vec_ok(g)) {
         // 8 x 4 outputs per thread where that still gives every SM several warps, else 4 x 4 (twice the warps
         // for the same tile), on tiles of 64, 32 or 16 rows
@@ -266,6 +469,14 @@ int run_gemm(const GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
 }
 
 }  // namespace
+
+// is_dw: dZ^T A, both operands with their unit stride along the output; else with the first one's along k.
+int fp32_gemm_slice(int M, int N, int K, int batch, bool is_dw, int sm_count) {
+    if (N % 4 || (is_dw ? M : K) % 4) return K;  // not for gemm_slice_kernel
+    const long long tiles = (long long)((M + kTileM - 1) / kTileM) * ((N + kTileN - 1) / kTileN) * batch;
+    if (tiles >= 4LL * sm_count || K < 32 * kSlices) return K;  // enough tiles, or slices of less than four steps
+    return ((K + kSlices - 1) / kSlices + kStepK - 1) / kStepK * kStepK;
+}
 
 int grad_fp32_alloc(dbw_handle* h) {
     const dbw_model_desc& m = h->model;
@@ -371,7 +582,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         }
         if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
         if (needs_db && !db_here) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
-            launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
+            launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l], g.slice);
             DBW_LAUNCHED();
         }
         if (l > 0) {  // dZ_{l}[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]

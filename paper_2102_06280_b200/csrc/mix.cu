@@ -224,8 +224,8 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
         return DBW_OK;
     });
     if (rc) return rc;
-    int per_sm = 0;
-    DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_panel_kernel<GS>, kMixThreads, smem));
+    int& per_sm = h->panel_per_sm[GS == 64 ? 4 : GS == 32 ? 3 : GS == 16 ? 2 : GS == 8 ? 1 : 0];  // asked once per handle: N sets it
+    if (per_sm < 1) DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_panel_kernel<GS>, kMixThreads, smem));
     if (per_sm < 1) return DBW_ERR_BAD_SHAPE;
     const int n_panels = (int)((h->ld + 4 * GS - 1) / (4 * GS));
     const int grid = n_panels < per_sm * h->sm_count ? n_panels : per_sm * h->sm_count;
@@ -248,8 +248,8 @@ int launch_active(dbw_handle* h, const float* X, const float* G, float lr, const
         return DBW_OK;
     });
     if (rc) return rc;
-    int per_sm = 0;
-    DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_active_kernel<GS>, kMixThreads, smem));
+    int& per_sm = h->active_per_sm[GS == 64 ? 4 : GS == 32 ? 3 : GS == 16 ? 2 : GS == 8 ? 1 : 0];  // asked once per handle: N sets it
+    if (per_sm < 1) DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mix_active_kernel<GS>, kMixThreads, smem));
     if (per_sm < 1) return DBW_ERR_BAD_SHAPE;
     const int n_panels = (int)((h->ld + 4 * GS - 1) / (4 * GS));
     WeightBlocks blocks{};

@@ -53,6 +53,7 @@ struct GemmArgs {
     const float* mask;  // same shape as C, nullable: C *= (mask > 0)
     long long sMz, sMm;
     int M, N, K;
+    int slice;  // k is summed in slices of this many (a multiple of 8, or at least K): each in ascending k, the slices added in order
     int relu;
     float* rowsum;  // nullable (gemm_vec_kernel only): sum over k of A(m, k), in ascending k
     long long sRz;
@@ -64,8 +65,8 @@ struct GemmArgs {
 // case with a long reduction, where a step costs one global-memory round trip whatever its depth
 // (the order of the additions is the same).
 // One tile (z, m0, n0) by a block of 256 threads; As / Bs are the block's staging tiles.  Ends with a
-// block barrier, so tiles may follow each other in a loop.  Every output element is summed over k in
-// ascending order whatever R and TK are.
+// block barrier, so tiles may follow each other in a loop.  Every output element is summed over k in the
+// order of g.slice whatever R and TK are.
 // NC = true reads the operands through the non-coherent path (they are constant while the kernel runs);
 // NC = false with plain loads, for operands written earlier in the same launch.
 template <bool NC, typename T>
@@ -74,7 +75,8 @@ __device__ __forceinline__ T load_g(const T* p) {
     else return *p;
 }
 
-template <int R, int TK, bool NC = true>
+// SLICED: g.slice may be less than K.
+template <int R, int TK, bool NC = true, bool SLICED = false>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int n0, float (*As)[16 * R + 4], float (*Bs)[16 * R + 4]) {
     constexpr int T = 16 * R;        // tile edge
     constexpr int PER = T * TK / 256;  // elements of each operand tile a thread stages
@@ -84,22 +86,23 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
     const int tx = tid & 15, ty = tid >> 4;
     const bool a_k_fast = g.sAk == 1;
     const bool b_k_fast = g.sBk == 1;
-    float acc[R][R] = {};
+    float acc[R][R] = {}, total[SLICED ? R : 1][SLICED ? R : 1];
     float pa[PER], pb[PER];  // next k-step's operand elements, in flight while this one is multiplied
+    int k_end = SLICED ? min(g.K, g.slice) : g.K;  // end of the current slice
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             const int e = tid + r * 256;
             const int ka = a_k_fast ? (e % TK) : (e / T);
             const int ma = a_k_fast ? (e / TK) : (e % T);
-            pa[r] = (m0 + ma < g.M && k0 + ka < g.K) ? load_g<NC>(A + (size_t)(m0 + ma) * g.sAm + (size_t)(k0 + ka) * g.sAk) : 0.f;
+            pa[r] = (m0 + ma < g.M && k0 + ka < k_end) ? load_g<NC>(A + (size_t)(m0 + ma) * g.sAm + (size_t)(k0 + ka) * g.sAk) : 0.f;
             const int kb = b_k_fast ? (e % TK) : (e / T);
             const int nb = b_k_fast ? (e / TK) : (e % T);
-            pb[r] = (n0 + nb < g.N && k0 + kb < g.K) ? load_g<NC>(B + (size_t)(n0 + nb) * g.sBn + (size_t)(k0 + kb) * g.sBk) : 0.f;
+            pb[r] = (n0 + nb < g.N && k0 + kb < k_end) ? load_g<NC>(B + (size_t)(n0 + nb) * g.sBn + (size_t)(k0 + kb) * g.sBk) : 0.f;
         }
     };
     fetch(0);
-    for (int k0 = 0; k0 < g.K; k0 += TK) {
+    for (int k0 = 0; k0 < g.K;) {
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             const int e = tid + r * 256;
@@ -107,7 +110,13 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
             Bs[b_k_fast ? (e % TK) : (e / T)][b_k_fast ? (e / TK) : (e % T)] = pb[r];
         }
         __syncthreads();
-        fetch(k0 + TK);  // all zero past the end
+        const int slice_of = k_end;
+        int next = k0 + TK;
+        if (SLICED && next >= k_end) {  // the next step begins the next slice
+            next = k_end;
+            k_end = min(g.K, k_end + g.slice);
+        }
+        fetch(next);  // all zero past the end
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
             float av[R], bv[R];
@@ -127,6 +136,18 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
 #pragma unroll
                 for (int j = 0; j < R; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
+        if (SLICED && next >= slice_of) {  // a slice is complete
+            const bool first = slice_of <= g.slice;
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < R; ++j) {
+                    float& t = total[SLICED ? i : 0][SLICED ? j : 0];
+                    t = first ? acc[i][j] : t + acc[i][j];
+                    acc[i][j] = 0.f;
+                }
+        }
+        k0 = next;
         __syncthreads();
     }
     float* C = g.C + (size_t)z * g.sCz;
@@ -140,7 +161,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
         for (int j = 0; j < R; ++j) {
             const int n = n0 + tx * R + j;
             if (n >= g.N) continue;
-            float v = acc[i][j];
+            float v = SLICED ? total[SLICED ? i : 0][SLICED ? j : 0] : acc[i][j];
             if (bias) v += bias[n];
             if (g.relu) v = fmaxf(v, 0.f);
             if (mask && !(mask[(size_t)m * g.sMm + n] > 0.f)) v = 0.f;
@@ -225,15 +246,20 @@ __device__ __forceinline__ void softmax_ce_worker(int i, int B, int C, const flo
     }
 }
 
-// db[i][o] = sum over the batch of dZ[i][m][o], in sample order
+// db[i][o] = sum over the batch of dZ[i][m][o], in the order of the dW GEMM: sample order within its slices, slices in order
 __device__ __forceinline__ void bias_grad_col(int i, int o, int B, int out_dim, const float* dz, float* G,
-                                              long long ld, long long b_off) {
+                                              long long ld, long long b_off, int slice) {
     if (o >= out_dim) return;
     const float* p = dz + (size_t)i * B * out_dim + o;
-    float s = 0.f;
+    float total = 0.f;
+    for (int m0 = 0; m0 < B; m0 += slice) {
+        float s = 0.f;
+        const int m1 = min(B, m0 + slice);
 #pragma unroll 8
-    for (int m = 0; m < B; ++m) s += p[(size_t)m * out_dim];
-    G[(size_t)i * ld + b_off + o] = s;
+        for (int m = m0; m < m1; ++m) s += p[(size_t)m * out_dim];
+        total = m0 == 0 ? s : total + s;
+    }
+    G[(size_t)i * ld + b_off + o] = total;
 }
 
 

@@ -32,7 +32,12 @@ constexpr int kMixGS = 32;                       // 128-column panels
 constexpr int kMaxWorkers = 64;                  // N * kMixGS * 16 bytes of panel <= 32 KiB
 constexpr int kSmemBytes = 2 * 128 * 36 * 4;     // the largest GEMM staging (32 x 32 tiles, 128-deep steps): 36,864 bytes
 constexpr int kBlocksPerSM = 1;                  // registers are spent on deep k-steps (a step costs one memory round trip)
-constexpr long long kAutoMaxMacs = 64ll << 20;   // multiply-adds of the forward pass up to which the launch is used unasked
+// Samples and multiply-adds of the forward pass up to which the launch is used unasked: above them the per-step kernels, placed
+// early and with as many blocks as they want, are the faster path.  Measured (single launch / step by step, us): 8 workers x
+// batch 32, 784-10: 19 / 33 and 256-64-64-10: 51 / 57; 5 x 70, 205-186-20-10: 73 / 75; 30 x 19, 784-53-10: 72 / 67; 42 x 56,
+// 37-10: 39 / 31; 63 x 75, 64-92-10: 91 / 58.
+constexpr long long kAutoMaxSamples = 512;
+constexpr long long kAutoMaxMacs = 16 << 20;
 
 // GEMM tile variants (R, TK) the kernel instantiates; which one a GEMM uses is chosen on the host.
 enum { V_2_16 = 0, V_2_64 = 1, V_4_16 = 2, V_4_64 = 3, V_2_128 = 4, kVariants = 5 };
@@ -68,12 +73,13 @@ struct FusedArgs {
     float lr;
     const float* lr_pw;
     float* loss;
+    int fwd_slice[DBW_MAX_LAYERS], dw_slice[DBW_MAX_LAYERS], da_slice[DBW_MAX_LAYERS];
     signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];
     float* head_part;
     int head;  // the last layer takes the small-output steps (at most 32 classes)
 };
 
-template <int R, int TK>
+template <int R, int TK, bool SLICED = false>
 __device__ __forceinline__ void gemm_tiles(const GemmArgs& g, int workers, float* smem) {
     constexpr int T = 16 * R;
     float(*As)[T + 4] = reinterpret_cast<float(*)[T + 4]>(smem);
@@ -82,11 +88,15 @@ __device__ __forceinline__ void gemm_tiles(const GemmArgs& g, int workers, float
     const int items = tiles_n * tiles_m * workers;
     for (int item = blockIdx.x; item < items; item += gridDim.x) {
         const int z = item / (tiles_n * tiles_m), rem = item % (tiles_n * tiles_m);
-        gemm_tile<R, TK, false>(g, z, (rem / tiles_n) * T, (rem % tiles_n) * T, As, Bs);
+        gemm_tile<R, TK, false, SLICED>(g, z, (rem / tiles_n) * T, (rem % tiles_n) * T, As, Bs);
     }
 }
 
 __device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int workers, float* smem) {
+    if (g.slice < g.K) {  // summed in slices of k: one tile shape serves them (the order does not depend on it)
+        gemm_tiles<2, 64, true>(g, workers, smem);
+        return;
+    }
     switch (variant) {
         case V_2_16: gemm_tiles<2, 16>(g, workers, smem); break;
         case V_2_64: gemm_tiles<2, 64>(g, workers, smem); break;
@@ -156,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.B = a.X + a.w_off[l]; g.sBz = a.ld; g.sBn = in; g.sBk = 1;
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
-        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1;
+        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = a.fwd_slice[l];
         gemm_any(a.fwd_var[l], g, N, smem);
         grid.sync();
     }
@@ -218,18 +228,18 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.A = a.dz[l + 1]; g.sAz = (long long)B * out; g.sAm = 1; g.sAk = out;
         g.B = a.act[l]; g.sBz = (long long)B * in; g.sBn = 1; g.sBk = in;
         g.C = a.G + a.w_off[l]; g.sCz = a.ld; g.sCm = in;
-        g.M = out; g.N = in; g.K = B;
+        g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l];
         gemm_any(a.dw_var[l], g, N, smem);
         if (l < L - 1 && !(a.head && l == L - 2))  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
             for (int e = blockIdx.x * kThreads + tid; e < N * out; e += gridDim.x * kThreads)
-                bias_grad_col(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l]);
+                bias_grad_col(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l], a.dw_slice[l]);
         if (l > 0) {  // dZ_l[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]
             GemmArgs d{};
             d.A = a.dz[l + 1]; d.sAz = (long long)B * out; d.sAm = out; d.sAk = 1;
             d.B = a.X + a.w_off[l]; d.sBz = a.ld; d.sBn = 1; d.sBk = in;
             d.C = a.dz[l]; d.sCz = (long long)B * in; d.sCm = in;
             d.mask = a.act[l]; d.sMz = (long long)B * in; d.sMm = in;
-            d.M = B; d.N = in; d.K = out;
+            d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l];
             gemm_any(a.da_var[l], d, N, smem);
         }
         grid.sync();
@@ -290,13 +300,11 @@ void round_fused_prepare(dbw_handle* h) {
     st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     long long macs = 0;
     for (int l = 0; l < h->model.n_layers; ++l) macs += (long long)h->N * h->model.batch * h->model.dims[l] * h->model.dims[l + 1];
-    st->auto_on = macs <= kAutoMaxMacs;
+    st->auto_on = macs <= kAutoMaxMacs && (long long)h->N * h->model.batch <= kAutoMaxSamples;
     st->usable = true;
 }
 
-// Used when asked for, or, left to itself, for networks so small that launch latency is most of the round
-// (measured: above roughly 1e8 multiply-adds per round the per-step kernels, which fill the SMs with more
-// blocks than a cooperative grid can hold, are faster).
+// Used when asked for, or, left to itself, for networks so small that launch latency is most of the round.
 bool round_fused_usable(const dbw_handle* h) {
     if (!h->fused || !h->fused->usable || !h->feat || h->fused_mode == 0) return false;
     return h->fused_mode > 0 || h->fused->auto_on;
@@ -343,6 +351,11 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
         a.fwd_var[l] = (signed char)pick_variant(B, m.dims[l + 1], m.dims[l], N, grid);
         a.dw_var[l] = (signed char)pick_variant(m.dims[l + 1], m.dims[l], B, N, grid);
         a.da_var[l] = (signed char)pick_variant(B, m.dims[l], m.dims[l + 1], N, grid);
+    }
+    for (int l = 0; l < m.n_layers; ++l) {
+        a.fwd_slice[l] = fp32_gemm_slice(B, m.dims[l + 1], m.dims[l], N, false, h->sm_count);
+        a.dw_slice[l] = fp32_gemm_slice(m.dims[l + 1], m.dims[l], B, N, true, h->sm_count);
+        a.da_slice[l] = fp32_gemm_slice(B, m.dims[l], m.dims[l + 1], N, false, h->sm_count);
     }
     void* params[] = {&a};
     DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(round_fused_kernel), dim3(grid), dim3(kThreads), params, kSmemBytes, s));

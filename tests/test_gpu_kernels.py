@@ -723,7 +723,11 @@ def test_round_with_few_participants_gives_the_bits_of_its_steps(dims, batch, n,
 
 @pytest.mark.parametrize("dims,batch,n", [([32, 10], 257, 3),           # two parts of the batch, the second of one sample
                                           ([40, 24, 32], 256, 3),       # one part, the most classes: the largest staging
-                                          ([64, 48, 36, 10], 520, 4)])  # three parts; a bias gradient out of a dW GEMM
+                                          ([64, 48, 36, 10], 520, 4),   # three parts; a bias gradient out of a dW GEMM
+                                          ([68, 36, 100, 12], 20, 3),   # GEMMs in slices of k: ragged tiles, a last slice of a few k
+                                          ([260, 64, 32, 10], 64, 5),   # ... whole tiles, a slice of less than a step more
+                                          ([128, 320, 64, 10], 64, 60),  # as many tiles as do without slices, and fewer
+                                          ([64, 30, 36, 10], 18, 3)])   # widths and a batch without 128-bit accesses beside some with
 def test_fp32_last_layer_in_parts_of_the_batch(dims, batch, n):
     """The last layer's backward step splits a large batch into parts whose sums are added in a fixed order.  Gradients and
     losses against the oracle (hidden units are far on one side of zero, so no ReLU decision is a matter of rounding), and
