@@ -488,42 +488,57 @@ gemm_dw_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 // ----------------------------------------------------------------------------- casts and gathers
-// fp32 [rows][cols] (row pitch src_pitch) -> bf16 [rows][cols] (row pitch cols).  Rows may be
-// indirect (row_idx: mini-batch gather, then the labels too).  cols % 8 == 0.  Every thread converts 16 consecutive floats
-// of one row: four 128-bit loads, two 128-bit stores.
 __device__ __forceinline__ uint4 pack8(const float* v) {
     return make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
 }
 
-__global__ void __launch_bounds__(256)
-cast_tile_kernel(int rows, int cols, const float* __restrict__ src, long long src_z, long long src_pitch,
-                 const int32_t* __restrict__ row_idx, int idx_z, int idx_limit, bf16* __restrict__ dst, long long dst_z,
-                 const int32_t* __restrict__ labels, int C, int32_t* __restrict__ ylab, uint32_t* status) {
+// Every fp32 -> bf16 copy of a gradient call in ONE launch (one for each layer's weights and one for the mini-batch before:
+// three launches of 4 - 11 us for 24 workers, 1000-328-136-10): the mini-batch rows with their labels, gathered through the batch
+// indices, and, unless the mix has left the copy, the weights of every tensor-core layer.  A task is [rows][cols] (row pitch
+// cols, a multiple of 8) for every worker; blockIdx.x walks the tasks' 64 x 64 tiles, blockIdx.y the workers.  Every thread converts
+// 16 consecutive floats of one row: four 128-bit loads, two 128-bit stores.
+struct CastArgs {
+    int n;
+    int first[DBW_MAX_LAYERS + 1], rows[DBW_MAX_LAYERS], cols[DBW_MAX_LAYERS];
+    const float* src[DBW_MAX_LAYERS];
+    long long src_z[DBW_MAX_LAYERS], dst_z[DBW_MAX_LAYERS];
+    bf16* dst[DBW_MAX_LAYERS];
+    // task 0: rows through row_idx [worker][rows[0]], one outside [0, samples) or a label outside [0, C) is clamped and reported
+    const int32_t* row_idx;
+    int samples, C;
+    const int32_t* labels;
+    int32_t* ylab;
+    uint32_t* status;
+};
+
+__global__ void __launch_bounds__(256) cast_kernel(const __grid_constant__ CastArgs a) {
     dependent_begin();
-    const int z = blockIdx.z;
-    const int t = threadIdx.x;
-    const int r = blockIdx.y * 64 + (t >> 2);
-    const int c0 = blockIdx.x * 64 + (t & 3) * 16;
+    const int z = blockIdx.y, t = threadIdx.x;
+    int task = 0;
+    while (task + 1 < a.n && (int)blockIdx.x >= a.first[task + 1]) ++task;
+    const int tile = blockIdx.x - a.first[task], rows = a.rows[task], cols = a.cols[task], tiles_x = (cols + 63) / 64;
+    const int r = (tile / tiles_x) * 64 + (t >> 2);
+    const int c0 = (tile % tiles_x) * 64 + (t & 3) * 16;
     if (r >= rows || c0 >= cols) return;
     long long sr = r;
-    if (row_idx) {
-        int s = row_idx[(size_t)z * idx_z + r];
-        if (s < 0 || s >= idx_limit) {
-            atomicOr(status, DBW_STATUS_BAD_INDEX);
-            s = s < 0 ? 0 : idx_limit - 1;
+    if (task == 0) {
+        int s = a.row_idx[(size_t)z * rows + r];
+        if (s < 0 || s >= a.samples) {
+            atomicOr(a.status, DBW_STATUS_BAD_INDEX);
+            s = s < 0 ? 0 : a.samples - 1;
         }
         sr = s;
-        if (c0 == 0) {  // the row's label; one outside [0, C) is clamped and reported
-            int y = labels[(size_t)z * idx_limit + s];
-            if (y < 0 || y >= C) {
-                atomicOr(status, DBW_STATUS_BAD_INDEX);
-                y = y < 0 ? 0 : C - 1;
+        if (c0 == 0) {
+            int y = a.labels[(size_t)z * a.samples + s];
+            if (y < 0 || y >= a.C) {
+                atomicOr(a.status, DBW_STATUS_BAD_INDEX);
+                y = y < 0 ? 0 : a.C - 1;
             }
-            ylab[(size_t)z * idx_z + r] = y;
+            a.ylab[(size_t)z * rows + r] = y;
         }
     }
-    const float* p = src + (size_t)z * src_z + sr * src_pitch + c0;
-    bf16* d = dst + (size_t)z * dst_z + (size_t)r * cols + c0;
+    const float* p = a.src[task] + (size_t)z * a.src_z[task] + sr * cols + c0;
+    bf16* d = a.dst[task] + (size_t)z * a.dst_z[task] + (size_t)r * cols + c0;
     float v[16];
 #pragma unroll
     for (int e = 0; e < 16; e += 4) {
@@ -1116,14 +1131,21 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     // bf16 copies of the weights of the tensor-core layers (inside the shadow rows), unless the
     // previous mix already wrote the shadow of this very X.
     const bool have_shadow = h->track_params && h->shadow_valid && h->shadow_of == X;
-    for (int l = 0; l <= L - 2 && !have_shadow; ++l) {
-        const int in = m.dims[l], out = m.dims[l + 1];
-        launch(cast_tile_kernel, dim3((in + 63) / 64, (out + 63) / 64, N), 256, 0, s, out, in, X + m.w_off[l], h->ld, in, nullptr, 0, 0, st->Wh[l], h->ld, nullptr, 0, nullptr, h->d_status);
-        DBW_LAUNCHED();
-    }
-    // mini-batch gather: A_0 in bf16, and the labels
-    launch(cast_tile_kernel, dim3((m.dims[0] + 63) / 64, (B + 63) / 64, N), 256, 0, s, B, m.dims[0], h->feat, (long long)h->S * m.dims[0], m.dims[0], batch_idx, B, h->S, st->A[0], (long long)B * m.dims[0],
-        h->labels, C, st->ylab, h->d_status);
+    CastArgs c{};
+    int blocks = 0;
+    auto task = [&](int rows, int cols, const float* src, long long src_z, bf16* dst, long long dst_z) {
+        c.first[c.n] = blocks;
+        c.rows[c.n] = rows; c.cols[c.n] = cols;
+        c.src[c.n] = src; c.src_z[c.n] = src_z;
+        c.dst[c.n] = dst; c.dst_z[c.n] = dst_z;
+        blocks += ((rows + 63) / 64) * ((cols + 63) / 64);
+        ++c.n;
+    };
+    task(B, m.dims[0], h->feat, (long long)h->S * m.dims[0], st->A[0], (long long)B * m.dims[0]);
+    for (int l = 0; l <= L - 2 && !have_shadow; ++l) task(m.dims[l + 1], m.dims[l], X + m.w_off[l], h->ld, st->Wh[l], h->ld);
+    c.row_idx = batch_idx; c.samples = h->S; c.C = C;
+    c.labels = h->labels; c.ylab = st->ylab; c.status = h->d_status;
+    launch(cast_kernel, dim3(blocks, N), 256, 0, s, c);
     DBW_LAUNCHED();
     // forward through the tensor-core layers
     for (int l = 0; l <= L - 2; ++l) {
