@@ -427,6 +427,13 @@ def test_grad_bf16_tensor_cores_match_oracle(dims, batch, n):
     h.close()
 
 
+@pytest.mark.parametrize("classes,batch,n", [(2, 8, 3), (8, 32, 2), (9, 40, 2), (12, 72, 3), (13, 24, 2), (16, 264, 2), (17, 16, 2)])
+def test_bf16_last_layer_at_the_edges_of_its_class_counts(classes, batch, n):
+    """Logits are summed over the lanes with samples and classes halved in turn: class counts on both sides of every halving and
+    of the kernel's variants, with the references and bars of the test above."""
+    test_grad_bf16_tensor_cores_match_oracle([128, 72, classes], batch, n)
+
+
 @pytest.mark.parametrize("flag", [0, 4])
 def test_label_out_of_range_is_clamped_and_reported(flag):
     """A label outside [0, classes) must not become an out-of-bounds read: it is clamped, the status word
