@@ -123,7 +123,9 @@ void free_all(dbw_handle* h) {
     if (h->side) cudaStreamDestroy(h->side);
     if (h->ev_loss) cudaEventDestroy(h->ev_loss);
     if (h->ev_read) cudaEventDestroy(h->ev_read);
-    h->ev_fork = h->ev_join = h->ev_loss = h->ev_read = nullptr;
+    if (h->ev_dz) cudaEventDestroy(h->ev_dz);
+    if (h->ev_tail) cudaEventDestroy(h->ev_tail);
+    h->ev_fork = h->ev_join = h->ev_loss = h->ev_read = h->ev_dz = h->ev_tail = nullptr;
     h->side = nullptr;
     grad_fp32_free(h);
     grad_bf16_free(h);
@@ -252,7 +254,9 @@ int dbw_init(dbw_handle** out, int32_t N, int64_t d, int64_t ld, const int32_t* 
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming)) ||
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming)) ||
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_loss, cudaEventDisableTiming)) ||
-        !cuda_ok(cudaEventCreateWithFlags(&h->ev_read, cudaEventDisableTiming)))
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_read, cudaEventDisableTiming)) ||
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_dz, cudaEventDisableTiming)) ||
+        !cuda_ok(cudaEventCreateWithFlags(&h->ev_tail, cudaEventDisableTiming)))
         return fail(DBW_ERR_CUDA);
     mix_sp_prepare(h);  // the 2:4 worker order of the sparse tensor-core mix, where that kernel can apply
     if (model) {

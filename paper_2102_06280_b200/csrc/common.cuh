@@ -182,6 +182,7 @@ struct dbw_handle {
     // into the caller's stream by the two events)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaEvent_t ev_dz = nullptr, ev_tail = nullptr;  // bf16 gradients: every dZ is there; the batch reductions beside the last GEMM are done
     cudaEvent_t ev_loss = nullptr, ev_read = nullptr;  // dbw_round_host: the losses are there; every result has been copied out
 
     // stage timing (dbw_profile): events[round][0..5] = start / end of the gradient, selection and mix stages
