@@ -282,8 +282,9 @@ inline bool fp32_head_usable(const dbw_handle* h) {
     return m.dims[L] <= 32 && (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 &&
            ((uintptr_t)h->feat & 15) == 0;
 }
-// Slices over k of an fp32 GEMM of `batch` problems M x N x K (GemmArgs::slice), the same for the per-step kernels and the
-// single launch, which sum in this order.
+// Slices over k of an fp32 backward GEMM of `batch` problems M x N x K (GemmArgs::slice), the same for the per-step kernels and
+// the single launch, which sum in this order.  Forward GEMMs are not sliced: whether a pre-activation of zero up to rounding
+// passes its ReLU follows from the order of its sum, which stays ascending in k for every shape.
 int fp32_gemm_slice(int M, int N, int K, int batch, bool is_dw, int sm_count);
 int grad_fp32_alloc(dbw_handle* h);
 void grad_fp32_free(dbw_handle* h);

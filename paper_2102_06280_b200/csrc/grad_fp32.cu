@@ -170,14 +170,14 @@ __global__ void __launch_bounds__(32 * WM) gemm_vec_kernel(GemmArgs g) {
     }
 }
 
-// The same for few tiles (fewer than the chip has schedulers).  Too few warps to hide latency behind, so a warp owns a tile of
+// The same for backward GEMMs of few tiles (fewer than the chip has schedulers).  Too few warps to hide latency behind, so a warp owns a tile of
 // 64 x 32 outputs, 8 x 8 per thread (below that shared-memory reads bound it: a 128-bit read takes four cycles of a pipe that
 // the SM's four schedulers share), with a ring of its own (three steps of eight k, asynchronous copies, no block barriers), and
 // the kSlices warps of a block share one tile: each sums its slice of k in ascending order and the slices are added in order.
-// Operands are staged as they lie in memory: one with its unit stride along k (AK / BK) as rows of eight k, of which a thread
+// Operands are staged as they lie in memory: one with its unit stride along k (AK) as rows of eight k, of which a thread
 // reads four at once (neighbouring lanes on neighbouring rows: distinct banks), one with its unit stride along the output as
-// eight rows.  (32 workers, 64 x 200 x 784: 29.8 us against 38.5; 10 workers, 256 x 256 x 1024: 46 against 60; with more tiles
-// the block-tile kernel is better: 10 workers, 1024 x 256 x 256: 41.5 against 45.5.)
+// eight rows.  (10 workers, 256 x 256 x 1024: 46 us against 60; with more tiles the block-tile kernel is better: 10 workers,
+// 1024 x 256 x 256: 41.5 against 45.5.)
 constexpr int kTileM = 64, kTileN = 32, kSlices = 4, kStepK = 8, kSteps = 3;
 
 // One operand of a warp's tile: R outputs, T of them per thread, LANES threads along it; KF: unit stride along k.
@@ -219,12 +219,12 @@ struct GemmOperand {
     }
 };
 
-template <bool SUMS, bool AK, bool BK>
+template <bool SUMS, bool AK>
 __global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __grid_constant__ GemmArgs g) {
     dependent_begin();
     constexpr int TM = 8, TN = 8, TX = kTileN / TN, TY = kTileM / TM;
     typedef GemmOperand<kTileM, TM, TY, AK> OpA;
-    typedef GemmOperand<kTileN, TN, TX, BK> OpB;
+    typedef GemmOperand<kTileN, TN, TX, false> OpB;
     constexpr int kRing = kSteps * (OpA::kFloats + OpB::kFloats), kExchange = TM * TN * 32 + 64;
     constexpr int kPerWarp = (kRing > kExchange ? kRing : kExchange + 3) / 4 * 4;
     __shared__ __align__(16) float sm[kSlices][kPerWarp];
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __gri
         if (step < steps) {
             float* st = ring + slot * (OpA::kFloats + OpB::kFloats);
             OpA::stage(st, A, AK ? g.sAm : g.sAk, m0, g.M, k_lo + step * kStepK, k_hi, lane);
-            OpB::stage(st + OpA::kFloats, B, BK ? g.sBn : g.sBk, n0, g.N, k_lo + step * kStepK, k_hi, lane);
+            OpB::stage(st + OpA::kFloats, B, g.sBk, n0, g.N, k_lo + step * kStepK, k_hi, lane);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
@@ -319,7 +319,6 @@ __global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __gri
             if (m0 + lane + 32 * h < g.M) g.rowsum[(size_t)z * g.sRz + m0 + lane + 32 * h] = rows[h];
     }
     float* C = g.C + (size_t)z * g.sCz;
-    const float* bias = g.bias ? g.bias + (size_t)z * g.sBiasz : nullptr;
     const float* mask = g.mask ? g.mask + (size_t)z * g.sMz : nullptr;
 #pragma unroll
     for (int i = 0; i < IPW; ++i) {
@@ -327,29 +326,16 @@ __global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __gri
         if (m >= g.M) continue;
         float* c = C + (size_t)m * g.sCm;
         const float* mk = mask ? mask + (size_t)m * g.sMm : nullptr;
-        if (BK) {
 #pragma unroll
-            for (int j = 0; j < TN; ++j) {
-                const int n = n0 + OpB::index(tx, j);
-                if (n >= g.N) continue;
-                float v = acc[i][j];
-                if (bias) v += __ldg(bias + n);
-                if (g.relu) v = fmaxf(v, 0.f);
-                if (mk && !(__ldg(mk + n) > 0.f)) v = 0.f;
-                c[n] = v;
+        for (int j = 0; j < TN; j += 4) {
+            const int n = n0 + OpB::index(tx, j);
+            if (n >= g.N) continue;  // N is a multiple of four: the four columns are inside or outside together
+            float4 v = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
+            if (mk) {
+                const float4 x = __ldg(reinterpret_cast<const float4*>(mk + n));
+                v.x = x.x > 0.f ? v.x : 0.f; v.y = x.y > 0.f ? v.y : 0.f; v.z = x.z > 0.f ? v.z : 0.f; v.w = x.w > 0.f ? v.w : 0.f;
             }
-        } else {
-#pragma unroll
-            for (int j = 0; j < TN; j += 4) {
-                const int n = n0 + OpB::index(tx, j);
-                if (n >= g.N) continue;  // N is a multiple of four: the four columns are inside or outside together
-                float4 v = make_float4(acc[i][j], acc[i][j + 1], acc[i][j + 2], acc[i][j + 3]);
-                if (mk) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(mk + n));
-                    v.x = x.x > 0.f ? v.x : 0.f; v.y = x.y > 0.f ? v.y : 0.f; v.z = x.z > 0.f ? v.z : 0.f; v.w = x.w > 0.f ? v.w : 0.f;
-                }
-                *reinterpret_cast<float4*>(c + n) = v;
-            }
+            *reinterpret_cast<float4*>(c + n) = v;
         }
     }
 }
@@ -422,17 +408,15 @@ void launch_gemm_vec(const GemmArgs& g, int batch, cudaStream_t s) {
 void launch_gemm_slice(const GemmArgs& g, int batch, cudaStream_t s) {
     const dim3 grid((g.N + kTileN - 1) / kTileN, (g.M + kTileM - 1) / kTileM, batch);
     if (g.sAk != 1 && g.rowsum)
-        launch<false>(gemm_slice_kernel<true, false, false>, grid, kSlices * 32, 0, s, g);
+        launch<false>(gemm_slice_kernel<true, false>, grid, kSlices * 32, 0, s, g);
     else if (g.sAk != 1)
-        launch<false>(gemm_slice_kernel<false, false, false>, grid, kSlices * 32, 0, s, g);
-    else if (g.sBk != 1)
-        launch<false>(gemm_slice_kernel<false, true, false>, grid, kSlices * 32, 0, s, g);
+        launch<false>(gemm_slice_kernel<false, false>, grid, kSlices * 32, 0, s, g);
     else
-        launch<false>(gemm_slice_kernel<false, true, true>, grid, kSlices * 32, 0, s, g);
+        launch<false>(gemm_slice_kernel<false, true>, grid, kSlices * 32, 0, s, g);
 }
 
 int run_gemm(GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
-    g.slice = fp32_gemm_slice(g.M, g.N, g.K, batch, g.sAk != 1, sm_count);
+    g.slice = g.bias ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, g.sAk != 1, sm_count);
     if (gemm_vec_ok(g) && g.slice < g.K) {
         launch_gemm_slice(g, batch, s);
         DBW_LAUNCHED();

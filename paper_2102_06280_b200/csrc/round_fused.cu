@@ -73,7 +73,7 @@ struct FusedArgs {
     float lr;
     const float* lr_pw;
     float* loss;
-    int fwd_slice[DBW_MAX_LAYERS], dw_slice[DBW_MAX_LAYERS], da_slice[DBW_MAX_LAYERS];
+    int dw_slice[DBW_MAX_LAYERS], da_slice[DBW_MAX_LAYERS];
     signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];
     float* head_part;
     int head;  // the last layer takes the small-output steps (at most 32 classes)
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.B = a.X + a.w_off[l]; g.sBz = a.ld; g.sBn = in; g.sBk = 1;
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
-        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = a.fwd_slice[l];
+        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in;
         gemm_any(a.fwd_var[l], g, N, smem);
         grid.sync();
     }
@@ -353,7 +353,6 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
         a.da_var[l] = (signed char)pick_variant(B, m.dims[l], m.dims[l + 1], N, grid);
     }
     for (int l = 0; l < m.n_layers; ++l) {
-        a.fwd_slice[l] = fp32_gemm_slice(B, m.dims[l + 1], m.dims[l], N, false, h->sm_count);
         a.dw_slice[l] = fp32_gemm_slice(m.dims[l + 1], m.dims[l], B, N, true, h->sm_count);
         a.da_slice[l] = fp32_gemm_slice(B, m.dims[l], m.dims[l + 1], N, false, h->sm_count);
     }
