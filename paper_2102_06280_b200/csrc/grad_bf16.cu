@@ -758,7 +758,7 @@ head_forward_staged_kernel(int N, int B, int K, int C, const bf16* __restrict__ 
         for (int c = 0; c < 2; ++c) z[c] = halve(b0, y3[c], y3[c + 2], 1);
         const int c0 = 8 * b2 + 4 * b1 + 2 * b0, s = s0 + 2 * b4 + b3;
         const int y = s < B ? ylab[(size_t)i * B + s] : -1;
-        float mx = -INFINITY, zy = -INFINITY, sum = 0.f, e[2];
+        float mx = -INFINITY, zy = -INFINITY, e[2], part[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             z[k] = c0 + k < C ? z[k] + __ldg(X + (size_t)i * ld + b_off + c0 + k) : -INFINITY;
@@ -772,11 +772,11 @@ head_forward_staged_kernel(int N, int B, int K, int C, const bf16* __restrict__ 
         }
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            e[k] = c0 + k < C ? expf(z[k] - mx) : 0.f;
-            sum += e[k];
-        }
+            e[k] = part[k] = c0 + k < C ? expf(z[k] - mx) : 0.f;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            for (int o = 4; o > 0; o >>= 1) part[k] += __shfl_xor_sync(0xffffffffu, part[k], o);
+        }
+        const float sum = part[0] + part[1];  // classes eight, four, two and one apart, as a sum over a warp's lanes takes them
         if (s < B) {
 #pragma unroll
             for (int k = 0; k < 2; ++k)
