@@ -340,6 +340,93 @@ __global__ void __launch_bounds__(kSlices * 32, 3) gemm_slice_kernel(const __gri
     }
 }
 
+// A forward GEMM (bias, ReLU), whose sums stay in ascending k.  A block is one warp with a tile of 32 x 32 outputs, 4 x 8 per
+// thread, and a ring of its own: no block barriers, hardly a partial tile, and an even spread over the schedulers.  What bounds it
+// is a step's latency, so operands are read from shared memory half a step ahead and a copy's addresses are formed once.
+constexpr int kWarpTile = 32, kWarpSteps = 6;
+__global__ void __launch_bounds__(32, 8) gemm_warp_kernel(const __grid_constant__ GemmArgs g) {
+    dependent_begin();
+    constexpr int TM = 4, TN = 8;
+    typedef GemmOperand<kWarpTile, TM, kWarpTile / TM, true> OpA;
+    typedef GemmOperand<kWarpTile, TN, kWarpTile / TN, true> OpB;
+    constexpr int kStep = OpA::kFloats + OpB::kFloats;
+    __shared__ __align__(16) float ring[kWarpSteps * kStep];
+    const int z = blockIdx.z, lane = threadIdx.x;
+    const int m0 = blockIdx.y * kWarpTile, n0 = blockIdx.x * kWarpTile;
+    const int ty = lane / (kWarpTile / TN), tx = lane % (kWarpTile / TN);
+    const float* A = g.A + (size_t)z * g.sAz;
+    const float* B = g.B + (size_t)z * g.sBz;
+    const int steps = (g.K + kStepK - 1) / kStepK;
+    // copies u = 0, 1 of each operand: 16 bytes at row (lane + 32 u) / 2, k = 4 (lane % 2) of a step
+    const int kc = 4 * (lane & 1);
+    const float *pa[2], *pb[2];
+    uint32_t to[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int r = (lane + 32 * u) / 2;
+        pa[u] = A + (long long)min(m0 + r, g.M - 1) * g.sAm + kc;
+        pb[u] = B + (long long)min(n0 + r, g.N - 1) * g.sBn + kc;
+        to[u] = (uint32_t)__cvta_generic_to_shared(ring + r * kStepK + kc);
+    }
+    auto fetch = [&](int step, int slot) {
+        const int k0 = step * kStepK;
+        if (step < steps) {
+            const int valid = k0 + kc < g.K ? 16 : 0, at = valid ? k0 : 0;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[u] + slot * kStep * 4), "l"(pa[u] + at - (valid ? 0 : kc)), "r"(valid) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to[u] + (slot * kStep + OpA::kFloats) * 4), "l"(pb[u] + at - (valid ? 0 : kc)), "r"(valid) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int s = 0; s < kWarpSteps - 1; ++s) fetch(s, s);
+    float acc[TM][TN] = {};
+    auto multiply = [&](const OpA& a, const OpB& b) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a.v[k][i], b.v[k][j], acc[i][j]);
+    };
+    OpA a[2];
+    OpB b[2];
+    asm volatile("cp.async.wait_group %0;" ::"n"(kWarpSteps - 2) : "memory");
+    __syncwarp();
+    a[0].load(ring, ty, 0);
+    b[0].load(ring + OpA::kFloats, tx, 0);
+    int slot = 0;
+#pragma unroll 1
+    for (int step = 0; step < steps; ++step) {
+        a[1].load(ring + slot * kStep, ty, 4);
+        b[1].load(ring + slot * kStep + OpA::kFloats, tx, 4);
+        multiply(a[0], b[0]);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kWarpSteps - 3) : "memory");
+        __syncwarp();  // the next step's copies have landed for every lane, and every lane is done with the step before
+        fetch(step + kWarpSteps - 1, slot == 0 ? kWarpSteps - 1 : slot - 1);
+        slot = slot == kWarpSteps - 1 ? 0 : slot + 1;
+        a[0].load(ring + slot * kStep, ty, 0);  // past the end: a slot's old values, not used
+        b[0].load(ring + slot * kStep + OpA::kFloats, tx, 0);
+        multiply(a[1], b[1]);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    float* C = g.C + (size_t)z * g.sCz;
+    const float* bias = g.bias + (size_t)z * g.sBiasz;
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+        const int n = n0 + OpB::index(tx, j);
+        if (n >= g.N) continue;
+        const float bn = __ldg(bias + n);
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            const int m = m0 + OpA::index(ty, i);
+            if (m < g.M) C[(size_t)m * g.sCm + n] = g.relu ? fmaxf(acc[i][j] + bn, 0.f) : acc[i][j] + bn;
+        }
+    }
+}
+
 // 128-bit accesses are possible: unit stride along k or along the output dimension, everything else a multiple of four floats
 bool gemm_vec_ok(const GemmArgs& g) {
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
@@ -419,6 +506,17 @@ int run_gemm(GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
     g.slice = g.bias ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, g.sAk != 1, sm_count);
     if (gemm_vec_ok(g) && g.slice < g.K) {
         launch_gemm_slice(g, batch, s);
+        DBW_LAUNCHED();
+        return DBW_OK;
+    }
+    // One-warp blocks where every SM gets at least two of them and none more than the eight that fit it at once.  Measured (workers,
+    // M x N x K, tiles: one-warp / block-tile kernel, us): 32, 64 x 200 x 784, 448: 30.3 / 38.2; 64 of them, 896: 48.8 / 64.7; 60,
+    // 128 x 128 x 256, 960: 19.4 / 23.2.  Fewer tiles leave the schedulers idle: 64, 64 x 64 x 784, 256: 29.8 / 28.6; 3, 64 x 200 x
+    // 784, 42: 27.6 / 24.9.  More run in waves: 10, 1024 x 256 x 784, 2560: 118 / 120, and a round with two such of K = 256
+    // 335 / 328.  A short sum does not pay for filling the ring: 60, 64 x 128 x 64, 480: 6.0 / 5.2.
+    const long long warp_tiles = (long long)((g.N + kWarpTile - 1) / kWarpTile) * ((g.M + kWarpTile - 1) / kWarpTile) * batch;
+    if (gemm_vec_ok(g) && g.bias && g.K >= 128 && warp_tiles >= 2LL * sm_count && warp_tiles <= 8LL * sm_count) {
+        launch<false>(gemm_warp_kernel, dim3((g.N + kWarpTile - 1) / kWarpTile, (g.M + kWarpTile - 1) / kWarpTile, batch), 32, 0, s, g);
         DBW_LAUNCHED();
         return DBW_OK;
     }

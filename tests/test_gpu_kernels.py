@@ -734,6 +734,8 @@ def test_round_with_few_participants_gives_the_bits_of_its_steps(dims, batch, n,
                                           ([68, 36, 100, 12], 20, 3),   # GEMMs in slices of k: ragged tiles, a last slice of a few k
                                           ([260, 64, 32, 10], 64, 5),   # ... whole tiles, a slice of less than a step more
                                           ([128, 320, 64, 10], 64, 60),  # as many tiles as do without slices, and fewer
+                                          ([132, 100, 12], 52, 40),     # one-warp forward tiles: ragged in every dimension
+                                          ([128, 320, 64, 10], 20, 60),  # ... one row of them, k of whole steps
                                           ([64, 30, 36, 10], 18, 3)])   # widths and a batch without 128-bit accesses beside some with
 def test_fp32_last_layer_in_parts_of_the_batch(dims, batch, n):
     """The last layer's backward step splits a large batch into parts whose sums are added in a fixed order.  Gradients and
