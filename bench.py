@@ -35,11 +35,8 @@ UNIT = "worker-rounds/s"
 DEFAULT_CONFIG = 4
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the mix kernel, from the ncu captures summarised
 # under profiles/ (config 4: the d = 65,536 case scaled by 16, the traffic being proportional to the columns
-# processed; configs 2 and 3: their mix at full size).  Reported only for the kernel the capture was taken of;
-# None = not captured for this workload.
-MIX_TRAFFIC_BYTES = {4: ("mix_staged_kernel", (537.05e6 + 220.89e6) * 16),
-                     3: ("mix_panel_kernel", 4.316048e9 + 3.227908e9),
-                     2: ("mix_panel_kernel", 875.2448e6 + 612.1979e6)}
+# processed).  Reported only for the kernel the capture was taken of; None = not captured for this workload.
+MIX_TRAFFIC_BYTES = {4: ("mix_staged_kernel", (537.05e6 + 220.89e6) * 16)}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
@@ -539,6 +536,8 @@ def measure(config, local, args, dist, overrides, col_range=None):
                stage_ms={k: v / max(stage_rounds, 1) for k, v in stage_ms.items()},
                bytes=job.host_bytes_per_step(), mix_bytes=job.mix_bytes_per_launch(),
                kept_last=int(job.kept.sum().item()), sms=torch.cuda.get_device_properties(local).multi_processor_count)
+    before = np.concatenate([[0], np.cumsum(job.kept.cpu().numpy() != 0)])
+    out["mixing_last"] = int(np.count_nonzero(before[job.w.rowptr[1:]] - before[job.w.rowptr[:-1]]))  # workers with a kept neighbour
     job.close()
     del job
     torch.cuda.empty_cache()
@@ -613,6 +612,14 @@ def summary(res, world, args):
         out["roofline"].update({"kernel": "round_fused_kernel", "achieved": None, "frac": None, "frac_of_8TBps_nominal": None,
                                 "note": "one cooperative launch per round; launch-bound, no separate mix kernel"})
         out["roofline"]["operand_delivery"].update({"achieved": None, "frac": None})
+    tc_flops, tc_bytes = tensor_core_gemm_work(w)
+    if tc_flops and res["mixing_last"] <= w.N // 2:
+        # the dW GEMMs take the step of the workers without a kept neighbour: x in, x' and its bf16 copy out instead of dW out
+        tc_bytes += (w.N - res["mixing_last"]) * 6 * sum(o * i for o, i in wl.layer_dims(w.layers)[:-1])
+        out["roofline"].update({"achieved": None, "frac": None, "frac_of_8TBps_nominal": None, "traffic": None,
+                                "note": "%d of %d workers have a kept neighbour: the dW GEMMs take the others' step (roofline_gemm), the mix "
+                                        "stage is left with the rest" % (res["mixing_last"], w.N)})
+        out["roofline"]["operand_delivery"].update({"achieved": None, "frac": None})
     if res.get("graph_ms"):
         out["cuda_graph"] = {"rounds_per_graph": args.graph, "ms_per_step": res["graph_ms"] / args.steps,
                              "value": aggregate_value(w.N, args.steps, res["graph_ms"], world, sharded),
@@ -622,7 +629,6 @@ def summary(res, world, args):
         out["gradients"] = {"dense_flop_per_round": flops,
                             "tflops_over_grad_stage": flops / (res["stage_ms"]["grad"] * 1e-3) / 1e12,
                             "note": "grad stage = gather, casts, GEMMs, loss and last layer together"}
-    tc_flops, tc_bytes = tensor_core_gemm_work(w)
     gemm_ms = res["stage_ms"].get("gemm", 0.0)
     if tc_flops and gemm_ms > 0:
         # The dense layers' GEMMs (batch 128-256 per worker) stream their weights or their fp32 result once: they sit
@@ -631,7 +637,7 @@ def summary(res, world, args):
         tf = tc_flops / (gemm_ms * 1e-3) / 1e12
         gbs = tc_bytes / (gemm_ms * 1e-3) / 1e9
         peak_tf = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
-        out["roofline_gemm"] = {"kernel": "gemm_tc_kernel (all tensor-core launches of a round)", "ms_per_round": gemm_ms,
+        out["roofline_gemm"] = {"kernel": "gemm_tc_kernel, gemm_dw_kernel (all tensor-core launches of a round)", "ms_per_round": gemm_ms,
                                 "flop_per_round": tc_flops, "achieved": tf, "peak": peak_tf, "unit": "TFLOP/s",
                                 "frac": tf / peak_tf, "peak_kind": "sustained bf16, of " + peak_kind,
                                 "hbm_bytes_per_round": tc_bytes, "achieved_gbs": gbs, "frac_hbm": gbs / peaks["hbm_gbs"],
