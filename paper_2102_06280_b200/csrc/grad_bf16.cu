@@ -1152,6 +1152,8 @@ int launch_grad_bf16(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     // bf16 copies of the weights of the tensor-core layers (inside the shadow rows), unless the
     // previous mix already wrote the shadow of this very X.
     const bool have_shadow = h->track_params && h->shadow_valid && h->shadow_of == X;
+    // From here on the copy is of this X, or (after a dW launch that steps) of no one matrix until the mix has written its part.
+    if (!have_shadow || (step && h->track_params)) h->shadow_valid = false;
     CastArgs c{};
     int blocks = 0;
     auto task = [&](int rows, int cols, const float* src, long long src_z, bf16* dst, long long dst_z) {

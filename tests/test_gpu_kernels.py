@@ -831,3 +831,38 @@ def test_staged_kernel_at_the_edges_of_its_panel_widths(n, deg, rule, order):
         assert torch.equal(Y, Z)
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("between", ["grad", "round_of_another_matrix"])
+def test_tracked_copy_is_forgotten_when_other_parameters_pass_through(between):
+    """With parameter tracking the bf16 copy belongs to the X_out of the call before.  Gradients of another matrix Z in between
+    (an averaged model, say) overwrite it: gradients of the tracked matrix Y afterwards are those without tracking, bit for bit."""
+    p = _dbw()
+    dims, batch, n = [128, 72, 64, 10], 32, 6
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m, flags=p.GEMM_BF16)
+    rng = np.random.default_rng(8)
+    S = 2 * batch
+    feat, labels = dev(rng.standard_normal((n, S, dims[0]), dtype=np.float32)), dev(rng.integers(0, dims[-1], size=(n, S)).astype(np.int32))
+    h.set_dataset(feat, labels, S)
+    X, Z = (dev(m.pack(0.1 * rng.standard_normal((n, m.d)).astype(np.float32))) for _ in range(2))
+    idx = dev(rng.integers(0, S, size=(n, batch)).astype(np.int32))
+    t = dev(1.0 + rng.random(n))
+    kept = torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+    for backups in (1, 2):  # everybody mixes / the dW GEMMs take everybody's step
+        b = torch.full((n,), backups, dtype=torch.int32, device="cuda")
+        h.set_param_tracking(True)
+        Y, other = torch.empty_like(X), torch.empty_like(X)
+        h.round(X, t, b, 0.05, Y, kept, batch_idx=idx)
+        G, G_ref = torch.zeros_like(X), torch.zeros_like(X)
+        if between == "grad":
+            h.grad(Z, idx, G)
+        else:
+            h.round(Z, t, b, 0.05, other, kept, batch_idx=idx)
+        h.grad(Y, idx, G)
+        h.set_param_tracking(False)
+        h.grad(Y, idx, G_ref)
+        assert torch.equal(G, G_ref), backups
+    assert h.status() == 0
+    h.close()
