@@ -305,8 +305,11 @@ int dbw_grad(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, 
     if (!h->has_model || !h->feat) return DBW_ERR_BAD_MODEL;
     if (!aligned16(X) || !aligned16(G)) return DBW_ERR_BAD_SHAPE;
     DeviceGuard guard(h->device);
-    return (h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, G, loss, (cudaStream_t)stream)
-                                      : launch_grad_fp32(h, X, batch_idx, G, loss, (cudaStream_t)stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int rc = (h->flags & DBW_GEMM_BF16) ? launch_grad_bf16(h, X, batch_idx, G, loss, s) : launch_grad_fp32(h, X, batch_idx, G, loss, s);
+    // what a failed call has left on the side stream is joined back too
+    if (rc != DBW_OK && cuda_ok(cudaEventRecord(h->ev_join, h->side))) cuda_ok(cudaStreamWaitEvent(s, h->ev_join, 0));
+    return rc;
 }
 
 static int check_mix_args(dbw_handle* h, const float* X, const float* G, float* X_out) {
@@ -454,7 +457,7 @@ static int run_round(dbw_handle* h, const float* X, const double* t, const int32
     // Tensor-core rounds: the dW GEMMs take the step of the workers that take no part, so they wait for the selection.
     const bool stepped = batch_idx && (h->flags & DBW_GEMM_BF16) && mix_active_usable(h);
     bool joinable = false;  // ev_join has been recorded behind everything queued on the side stream
-    const std::function<int()> select = [&]() -> int {
+    auto queue_selection = [&]() -> int {
         int code = io ? copy_inputs(h, *io, sel) : DBW_OK;
         if (ev) cuda(cudaEventRecord(ev[2], sel));
         if (code == DBW_OK) code = launch_select(h, t, b, kept, T_worker, T_nbr, T_round, true, sel, stepped);
@@ -463,6 +466,7 @@ static int run_round(dbw_handle* h, const float* X, const double* t, const int32
         joinable = true;
         return code;
     };
+    const std::function<int()> select = std::ref(queue_selection);  // (holds a reference: nothing is allocated, nothing thrown)
     if (io) note(copy_batch(h, *io, s));
     if (ev) cuda(cudaEventRecord(ev[0], s));
     const StepArgs step{lr, lr_per_worker, X_out, h->ev_join};
@@ -471,7 +475,7 @@ static int run_round(dbw_handle* h, const float* X, const double* t, const int32
                                         : launch_grad_fp32(h, X, batch_idx, h->d_G, loss, s, &select));
     else if (first == DBW_OK)
         note(select());
-    if (forked && !joinable) cuda(cudaEventRecord(h->ev_join, sel));
+    if (forked && (!joinable || first != DBW_OK)) cuda(cudaEventRecord(h->ev_join, sel));  // again: the gradients may have queued work there too
     if (ev) cuda(cudaEventRecord(ev[1], s));
     if (io) cuda(cudaEventRecord(h->ev_loss, s));
     // whatever failed above, the side stream is joined back: it never dangles, a capture stays valid
@@ -483,7 +487,10 @@ static int run_round(dbw_handle* h, const float* X, const double* t, const int32
     }
     if (io) {
         if (first == DBW_OK) note(copy_results(h, *io, h->ev_loss, sel));
-        cuda(cudaEventRecord(h->ev_read, sel));
+        if (!cuda_ok(cudaEventRecord(h->ev_read, sel))) {
+            note(DBW_ERR_CUDA);
+            cuda(cudaEventRecord(h->ev_read, sel));  // again: the copies are on their way
+        }
         cuda(cudaStreamWaitEvent(s, h->ev_read, 0));
     }
     return first;
