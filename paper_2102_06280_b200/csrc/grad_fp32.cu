@@ -36,9 +36,9 @@ softmax_ce_kernel(int B, int C, const float* __restrict__ logits, const int32_t*
 }
 
 __global__ void bias_grad_kernel(int B, int out_dim, const float* __restrict__ dz, float* __restrict__ G,
-                                 long long ld, long long b_off, int slice) {
+                                 long long ld, long long b_off) {
     dependent_begin();
-    bias_grad_col(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, B, out_dim, dz, G, ld, b_off, slice);
+    bias_grad_col(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, B, out_dim, dz, G, ld, b_off, B);
 }
 
 // The GEMM for operands whose unit-stride dimension allows 128-bit accesses (every layer whose width and
@@ -502,8 +502,9 @@ void launch_gemm_slice(const GemmArgs& g, int batch, cudaStream_t s) {
         launch<false>(gemm_slice_kernel<false, true>, grid, kSlices * 32, 0, s, g);
 }
 
-int run_gemm(GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
-    g.slice = g.bias ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, g.sAk != 1, sm_count);
+enum GemmStep { GEMM_FORWARD, GEMM_DW, GEMM_DA };
+int run_gemm(GemmArgs& g, GemmStep step, int batch, int sm_count, cudaStream_t s) {
+    g.slice = step == GEMM_FORWARD ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, step == GEMM_DW, sm_count);
     if (gemm_vec_ok(g) && g.slice < g.K) {
         launch_gemm_slice(g, batch, s);
         DBW_LAUNCHED();
@@ -515,7 +516,7 @@ int run_gemm(GemmArgs& g, int batch, int sm_count, cudaStream_t s) {
     // 784, 42: 27.6 / 24.9.  More run in waves: 10, 1024 x 256 x 784, 2560: 118 / 120, and a round with two such of K = 256
     // 335 / 328.  A short sum does not pay for filling the ring: 60, 64 x 128 x 64, 480: 6.0 / 5.2.
     const long long warp_tiles = (long long)((g.N + kWarpTile - 1) / kWarpTile) * ((g.M + kWarpTile - 1) / kWarpTile) * batch;
-    if (gemm_vec_ok(g) && g.bias && g.K >= 128 && warp_tiles >= 2LL * sm_count && warp_tiles <= 8LL * sm_count) {
+    if (gemm_vec_ok(g) && step == GEMM_FORWARD && g.K >= 128 && warp_tiles >= 2LL * sm_count && warp_tiles <= 8LL * sm_count) {
         launch<false>(gemm_warp_kernel, dim3((g.N + kWarpTile - 1) / kWarpTile, (g.M + kWarpTile - 1) / kWarpTile, batch), 32, 0, s, g);
         DBW_LAUNCHED();
         return DBW_OK;
@@ -609,7 +610,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.C = h->d_act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = X + m.b_off[l]; g.sBiasz = h->ld;
         g.M = B; g.N = out; g.K = in; g.relu = l < L - 1;
-        if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
+        if ((rc = run_gemm(g, GEMM_FORWARD, N, h->sm_count, s)) != DBW_OK) return rc;
     }
     if (beside && (rc = (*beside)())) return rc;
     if (head) {
@@ -662,9 +663,9 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
             g.rowsum = G + m.b_off[l];
             g.sRz = h->ld;
         }
-        if ((rc = run_gemm(g, N, h->sm_count, s)) != DBW_OK) return rc;
+        if ((rc = run_gemm(g, GEMM_DW, N, h->sm_count, s)) != DBW_OK) return rc;
         if (needs_db && !db_here) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
-            launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l], g.slice);
+            launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
             DBW_LAUNCHED();
         }
         if (l > 0) {  // dZ_{l}[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]
@@ -674,7 +675,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
             a.C = h->d_dz[l]; a.sCz = (long long)B * in; a.sCm = in;
             a.mask = h->d_act[l]; a.sMz = (long long)B * in; a.sMm = in;
             a.M = B; a.N = in; a.K = out;
-            if ((rc = run_gemm(a, N, h->sm_count, s)) != DBW_OK) return rc;
+            if ((rc = run_gemm(a, GEMM_DA, N, h->sm_count, s)) != DBW_OK) return rc;
         }
     }
     return DBW_OK;

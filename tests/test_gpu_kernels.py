@@ -866,3 +866,30 @@ def test_tracked_copy_is_forgotten_when_other_parameters_pass_through(between):
         assert torch.equal(G, G_ref), backups
     assert h.status() == 0
     h.close()
+
+
+def test_bias_gradient_of_a_layer_of_one_unit():
+    """One unit: its dW GEMM has unit stride along k on both sides and no slices, and its bias gradient is summed in the same order,
+    step by step and in one launch."""
+    p = _dbw()
+    dims, batch, n = [64, 1, 10], 128, 3
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    rng = np.random.default_rng(12)
+    feat, labels = dev(rng.random((n, batch, dims[0]), dtype=np.float32)), dev(rng.integers(0, 10, size=(n, batch)).astype(np.int32))
+    h.set_dataset(feat, labels, batch)
+    X = m.pack((0.3 * rng.standard_normal((n, m.d))).astype(np.float32))
+    X[:, m.w_off[0]: m.w_off[0] + dims[0]] = np.abs(X[:, m.w_off[0]: m.w_off[0] + dims[0]])  # every sample passes the ReLU
+    X[:, m.b_off[0]] = 0.0  # its step is all that is left of it
+    idx = dev(np.stack([rng.permutation(batch) for _ in range(n)]).astype(np.int32))
+    t, b = dev(1.0 + rng.random(n)), torch.full((n,), 2, dtype=torch.int32, device="cuda")
+    outs = []
+    for fused in (True, False):
+        h.set_fused_round(fused)
+        Y, kept = dev(X), torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+        h.round(Y, t, b, 0.05, Y, kept, batch_idx=idx)
+        outs.append(Y)
+    assert torch.equal(outs[0], outs[1])
+    assert h.status() == 0
+    h.close()
