@@ -95,14 +95,14 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
             const int e = tid + r * 256;
             const int ka = a_k_fast ? (e % TK) : (e / T);
             const int ma = a_k_fast ? (e / TK) : (e % T);
-            pa[r] = (m0 + ma < g.M && k0 + ka < k_end) ? load_g<NC>(A + (size_t)(m0 + ma) * g.sAm + (size_t)(k0 + ka) * g.sAk) : 0.f;
+            pa[r] = (m0 + ma < g.M && k0 + ka < (SLICED ? k_end : g.K)) ? load_g<NC>(A + (size_t)(m0 + ma) * g.sAm + (size_t)(k0 + ka) * g.sAk) : 0.f;
             const int kb = b_k_fast ? (e % TK) : (e / T);
             const int nb = b_k_fast ? (e / TK) : (e % T);
-            pb[r] = (n0 + nb < g.N && k0 + kb < k_end) ? load_g<NC>(B + (size_t)(n0 + nb) * g.sBn + (size_t)(k0 + kb) * g.sBk) : 0.f;
+            pb[r] = (n0 + nb < g.N && k0 + kb < (SLICED ? k_end : g.K)) ? load_g<NC>(B + (size_t)(n0 + nb) * g.sBn + (size_t)(k0 + kb) * g.sBk) : 0.f;
         }
     };
     fetch(0);
-    for (int k0 = 0; k0 < g.K;) {
+    auto step = [&](int next) {  // the staged step is multiplied while the one from k = next on is fetched
 #pragma unroll
         for (int r = 0; r < PER; ++r) {
             const int e = tid + r * 256;
@@ -110,12 +110,6 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
             Bs[b_k_fast ? (e % TK) : (e / T)][b_k_fast ? (e / TK) : (e % T)] = pb[r];
         }
         __syncthreads();
-        const int slice_of = k_end;
-        int next = k0 + TK;
-        if (SLICED && next >= k_end) {  // the next step begins the next slice
-            next = k_end;
-            k_end = min(g.K, k_end + g.slice);
-        }
         fetch(next);  // all zero past the end
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
@@ -136,19 +130,31 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
 #pragma unroll
                 for (int j = 0; j < R; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
-        if (SLICED && next >= slice_of) {  // a slice is complete
-            const bool first = slice_of <= g.slice;
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int j = 0; j < R; ++j) {
-                    float& t = total[SLICED ? i : 0][SLICED ? j : 0];
-                    t = first ? acc[i][j] : t + acc[i][j];
-                    acc[i][j] = 0.f;
-                }
-        }
-        k0 = next;
         __syncthreads();
+    };
+    if constexpr (!SLICED) {
+        for (int k0 = 0; k0 < g.K; k0 += TK) step(k0 + TK);
+    } else {
+        for (int k0 = 0; k0 < g.K;) {
+            const int slice_of = k_end;
+            int next = k0 + TK;
+            if (next >= k_end) {  // the next step begins the next slice
+                next = k_end;
+                k_end = min(g.K, k_end + g.slice);
+            }
+            step(next);
+            if (next >= slice_of) {  // a slice is complete
+                const bool first = slice_of <= g.slice;
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        total[i][j] = first ? acc[i][j] : total[i][j] + acc[i][j];
+                        acc[i][j] = 0.f;
+                    }
+            }
+            k0 = next;
+        }
     }
     float* C = g.C + (size_t)z * g.sCz;
     const float* bias = g.bias ? g.bias + (size_t)z * g.sBiasz : nullptr;
@@ -246,18 +252,25 @@ __device__ __forceinline__ void softmax_ce_worker(int i, int B, int C, const flo
     }
 }
 
-// db[i][o] = sum over the batch of dZ[i][m][o], in the order of the dW GEMM: sample order within its slices, slices in order
+// db[i][o] = sum over the batch of dZ[i][m][o], in the order of the dW GEMM: sample order within its slices, slices in order.
+// SLICED: slice may be less than B.
+template <bool SLICED>
 __device__ __forceinline__ void bias_grad_col(int i, int o, int B, int out_dim, const float* dz, float* G,
                                               long long ld, long long b_off, int slice) {
     if (o >= out_dim) return;
     const float* p = dz + (size_t)i * B * out_dim + o;
     float total = 0.f;
-    for (int m0 = 0; m0 < B; m0 += slice) {
-        float s = 0.f;
-        const int m1 = min(B, m0 + slice);
+    if constexpr (!SLICED) {
 #pragma unroll 8
-        for (int m = m0; m < m1; ++m) s += p[(size_t)m * out_dim];
-        total = m0 == 0 ? s : total + s;
+        for (int m = 0; m < B; ++m) total += p[(size_t)m * out_dim];
+    } else {
+        for (int m0 = 0; m0 < B; m0 += slice) {
+            float s = 0.f;
+            const int m1 = min(B, m0 + slice);
+#pragma unroll 8
+            for (int m = m0; m < m1; ++m) s += p[(size_t)m * out_dim];
+            total = m0 == 0 ? s : total + s;
+        }
     }
     G[(size_t)i * ld + b_off + o] = total;
 }

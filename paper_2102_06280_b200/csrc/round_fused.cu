@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         gemm_any(a.dw_var[l], g, N, smem);
         if (l < L - 1 && !(a.head && l == L - 2))  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
             for (int e = blockIdx.x * kThreads + tid; e < N * out; e += gridDim.x * kThreads)
-                bias_grad_col(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l], a.dw_slice[l]);
+                bias_grad_col<true>(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l], a.dw_slice[l]);
         if (l > 0) {  // dZ_l[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]
             GemmArgs d{};
             d.A = a.dz[l + 1]; d.sAz = (long long)B * out; d.sAm = out; d.sAk = 1;
