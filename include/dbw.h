@@ -224,8 +224,10 @@ int dbw_round(dbw_handle* h, const float* X, const double* t, const int32_t* b,
  * gather, forward, loss, backward, selection, weights, times and the mix inside one persistent kernel with
  * grid-wide barriers between dependent steps.  The results are bit-identical to the multi-launch path (the
  * same device functions in the same order per output element).  enable = -1 (the default) uses it where it
- * is the faster path (up to 512 samples over all workers and 1.6e7 multiply-adds per forward pass: above that the per-step
- * kernels, which put more blocks on an SM than a cooperative grid can, win), 1 wherever it applies, 0 never.
+ * is the faster path: up to 2560 samples over all workers for one layer, 2048 of at most 20 workers for more, where the last layer
+ * has at most 32 classes and a width that is a multiple of four (else 64 and 512 samples, the latter with no more than 148 tiles
+ * and 1.6e7 multiply-adds per forward pass): above that the per-step kernels, which put more blocks on an SM than a
+ * cooperative grid can, win.  1 wherever it applies, 0 never.
  * dbw_round_is_fused() tells which path dbw_round would take (1 = single launch).  With stage timing on, the
  * whole launch is reported under stage 0.
  */

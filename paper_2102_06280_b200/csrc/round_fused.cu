@@ -32,12 +32,22 @@ constexpr int kMixGS = 32;                       // 128-column panels
 constexpr int kMaxWorkers = 64;                  // N * kMixGS * 16 bytes of panel <= 32 KiB
 constexpr int kSmemBytes = 2 * 128 * 36 * 4;     // the largest GEMM staging (32 x 32 tiles, 128-deep steps): 36,864 bytes
 constexpr int kBlocksPerSM = 1;                  // registers are spent on deep k-steps (a step costs one memory round trip)
-// Samples and multiply-adds of the forward pass up to which the launch is used unasked: above them the per-step kernels, placed
-// early and with as many blocks as they want, are the faster path.  Measured (single launch / step by step, us): 8 workers x
-// batch 32, 784-10: 19 / 33 and 256-64-64-10: 51 / 57; 5 x 70, 205-186-20-10: 73 / 75; 30 x 19, 784-53-10: 72 / 67; 42 x 56,
-// 37-10: 39 / 31; 63 x 75, 64-92-10: 91 / 58.
-constexpr long long kAutoMaxSamples = 512;
-constexpr long long kAutoMaxMacs = 16 << 20;
+// Networks for which the launch is used unasked: those where it is the faster path, which depends on the steps it has to make.  What
+// it saves is launches; what it costs is that one block to an SM works off all samples and tiles, and that its steps wait for
+// the slowest block.  Where the lines lie was measured on 1700 networks of 3 - 64 workers (single launch / step by step, us):
+//  - one layer, whose last layer's two steps read the data set themselves: up to 2560 samples over all workers (8 workers x batch 32,
+//    784-10: 19 / 33, 16 x 64, 784-10: 24 / 36, 41 x 52, 784-10: 39 / 40; 25 x 265, 121-10 is of the next kind: 92 / 62);
+//  - one layer as a GEMM (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26);
+//  - more layers, the last one in those two steps: 2048 samples of at most 20 workers (8 x 128, 256-64-10: 50 / 59, 8 x 268, 64-96-10:
+//    74 / 79; 40 x 17, 16-108-10: 45 / 36);
+//  - more layers, all of them GEMMs: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16 million multiply-adds.
+// Never above 64 million multiply-adds of the forward pass.
+struct AutoLimits {
+    long long samples, tiles, workers, macs;
+};
+constexpr long long kAny = 1ll << 40;
+constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {2560, kAny, kAny, 64 << 20}},   // one layer: a GEMM / small outputs
+                                    {{512, 148, kAny, 16 << 20}, {2048, kAny, 20, 64 << 20}}};    // more
 
 // GEMM tile variants (R, TK) the kernel instantiates; which one a GEMM uses is chosen on the host.
 enum { V_2_16 = 0, V_2_64 = 1, V_4_16 = 2, V_4_64 = 3, V_2_128 = 4, kVariants = 5 };
@@ -298,9 +308,15 @@ void round_fused_prepare(dbw_handle* h) {
     if (!cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device)) || !coop) return;
     if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, round_fused_kernel, kThreads, kSmemBytes)) || per_sm < 1) return;
     st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
-    long long macs = 0;
-    for (int l = 0; l < h->model.n_layers; ++l) macs += (long long)h->N * h->model.batch * h->model.dims[l] * h->model.dims[l + 1];
-    st->auto_on = macs <= kAutoMaxMacs && (long long)h->N * h->model.batch <= kAutoMaxSamples;
+    const dbw_model_desc& m = h->model;
+    const long long samples = (long long)h->N * m.batch;
+    long long macs = 0, tiles = 0;
+    for (int l = 0; l < m.n_layers; ++l) {
+        macs += samples * m.dims[l] * m.dims[l + 1];
+        if (l + 1 < m.n_layers) tiles = std::max(tiles, (long long)h->N * ((m.batch + 31) / 32) * ((m.dims[l + 1] + 31) / 32));
+    }
+    const AutoLimits& a = kAuto[m.n_layers > 1][fp32_head_usable(h)];
+    st->auto_on = samples <= a.samples && tiles <= a.tiles && h->N <= a.workers && macs <= a.macs;
     st->usable = true;
 }
 

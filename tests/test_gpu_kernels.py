@@ -893,3 +893,20 @@ def test_bias_gradient_of_a_layer_of_one_unit():
     assert torch.equal(outs[0], outs[1])
     assert h.status() == 0
     h.close()
+
+
+# both sides measured where the lines were drawn (csrc/round_fused.cu)
+@pytest.mark.parametrize("dims,batch,n,single", [([784, 10], 32, 8, True), ([784, 10], 64, 16, True), ([256, 10], 128, 20, True), ([256, 10], 129, 20, False),
+                                                 ([121, 10], 16, 4, True), ([121, 10], 17, 4, False),
+                                                 ([256, 64, 10], 128, 8, True), ([64, 40, 10], 24, 21, False), ([64, 40, 10], 102, 20, True),
+                                                 ([64, 41, 10], 32, 16, True), ([64, 41, 10], 33, 16, False), ([64, 41, 41, 10], 4, 50, True),
+                                                 ([784, 200, 10], 64, 32, False), ([784, 320, 10], 128, 4, False)])
+def test_which_rounds_are_one_launch(dims, batch, n, single):
+    p = _dbw()
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    feat, labels = torch.zeros(n, batch, dims[0], device="cuda"), torch.zeros(n, batch, dtype=torch.int32, device="cuda")
+    h.set_dataset(feat, labels, batch)
+    assert h.round_is_fused() == single
+    h.close()
