@@ -249,6 +249,20 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
     return DBW_OK;
 }
 
+// 64 columns to a panel instead of 128 where the panels are then walked in fewer turns of all blocks, by a twelfth at least, or with
+// more than twelve neighbours a sixth: as many turns of half the width cost more (rows of 256 bytes instead of 512, and the
+// mixing plan read twice as often).  Measured with 128 / 64 columns: 96 workers x
+// 300,007 columns (6 turns or 11 halves) 111 / 104 us, 78 x 8372 (1 / 1) 10.4 / 7.8, 173 x 166,798 (two blocks an SM, 5 / 6) 125 /
+// 108; 109 x 1,298,095 (23 / 46) 950 / 1397, 116 x 1,614,144 (29 / 57) 2074 / 2244, 74 x 660,293 (12 / 24) 138 / 156,
+// with 16 neighbours 113 x 253,162 (5 / 9) 147 / 168.
+int narrower_panel(dbw_handle* h, bool* narrower) {
+    int wide = 0, narrow = 0, rc;
+    if ((rc = panel_blocks<32>(h, &wide)) || (rc = panel_blocks<16>(h, &narrow))) return rc;
+    auto turns = [h](int cols, int per_sm) { return (((h->ld + cols - 1) / cols) + per_sm * h->sm_count - 1) / (per_sm * h->sm_count); };
+    *narrower = 100 * turns(64, narrow) < (h->nnz > 12 * h->N ? 168 : 184) * turns(128, wide);
+    return DBW_OK;
+}
+
 template <int GS>
 int launch_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow,
                   cudaStream_t s) {
@@ -362,10 +376,12 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     if (use_tc(h)) return launch_mix_tc(h, X, G, lr, lr_pw, X_out, shadow, s);
     if (use_staged(h)) return launch_mix_staged(h, X, G, lr, lr_pw, X_out, shadow, s);
     int gs = auto_group_size(h);
-    // 64 instead of 128 columns: twice the panels spread more evenly over the blocks, and the row segments are still two lines
-    // (96 workers x 300,007 columns, 5.3 or 10.6 panels a block: 111 -> 104 us in Eq. 3's order, 114 -> 108 in Algorithm 1's;
-    // 128 x 2,000,000, 35 or 70 panels a block: 757 and 760)
-    if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) gs = 16;
+    if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) {
+        bool narrower = false;
+        const int rc = narrower_panel(h, &narrower);
+        if (rc) return rc;
+        if (narrower) gs = 16;
+    }
     switch (gs) {
         case 64: return launch_panel<64>(h, X, G, lr, lr_pw, X_out, shadow, s);
         case 32: return launch_panel<32>(h, X, G, lr, lr_pw, X_out, shadow, s);
