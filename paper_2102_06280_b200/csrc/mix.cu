@@ -22,7 +22,7 @@ constexpr int kMixThreads = 512;
 
 using namespace dev;
 
-template <int GS>
+template <int GS, bool LOCAL>
 __global__ void __launch_bounds__(kMixThreads, 3)
 mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ G, float lr,
                  const float* __restrict__ lr_pw, float* Xout, uint16_t* __restrict__ shadow, MixPlan plan,
@@ -31,7 +31,7 @@ mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ 
     extern __shared__ float4 sm[];  // [N][GS]
     if (active_count && *active_count <= active_limit(N)) return;  // mix_active_kernel's round
     for (int panel = blockIdx.x; panel < n_panels; panel += gridDim.x) {
-        mix_panel_body<GS, kMixThreads>(panel, sm, N, ld, X, G, lr, lr_pw, Xout, shadow, plan, mix_then_correct);
+        mix_panel_body<GS, kMixThreads, true, LOCAL>(panel, sm, N, ld, X, G, lr, lr_pw, Xout, shadow, plan, mix_then_correct);
         __syncthreads();
     }
 }
@@ -213,27 +213,32 @@ int auto_group_size(const dbw_handle* h) {
     return ((size_t)h->N * 4 * 16 <= (size_t)h->smem_optin) ? 4 : 0;
 }
 
+// Algorithm 1's order as a kernel of its own for graphs of many neighbours: without Eq. 3's gradient the registers go to the rows that
+// are summed (1965 workers x 74,459 columns, 60 neighbours: 2823 us against 2957; 303 x 197,748: 878 / 911; within 1 % at up to 12
+// neighbours).
+bool panel_local(const dbw_handle* h) { return !(h->flags & DBW_ORDER_MIX_THEN_CORRECT) && h->nnz > 12 * h->N; }
+
 // Blocks of the panel kernel that share an SM; asked once per handle and width: N and the flags set it.
-template <int GS>
+template <int GS, bool LOCAL>
 int panel_blocks(dbw_handle* h, int* per_sm) {
     static PerDeviceOnce once;
     const int rc = once.run(h->device, [h]() -> int {
-        DBW_CUDA(cudaFuncSetAttribute(mix_panel_kernel<GS>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin));
+        DBW_CUDA(cudaFuncSetAttribute(mix_panel_kernel<GS, LOCAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_optin));
         return DBW_OK;
     });
     if (rc) return rc;
     int& known = h->panel_per_sm[GS == 64 ? 4 : GS == 32 ? 3 : GS == 16 ? 2 : GS == 8 ? 1 : 0];
-    if (known < 1) DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&known, mix_panel_kernel<GS>, kMixThreads, (size_t)h->N * GS * 16));
+    if (known < 1) DBW_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&known, mix_panel_kernel<GS, LOCAL>, kMixThreads, (size_t)h->N * GS * 16));
     *per_sm = known;
     return known < 1 ? DBW_ERR_BAD_SHAPE : DBW_OK;
 }
 
-template <int GS>
-int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
-                          const int* active_count = nullptr) {
+template <int GS, bool LOCAL>
+int launch_panel_of(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
+                          const int* active_count) {
     const size_t smem = (size_t)h->N * GS * 16;
     int per_sm = 0;
-    const int rc = panel_blocks<GS>(h, &per_sm);
+    const int rc = panel_blocks<GS, LOCAL>(h, &per_sm);
     if (rc) return rc;
     const int n_panels = (int)((h->ld + 4 * GS - 1) / (4 * GS)), slots = per_sm * h->sm_count;
     const int mtc = (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0;
@@ -241,12 +246,19 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
     // that end up several to an SM when they are placed among those of the kernel before (502 workers x 4545 columns, 60
     // neighbours: 75 us early, 51 in order; 1032 x 1196: 141 / 62; up to 256 workers early is the better one, by 1 - 2 us).
     if (n_panels >= slots || h->N <= 256)
-        launch(mix_panel_kernel<GS>, std::min(n_panels, slots), kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels,
+        launch(mix_panel_kernel<GS, LOCAL>, std::min(n_panels, slots), kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels,
                active_count);
     else
-        launch<false>(mix_panel_kernel<GS>, n_panels, kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels, active_count);
+        launch<false>(mix_panel_kernel<GS, LOCAL>, n_panels, kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels, active_count);
     DBW_LAUNCHED();
     return DBW_OK;
+}
+
+template <int GS>
+int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
+                 const int* active_count = nullptr) {
+    return panel_local(h) ? launch_panel_of<GS, true>(h, X, G, lr, lr_pw, X_out, shadow, s, active_count)
+                          : launch_panel_of<GS, false>(h, X, G, lr, lr_pw, X_out, shadow, s, active_count);
 }
 
 // 64 columns to a panel instead of 128 where the panels are then walked in fewer turns of all blocks, by a twelfth at least, or with
@@ -255,9 +267,10 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
 // 300,007 columns (6 turns or 11 halves) 111 / 104 us, 78 x 8372 (1 / 1) 10.4 / 7.8, 173 x 166,798 (two blocks an SM, 5 / 6) 125 /
 // 108; 109 x 1,298,095 (23 / 46) 950 / 1397, 116 x 1,614,144 (29 / 57) 2074 / 2244, 74 x 660,293 (12 / 24) 138 / 156,
 // with 16 neighbours 113 x 253,162 (5 / 9) 147 / 168.
+template <bool LOCAL>
 int narrower_panel(dbw_handle* h, bool* narrower) {
     int wide = 0, narrow = 0, rc;
-    if ((rc = panel_blocks<32>(h, &wide)) || (rc = panel_blocks<16>(h, &narrow))) return rc;
+    if ((rc = panel_blocks<32, LOCAL>(h, &wide)) || (rc = panel_blocks<16, LOCAL>(h, &narrow))) return rc;
     auto turns = [h](int cols, int per_sm) { return (((h->ld + cols - 1) / cols) + per_sm * h->sm_count - 1) / (per_sm * h->sm_count); };
     *narrower = 100 * turns(64, narrow) < (h->nnz > 12 * h->N ? 168 : 184) * turns(128, wide);
     return DBW_OK;
@@ -378,7 +391,7 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     int gs = auto_group_size(h);
     if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) {
         bool narrower = false;
-        const int rc = narrower_panel(h, &narrower);
+        const int rc = panel_local(h) ? narrower_panel<true>(h, &narrower) : narrower_panel<false>(h, &narrower);
         if (rc) return rc;
         if (narrower) gs = 16;
     }

@@ -666,13 +666,15 @@ __device__ __forceinline__ float4 fma4(float w, float4 v, float4 a) {
 // row is the weighted sum of staged rows in plan order (self first, then the kept neighbours in CSR order).
 // The caller puts a block barrier after it before the next panel.  G == nullptr: G = 0.
 // `mine(i)`: whether row i is wanted here, as a staged row and as an output (all of them by default).
+// LOCAL: Algorithm 1's order, known to the compiler (mix_then_correct is not looked at).
 struct AllRows {
     __device__ __forceinline__ bool operator()(int) const { return true; }
 };
-template <int GS, int THREADS, bool NC = true, class Mine = AllRows>
+template <int GS, int THREADS, bool NC = true, bool LOCAL = false, class Mine = AllRows>
 __device__ __forceinline__ void mix_panel_body(int panel, float4* sm, int N, long long ld, const float* X, const float* G,
                                                float lr, const float* __restrict__ lr_pw, float* Xout, uint16_t* __restrict__ shadow,
                                                const MixPlan& plan, int mix_then_correct, Mine mine = Mine()) {
+    if (LOCAL) mix_then_correct = 0;
     const int tid = threadIdx.x;
     const int q = tid % GS;
     const int gid = tid / GS;
