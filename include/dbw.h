@@ -182,7 +182,10 @@ int dbw_grad(dbw_handle* h, const float* X, const int32_t* batch_idx, float* G, 
  *             the weights of Assumption 1 the counts p = deg - b of both ends are used.  A row of kept
  *             that does not hold deg_i - b_i entries sets DBW_STATUS_BAD_B.
  * DEVICE out: X_out [N][ld].  X_out may alias X exactly (in place) when dbw_mix_in_place_ok()
- *             is 1; partial overlap is an error.  G is read only.
+ *             is 1; partial overlap is an error.  G is read only.  (Beyond about 3600 workers, where no
+ *             panel of all rows fits shared memory, large matrices of graphs with six neighbours or more a
+ *             worker are mixed in place too, but out of place rounds in which few neighbours are kept are
+ *             the faster ones: dbw_mix_in_place_ok() is 0.)
  * Summation order per element is fixed (self, then kept neighbours in CSR order), so results
  * are reproducible run to run.
  */
@@ -191,8 +194,8 @@ int dbw_mix(dbw_handle* h, const float* X, const float* G, const uint8_t* kept, 
 int dbw_mix_in_place_ok(const dbw_handle* h);
 /* Expert knob: columns per shared-memory panel of the mix kernel: 0 = automatic, 16 / 32 / 64 /
  * 128 / 256 = fixed (falls back to the direct kernel when N * cols * 4 bytes exceed shared memory),
- * 1 = the tensor-memory staged kernel wherever it applies (64 <= N <= 1024; with the Metropolis
- *     weights degrees up to 62),
+ * 1 = the tensor-memory staged kernel wherever it applies (64 <= N <= 4096; with the Metropolis
+ *     weights degrees up to 62, above 1024 workers 30, above 2048 workers 14),
  * 2 = the tensor-core kernel wherever it applies (uniform weights, 256 <= N <= 1024): the mix as a
  *     dense product with the 0/1 selection matrix, every fp32 value split exactly into three BF16
  *     pieces, fp32 accumulation; with N > 512 it cannot run in place (dbw_mix_in_place_ok() = 0),
@@ -202,7 +205,8 @@ int dbw_mix_in_place_ok(const dbw_handle* h);
  * -1 = always the direct (L2 re-read, out-of-place only) kernel. */
 int dbw_set_mix_panel(dbw_handle* h, int32_t cols);
 /* Which mix kernel the current settings select: 0 = direct (L2 re-read), 1 = shared-memory panel,
- * 2 = tensor-memory staged, 3 = tensor-core, 4 = structured-sparse tensor-core.  Negative on error. */
+ * 2 = tensor-memory staged (beyond about 3600 workers, out of place, for rounds of six kept neighbours a worker and
+ * more; the others are the direct kernel's), 3 = tensor-core, 4 = structured-sparse tensor-core.  Negative on error. */
 int dbw_mix_kernel(const dbw_handle* h);
 
 /*

@@ -350,7 +350,7 @@ int dbw_set_fused_round(dbw_handle* h, int enable) {
 
 int dbw_round_is_fused(const dbw_handle* h) { return h ? (round_fused_usable(h) ? 1 : 0) : DBW_ERR_NULL; }
 
-int dbw_mix_in_place_ok(const dbw_handle* h) { return h && mix_panel_fits(h) ? 1 : 0; }
+int dbw_mix_in_place_ok(const dbw_handle* h) { return h && mix_in_place_advised(h) ? 1 : 0; }
 
 int dbw_mix_kernel(const dbw_handle* h) { return h ? mix_kernel_kind(h) : DBW_ERR_NULL; }
 

@@ -223,6 +223,7 @@ __device__ __forceinline__ uint2 pack_bf16x4_rn(float a, float b, float c, float
     return make_uint2(lo, hi);
 }
 bool mix_panel_fits(const dbw_handle* h);
+bool mix_in_place_advised(const dbw_handle* h);
 // The mix of a round whose dW GEMMs may already have taken the step x' = x - lr g of every worker that takes no part.
 bool mix_active_usable(const dbw_handle* h);
 int launch_mix_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, cudaStream_t s);
@@ -230,8 +231,9 @@ int mix_kernel_kind(const dbw_handle* h);
 
 // mix_staged.cu
 bool mix_staged_usable(const dbw_handle* h);
+size_t mix_staged_smem(const dbw_handle* h);  // of one block, without the row weights and list lengths it can do without
 int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
-                      uint16_t* shadow, cudaStream_t s);
+                      uint16_t* shadow, long long kept_limit, cudaStream_t s);
 
 // mix_tc.cu
 bool mix_tc_usable(const dbw_handle* h);

@@ -45,7 +45,8 @@ mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ 
 __global__ void __launch_bounds__(256)
 mix_direct_kernel(int N, long long ld, const float* __restrict__ X, const float* __restrict__ G, float lr,
                   const float* __restrict__ lr_pw, float* __restrict__ Xout, uint16_t* __restrict__ shadow,
-                  MixPlan plan, int mix_then_correct, int panel_cols, long long n_items) {
+                  MixPlan plan, int mix_then_correct, int panel_cols, long long n_items, long long kept_limit) {
+    if (kept_limit > 0 && keeps_at_least(plan, N, kept_limit)) return;  // mix_staged_kernel's round
     for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
         const int i = (int)(item % N);
         const long long c = (item / N) * panel_cols + 4 * (long long)threadIdx.x;
@@ -322,22 +323,41 @@ constexpr bool kSparseByDefault = false;
 // The tensor-memory staged kernel takes over when it applies and the plain panel kernel could not keep a 32-column
 // (128-byte segment) panel with two CTAs per SM.  Beyond 1024 workers its own panels are narrower too (16 columns, from 2049
 // workers 8): measured with 8 neighbours, 1300 workers x 131,072 columns 659 us against 847 (16-column panel kernel), 2048
-// workers 968 / 1669, 3000 x 65,536 907 / 1303.  The panel kernel stays better where two of its CTAs share an SM and the
-// matrix is a fraction of L2 (1100 x 4096: 31 us against 35; x 8192: 51 / 50).  Where no panel of all rows leaves the panel
-// kernel any room, the L2 kernel stays when few neighbours are read or the matrix does not stream from HBM (4096 workers, 2
-// neighbours: 837 us against 1016, 4 neighbours 1046 / 1016, 8 neighbours 1541 / 1348; 16,384 columns 396 / 371).
+// workers 968 / 1669, 3000 x 65,536 907 / 1303.  The panel kernel stays better
+//  - where two of its CTAs share an SM and the matrix is a fraction of L2 (1100 x 4096: 31 us against 35; x 8192: 51 / 50);
+//  - with eight-column panels, weights and eight neighbours or more on a matrix that stays in L2 (2652 x 1507, 8 neighbours: 37
+//    against 43; 2922 x 4415, 14 neighbours: 115 / 139; uniform weights 2363 x 2376, 12 neighbours: 58 / 45);
+//  - where panel and lists leave L1 hardly a line (kCrowdedBytes), unless panels are wide and the matrix streams from HBM (1019 x
+//    10,653, 48 neighbours: 36 / 48; 3049 x 11,692, 20 neighbours: 334 / 366; but 926 x 70,855, 48 neighbours: 910 / 507).
+// Where no panel of all rows leaves the panel kernel any room, the L2 kernel stays for graphs of few neighbours (3790 x 56,509,
+// 2 neighbours: 569 us against 840) and for matrices that do not stream from HBM (4033 x 3563, 4 neighbours: 60 / 93); between the
+// two where both apply see kept_decides.
+constexpr size_t kCrowdedBytes = 200 * 1024;
 static bool use_staged(const dbw_handle* h) {
     if (!mix_staged_usable(h)) return false;
     if (h->mix_panel_cols == 1) return true;
     if (h->mix_panel_cols != 0) return false;
     const int gs = auto_group_size(h);
-    const size_t matrix = (size_t)h->N * h->ld * sizeof(float);
+    const size_t matrix = (size_t)h->N * h->ld * sizeof(float), MB = (size_t)1 << 20;
+    const bool crowded = mix_staged_smem(h) > kCrowdedBytes;
     if (gs >= 8) return false;
-    if (gs == 0) return h->nnz >= 6 * h->N && matrix > ((size_t)256 << 20);
+    if (gs == 0) return h->nnz >= 6 * h->N && matrix > 256 * MB;
+    if (crowded && (h->N > 2048 || matrix <= 64 * MB)) return false;
     if (h->N <= 1024) return true;
+    if (h->N > 2048 && !(h->flags & DBW_WEIGHT_UNIFORM) && h->nnz >= 8 * h->N && matrix <= 64 * MB) return false;
     const bool two_ctas = (size_t)h->N * gs * 16 <= (size_t)h->smem_optin / 2 - 1024;
-    return !two_ctas || matrix > ((size_t)32 << 20);
+    return !two_ctas || matrix > 32 * MB;
 }
+
+// Workers that keep few neighbours, as in most rounds of the threshold rule, leave the L2 kernel little to read again, while the
+// staged kernel moves every row through its narrow panels whatever is kept.  How many are kept only the device knows: where the
+// two compete (no panel of all rows fits) both are launched, and the one whose round it is not leaves after a look at the
+// plan's counts.  At six a worker and more the staged kernel is the faster one (4065 workers x 40,364 columns, 6 neighbours, few
+// kept: 370 us against 720; 3971 x 32,355, all 6 kept: 704 / 633; 3848 x 38,685, 5 kept: 691 / 762).
+// Always the L2 kernel's are rounds in Eq. 3's order, whose gradient the staged kernel reads in 32-byte pieces (3811 x 65,782, 6
+// neighbours: 1004 against 1330), and rounds without gradients (3818 x 36,482, 12 neighbours: 652 / 907).
+static bool kept_decides(const dbw_handle* h) { return h->mix_panel_cols == 0 && auto_group_size(h) == 0; }
+static bool direct_always(const dbw_handle* h, const float* G) { return kept_decides(h) && (!G || (h->flags & DBW_ORDER_MIX_THEN_CORRECT)); }
 
 // The tensor-core kernel (dense 0/1 selection product) when asked for and applicable.
 static bool use_tc(const dbw_handle* h) { return h->mix_panel_cols == 2 && mix_tc_usable(h); }
@@ -354,7 +374,14 @@ bool mix_panel_fits(const dbw_handle* h) {
     if (use_sp(h)) return mix_sp_in_place_ok(h);
     return use_tc(h) ? mix_tc_in_place_ok(h) : (use_staged(h) || auto_group_size(h) != 0);
 }
-int mix_kernel_kind(const dbw_handle* h) { return use_sp(h) ? 4 : use_tc(h) ? 3 : use_staged(h) ? 2 : (auto_group_size(h) != 0 ? 1 : 0); }
+// In place only the staged kernel is left where it would share the rounds with the L2 kernel, so a caller is advised against it.
+bool mix_in_place_advised(const dbw_handle* h) { return mix_panel_fits(h) && !(use_staged(h) && kept_decides(h)); }
+int mix_kernel_kind(const dbw_handle* h) {
+    if (use_sp(h)) return 4;
+    if (use_tc(h)) return 3;
+    if (use_staged(h)) return kept_decides(h) && (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 0 : 2;
+    return auto_group_size(h) != 0 ? 1 : 0;
+}
 
 // With tensor-core layers and a panel of all workers in shared memory the dW GEMMs can take the step of the workers that
 // take no part in the round, whose weights then cross HBM once (read x, write x' and its bf16 copy: 10 bytes an element)
@@ -387,7 +414,12 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     h->shadow_of = X_out;
     if (use_sp(h)) return launch_mix_sp(h, X, G, lr, lr_pw, X_out, shadow, s);
     if (use_tc(h)) return launch_mix_tc(h, X, G, lr, lr_pw, X_out, shadow, s);
-    if (use_staged(h)) return launch_mix_staged(h, X, G, lr, lr_pw, X_out, shadow, s);
+    long long kept_limit = 0;
+    if (use_staged(h) && (X_out == X || !direct_always(h, G))) {
+        if (X_out != X && kept_decides(h)) kept_limit = 6ll * h->N;
+        const int rc = launch_mix_staged(h, X, G, lr, lr_pw, X_out, shadow, kept_limit, s);
+        if (rc || kept_limit == 0) return rc;
+    }
     int gs = auto_group_size(h);
     if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) {
         bool narrower = false;
@@ -415,7 +447,7 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
     // In order: its blocks keep their places for the whole launch, and placed among those of the kernel before they end up
     // unevenly spread (4229 workers x 29,718 columns, 48 neighbours: 1790 us, placed early 2810).
     launch<false>(mix_direct_kernel, (int)blocks, panel_cols / 4, 0, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan,
-                  (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, panel_cols, n_items);
+                  (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0, panel_cols, n_items, kept_limit);
     DBW_LAUNCHED();
     return DBW_OK;
 }

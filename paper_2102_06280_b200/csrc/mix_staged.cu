@@ -15,6 +15,7 @@
 // in shared memory for the whole launch.  HBM traffic is the algorithmic 12 bytes per element; a panel
 // is fully staged before any of it is written and panels are disjoint, so X' may overwrite X.
 #include "common.cuh"
+#include "round_dev.cuh"
 
 namespace dbw {
 
@@ -90,6 +91,7 @@ struct StagedArgs {
     float* Xout;
     uint16_t* shadow;
     MixPlan plan;
+    long long kept_limit;  // 0, or the kept entries of the round from which on it is this kernel's
 };
 
 // Shared memory: panel float4 [N + 1][W / 4] (row N is all zero: the target of list padding), then the neighbour lists
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(kThreads, 1) mix_staged_kernel(StagedArgs a) {
     extern __shared__ float4 smem4[];
     float4* panel = smem4;
     const int N = a.N;
+    if (a.kept_limit > 0 && !dev::keeps_at_least(a.plan, N, a.kept_limit)) return;  // mix_direct_kernel's round
     const int lrow = a.list_row;
     uint16_t* lists = reinterpret_cast<uint16_t*>(panel + (size_t)(N + 1) * SLOTS);
     float* wtab = reinterpret_cast<float*>(lists + (size_t)N * lrow);  // weights by code (weighted lists)
@@ -344,8 +347,10 @@ bool mix_staged_usable(const dbw_handle* h) {
     return staged_smem(h, false) + 256 <= (size_t)h->smem_optin;
 }
 
+size_t mix_staged_smem(const dbw_handle* h) { return staged_smem(h, false); }
+
 int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out,
-                      uint16_t* shadow, cudaStream_t s) {
+                      uint16_t* shadow, long long kept_limit, cudaStream_t s) {
     StagedArgs a{};
     a.N = h->N;
     a.ld = h->ld;
@@ -353,6 +358,7 @@ int launch_mix_staged(dbw_handle* h, const float* X, const float* G, float lr, c
     const int W = staged_width(h->N);
     a.list_row = list_entries(h->maxdeg);
     a.X = X; a.G = G; a.lr = lr; a.lr_pw = lr_pw; a.Xout = X_out; a.shadow = shadow; a.plan = h->plan;
+    a.kept_limit = kept_limit;
     switch (W) {
         case 32: return launch_staged_width<32>(h, a, s);
         case 16: return launch_staged_width<16>(h, a, s);

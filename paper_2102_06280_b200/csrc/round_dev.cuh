@@ -610,6 +610,20 @@ __device__ __forceinline__ void select_worker(int i, int lane, const int32_t* __
     }
 }
 
+// Whether the workers keep at least `limit` neighbours in all; called by all threads of a block.
+__device__ __forceinline__ bool keeps_at_least(const MixPlan& plan, int N, long long limit) {
+    __shared__ unsigned kept_in_all;
+    if (threadIdx.x == 0) kept_in_all = 0u;
+    __syncthreads();
+    unsigned kept = 0u;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) kept += (unsigned)__ldg(plan.cnt + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&kept_in_all, kept);
+    __syncthreads();
+    return (long long)kept_in_all >= limit;
+}
+
 // Per-worker and per-round times (Section 3.2.2) once every worker's selection is visible: the calling
 // block's threads share the workers; returns this thread's part of max T_worker over the participants
 // (the caller reduces it over the block).  Clears the "waited for" flags for the next round.

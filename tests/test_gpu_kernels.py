@@ -910,3 +910,50 @@ def test_which_rounds_are_one_launch(dims, batch, n, single):
     h.set_dataset(feat, labels, batch)
     assert h.round_is_fused() == single
     h.close()
+
+
+@pytest.mark.parametrize("n,deg,d,flags,kernel,in_place", [
+    (1019, 48, 10_653, 0, "mix_panel_kernel", True), (1000, 32, 10_653, 0, "mix_staged_kernel", True),    # lists that crowd L1 out
+    (2652, 8, 1507, 0, "mix_panel_kernel", True), (2652, 8, 1507, 1, "mix_staged_kernel", True),          # weighted lists, a matrix in L2
+    (3049, 20, 11_692, 1, "mix_panel_kernel", True), (2500, 8, 30_000, 0, "mix_staged_kernel", True),
+    (3700, 6, 20_000, 0, "mix_staged_kernel", False), (3700, 6, 20_000, 2, "mix_direct_kernel", False)])   # no panel of all rows fits
+def test_which_kernel_mixes_many_workers(n, deg, d, flags, kernel, in_place):
+    p = _dbw()
+    h = p.Dbw(*wl.random_regular(n, deg, 7), d=d, flags=flags)
+    assert h.mix_kernel() == kernel and h.mix_in_place_ok() == in_place
+    h.close()
+
+
+@pytest.mark.parametrize("order", ["local_then_mix", "mix_then_correct"])
+def test_kernel_by_the_kept_count_where_no_panel_fits(order):
+    """Out of place the L2 kernel takes the rounds of fewer than six kept neighbours a worker (in Eq. 3's order, and without
+    gradients, every round) and the staged kernel the others; in place it is the staged kernel's alone.  Uniform weights, which
+    the two apply at different places of the sum, tell them apart by their bits."""
+    p = _dbw()
+    n, deg, d = 3640, 8, 19_000
+    rowptr, col = wl.random_regular(n, deg, 3)
+    flags = p.WEIGHT_UNIFORM | (p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    h = p.Dbw(rowptr, col, d=d, flags=flags)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    X, G = (torch.randn(n, h.ld, device="cuda", generator=gen) for _ in range(2))
+    X[:, d:] = 0
+    G[:, d:] = 0
+    kept = torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+    t = dev(1.0 + np.random.default_rng(2).random(n))
+    out, direct, staged = (torch.empty_like(X) for _ in range(3))
+    for total in (0, 6 * n - 1, 6 * n, deg * n):
+        p_i = np.full(n, total // n) + (np.arange(n) < total % n)
+        b = dev((deg - p_i).astype(np.int32))
+        h.select(t, b, kept)
+        for g in (G, None):
+            for panel, to in ((-1, direct), (1, staged), (0, out)):
+                h.set_mix_panel(panel)
+                h.mix(X, g, kept, b, 0.05, to)
+            assert total == 0 or not torch.equal(direct, staged)
+            wants = direct if total < 6 * n or g is None or order == "mix_then_correct" else staged
+            assert torch.equal(out, wants), (total, g is None)
+            Y = X.clone()
+            h.mix(Y, g, kept, b, 0.05, Y)  # in place: accepted, by the staged kernel
+            assert torch.equal(Y, staged), (total, g is None)
+    assert h.status() == 0
+    h.close()
