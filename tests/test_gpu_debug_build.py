@@ -20,7 +20,8 @@ def test_kernel_parity_tests_pass_against_the_bounds_checked_library():
     build.build(debug=True)
     env = dict(os.environ, DBW_LIBRARY="debug")
     select = ("selection_bit_exact or mix_matches_oracle or tensor_core_kernel or staged_kernel or large_worker_count or "
-              "update_backups or grad_fp32 or consensus_only_mix or degenerate or per_link_times or kept_count")
+              "update_backups or grad_fp32 or consensus_only_mix or degenerate or per_link_times or few_participants or merged_panels or "
+              "parts_of_the_batch or one_unit or kept_count")
     cmd = [sys.executable, "-m", "pytest", "tests/debug_bounds_checks.py", "tests/test_gpu_kernels.py", "tests/test_zz_no_alloc.py",
            "-m", "gpu", "-q", "-x", "-p", "no:cacheprovider", "-k", select + " or bounds_checked or bad_neighbour or static_selection"]
     r = subprocess.run(cmd, cwd=ROOT, env=env, capture_output=True, text=True, timeout=1500)

@@ -957,3 +957,118 @@ def test_kernel_by_the_kept_count_where_no_panel_fits(order):
             assert torch.equal(Y, staged), (total, g is None)
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("n,cols", [(10, 16), (10, 32), (10, 64), (10, 256), (80, 0), (80, 16)])  # 80 workers: four and five dW tiles to an SM
+def test_stepping_rounds_with_merged_panels_of_every_width(n, cols):
+    """Rounds whose dW GEMMs step, on a matrix wide enough that several panels of the participants are staged together, the last
+    group of a block a ragged one, with every panel width, and with several dW tiles to an SM: the bits of the round's steps.  One
+    launch more than with a mix that cannot leave rows out says that this is the path."""
+    p = _dbw()
+    from paper_2102_06280_b200 import binding
+    dims, batch = [1024, 264, 10], 64
+    rowptr, col = wl.ring(n)
+    deg = np.diff(rowptr)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m, flags=p.GEMM_BF16)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    feat, labels = torch.randn(n, batch, dims[0], device="cuda", generator=gen), torch.randint(0, 10, (n, batch), dtype=torch.int32, device="cuda", generator=gen)
+    h.set_dataset(feat, labels, batch)
+    X = torch.zeros(n, m.ld, device="cuda")
+    for l in range(2):
+        X[:, m.w_off[l]: m.w_off[l] + dims[l] * dims[l + 1]].normal_(0.0, 0.05, generator=gen)
+    idx = torch.stack([torch.randperm(batch, device="cuda", generator=gen) for _ in range(n)]).int()
+    rng = np.random.default_rng(1)
+    kept, kept2 = (torch.zeros(len(col), dtype=torch.uint8, device="cuda") for _ in range(2))
+    G, ref, out = (torch.zeros_like(X) for _ in range(3))
+
+    def launches(f):
+        before = binding.launch_count()
+        f()
+        return binding.launch_count() - before
+
+    for k in (0, 2, 3, n // 2):
+        inside = np.arange(n) < k
+        t = dev(np.where(inside, 1.0, 9.0) + rng.random(n))
+        mates = np.array([inside[col[rowptr[i]:rowptr[i + 1]]].sum() for i in range(n)])
+        b = dev(np.where(inside, deg - mates, deg).astype(np.int32))
+        h.set_mix_panel(cols)
+        h.grad(X, idx, G)
+        h.select(t, b, kept)
+        h.mix(X, G, kept, b, 0.05, ref)
+        for track in (False, True):
+            h.set_param_tracking(track)
+            out.fill_(float("nan"))
+            stepping = launches(lambda: h.round(X, t, b, 0.05, out, kept2, batch_idx=idx))
+            assert torch.equal(out, ref) and torch.equal(kept, kept2), (k, track)
+            Y = X.clone()
+            h.set_param_tracking(track)
+            h.round(Y, t, b, 0.05, Y, kept2, batch_idx=idx)
+            assert torch.equal(Y, ref), (k, track)
+            h.set_param_tracking(False)
+            h.set_mix_panel(-1)
+            assert stepping == launches(lambda: h.round(X, t, b, 0.05, out, kept2, batch_idx=idx)) + 1
+            h.set_mix_panel(cols)
+    assert h.status() == 0
+    h.close()
+
+
+@pytest.mark.parametrize("kind", ["fp32_steps", "bf16", "bf16_tracked", "mix_only", "consensus_only", "one_launch"])
+@pytest.mark.parametrize("dynamic", [False, True])
+def test_round_host_on_two_streams_gives_the_bits_of_dbw_round(kind, dynamic):
+    """dbw_round_host with its copies beside the gradients and the mix: several rounds queued without a wait in between, each with host
+    buffers of its own, with given backup counts and with the threshold rule's, against dbw_update_backups and dbw_round."""
+    p = _dbw()
+    n, rounds = 12, 5
+    rowptr, col = wl.random_regular(n, 4, 1)
+    rng = np.random.default_rng(6)
+    model = kind in ("fp32_steps", "one_launch") or kind.startswith("bf16")
+    if model:
+        dims, batch, S = [136, 72, 10], 40, 90
+        m = p.model_layout(dims, batch)
+        handles = [p.Dbw(rowptr, col, d=m.d, model=m, flags=p.GEMM_BF16 if kind.startswith("bf16") else 0) for _ in range(2)]
+        feat, labels = dev(rng.random((n, S, dims[0]), dtype=np.float32)), dev(rng.integers(0, 10, size=(n, S)).astype(np.int32))
+        X0 = dev(m.pack((0.1 * rng.standard_normal((n, m.d))).astype(np.float32)))
+        for h in handles:
+            h.set_dataset(feat, labels, S)
+            h.set_fused_round(kind == "one_launch")
+            h.set_param_tracking(kind == "bf16_tracked")
+        G = None
+    else:
+        handles = [p.Dbw(rowptr, col, d=5000) for _ in range(2)]
+        X0 = dev(rng.standard_normal((n, 5000), dtype=np.float32))
+        G = dev(0.1 * rng.standard_normal((n, 5000), dtype=np.float32)) if kind == "mix_only" else None
+    pin = lambda a: torch.from_numpy(np.ascontiguousarray(a)).pin_memory()
+    times = [pin(1.0 + rng.exponential(1.0, size=n)) for _ in range(rounds)]
+    counts = [pin(rng.integers(0, 5, size=n).astype(np.int32)) for _ in range(rounds)]
+    idx = [pin(np.stack([rng.permutation(90)[:40] for _ in range(n)]).astype(np.int32)) for _ in range(rounds)] if model else [None] * rounds
+
+    def results():
+        return {"kept": torch.zeros(len(col), dtype=torch.uint8), "T_worker": torch.zeros(n, dtype=torch.float64), "T_round": torch.zeros(1, dtype=torch.float64),
+                "loss": torch.zeros(n), "b_out": torch.zeros(n, dtype=torch.int32)}
+
+    # on the host's buffers
+    h, X, got = handles[0], X0.clone(), []
+    for k in range(rounds):
+        r = {name: v.pin_memory() for name, v in results().items()}
+        h.round_host(X, times[k], None if dynamic else counts[k], 0.05, X, h_batch_idx=idx[k], G_ext=G, h_kept=r["kept"], h_T_worker=r["T_worker"],
+                     h_T_round=r["T_round"], h_loss=r["loss"] if model else None, h_b_out=r["b_out"])
+        got.append(r)
+    torch.cuda.current_stream().synchronize()
+    # on the device's
+    h, Y = handles[1], X0.clone()
+    for k in range(rounds):
+        r = {name: v.cuda() for name, v in results().items()}
+        t = times[k].cuda()
+        if dynamic:
+            h.update_backups(t, r["b_out"])
+        else:
+            r["b_out"].copy_(counts[k])
+        h.round(Y, t, r["b_out"], 0.05, Y, r["kept"], batch_idx=None if idx[k] is None else idx[k].cuda(), G_ext=G, T_worker=r["T_worker"],
+                T_round=r["T_round"], loss=r["loss"] if model else None)
+        for name, v in r.items():
+            assert torch.equal(v.cpu(), got[k][name]), (k, name)
+    assert torch.equal(X, Y)
+    for h in handles:
+        assert h.status() == 0
+        h.close()
