@@ -35,8 +35,9 @@ UNIT = "worker-rounds/s"
 DEFAULT_CONFIG = 4
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the mix kernel, from the ncu captures summarised
 # under profiles/ (config 4: the d = 65,536 case scaled by 16, the traffic being proportional to the columns
-# processed).  Reported only for the kernel the capture was taken of; None = not captured for this workload.
-MIX_TRAFFIC_BYTES = {4: ("mix_staged_kernel", (537.05e6 + 220.89e6) * 16)}
+# processed; taken of the kernel with its lists in blocks of four).  Reported only for the kernel the capture was taken
+# of; None = not captured for this workload.
+MIX_TRAFFIC_BYTES = {4: ("mix_staged_kernel", (537.04e6 + 219.48e6) * 16)}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
@@ -185,6 +186,23 @@ class Job:
         self.torch.cuda.current_stream().synchronize()      # the caller reads the round's results
         self._swap(out)
         self.k += 1
+
+    def participants(self, first, rounds, threshold_state):
+        """Workers that take part (keep a neighbour or are kept by one) in each of the given rounds, by their selections
+        alone, replayed from the threshold rule's state before them."""
+        w, counts = self.w, []
+        row = np.repeat(np.arange(w.N), np.diff(w.rowptr))
+        self.h.state_import(threshold_state)
+        for k in range(first, first + rounds):
+            r = k % self.n_rounds
+            b = self.d_b[r]
+            if w.backups == "dtur" and k > 0:
+                self.h.update_backups(self.d_t[r], self.b_dyn)
+                b = self.b_dyn
+            self.h.select(self.d_t[r], b, self.kept)
+            kept = self.kept.cpu().numpy() != 0
+            counts.append(len(np.union1d(row[kept], np.asarray(w.col)[kept])))
+        return counts
 
     def host_bytes_per_step(self):
         w = self.w
@@ -515,6 +533,7 @@ def measure(config, local, args, dist, overrides, col_range=None):
     for _ in range(args.warmup):
         job.step()
     torch.cuda.synchronize()
+    timed_from, threshold_state = job.k, job.h.state_export() if job.w.precision == "bf16" and job.w.layers is not None else None
     job.h.profile(True)
     job.h.profile_read()
     launches0 = binding.launch_count()
@@ -536,8 +555,7 @@ def measure(config, local, args, dist, overrides, col_range=None):
                stage_ms={k: v / max(stage_rounds, 1) for k, v in stage_ms.items()},
                bytes=job.host_bytes_per_step(), mix_bytes=job.mix_bytes_per_launch(),
                kept_last=int(job.kept.sum().item()), sms=torch.cuda.get_device_properties(local).multi_processor_count)
-    before = np.concatenate([[0], np.cumsum(job.kept.cpu().numpy() != 0)])
-    out["mixing_last"] = int(np.count_nonzero(before[job.w.rowptr[1:]] - before[job.w.rowptr[:-1]]))  # workers with a kept neighbour
+    out["mixing"] = job.participants(timed_from, args.steps, threshold_state) if threshold_state is not None else []
     job.close()
     del job
     torch.cuda.empty_cache()
@@ -613,12 +631,15 @@ def summary(res, world, args):
                                 "note": "one cooperative launch per round; launch-bound, no separate mix kernel"})
         out["roofline"]["operand_delivery"].update({"achieved": None, "frac": None})
     tc_flops, tc_bytes = tensor_core_gemm_work(w)
-    if tc_flops and res["mixing_last"] <= w.N // 2:
-        # the dW GEMMs take the step of the workers without a kept neighbour: x in, x' and its bf16 copy out instead of dW out
-        tc_bytes += (w.N - res["mixing_last"]) * 6 * sum(o * i for o, i in wl.layer_dims(w.layers)[:-1])
+    # in a round of at most N / 2 participants the dW GEMMs take the step of the others: x in, x' and its bf16 copy out instead of
+    # dW out; bytes are the mean over the timed rounds, as the times are
+    stepped = [w.N - m for m in res["mixing"] if m <= w.N // 2]
+    if tc_flops and stepped:
+        tc_bytes += sum(stepped) / len(res["mixing"]) * 6 * sum(o * i for o, i in wl.layer_dims(w.layers)[:-1])
         out["roofline"].update({"achieved": None, "frac": None, "frac_of_8TBps_nominal": None, "traffic": None,
-                                "note": "%d of %d workers have a kept neighbour: the dW GEMMs take the others' step (roofline_gemm), the mix "
-                                        "stage is left with the rest" % (res["mixing_last"], w.N)})
+                                "note": "in %d of %d rounds at most half of the %d workers take part (%.1f of them on average over all rounds): the dW "
+                                        "GEMMs take the others' step (roofline_gemm), the mix stage is left with the rest"
+                                        % (len(stepped), len(res["mixing"]), w.N, sum(res["mixing"]) / len(res["mixing"]))})
         out["roofline"]["operand_delivery"].update({"achieved": None, "frac": None})
     if res.get("graph_ms"):
         out["cuda_graph"] = {"rounds_per_graph": args.graph, "ms_per_step": res["graph_ms"] / args.steps,
