@@ -36,8 +36,8 @@ constexpr int kBlocksPerSM = 1;                  // registers are spent on deep 
 // it saves is launches; what it costs is that one block to an SM works off all samples and tiles, and that its steps wait for
 // the slowest block.  Where the lines lie was measured on 1700 networks of 3 - 64 workers (single launch / step by step, us):
 //  - one layer, whose last layer's two steps read the data set themselves: up to 2560 samples over all workers (8 workers x batch 32,
-//    784-10: 19 / 33, 16 x 64, 784-10: 24 / 36, 41 x 52, 784-10: 39 / 40; 25 x 265, 121-10 is of the next kind: 92 / 62);
-//  - one layer as a GEMM (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26);
+//    784-10: 19 / 33, 16 x 64, 784-10: 24 / 36, 41 x 52, 784-10: 39 / 40, 23 x 372, 256-10: 60 / 49);
+//  - one layer as a GEMM (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26, 25 x 265, 121-10: 92 / 62);
 //  - more layers, the last one in those two steps: 2048 samples of at most 20 workers (8 x 128, 256-64-10: 50 / 59, 8 x 268, 64-96-10:
 //    74 / 79; 40 x 17, 16-108-10: 45 / 36);
 //  - more layers, all of them GEMMs: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16 million multiply-adds.
