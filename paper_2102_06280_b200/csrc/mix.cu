@@ -245,12 +245,14 @@ int launch_panel_of(dbw_handle* h, const float* X, const float* G, float lr, con
     const int mtc = (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0;
     // Placed early where the blocks fill the chip, or are so short that it does not matter where they lie.  Fewer blocks than
     // that end up several to an SM when they are placed among those of the kernel before (502 workers x 4545 columns, 60
-    // neighbours: 75 us early, 51 in order; 1032 x 1196: 141 / 62; up to 256 workers early is the better one, by 1 - 2 us).
-    if (n_panels >= slots || h->N <= 256)
+    // neighbours: 75 us early, 51 in order; 1032 x 1196: 141 / 62; up to 256 workers early is the better one, by 1 - 2 us), and so
+    // do the blocks with a second panel of two, which counts where rows are many neighbours long (1091 x 10,761, 48 neighbours:
+    // 242 early, 209 in order).
+    if (n_panels >= (h->nnz > 12 * h->N ? 2 : 1) * slots || h->N <= 256)
         launch(mix_panel_kernel<GS, LOCAL>, std::min(n_panels, slots), kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels,
                active_count);
     else
-        launch<false>(mix_panel_kernel<GS, LOCAL>, n_panels, kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels, active_count);
+        launch<false>(mix_panel_kernel<GS, LOCAL>, std::min(n_panels, slots), kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels, active_count);
     DBW_LAUNCHED();
     return DBW_OK;
 }
