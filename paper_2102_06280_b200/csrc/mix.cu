@@ -329,19 +329,19 @@ constexpr bool kSparseByDefault = false;
 //  - where two of its CTAs share an SM and the matrix is a fraction of L2 (1100 x 4096: 31 us against 35; x 8192: 51 / 50);
 //  - with eight-column panels, weights and eight neighbours or more on a matrix that stays in L2 (2652 x 1507, 8 neighbours: 37
 //    against 43; 2922 x 4415, 14 neighbours: 115 / 139; uniform weights 2363 x 2376, 12 neighbours: 58 / 45);
-//  - where panel and lists leave L1 hardly a line (kCrowdedBytes), unless panels are wide and the matrix streams from HBM (1019 x
-//    10,653, 48 neighbours: 36 / 48; 3049 x 11,692, 20 neighbours: 334 / 366; but 926 x 70,855, 48 neighbours: 910 / 507).
+//  - where panel and lists leave L1 hardly a line (crowded), unless panels are wide and the matrix streams from HBM (1019 x
+//    10,653, 48 neighbours: 36 / 48; 3049 x 11,692, 20 neighbours: 334 / 366; but 926 x 70,855, 48 neighbours: 910 / 507, and a little
+//    less crowded 922 x 13,110: 191 / 150).
 // Where no panel of all rows leaves the panel kernel any room, the L2 kernel stays for graphs of few neighbours (3790 x 56,509,
 // 2 neighbours: 569 us against 840) and for matrices that do not stream from HBM (4033 x 3563, 4 neighbours: 60 / 93); between the
 // two where both apply see kept_decides.
-constexpr size_t kCrowdedBytes = 200 * 1024;
 static bool use_staged(const dbw_handle* h) {
     if (!mix_staged_usable(h)) return false;
     if (h->mix_panel_cols == 1) return true;
     if (h->mix_panel_cols != 0) return false;
     const int gs = auto_group_size(h);
     const size_t matrix = (size_t)h->N * h->ld * sizeof(float), MB = (size_t)1 << 20;
-    const bool crowded = mix_staged_smem(h) > kCrowdedBytes;
+    const bool crowded = mix_staged_smem(h) > (size_t)(h->N <= 1024 ? 207 : 200) * 1024;
     if (gs >= 8) return false;
     if (gs == 0) return h->nnz >= 6 * h->N && matrix > 256 * MB;
     if (crowded && (h->N > 2048 || matrix <= 64 * MB)) return false;

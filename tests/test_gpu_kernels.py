@@ -914,6 +914,7 @@ def test_which_rounds_are_one_launch(dims, batch, n, single):
 
 @pytest.mark.parametrize("n,deg,d,flags,kernel,in_place", [
     (1019, 48, 10_653, 0, "mix_panel_kernel", True), (1000, 32, 10_653, 0, "mix_staged_kernel", True),    # lists that crowd L1 out
+    (922, 48, 13_110, 0, "mix_staged_kernel", True),
     (2652, 8, 1507, 0, "mix_panel_kernel", True), (2652, 8, 1507, 1, "mix_staged_kernel", True),          # weighted lists, a matrix in L2
     (3049, 20, 11_692, 1, "mix_panel_kernel", True), (2500, 8, 30_000, 0, "mix_staged_kernel", True),
     (3700, 6, 20_000, 0, "mix_staged_kernel", False), (3700, 6, 20_000, 2, "mix_direct_kernel", False)])   # no panel of all rows fits
