@@ -264,18 +264,18 @@ int launch_panel(dbw_handle* h, const float* X, const float* G, float lr, const 
                           : launch_panel_of<GS, false>(h, X, G, lr, lr_pw, X_out, shadow, s, active_count);
 }
 
-// 64 columns to a panel instead of 128 where the panels are then walked in fewer turns of all blocks, by a twelfth at least, or with
-// more than twelve neighbours a sixth: as many turns of half the width cost more (rows of 256 bytes instead of 512, and the
-// mixing plan read twice as often).  Measured with 128 / 64 columns: 96 workers x
-// 300,007 columns (6 turns or 11 halves) 111 / 104 us, 78 x 8372 (1 / 1) 10.4 / 7.8, 173 x 166,798 (two blocks an SM, 5 / 6) 125 /
-// 108; 109 x 1,298,095 (23 / 46) 950 / 1397, 116 x 1,614,144 (29 / 57) 2074 / 2244, 74 x 660,293 (12 / 24) 138 / 156,
-// with 16 neighbours 113 x 253,162 (5 / 9) 147 / 168.
+// 64 columns to a panel instead of 128 where the panels are then walked in fewer turns of all blocks: by a twelfth at least, with more
+// than twelve neighbours by two fifths.  As many turns of half the width cost more (rows of 256 bytes instead of 512, the mixing
+// plan read twice as often), and two rows to a warp take as long as the longer one, which counts where many are kept and not
+// equally many.  Measured with 128 / 64 columns: 96 workers x 300,007 columns (6 turns or 11 halves) 111 / 104 us, 78 x 8372 (1 / 1)
+// 10.4 / 7.8, 173 x 166,798 (two blocks an SM, 5 / 6) 125 / 108; 109 x 1,298,095 (23 / 46) 950 / 1397, 116 x 1,614,144 (29 / 57) 2074 /
+// 2244, 74 x 660,293 (12 / 24) 138 / 156; 205 x 181,206, 24 to 32 of 32 neighbours kept (5 / 7) 300 / 360.
 template <bool LOCAL>
 int narrower_panel(dbw_handle* h, bool* narrower) {
     int wide = 0, narrow = 0, rc;
     if ((rc = panel_blocks<32, LOCAL>(h, &wide)) || (rc = panel_blocks<16, LOCAL>(h, &narrow))) return rc;
     auto turns = [h](int cols, int per_sm) { return (((h->ld + cols - 1) / cols) + per_sm * h->sm_count - 1) / (per_sm * h->sm_count); };
-    *narrower = 100 * turns(64, narrow) < (h->nnz > 12 * h->N ? 168 : 184) * turns(128, wide);
+    *narrower = 100 * turns(64, narrow) < (h->nnz > 12 * h->N ? 120 : 184) * turns(128, wide);
     return DBW_OK;
 }
 
