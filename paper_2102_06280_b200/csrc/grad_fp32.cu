@@ -2,6 +2,7 @@
 // CUDA cores, for all workers at once: every kernel is batched over workers (blockIdx.z), whose
 // weights are slices of their rows of X.
 #include "common.cuh"
+#include "gemm_split.cuh"
 #include "round_dev.cuh"
 
 namespace dbw {
@@ -427,6 +428,46 @@ __global__ void __launch_bounds__(32, 8) gemm_warp_kernel(const __grid_constant_
     }
 }
 
+// On the tensor cores (gemm_split.cuh), a block to a tile.  DEEP: a block to an SM with loads two steps ahead and a ring of four, for
+// launches of no more tiles than SMs, which wait for their chain of k steps; else two blocks to an SM with half of that each.
+template <int KIND, bool VEC, bool DEEP>
+__global__ void __launch_bounds__(split::kFillThreads + 32, DEEP ? 1 : 2) gemm_split_kernel(const __grid_constant__ GemmArgs g, const split::Tiles tiles) {
+    dependent_begin();
+    constexpr int RING = DEEP ? 4 : 2, AHEAD = DEEP ? 2 : 1;
+    extern __shared__ uint8_t split_smem[];
+    __shared__ split::BlockSmem fixed;
+    split::Block blk;
+    if (threadIdx.x < split::kFillThreads) {
+        split::gemm_tile<KIND, VEC, true, RING, AHEAD, true>(blk, g, tiles, blockIdx.x, [&] { split::block_begin(blk, split_smem, fixed); });
+    } else {
+        split::block_begin(blk, split_smem, fixed);
+        split::issue_tile<KIND, RING>(blk, g);
+    }
+    split::block_end(blk);
+}
+
+template <int KIND, bool VEC, bool DEEP>
+int launch_split_of(dbw_handle* h, const GemmArgs& g, const split::Tiles& tiles, cudaStream_t s) {
+    static PerDeviceOnce once;
+    constexpr size_t smem = split::smem_bytes(DEEP ? 4 : 2);
+    const int rc = once.run(h->device, []() -> int {
+        DBW_CUDA(cudaFuncSetAttribute(gemm_split_kernel<KIND, VEC, DEEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        return DBW_OK;
+    });
+    if (rc) return rc;
+    launch<false>(gemm_split_kernel<KIND, VEC, DEEP>, tiles.total, split::kFillThreads + 32, smem, s, g, tiles);
+    DBW_LAUNCHED();
+    return DBW_OK;
+}
+
+template <int KIND>
+int launch_split(dbw_handle* h, const GemmArgs& g, int batch, cudaStream_t s) {
+    const split::Tiles tiles(g.M, g.N, batch);
+    if (tiles.total <= h->sm_count)
+        return split::aligned<KIND>(g) ? launch_split_of<KIND, true, true>(h, g, tiles, s) : launch_split_of<KIND, false, true>(h, g, tiles, s);
+    return split::aligned<KIND>(g) ? launch_split_of<KIND, true, false>(h, g, tiles, s) : launch_split_of<KIND, false, false>(h, g, tiles, s);
+}
+
 // 128-bit accesses are possible: unit stride along k or along the output dimension, everything else a multiple of four floats
 bool gemm_vec_ok(const GemmArgs& g) {
     auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
@@ -503,7 +544,11 @@ void launch_gemm_slice(const GemmArgs& g, int batch, cudaStream_t s) {
 }
 
 enum GemmStep { GEMM_FORWARD, GEMM_DW, GEMM_DA };
-int run_gemm(GemmArgs& g, GemmStep step, int batch, int sm_count, cudaStream_t s) {
+int run_gemm(dbw_handle* h, GemmArgs& g, GemmStep step, int batch, cudaStream_t s) {
+    const int sm_count = h->sm_count;
+    g.status = h->d_status;
+    if (fp32_gemm_split(g.M, g.N, g.K, batch, step == GEMM_DW))
+        return step == GEMM_FORWARD ? launch_split<split::FORWARD>(h, g, batch, s) : step == GEMM_DW ? launch_split<split::DW>(h, g, batch, s) : launch_split<split::DA>(h, g, batch, s);
     g.slice = step == GEMM_FORWARD ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, step == GEMM_DW, sm_count);
     if (gemm_vec_ok(g) && g.slice < g.K) {
         launch_gemm_slice(g, batch, s);
@@ -552,6 +597,17 @@ int run_gemm(GemmArgs& g, GemmStep step, int batch, int sm_count, cudaStream_t s
 }
 
 }  // namespace
+
+// Which GEMMs run on the tensor cores: those of many multiply-adds; fewer where operand rows are not whole 16-byte groups and the CUDA-core
+// kernel is the scalar one.  Measured on 900 GEMMs of 4 - 64 workers (us, CUDA cores / tensor cores): 10 workers, M x N x K =
+// 1024 x 256 x 256 42 / 22.6, 32, 64 x 200 x 784 30.6 / 20.7; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4, 36, 168 x 256 x
+// 45 (40 million) 8.3 / 10.4; unaligned 14, 124 x 52 x 578 (52 million) 16.5 / 20.6 and 37, 57 x 157 x 128 (42 million) 12.4 / 8.9.  What it
+// costs is a launch's chain: operands to bf16 pieces, MMAs and a barrier between them for every 32 k, about 0.5 us whatever the
+// size; a k of one such step does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5).
+bool fp32_gemm_split(int M, int N, int K, int batch, bool is_dw) {
+    const bool rows_aligned = N % 4 == 0 && (is_dw ? M : K) % 4 == 0;
+    return (long long)M * N * K * batch >= (rows_aligned ? 60000000 : 30000000) && (K > split::kStep || !rows_aligned);
+}
 
 // is_dw: dZ^T A, both operands with their unit stride along the output; else with the first one's along k.
 int fp32_gemm_slice(int M, int N, int K, int batch, bool is_dw, int sm_count) {
@@ -614,7 +670,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.C = h->d_act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = X + m.b_off[l]; g.sBiasz = h->ld;
         g.M = B; g.N = out; g.K = in; g.relu = l < L - 1;
-        if ((rc = run_gemm(g, GEMM_FORWARD, N, h->sm_count, s)) != DBW_OK) return rc;
+        if ((rc = run_gemm(h, g, GEMM_FORWARD, N, s)) != DBW_OK) return rc;
     }
     if (beside && (rc = (*beside)())) return rc;
     if (head) {
@@ -662,12 +718,12 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         g.B = h->d_act[l]; g.sBz = (long long)B * in; g.sBn = 1; g.sBk = in;
         g.C = G + m.w_off[l]; g.sCz = h->ld; g.sCm = in;
         g.M = out; g.N = in; g.K = B;
-        const bool needs_db = l < L - 1 && !(head && l == L - 2), db_here = needs_db && gemm_vec_ok(g);
+        const bool needs_db = l < L - 1 && !(head && l == L - 2), db_here = needs_db && (fp32_gemm_split(g.M, g.N, g.K, N, true) || gemm_vec_ok(g));
         if (db_here) {  // the sums of dZ's columns come with the GEMM that reads them
             g.rowsum = G + m.b_off[l];
             g.sRz = h->ld;
         }
-        if ((rc = run_gemm(g, GEMM_DW, N, h->sm_count, s)) != DBW_OK) return rc;
+        if ((rc = run_gemm(h, g, GEMM_DW, N, s)) != DBW_OK) return rc;
         if (needs_db && !db_here) {  // the last layer's bias gradient came out of the loss kernel, the one before's out of the last layer's backward kernel
             launch<false>(bias_grad_kernel, dim3((out + 127) / 128, N), 128, 0, s, B, out, h->d_dz[l + 1], G, h->ld, m.b_off[l]);
             DBW_LAUNCHED();
@@ -679,7 +735,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
             a.C = h->d_dz[l]; a.sCz = (long long)B * in; a.sCm = in;
             a.mask = h->d_act[l]; a.sMz = (long long)B * in; a.sMm = in;
             a.M = B; a.N = in; a.K = out;
-            if ((rc = run_gemm(a, GEMM_DA, N, h->sm_count, s)) != DBW_OK) return rc;
+            if ((rc = run_gemm(h, a, GEMM_DA, N, s)) != DBW_OK) return rc;
         }
     }
     return DBW_OK;

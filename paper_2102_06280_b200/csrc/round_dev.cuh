@@ -55,8 +55,9 @@ struct GemmArgs {
     int M, N, K;
     int slice;  // k is summed in slices of this many (a multiple of 8, or at least K): each in ascending k, the slices added in order
     int relu;
-    float* rowsum;  // nullable (gemm_vec_kernel only): sum over k of A(m, k), in ascending k
+    float* rowsum;  // nullable (not for gemm_tile): sum over k of A(m, k)
     long long sRz;
+    uint32_t* status;
 };
 
 

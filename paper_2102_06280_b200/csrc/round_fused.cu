@@ -18,6 +18,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "gemm_split.cuh"
 #include "round_dev.cuh"
 
 namespace dbw {
@@ -31,6 +32,10 @@ constexpr int kThreads = 256;
 constexpr int kMixGS = 32;                       // 128-column panels
 constexpr int kMaxWorkers = 64;                  // N * kMixGS * 16 bytes of panel <= 32 KiB
 constexpr int kSmemBytes = 2 * 128 * 36 * 4;     // the largest GEMM staging (32 x 32 tiles, 128-deep steps): 36,864 bytes
+// With GEMMs on the tensor cores: their buffer, and more than half of an SM's shared memory, so that no two launches of this kernel share an
+// SM and wait for each other's tensor memory there.
+constexpr int kSplitSmemBytes = 116 * 1024;
+static_assert(split::smem_bytes(2) <= kSplitSmemBytes && split::kFillThreads == kThreads, "");
 constexpr int kBlocksPerSM = 1;                  // registers are spent on deep k-steps (a step costs one memory round trip)
 // Networks for which the launch is used unasked: those where it is the faster path, which depends on the steps it has to make.  What
 // it saves is launches; what it costs is that one block to an SM works off all samples and tiles, and that its steps wait for
@@ -50,7 +55,7 @@ constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {2560, kAny, kA
                                     {{512, 148, kAny, 16 << 20}, {2048, kAny, 20, 64 << 20}}};    // more
 
 // GEMM tile variants (R, TK) the kernel instantiates; which one a GEMM uses is chosen on the host.
-enum { V_2_16 = 0, V_2_64 = 1, V_4_16 = 2, V_4_64 = 3, V_2_128 = 4, kVariants = 5 };
+enum { V_2_16 = 0, V_2_64 = 1, V_4_16 = 2, V_4_64 = 3, V_2_128 = 4, kVariants = 5, V_SPLIT = 5 };
 
 struct FusedArgs {
     int N, B, S, L, C;
@@ -84,7 +89,8 @@ struct FusedArgs {
     const float* lr_pw;
     float* loss;
     int dw_slice[DBW_MAX_LAYERS], da_slice[DBW_MAX_LAYERS];
-    signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];
+    signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];  // V_SPLIT: on the tensor cores (gemm_split.cuh)
+    int any_split;
     float* head_part;
     int head;  // the last layer takes the small-output steps (at most 32 classes)
 };
@@ -102,7 +108,14 @@ __device__ __forceinline__ void gemm_tiles(const GemmArgs& g, int workers, float
     }
 }
 
-__device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int workers, float* smem) {
+template <int KIND>
+__device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int workers, float* smem, split::Block& blk) {
+    if (variant == V_SPLIT) {
+        const split::Tiles tiles(g.M, g.N, workers);
+        for (int tile = blockIdx.x; tile < tiles.total; tile += gridDim.x) split::gemm_tile<KIND, false, false, 2, 1, false>(blk, g, tiles, tile, [] {});
+        __syncthreads();
+        return;
+    }
     if (g.slice < g.K) {  // summed in slices of k: one tile shape serves them (the order does not depend on it)
         gemm_tiles<2, 64, true>(g, workers, smem);
         return;
@@ -120,6 +133,9 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
     extern __shared__ __align__(16) float smem[];
     __shared__ float sl[8];
     __shared__ double red[kThreads / 32];
+    __shared__ split::BlockSmem fixed;
+    split::Block blk{};
+    if (a.any_split) split::block_begin(blk, reinterpret_cast<uint8_t*>(smem), fixed);
     cg::grid_group grid = cg::this_grid();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.B, N = a.N, L = a.L;
@@ -176,8 +192,8 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.B = a.X + a.w_off[l]; g.sBz = a.ld; g.sBn = in; g.sBk = 1;
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
-        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in;
-        gemm_any(a.fwd_var[l], g, N, smem);
+        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in; g.status = a.status;
+        gemm_any<split::FORWARD>(a.fwd_var[l], g, N, smem, blk);
         grid.sync();
     }
 
@@ -238,9 +254,14 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.A = a.dz[l + 1]; g.sAz = (long long)B * out; g.sAm = 1; g.sAk = out;
         g.B = a.act[l]; g.sBz = (long long)B * in; g.sBn = 1; g.sBk = in;
         g.C = a.G + a.w_off[l]; g.sCz = a.ld; g.sCm = in;
-        g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l];
-        gemm_any(a.dw_var[l], g, N, smem);
-        if (l < L - 1 && !(a.head && l == L - 2))  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
+        g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l]; g.status = a.status;
+        const bool needs_db = l < L - 1 && !(a.head && l == L - 2);  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
+        if (needs_db && a.dw_var[l] == V_SPLIT) {  // the sums of dZ's columns come with the GEMM
+            g.rowsum = a.G + a.b_off[l];
+            g.sRz = a.ld;
+        }
+        gemm_any<split::DW>(a.dw_var[l], g, N, smem, blk);
+        if (needs_db && a.dw_var[l] != V_SPLIT)
             for (int e = blockIdx.x * kThreads + tid; e < N * out; e += gridDim.x * kThreads)
                 bias_grad_col<true>(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l], a.dw_slice[l]);
         if (l > 0) {  // dZ_l[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]
@@ -249,8 +270,8 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
             d.B = a.X + a.w_off[l]; d.sBz = a.ld; d.sBn = 1; d.sBk = in;
             d.C = a.dz[l]; d.sCz = (long long)B * in; d.sCm = in;
             d.mask = a.act[l]; d.sMz = (long long)B * in; d.sMm = in;
-            d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l];
-            gemm_any(a.da_var[l], d, N, smem);
+            d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l]; d.status = a.status;
+            gemm_any<split::DA>(a.da_var[l], d, N, smem, blk);
         }
         grid.sync();
     }
@@ -262,6 +283,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
                                                a.plan, a.mix_then_correct);
         __syncthreads();
     }
+    if (a.any_split) split::block_end(blk);
 }
 
 // Which tile variant a GEMM of `workers` problems M x N x K should take on a grid of `grid` blocks: the
@@ -307,6 +329,7 @@ void round_fused_prepare(dbw_handle* h) {
     int coop = 0, per_sm = 0;
     if (!cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device)) || !coop) return;
     if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, round_fused_kernel, kThreads, kSmemBytes)) || per_sm < 1) return;
+    if (!cuda_ok(cudaFuncSetAttribute(round_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
     st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     const dbw_model_desc& m = h->model;
     const long long samples = (long long)h->N * m.batch;
@@ -364,16 +387,22 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     widest = std::max<long long>(widest, (long long)N * (((m.dims[m.n_layers - 1] >> 2) + kHeadChunk4 - 1) / kHeadChunk4));
     const int grid = (int)std::min<long long>(h->fused->max_blocks, std::max<long long>(widest + 1, 2));
     for (int l = 0; l < m.n_layers; ++l) {
-        a.fwd_var[l] = (signed char)pick_variant(B, m.dims[l + 1], m.dims[l], N, grid);
-        a.dw_var[l] = (signed char)pick_variant(m.dims[l + 1], m.dims[l], B, N, grid);
-        a.da_var[l] = (signed char)pick_variant(B, m.dims[l], m.dims[l + 1], N, grid);
+        auto variant = [&](int M, int Nn, int K, bool is_dw) {
+            if (l >= (a.head ? m.n_layers - 1 : m.n_layers)) return 0;  // not a GEMM
+            const bool on_tensor_cores = fp32_gemm_split(M, Nn, K, N, is_dw);
+            a.any_split |= on_tensor_cores;
+            return on_tensor_cores ? (int)V_SPLIT : pick_variant(M, Nn, K, N, grid);
+        };
+        a.fwd_var[l] = (signed char)variant(B, m.dims[l + 1], m.dims[l], false);
+        a.dw_var[l] = (signed char)variant(m.dims[l + 1], m.dims[l], B, true);
+        a.da_var[l] = (signed char)variant(B, m.dims[l], m.dims[l + 1], false);
     }
     for (int l = 0; l < m.n_layers; ++l) {
         a.dw_slice[l] = fp32_gemm_slice(m.dims[l + 1], m.dims[l], B, N, true, h->sm_count);
         a.da_slice[l] = fp32_gemm_slice(B, m.dims[l], m.dims[l + 1], N, false, h->sm_count);
     }
     void* params[] = {&a};
-    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(round_fused_kernel), dim3(grid), dim3(kThreads), params, kSmemBytes, s));
+    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(round_fused_kernel), dim3(grid), dim3(kThreads), params, a.any_split ? kSplitSmemBytes : kSmemBytes, s));
     DBW_LAUNCHED();
     return DBW_OK;
 }

@@ -1073,3 +1073,52 @@ def test_round_host_on_two_streams_gives_the_bits_of_dbw_round(kind, dynamic):
     for h in handles:
         assert h.status() == 0
         h.close()
+
+
+@pytest.mark.parametrize("dims,batch,n", [([129, 127, 65, 10], 97, 40),   # nothing a multiple of four: rows at every shift, partial tiles one short and one over
+                                          ([132, 128, 64, 10], 128, 64),  # whole tiles, a last step of a few k, more tiles than SMs
+                                          ([784, 64, 10], 64, 20),        # one tile a worker: the deep ring, an odd number of steps
+                                          ([36, 256, 10], 128, 60),       # a step and four k
+                                          ([31, 301, 10], 100, 40),       # less than a step
+                                          ([300, 201, 10], 33, 20),       # dW of a step and one sample
+                                          ([65, 500, 130, 10], 250, 12)])
+def test_fp32_gemms_on_the_tensor_cores(dims, batch, n):
+    """fp32 GEMMs of three bf16 pieces per value: gradients and losses against the oracle within 1e-5 of the largest entry (fp32 sums;
+    hidden units far from zero, so no ReLU decision is a matter of rounding), single launch and steps bit for bit, and an infinite
+    weight that stays its worker's own and shows in its loss."""
+    p = _dbw()
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    rng = np.random.default_rng(4)
+    S = batch + 11
+    feat = rng.random((n, S, dims[0]), dtype=np.float32)
+    labels = rng.integers(0, dims[-1], size=(n, S)).astype(np.int32)
+    X = m.pack((0.05 * rng.standard_normal((n, m.d))).astype(np.float32))
+    for l in range(len(dims) - 2):
+        X[:, m.b_off[l]: m.b_off[l] + dims[l + 1]] = np.where(np.arange(dims[l + 1]) % 3 == 0, -9.0, 9.0) * 0.5 ** l
+    idx = np.stack([rng.permutation(S)[:batch] for _ in range(n)]).astype(np.int32)
+    h.set_dataset(dev(feat), dev(labels), S)
+    G, loss = torch.zeros(n, m.ld, device="cuda"), torch.zeros(n, device="cuda")
+    h.grad(dev(X), dev(idx), G, loss)
+    got = m.unpack(G.cpu().numpy())
+    for i in range(n):
+        g, l = orc.mlp_grad(m.unpack(X[i:i + 1])[0], dims, feat[i][idx[i]], labels[i][idx[i]])
+        assert np.abs(got[i] - g).max() <= 1e-5 * np.abs(g).max()
+        assert abs(float(loss[i]) - l) <= 1e-5 * max(abs(l), 1.0)
+    if n <= 64:
+        t, b = dev(1.0 + rng.random(n)), torch.ones(n, dtype=torch.int32, device="cuda")
+        outs = []
+        for fused in (True, False):
+            h.set_fused_round(fused)
+            Y, kept = dev(X), torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+            h.round(Y, t, b, 0.05, Y, kept, batch_idx=dev(idx), loss=loss)
+            outs.append((Y, loss.clone()))
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    X[1, m.w_off[0] + dims[0] + 1] = np.inf  # a unit that passes its ReLU
+    G2, loss2 = torch.zeros_like(G), torch.zeros_like(loss)
+    h.grad(dev(X), dev(idx), G2, loss2)
+    others = [i for i in range(n) if i != 1]
+    assert torch.equal(G2[others], G[others]) and not np.isfinite(float(loss2[1]))
+    assert h.status() == 0
+    h.close()
