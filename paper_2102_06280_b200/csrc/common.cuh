@@ -276,13 +276,24 @@ inline size_t fp32_head_smem_bytes(int B, int C) {
 }
 // floats of one worker's partial sums: dW, db, the bias gradient of the layer before, the loss
 __host__ __device__ inline long long fp32_head_partial(int in, int C) { return (long long)C * in + (C + in + 1 + 3) / 4 * 4; }
-// Whether the last layer can take the small-output path (at most 32 classes, 16-byte rows).
-inline bool fp32_head_usable(const dbw_handle* h) {
+// Whether the last layer takes the small-output path (at most 32 classes), and whether its rows are 16-byte aligned there.
+inline bool fp32_head_usable(const dbw_handle* h) { return h->model.dims[h->model.n_layers] <= 32; }
+inline bool fp32_head_aligned(const dbw_handle* h) {
     const dbw_model_desc& m = h->model;
     const int L = m.n_layers;
-    if (L < 1) return false;
-    return m.dims[L] <= 32 && (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 &&
-           ((uintptr_t)h->feat & 15) == 0;
+    return (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 && ((uintptr_t)h->feat & 15) == 0;
+}
+// Lanes that share a feature group's samples in the last layer's backward step, and the feature groups of a block.  Sixteen instead of
+// eight make twice the blocks, each half as long, which pays where the blocks are few and their samples many (us, 8 / 16: 10 workers
+// x batch 1024, 256 features 46 / 32, 32 x 64, 200 features 13.4 / 10.3), not where a lane is left with a few samples for as many
+// shuffles, nor in the networks that the single launch takes unasked, where its blocks then have a second turn (21 x 57, 784 features, a
+// round 31 / 37).  The same for the per-step kernels and the single launch, which sum in this order.
+__host__ __device__ constexpr int head_chunk4(int slices) { return 8 * 32 / slices; }
+inline int fp32_head_slices(const dbw_handle* h) {
+    const int B = h->model.batch, in4 = (h->model.dims[h->model.n_layers - 1] + 3) / 4;
+    const long long blocks = (long long)h->N * ((in4 + head_chunk4(8) - 1) / head_chunk4(8)) * fp32_head_parts(B);
+    const bool large = (long long)h->N * B > 2560 || (h->model.n_layers > 1 && h->N > 20);
+    return large && B >= 64 && 2 * blocks <= h->sm_count + h->sm_count / 4 ? 16 : 8;
 }
 // Slices over k of an fp32 backward GEMM of `batch` problems M x N x K (GemmArgs::slice), the same for the per-step kernels and
 // the single launch, which sum in this order.  Forward GEMMs are not sliced: whether a pre-activation of zero up to rounding

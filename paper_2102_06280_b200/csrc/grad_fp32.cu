@@ -479,28 +479,28 @@ bool gemm_vec_ok(const GemmArgs& g) {
     return a_ok && b_ok && c_ok && m_ok && g.sAz % 4 == 0 && g.sBz % 4 == 0 && al(g.A) && al(g.B);
 }
 
-// Last layer with at most 32 classes: forward + loss by a warp per sample, backward by a block per worker
-// and 128 features (bodies in round_dev.cuh).
-template <int CP>
+// Last layer with at most 32 classes: forward + loss by a warp per U samples, backward by a block per worker
+// and 128 or 64 features (bodies in round_dev.cuh).
+template <int CP, int U, bool VEC>
 __global__ void __launch_bounds__(256)
 last_layer_forward_kernel(int N, int B, int in, int C, HeadRows rows, const float* __restrict__ X, long long ld, long long w_off,
                           long long b_off, float* __restrict__ dz, float* __restrict__ loss_s, uint32_t* status) {
     dependent_begin();
-    const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (item >= N * B) return;
-    const int i = item / B;
-    head_forward_sample<CP, true>(i, item % B, B, in, C, rows, X + (size_t)i * ld + w_off, X + (size_t)i * ld + b_off, dz, loss_s, status);
+    const int item = blockIdx.x * 8 + (threadIdx.x >> 5), groups = (B + U - 1) / U;
+    if (item >= N * groups) return;
+    const int i = item / groups;
+    head_forward_samples<CP, U, VEC, true>(i, item % groups * U, B, in, C, rows, X + (size_t)i * ld + w_off, X + (size_t)i * ld + b_off, dz, loss_s, status);
 }
 
-template <int CP>
+template <int CP, int SLICES, bool VEC>
 __global__ void __launch_bounds__(256)
 last_layer_backward_kernel(int B, int in, int C, HeadRows rows, const float* __restrict__ dz, const float* __restrict__ loss_s,
                            const float* __restrict__ X, float* __restrict__ G, long long ld, long long w_off, long long b_off,
                            float* __restrict__ loss, float* __restrict__ dz_prev, long long b_off_prev, float* __restrict__ partial, uint32_t* status) {
     dependent_begin();
     extern __shared__ __align__(16) float head_smem[];
-    const int i = blockIdx.y, k_lo = blockIdx.x * kHeadChunk4;
-    const int k_hi = min(in >> 2, k_lo + kHeadChunk4);
+    const int i = blockIdx.y, k_lo = blockIdx.x * head_chunk4(SLICES);
+    const int k_hi = min((in + 3) >> 2, k_lo + head_chunk4(SLICES));
     const int s_lo = blockIdx.z * kHeadPart, s_hi = min(B, s_lo + kHeadPart);
     float *Gw = G + (size_t)i * ld + w_off, *Gb = G + (size_t)i * ld + b_off, *Gp = G + (size_t)i * ld + b_off_prev, *li = loss ? loss + i : nullptr;
     float scale = 1.0f / (float)B;
@@ -511,8 +511,8 @@ last_layer_backward_kernel(int B, int in, int C, HeadRows rows, const float* __r
         li = Gp + in;
         scale = 1.f;
     }
-    head_backward_part<CP, true>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, C, rows, dz, loss_s, X + (size_t)i * ld + w_off, Gw, Gb, li, dz_prev, Gp,
-                                 head_smem, status);
+    head_backward_part<CP, SLICES, VEC, true>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, C, rows, dz, loss_s, X + (size_t)i * ld + w_off, Gw, Gb, li, dz_prev, Gp,
+                                      head_smem, status);
 }
 
 __global__ void __launch_bounds__(256)
@@ -603,10 +603,11 @@ int run_gemm(dbw_handle* h, GemmArgs& g, GemmStep step, int batch, cudaStream_t 
 // 1024 x 256 x 256 42 / 22.6, 32, 64 x 200 x 784 30.6 / 20.7; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4, 36, 168 x 256 x
 // 45 (40 million) 8.3 / 10.4; unaligned 14, 124 x 52 x 578 (52 million) 16.5 / 20.6 and 37, 57 x 157 x 128 (42 million) 12.4 / 8.9.  What it
 // costs is a launch's chain: operands to bf16 pieces, MMAs and a barrier between them for every 32 k, about 0.5 us whatever the
-// size; a k of one such step does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5).
+// size; a k of one such step does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5), nor does a long one of few multiply-adds (5, 49 x
+// 240 x 563, 33 million: a gradient call 48 / 52).
 bool fp32_gemm_split(int M, int N, int K, int batch, bool is_dw) {
     const bool rows_aligned = N % 4 == 0 && (is_dw ? M : K) % 4 == 0;
-    return (long long)M * N * K * batch >= (rows_aligned ? 60000000 : 30000000) && (K > split::kStep || !rows_aligned);
+    return (long long)M * N * K * batch >= (rows_aligned || K > 512 ? 60000000 : 30000000) && (K > split::kStep || !rows_aligned);
 }
 
 // is_dw: dZ^T A, both operands with their unit stride along the output; else with the first one's along k.
@@ -649,7 +650,7 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
     const int B = m.batch, L = m.n_layers, N = h->N;
     // A last layer of at most 32 classes runs as two kernels of its own instead of a GEMM, the loss kernel and
     // two more GEMMs; a one-layer model then needs no gathered copy of the mini-batch either.
-    const bool head = fp32_head_usable(h) && (((uintptr_t)X | (uintptr_t)G) & 15) == 0;
+    const bool head = fp32_head_usable(h), head_aligned = fp32_head_aligned(h) && (((uintptr_t)X | (uintptr_t)G) & 15) == 0;
     const int Lg = head ? L - 1 : L;  // layers that run as GEMMs
     if (Lg > 0 || !head) {
         if ((long long)B * N <= 16LL * h->sm_count)
@@ -684,23 +685,34 @@ int launch_grad_fp32(dbw_handle* h, const float* X, const int32_t* batch_idx, fl
         float* loss_s = h->d_act[L];  // [N][B] of the logits' buffer: the logits themselves are never stored
         float* dz_prev = L > 1 ? h->d_dz[L - 1] : nullptr;
         const int parts = fp32_head_parts(B);
-        const dim3 bgrid(((in >> 2) + kHeadChunk4 - 1) / kHeadChunk4, N, parts);
+        const int slices = fp32_head_slices(h);
+        const dim3 bgrid(((in + 3) / 4 + head_chunk4(slices) - 1) / head_chunk4(slices), N, parts);
         const long long b_prev = L > 1 ? m.b_off[L - 2] : -1;
         const size_t smem = fp32_head_smem_bytes(B, C);
-        if (C <= 16) {
-            launch<false>(last_layer_forward_kernel<16>, (N * B + 7) / 8, 256, 0, s, N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
-                                                                          h->d_dz[L], loss_s, h->d_status);
+        // Four samples to a warp once that still gives every SM a dozen warps.
+        const bool four = (long long)N * ((B + 3) / 4) >= 12LL * h->sm_count && C <= 16;
+        const long long b_prev_off = L > 1 ? b_prev : 0;
+        auto both = [&](auto cp, auto samples, auto vec) -> int {
+            constexpr int CP = decltype(cp)::value, U = decltype(samples)::value;
+            constexpr bool VEC = decltype(vec)::value;
+            launch<false>(last_layer_forward_kernel<CP, U, VEC>, (N * ((B + U - 1) / U) + 7) / 8, 256, 0, s, N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1], h->d_dz[L],
+                          loss_s, h->d_status);
             DBW_LAUNCHED();
-            launch<false>(last_layer_backward_kernel<16>, bgrid, 256, smem, s, B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
-                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
-        } else {
-            launch<false>(last_layer_forward_kernel<32>, (N * B + 7) / 8, 256, 0, s, N, B, in, C, rows, X, h->ld, m.w_off[L - 1], m.b_off[L - 1],
-                                                                          h->d_dz[L], loss_s, h->d_status);
+            launch<false>(slices == 16 ? last_layer_backward_kernel<CP, 16, VEC> : last_layer_backward_kernel<CP, 8, VEC>, bgrid, 256, smem, s, B, in, C, rows, h->d_dz[L], loss_s,
+                          X, G, h->ld, m.w_off[L - 1], m.b_off[L - 1], loss, dz_prev, b_prev_off, h->d_head_part, h->d_status);
             DBW_LAUNCHED();
-            launch<false>(last_layer_backward_kernel<32>, bgrid, 256, smem, s, B, in, C, rows, h->d_dz[L], loss_s, X, G, h->ld, m.w_off[L - 1],
-                                                                    m.b_off[L - 1], loss, dz_prev, L > 1 ? b_prev : 0, h->d_head_part, h->d_status);
-        }
-        DBW_LAUNCHED();
+            return DBW_OK;
+        };
+        using std::integral_constant;
+        using one = integral_constant<int, 1>;
+        using several = integral_constant<int, 4>;
+        if (C > 16)
+            rc = head_aligned ? both(integral_constant<int, 32>{}, one{}, std::true_type{}) : both(integral_constant<int, 32>{}, one{}, std::false_type{});
+        else if (four)
+            rc = head_aligned ? both(integral_constant<int, 16>{}, several{}, std::true_type{}) : both(integral_constant<int, 16>{}, several{}, std::false_type{});
+        else
+            rc = head_aligned ? both(integral_constant<int, 16>{}, one{}, std::true_type{}) : both(integral_constant<int, 16>{}, one{}, std::false_type{});
+        if (rc) return rc;
         if (parts > 1) {
             launch(last_layer_add_parts_kernel, dim3((C * in + C + in + 256) / 256, N), 256, 0, s, parts, N, B, in, C, h->d_head_part, G, h->ld, m.w_off[L - 1],
                                                                                             m.b_off[L - 1], b_prev, loss);

@@ -320,72 +320,148 @@ __device__ __forceinline__ const float* head_row(const HeadRows& r, int i, int s
     return r.feat + ((size_t)i * r.S + src) * in;
 }
 
-// Sample s of worker i by one warp: z = W a + b, dZ = (softmax(z) - onehot(y)) / B, the sample's loss
-// logsumexp(z) - z_y into loss_s[i][s].  CP = compile-time bound on the classes (16 or 32); in is a multiple of 4.
-// A lane adds its features in ascending order, the lanes are then added by a butterfly.
-template <int CP, bool NC>
-__device__ __forceinline__ void head_forward_sample(int i, int s, int B, int in, int C, const HeadRows& rows, const float* W,
-                                                    const float* bias, float* dz, float* loss_s, uint32_t* status) {
+// Four neighbouring features 4 k .. of a row of `in`; VEC: rows are 16-byte aligned and `in` is a multiple of four, else features past the
+// end are zero.
+template <bool VEC, bool NC>
+__device__ __forceinline__ float4 head_load4(const float* row, int k, int in) {
+    if (VEC) return load_g<NC>(reinterpret_cast<const float4*>(row) + k);
+    const float* p = row + 4 * k;
+    const int left = in - 4 * k;
+    return make_float4(load_g<NC>(p), left > 1 ? load_g<NC>(p + 1) : 0.f, left > 2 ? load_g<NC>(p + 2) : 0.f, left > 3 ? load_g<NC>(p + 3) : 0.f);
+}
+template <bool VEC>
+__device__ __forceinline__ void head_store4(float* row, int k, int in, float4 v) {
+    if (VEC) {
+        reinterpret_cast<float4*>(row)[k] = v;
+    } else {
+        float* p = row + 4 * k;
+        const int left = in - 4 * k;
+        p[0] = v.x;
+        if (left > 1) p[1] = v.y;
+        if (left > 2) p[2] = v.z;
+        if (left > 3) p[3] = v.w;
+    }
+}
+
+// Samples s .. s + U - 1 of worker i by one warp: z = W a + b, dZ = (softmax(z) - onehot(y)) / B, the sample's loss
+// logsumexp(z) - z_y into loss_s[i][s].  CP = compile-time bound on the classes.  A lane adds its features in ascending order (VEC: every
+// 32nd group of four, else every 32nd feature), the lanes are then added by a butterfly; the same bits whatever U is.  A weight that
+// has been read serves U samples, and with U = 4 eight lanes end up with each sample: 60 shuffles for ten classes of four samples
+// instead of 200.  (10 workers x batch 1024, 256 features, ten classes: U = 1 21 us.)
+template <int CP, int U, bool VEC, bool NC>
+__device__ __forceinline__ void head_forward_samples(int i, int s, int B, int in, int C, const HeadRows& rows, const float* W,
+                                                     const float* bias, float* dz, float* loss_s, uint32_t* status) {
+    static_assert(U == 1 || U == 4, "");
     const int lane = threadIdx.x & 31;
-    int y;
-    const float4* arow = reinterpret_cast<const float4*>(head_row<NC>(rows, i, s, B, in, C, status, &y));
-    const float4* w4 = reinterpret_cast<const float4*>(W);
-    const int in4 = in >> 2;
-    float acc[CP];
+    const float* arow[U];
+    int label[U];
 #pragma unroll
-    for (int c = 0; c < CP; ++c) acc[c] = 0.f;
-    for (int k0 = lane; k0 < in4; k0 += 64) {  // two float4 per lane and pass: twice the loads in flight
-        const int k1 = k0 + 32;
-        const bool two = k1 < in4;
-        const float4 a0 = arow[k0];
-        const float4 a1 = two ? arow[k1] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int u = 0; u < U; ++u) arow[u] = head_row<NC>(rows, i, min(s + u, B - 1), B, in, C, status, &label[u]);
+    float acc[U][CP];
 #pragma unroll
-        for (int c0 = 0; c0 < CP; c0 += 8) {  // eight classes at a time: sixteen weight loads in flight per lane
-            if (c0 >= C) break;
-            float4 w0[8], w1[8];
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int c = c0 + u;
-                w0[u] = c < C ? load_g<NC>(w4 + (size_t)c * in4 + k0) : make_float4(0.f, 0.f, 0.f, 0.f);
-                w1[u] = (c < C && two) ? load_g<NC>(w4 + (size_t)c * in4 + k1) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < CP; ++c) acc[u][c] = 0.f;
+    if (VEC) {
+        const float4* w4 = reinterpret_cast<const float4*>(W);
+        const int in4 = in >> 2;
+        constexpr int CB = U == 1 ? 8 : 2;  // classes whose weights are on their way together
+        for (int k0 = lane; k0 < in4; k0 += 64) {  // two float4 per lane and pass: twice the loads in flight
+            const int k1 = k0 + 32;
+            const bool two = k1 < in4;
+            float4 a0[U], a1[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                a0[u] = *(reinterpret_cast<const float4*>(arow[u]) + k0);
+                a1[u] = two ? *(reinterpret_cast<const float4*>(arow[u]) + k1) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                float t = acc[c0 + u];
-                t = fmaf(a0.x, w0[u].x, t); t = fmaf(a0.y, w0[u].y, t); t = fmaf(a0.z, w0[u].z, t); t = fmaf(a0.w, w0[u].w, t);
-                t = fmaf(a1.x, w1[u].x, t); t = fmaf(a1.y, w1[u].y, t); t = fmaf(a1.z, w1[u].z, t); t = fmaf(a1.w, w1[u].w, t);
-                acc[c0 + u] = t;
+            for (int c0 = 0; c0 < CP; c0 += CB) {
+                if (c0 >= C) break;
+                float4 w0[CB], w1[CB];
+#pragma unroll
+                for (int e = 0; e < CB; ++e) {
+                    const int c = c0 + e;
+                    w0[e] = c < C ? load_g<NC>(w4 + (size_t)c * in4 + k0) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    w1[e] = (c < C && two) ? load_g<NC>(w4 + (size_t)c * in4 + k1) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int e = 0; e < CB; ++e) {
+                    if (c0 + e >= CP) break;
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        float t = acc[u][c0 + e];
+                        t = fmaf(a0[u].x, w0[e].x, t); t = fmaf(a0[u].y, w0[e].y, t); t = fmaf(a0[u].z, w0[e].z, t); t = fmaf(a0[u].w, w0[e].w, t);
+                        t = fmaf(a1[u].x, w1[e].x, t); t = fmaf(a1[u].y, w1[e].y, t); t = fmaf(a1[u].z, w1[e].z, t); t = fmaf(a1[u].w, w1[e].w, t);
+                        acc[u][c0 + e] = t;
+                    }
+                }
             }
+        }
+    } else {
+#pragma unroll 2
+        for (int k = lane; k < in; k += 32) {
+            float a[U], w[CP];
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] = arow[u][k];
+#pragma unroll
+            for (int c = 0; c < CP; ++c) w[c] = c < C ? load_g<NC>(W + (size_t)c * in + k) : 0.f;
+#pragma unroll
+            for (int c = 0; c < CP; ++c)
+#pragma unroll
+                for (int u = 0; u < U; ++u) acc[u][c] = fmaf(a[u], w[c], acc[u][c]);
+        }
+    }
+    // the sums over the lanes; with U = 4 a lane keeps the samples 2 (lane / 16) .. of a pair first, then sample lane / 8
+    float z[CP];
+    int y = label[0];
+    if (U == 4) y = lane & 16 ? (lane & 8 ? label[U - 1] : label[U / 2]) : (lane & 8 ? label[U > 1] : label[0]);
+#pragma unroll
+    for (int c = 0; c < CP; ++c) {
+        if (c < C) {
+            if (U == 1) {
+                z[c] = warp_sum(acc[0][c]);
+            } else {
+                auto halve = [](bool upper, float lo, float hi, int o) { return (upper ? hi : lo) + __shfl_xor_sync(0xffffffffu, upper ? lo : hi, o); };
+                const float lo = halve(lane & 16, acc[0][c], acc[U / 2][c], 16), hi = halve(lane & 16, acc[U > 1][c], acc[U - 1][c], 16);
+                z[c] = halve(lane & 8, lo, hi, 8);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) z[c] += __shfl_xor_sync(0xffffffffu, z[c], o);
+            }
+            z[c] += load_g<NC>(bias + c);
         }
     }
     float mx = -INFINITY;
 #pragma unroll
-    for (int c = 0; c < CP; ++c) {
-        if (c < C) {
-            acc[c] = warp_sum(acc[c]) + load_g<NC>(bias + c);
-            mx = fmaxf(mx, acc[c]);
-        }
-    }
+    for (int c = 0; c < CP; ++c)
+        if (c < C) mx = fmaxf(mx, z[c]);
     float sum = 0.f, zy = 0.f;
 #pragma unroll
     for (int c = 0; c < CP; ++c) {
         if (c < C) {
-            if (c == y) zy = acc[c];
-            acc[c] = expf(acc[c] - mx);
-            sum += acc[c];
+            if (c == y) zy = z[c];
+            z[c] = expf(z[c] - mx);
+            sum += z[c];
         }
     }
     const float inv = 1.0f / sum, invB = 1.0f / (float)B;
-    float mine = 0.f;
+    constexpr int LPS = 32 / U;  // lanes to a sample
+    const int mine = s + lane / LPS;
+    if (mine >= B) return;
 #pragma unroll
-    for (int c = 0; c < CP; ++c)
-        if (c < C && c == lane) mine = (acc[c] * inv - (c == y ? 1.f : 0.f)) * invB;
-    if (lane < C) dz[((size_t)i * B + s) * C + lane] = mine;
-    if (lane == 0) loss_s[(size_t)i * B + s] = (mx + logf(sum)) - zy;
+    for (int c0 = 0; c0 < CP; c0 += LPS) {
+        float d = 0.f;
+        const int own = c0 + lane % LPS;
+#pragma unroll
+        for (int c = c0; c < CP && c < c0 + LPS; ++c)
+            if (c < C && c == own) d = (z[c] * inv - (c == y ? 1.f : 0.f)) * invB;
+        if (own < C) dz[((size_t)i * B + mine) * C + own] = d;
+    }
+    if (lane % LPS == 0) loss_s[(size_t)i * B + mine] = (mx + logf(sum)) - zy;
 }
 
-// Backward of the last layer for worker i, features [4 k_lo, 4 k_hi) (at most kHeadChunk4 groups of four) by a
-// block of 256 threads.  A warp owns four feature groups; its lanes split the samples eight ways (lane mod 8):
+// Backward of the last layer for worker i, features [4 k_lo, 4 k_hi) (at most head_chunk4(SLICES) groups of four) by a
+// block of 256 threads.  A warp owns 32 / SLICES feature groups; its lanes split the samples SLICES ways (lane mod SLICES):
 //   dW[c][f] = sum_s dZ[s][c] a[s][f]: each lane adds its samples in ascending order, a butterfly adds the lanes;
 //   with dz_prev also dZ of the layer before, (sum_c dZ[s][c] W[c][f]) [a[s][f] > 0], classes in ascending order,
 //   and that layer's bias gradient (the sum of its dZ over the samples) into Gb_prev.
@@ -393,8 +469,7 @@ __device__ __forceinline__ void head_forward_sample(int i, int s, int B, int in,
 // Only samples [s_lo, s_hi): all of them, with `scale` = 1 / B for the mean loss, or one part of a large batch, whose sums
 // go to partial buffers (scale 1) and are added by head_add_parts.
 // smem: (s_hi - s_lo) * C floats + as many 64-bit offsets + as many floats.  Ends with a block barrier (shared memory free again).
-constexpr int kHeadChunk4 = 32;
-template <int CP, bool NC>
+template <int CP, int SLICES, bool VEC, bool NC>
 __device__ __forceinline__ void head_backward_part(int i, int s_lo, int s_hi, float scale, int k_lo, int k_hi, int B, int in, int C, const HeadRows& rows,
                                                    const float* dz, const float* loss_s, const float* W, float* Gw, float* Gb,
                                                    float* loss, float* dz_prev, float* Gb_prev, float* smem, uint32_t* status) {
@@ -423,15 +498,15 @@ __device__ __forceinline__ void head_backward_part(int i, int s_lo, int s_hi, fl
             *loss = t * scale;
         }
     }
-    const int lane = threadIdx.x & 31, slice = lane & 7;
-    const int k = k_lo + (int)(threadIdx.x >> 5) * 4 + (lane >> 3);
-    if (k < k_hi) {  // the eight lanes of a feature group stay together
+    const int lane = threadIdx.x & 31, slice = lane % SLICES;
+    const int k = k_lo + (int)(threadIdx.x >> 5) * (32 / SLICES) + lane / SLICES;
+    if (k < k_hi) {  // the lanes of a feature group stay together
         float4 acc[CP];
 #pragma unroll
         for (int c = 0; c < CP; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-        for (int s = slice; s < S; s += 8) {
-            const float4 a = *(reinterpret_cast<const float4*>(base + rowoff[s]) + k);
+        for (int s = slice; s < S; s += SLICES) {
+            const float4 a = head_load4<VEC, false>(base + rowoff[s], k, in);
 #pragma unroll
             for (int c = 0; c < CP; ++c) {
                 if (c < C) {
@@ -441,26 +516,26 @@ __device__ __forceinline__ void head_backward_part(int i, int s_lo, int s_hi, fl
                 }
             }
         }
-        const unsigned grp = 0xffu << (lane & 24);
+        const unsigned grp = ((1u << SLICES) - 1u) << (lane & ~(SLICES - 1));
 #pragma unroll
         for (int c = 0; c < CP; ++c) {
             if (c < C) {
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) {
+                for (int o = 1; o < SLICES; o <<= 1) {
                     acc[c].x += __shfl_xor_sync(grp, acc[c].x, o); acc[c].y += __shfl_xor_sync(grp, acc[c].y, o);
                     acc[c].z += __shfl_xor_sync(grp, acc[c].z, o); acc[c].w += __shfl_xor_sync(grp, acc[c].w, o);
                 }
-                if ((c & 7) == slice) reinterpret_cast<float4*>(Gw + (size_t)c * in)[k] = acc[c];
+                if (c % SLICES == slice) head_store4<VEC>(Gw + (size_t)c * in, k, in, acc[c]);
             }
         }
         if (dz_prev) {
 #pragma unroll
             for (int c = 0; c < CP; ++c)
-                if (c < C) acc[c] = load_g<NC>(reinterpret_cast<const float4*>(W + (size_t)c * in) + k);
+                if (c < C) acc[c] = head_load4<VEC, NC>(W + (size_t)c * in, k, in);
             float4 db = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-            for (int s = slice; s < S; s += 8) {
-                const float4 a = *(reinterpret_cast<const float4*>(base + rowoff[s]) + k);
+            for (int s = slice; s < S; s += SLICES) {
+                const float4 a = head_load4<VEC, false>(base + rowoff[s], k, in);
                 float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int c = 0; c < CP; ++c) {
@@ -472,17 +547,20 @@ __device__ __forceinline__ void head_backward_part(int i, int s_lo, int s_hi, fl
                 }
                 v.x = a.x > 0.f ? v.x : 0.f; v.y = a.y > 0.f ? v.y : 0.f;
                 v.z = a.z > 0.f ? v.z : 0.f; v.w = a.w > 0.f ? v.w : 0.f;
-                reinterpret_cast<float4*>(dz_prev + ((size_t)i * B + s_lo + s) * in)[k] = v;
+                head_store4<VEC>(dz_prev + ((size_t)i * B + s_lo + s) * in, k, in, v);
                 db.x += v.x; db.y += v.y; db.z += v.z; db.w += v.w;
             }
-            // bias gradient of the layer before: this lane's samples in ascending order, then the eight lanes
+            // bias gradient of the layer before: this lane's samples in ascending order, then the lanes
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
+            for (int o = 1; o < SLICES; o <<= 1) {
                 db.x += __shfl_xor_sync(grp, db.x, o); db.y += __shfl_xor_sync(grp, db.y, o);
                 db.z += __shfl_xor_sync(grp, db.z, o); db.w += __shfl_xor_sync(grp, db.w, o);
             }
             if (slice == 0) {
-                Gb_prev[4 * k] = db.x; Gb_prev[4 * k + 1] = db.y; Gb_prev[4 * k + 2] = db.z; Gb_prev[4 * k + 3] = db.w;
+                Gb_prev[4 * k] = db.x;
+                if (VEC || 4 * k + 1 < in) Gb_prev[4 * k + 1] = db.y;
+                if (VEC || 4 * k + 2 < in) Gb_prev[4 * k + 2] = db.z;
+                if (VEC || 4 * k + 3 < in) Gb_prev[4 * k + 3] = db.w;
             }
         }
     }

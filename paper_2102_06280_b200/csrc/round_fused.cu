@@ -42,16 +42,16 @@ constexpr int kBlocksPerSM = 1;                  // registers are spent on deep 
 // the slowest block.  Where the lines lie was measured on 1700 networks of 3 - 64 workers (single launch / step by step, us):
 //  - one layer, whose last layer's two steps read the data set themselves: up to 2560 samples over all workers (8 workers x batch 32,
 //    784-10: 19 / 33, 16 x 64, 784-10: 24 / 36, 41 x 52, 784-10: 39 / 40, 23 x 372, 256-10: 60 / 49);
-//  - one layer as a GEMM (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26, 25 x 265, 121-10: 92 / 62);
+//  - one layer whose rows are not aligned (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26, 25 x 265, 121-10: 92 / 62);
 //  - more layers, the last one in those two steps: 2048 samples of at most 20 workers (8 x 128, 256-64-10: 50 / 59, 8 x 268, 64-96-10:
 //    74 / 79; 40 x 17, 16-108-10: 45 / 36);
-//  - more layers, all of them GEMMs: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16 million multiply-adds.
+//  - more layers, the last one's rows not aligned: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16 million multiply-adds.
 // Never above 64 million multiply-adds of the forward pass.
 struct AutoLimits {
     long long samples, tiles, workers, macs;
 };
 constexpr long long kAny = 1ll << 40;
-constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {2560, kAny, kAny, 64 << 20}},   // one layer: a GEMM / small outputs
+constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {2560, kAny, kAny, 64 << 20}},   // one layer: rows not aligned / aligned
                                     {{512, 148, kAny, 16 << 20}, {2048, kAny, 20, 64 << 20}}};    // more
 
 // GEMM tile variants (R, TK) the kernel instantiates; which one a GEMM uses is chosen on the host.
@@ -92,7 +92,7 @@ struct FusedArgs {
     signed char fwd_var[DBW_MAX_LAYERS], dw_var[DBW_MAX_LAYERS], da_var[DBW_MAX_LAYERS];  // V_SPLIT: on the tensor cores (gemm_split.cuh)
     int any_split;
     float* head_part;
-    int head;  // the last layer takes the small-output steps (at most 32 classes)
+    int head, head_slices, head_aligned;  // the last layer takes the small-output steps (at most 32 classes); its rows are 16-byte aligned
 };
 
 template <int R, int TK, bool SLICED = false>
@@ -108,9 +108,9 @@ __device__ __forceinline__ void gemm_tiles(const GemmArgs& g, int workers, float
     }
 }
 
-template <int KIND>
+template <int KIND, bool GENERAL>
 __device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int workers, float* smem, split::Block& blk) {
-    if (variant == V_SPLIT) {
+    if (GENERAL && variant == V_SPLIT) {
         const split::Tiles tiles(g.M, g.N, workers);
         for (int tile = blockIdx.x; tile < tiles.total; tile += gridDim.x) split::gemm_tile<KIND, false, false, 2, 1, false>(blk, g, tiles, tile, [] {});
         __syncthreads();
@@ -129,13 +129,17 @@ __device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int wor
     }
 }
 
+// GENERAL = false leaves out what most rounds of this size have no use for: GEMMs on the tensor cores, last layers whose rows are not
+// aligned or whose backward step has sixteen lanes to a feature group.  The launch is short enough for code that is not run to show
+// (21 workers, 784-10, batch 57: 33.0 us a round with it, 30.0 without).
+template <bool GENERAL>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(FusedArgs a) {
     extern __shared__ __align__(16) float smem[];
     __shared__ float sl[8];
     __shared__ double red[kThreads / 32];
     __shared__ split::BlockSmem fixed;
     split::Block blk{};
-    if (a.any_split) split::block_begin(blk, reinterpret_cast<uint8_t*>(smem), fixed);
+    if (GENERAL && a.any_split) split::block_begin(blk, reinterpret_cast<uint8_t*>(smem), fixed);
     cg::grid_group grid = cg::this_grid();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int B = a.B, N = a.N, L = a.L;
@@ -150,14 +154,19 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         rows.feat = a.feat; rows.labels = a.labels; rows.batch_idx = a.batch_idx; rows.S = a.S;
     }
     float* loss_s = a.act[L];
+    auto head_variant = [&](auto f) {  // by the number of classes, and whether rows are aligned
+        if (a.C <= 16) !GENERAL || a.head_aligned ? f(std::integral_constant<int, 16>{}, std::true_type{}) : f(std::integral_constant<int, 16>{}, std::bool_constant<!GENERAL>{});
+        else !GENERAL || a.head_aligned ? f(std::integral_constant<int, 32>{}, std::true_type{}) : f(std::integral_constant<int, 32>{}, std::bool_constant<!GENERAL>{});
+    };
     auto head_forward = [&](int first, int step) {
         for (int item = first * (kThreads / 32) + warp; item < N * B; item += step * (kThreads / 32)) {
             const int i = item / B;
             const float* Xi = a.X + (size_t)i * a.ld;
-            if (a.C <= 16)
-                head_forward_sample<16, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
-            else
-                head_forward_sample<32, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+            auto sample = [&](auto cp, auto vec) {
+                head_forward_samples<decltype(cp)::value, 1, decltype(vec)::value, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1],
+                                                                                        Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+            };
+            head_variant(sample);
         }
     };
 
@@ -193,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
         g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in; g.status = a.status;
-        gemm_any<split::FORWARD>(a.fwd_var[l], g, N, smem, blk);
+        gemm_any<split::FORWARD, GENERAL>(a.fwd_var[l], g, N, smem, blk);
         grid.sync();
     }
 
@@ -203,13 +212,13 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
             grid.sync();
         }
         // ---- last layer backward: dW_L, db_L, the loss, dZ_{L-1} ----
-        const int in = a.dims[L - 1], in4 = in >> 2;
-        const int chunks = (in4 + kHeadChunk4 - 1) / kHeadChunk4;
+        const int in = a.dims[L - 1], in4 = (in + 3) >> 2;
+        const int chunk4 = head_chunk4(GENERAL ? a.head_slices : 8), chunks = (in4 + chunk4 - 1) / chunk4;
         const int parts = fp32_head_parts(B);
         const long long b_prev = L > 1 ? a.b_off[L - 2] : 0;
         for (int item = blockIdx.x; item < N * chunks * parts; item += gridDim.x) {
-            const int i = item / chunks % N, part = item / (chunks * N), k_lo = (item % chunks) * kHeadChunk4;
-            const int k_hi = min(in4, k_lo + kHeadChunk4), s_lo = part * kHeadPart, s_hi = min(B, s_lo + kHeadPart);
+            const int i = item / chunks % N, part = item / (chunks * N), k_lo = (item % chunks) * chunk4;
+            const int k_hi = min(in4, k_lo + chunk4), s_lo = part * kHeadPart, s_hi = min(B, s_lo + kHeadPart);
             const float* Xi = a.X + (size_t)i * a.ld;
             float* Gi = a.G + (size_t)i * a.ld;
             float *Gw = Gi + a.w_off[L - 1], *Gb = Gi + a.b_off[L - 1], *Gp = Gi + b_prev, *li = a.loss ? a.loss + i : nullptr;
@@ -222,10 +231,16 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
                 scale = 1.f;
             }
             float* dz_prev = L > 1 ? a.dz[L - 1] : nullptr;
-            if (a.C <= 16)
-                head_backward_part<16, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gw, Gb, li, dz_prev, Gp, smem, a.status);
-            else
-                head_backward_part<32, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, Xi + a.w_off[L - 1], Gw, Gb, li, dz_prev, Gp, smem, a.status);
+            auto part_of = [&](auto cp, auto vec) {
+                constexpr int CP = decltype(cp)::value;
+                constexpr bool VEC = decltype(vec)::value;
+                const float* W = Xi + a.w_off[L - 1];
+                if (GENERAL && a.head_slices == 16)
+                    head_backward_part<CP, 16, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+                else
+                    head_backward_part<CP, 8, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+            };
+            head_variant(part_of);
         }
         if (parts > 1) {
             grid.sync();
@@ -256,12 +271,12 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.C = a.G + a.w_off[l]; g.sCz = a.ld; g.sCm = in;
         g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l]; g.status = a.status;
         const bool needs_db = l < L - 1 && !(a.head && l == L - 2);  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
-        if (needs_db && a.dw_var[l] == V_SPLIT) {  // the sums of dZ's columns come with the GEMM
+        if (GENERAL && needs_db && a.dw_var[l] == V_SPLIT) {  // the sums of dZ's columns come with the GEMM
             g.rowsum = a.G + a.b_off[l];
             g.sRz = a.ld;
         }
-        gemm_any<split::DW>(a.dw_var[l], g, N, smem, blk);
-        if (needs_db && a.dw_var[l] != V_SPLIT)
+        gemm_any<split::DW, GENERAL>(a.dw_var[l], g, N, smem, blk);
+        if (needs_db && (!GENERAL || a.dw_var[l] != V_SPLIT))
             for (int e = blockIdx.x * kThreads + tid; e < N * out; e += gridDim.x * kThreads)
                 bias_grad_col<true>(e / out, e % out, B, out, a.dz[l + 1], a.G, a.ld, a.b_off[l], a.dw_slice[l]);
         if (l > 0) {  // dZ_l[m][k] = (sum_o dZ_{l+1}[m][o] W_l[o][k]) * [A_l[m][k] > 0]
@@ -271,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
             d.C = a.dz[l]; d.sCz = (long long)B * in; d.sCm = in;
             d.mask = a.act[l]; d.sMz = (long long)B * in; d.sMm = in;
             d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l]; d.status = a.status;
-            gemm_any<split::DA>(a.da_var[l], d, N, smem, blk);
+            gemm_any<split::DA, GENERAL>(a.da_var[l], d, N, smem, blk);
         }
         grid.sync();
     }
@@ -283,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
                                                a.plan, a.mix_then_correct);
         __syncthreads();
     }
-    if (a.any_split) split::block_end(blk);
+    if (GENERAL && a.any_split) split::block_end(blk);
 }
 
 // Which tile variant a GEMM of `workers` problems M x N x K should take on a grid of `grid` blocks: the
@@ -328,8 +343,9 @@ void round_fused_prepare(dbw_handle* h) {
     h->fused = st;
     int coop = 0, per_sm = 0;
     if (!cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device)) || !coop) return;
-    if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, round_fused_kernel, kThreads, kSmemBytes)) || per_sm < 1) return;
-    if (!cuda_ok(cudaFuncSetAttribute(round_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
+    for (auto kernel : {round_fused_kernel<false>, round_fused_kernel<true>})
+        if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, kSmemBytes)) || per_sm < 1) return;
+    if (!cuda_ok(cudaFuncSetAttribute(round_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
     st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     const dbw_model_desc& m = h->model;
     const long long samples = (long long)h->N * m.batch;
@@ -338,7 +354,7 @@ void round_fused_prepare(dbw_handle* h) {
         macs += samples * m.dims[l] * m.dims[l + 1];
         if (l + 1 < m.n_layers) tiles = std::max(tiles, (long long)h->N * ((m.batch + 31) / 32) * ((m.dims[l + 1] + 31) / 32));
     }
-    const AutoLimits& a = kAuto[m.n_layers > 1][fp32_head_usable(h)];
+    const AutoLimits& a = kAuto[m.n_layers > 1][fp32_head_usable(h) && fp32_head_aligned(h)];
     st->auto_on = samples <= a.samples && tiles <= a.tiles && h->N <= a.workers && macs <= a.macs;
     st->usable = true;
 }
@@ -374,7 +390,9 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     a.uniform = (h->flags & DBW_WEIGHT_UNIFORM) ? 1 : 0;
     a.mix_then_correct = (h->flags & DBW_ORDER_MIX_THEN_CORRECT) ? 1 : 0;
     a.lr = lr; a.lr_pw = lr_pw; a.loss = loss;
-    a.head = (fp32_head_usable(h) && (((uintptr_t)X | (uintptr_t)h->d_G) & 15) == 0) ? 1 : 0;
+    a.head = fp32_head_usable(h) ? 1 : 0;
+    a.head_slices = fp32_head_slices(h);
+    a.head_aligned = (fp32_head_aligned(h) && (((uintptr_t)X | (uintptr_t)h->d_G) & 15) == 0) ? 1 : 0;
     // grid: as many blocks as the widest step has work items, at most one per SM
     const int B = m.batch, N = h->N;
     long long widest = (long long)N * B;  // gather rows
@@ -384,7 +402,7 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     }
     widest = std::max<long long>(widest, (h->ld + 4 * kMixGS - 1) / (4 * kMixGS));
     widest = std::max<long long>(widest, ((long long)N * B + kThreads / 32 - 1) / (kThreads / 32));  // last layer: a warp per sample
-    widest = std::max<long long>(widest, (long long)N * (((m.dims[m.n_layers - 1] >> 2) + kHeadChunk4 - 1) / kHeadChunk4));
+    widest = std::max<long long>(widest, (long long)N * (((m.dims[m.n_layers - 1] + 3) / 4 + head_chunk4(a.head_slices) - 1) / head_chunk4(a.head_slices)));
     const int grid = (int)std::min<long long>(h->fused->max_blocks, std::max<long long>(widest + 1, 2));
     for (int l = 0; l < m.n_layers; ++l) {
         auto variant = [&](int M, int Nn, int K, bool is_dw) {
@@ -402,7 +420,8 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
         a.da_slice[l] = fp32_gemm_slice(B, m.dims[l], m.dims[l + 1], N, false, h->sm_count);
     }
     void* params[] = {&a};
-    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(round_fused_kernel), dim3(grid), dim3(kThreads), params, a.any_split ? kSplitSmemBytes : kSmemBytes, s));
+    const bool general = a.any_split || (a.head && (!a.head_aligned || a.head_slices == 16));
+    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(general ? round_fused_kernel<true> : round_fused_kernel<false>), dim3(grid), dim3(kThreads), params, a.any_split ? kSplitSmemBytes : kSmemBytes, s));
     DBW_LAUNCHED();
     return DBW_OK;
 }

@@ -1122,3 +1122,45 @@ def test_fp32_gemms_on_the_tensor_cores(dims, batch, n):
     assert torch.equal(G2[others], G[others]) and not np.isfinite(float(loss2[1]))
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("dims,batch,n", [([33, 10], 65, 3),             # one layer, rows of the data set at every shift
+                                          ([64, 131, 10], 72, 35),       # sixteen lanes to a feature group, a last group of three features
+                                          ([64, 132, 12], 301, 30),      # ... aligned, two parts, four samples to a warp and one left over
+                                          ([64, 35, 16], 258, 41),       # ... unaligned
+                                          ([64, 130, 32], 50, 30),       # the most classes
+                                          ([20, 1, 3], 9, 4)])           # a single feature
+def test_fp32_last_layer_of_any_width(dims, batch, n):
+    """The last layer's two steps with rows that are not 16-byte aligned, and their variants by size: gradients and losses against the
+    oracle within 1e-5 of the largest entry (fp32 sums; hidden units far from zero), single launch and steps bit for bit."""
+    p = _dbw()
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    rng = np.random.default_rng(8)
+    S = batch + 5
+    feat = rng.random((n, S, dims[0]), dtype=np.float32)
+    labels = rng.integers(0, dims[-1], size=(n, S)).astype(np.int32)
+    X = m.pack((0.05 * rng.standard_normal((n, m.d))).astype(np.float32))
+    for l in range(len(dims) - 2):
+        X[:, m.b_off[l]: m.b_off[l] + dims[l + 1]] = np.where(np.arange(dims[l + 1]) % 3 == 0, 9.0, -9.0)
+    idx = np.stack([rng.permutation(S)[:batch] for _ in range(n)]).astype(np.int32)
+    h.set_dataset(dev(feat), dev(labels), S)
+    G, loss = torch.zeros(n, m.ld, device="cuda"), torch.zeros(n, device="cuda")
+    h.grad(dev(X), dev(idx), G, loss)
+    got = m.unpack(G.cpu().numpy())
+    for i in range(n):
+        g, l = orc.mlp_grad(m.unpack(X[i:i + 1])[0], dims, feat[i][idx[i]], labels[i][idx[i]])
+        assert np.abs(got[i] - g).max() <= 1e-5 * np.abs(g).max()
+        assert abs(float(loss[i]) - l) <= 1e-5 * max(abs(l), 1.0)
+    assert np.count_nonzero(G.cpu().numpy()) == np.count_nonzero(got)  # padding untouched
+    t, b = dev(1.0 + rng.random(n)), torch.ones(n, dtype=torch.int32, device="cuda")
+    outs = []
+    for fused in (True, False):
+        h.set_fused_round(fused)
+        Y, kept = dev(X), torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+        h.round(Y, t, b, 0.05, Y, kept, batch_idx=dev(idx), loss=loss)
+        outs.append((Y, loss.clone()))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    assert h.status() == 0
+    h.close()
