@@ -11,7 +11,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libdbw.so")
 LIB_DEBUG = os.path.join(PKG, "libdbw_dbg.so")   # the same sources with -DDBW_BOUNDS: every index a kernel reads is checked
-SOURCES = ["api.cu", "select.cu", "mix.cu", "mix_staged.cu", "mix_tc.cu", "mix_sp.cu", "dtur.cu", "grad_fp32.cu", "grad_bf16.cu", "round_fused.cu", "probe.cu"]
+SOURCES = ["api.cu", "select.cu", "mix.cu", "mix_staged.cu", "mix_pipe.cu", "mix_tc.cu", "mix_sp.cu", "dtur.cu", "grad_fp32.cu", "grad_bf16.cu", "round_fused.cu", "probe.cu"]
 
 
 def _nvcc() -> str:

@@ -229,6 +229,11 @@ bool mix_active_usable(const dbw_handle* h);
 int launch_mix_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, cudaStream_t s);
 int mix_kernel_kind(const dbw_handle* h);
 
+// mix_pipe.cu: the panel mix as a pipeline, where that is the faster one
+bool mix_pipe_usable(const dbw_handle* h, bool gradient);
+int launch_mix_pipe(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
+                    const int* active_count = nullptr);
+
 // mix_staged.cu
 bool mix_staged_usable(const dbw_handle* h);
 size_t mix_staged_smem(const dbw_handle* h);  // of one block, without the row weights and list lengths it can do without

@@ -85,7 +85,7 @@ mix_direct_kernel(int N, long long ld, const float* __restrict__ X, const float*
 // panels are staged together, up to half of the buffer with x and the other half with g: copied asynchronously, every
 // load of the panels is in flight at once whatever the registers hold.  A panel that reaches outside the weight blocks
 // is mixed as by mix_panel_kernel, without the stores that are already done.
-// With more participants the round is mix_panel_kernel's: both are launched, and the one whose round it is not leaves at
+// With more participants the round is mix_panel_kernel's (or mix_pipe_kernel's): both are launched, and the one whose round it is not leaves at
 // once (about 2 us; as one kernel for both cases the registers of either spilled: 2.01 ms instead of 1.74 for 128 workers
 // x 4.2 million columns with all 8 neighbours kept).
 struct WeightBlocks {
@@ -283,7 +283,8 @@ template <int GS>
 int launch_active(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow,
                   cudaStream_t s) {
     const size_t smem = active_smem(h->N, GS);
-    int rc = launch_panel<GS>(h, X, G, lr, lr_pw, X_out, shadow, s, h->active.count);
+    int rc = h->mix_panel_cols == 0 && mix_pipe_usable(h, true) ? launch_mix_pipe(h, X, G, lr, lr_pw, X_out, shadow, s, h->active.count)
+                                                                 : launch_panel<GS>(h, X, G, lr, lr_pw, X_out, shadow, s, h->active.count);
     if (rc) return rc;
     static PerDeviceOnce once;
     rc = once.run(h->device, [h]() -> int {
@@ -423,6 +424,7 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
         if (rc || kept_limit == 0) return rc;
     }
     int gs = auto_group_size(h);
+    if (gs >= 8 && h->mix_panel_cols == 0 && mix_pipe_usable(h, G != nullptr)) return launch_mix_pipe(h, X, G, lr, lr_pw, X_out, shadow, s);
     if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) {
         bool narrower = false;
         const int rc = panel_local(h) ? narrower_panel<true>(h, &narrower) : narrower_panel<false>(h, &narrower);

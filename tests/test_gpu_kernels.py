@@ -1164,3 +1164,35 @@ def test_fp32_last_layer_of_any_width(dims, batch, n):
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("n,deg,d", [(5, 2, 3_000_001), (17, 4, 900_000), (33, 4, 450_003),   # panels of 256, 128 and 64 columns
+                                     (70, 32, 210_000),                                        # a long plan
+                                     (129, 8, 120_001), (200, 6, 40_002), (257, 8, 20_000),    # 32 columns, two blocks an SM and one; two boxes of rows
+                                     (439, 6, 19_000), (750, 4, 20_000)])                      # without gradients alone
+@pytest.mark.parametrize("order", ["local_then_mix", "mix_then_correct"])
+def test_pipelined_panel_mix_gives_the_bits_of_the_plain_one(n, deg, d, order):
+    """The panel mix with its next panels on their way, at the edges of its panel widths: with and without gradients, with a learning rate per
+    worker and in place, against the plain panel kernel (asked for by its width) bit for bit."""
+    p = _dbw()
+    rowptr, col = wl.ring(n) if deg == 2 else wl.random_regular(n, deg, 3)
+    h = p.Dbw(rowptr, col, d=d, flags=p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X, G = (torch.randn(n, h.ld, device="cuda", generator=gen) for _ in range(2))
+    lr = torch.rand(n, device="cuda", generator=gen)
+    t = torch.rand(n, device="cuda", generator=gen, dtype=torch.float64)
+    b = torch.randint(0, deg, (n,), device="cuda", generator=gen, dtype=torch.int32)
+    kept = torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+    h.select(t, b, kept)
+    for g, rate in ((G, None), (G, lr), (None, None)):
+        want, got = torch.empty_like(X), torch.empty_like(X)
+        h.set_mix_panel(16)
+        h.mix(X, g, kept, b, 0.05, want, lr_per_worker=rate)
+        h.set_mix_panel(0)
+        h.mix(X, g, kept, b, 0.05, got, lr_per_worker=rate)
+        assert torch.equal(got, want)
+        Y = X.clone()
+        h.mix(Y, g, kept, b, 0.05, Y, lr_per_worker=rate)
+        assert torch.equal(Y, want)
+    assert h.status() == 0
+    h.close()
