@@ -304,7 +304,7 @@ inline int fp32_head_slices(const dbw_handle* h) {
 // the single launch, which sum in this order.  Forward GEMMs are not sliced: whether a pre-activation of zero up to rounding
 // passes its ReLU follows from the order of its sum, which stays ascending in k for every shape.
 int fp32_gemm_slice(int M, int N, int K, int batch, bool is_dw, int sm_count);
-// Whether an fp32 GEMM runs on the tensor cores, each operand value as three bf16 pieces (gemm_split.cuh): the same for both again.
+// Whether a backward fp32 GEMM runs on the tensor cores, each operand value as three bf16 pieces (gemm_split.cuh): the same for both again.
 bool fp32_gemm_split(int M, int N, int K, int batch, bool is_dw);
 int grad_fp32_alloc(dbw_handle* h);
 void grad_fp32_free(dbw_handle* h);

@@ -1,4 +1,5 @@
-// fp32 GEMM tiles of the gradient path on the tensor cores, at fp32 precision.  Every fp32 operand value is the exact sum of three
+// The backward fp32 GEMM tiles of the gradient path on the tensor cores, at fp32 precision.  (Forward sums stay in ascending k: whether a
+// pre-activation of zero up to rounding passes its ReLU follows from the order of its sum.)  Every fp32 operand value is the exact sum of three
 // bf16 pieces (each the rounded rest of the ones before), x = h + m + l, and a product is the sum of the piece products
 //   h h + (h m + m h) + (h l + m m + l h),
 // what is left out being below 2^-25 of the product.  Pieces are formed while an operand tile is staged in shared memory and the
@@ -225,13 +226,13 @@ __device__ __forceinline__ float sum_directly(const GemmArgs& g, int z, int m, i
     return t;
 }
 
-enum { FORWARD = 0, DW = 1, DA = 2 };
+enum { DW = 0, DA = 1 };
 __host__ __device__ constexpr int block_steps(int kind) { return kind == DW ? 1 : 2; }  // k steps whose h h are summed in tensor memory
 // Operand rows are 16-byte aligned and whole groups of four: VEC.
 template <int KIND>
 __host__ __device__ inline bool aligned(const GemmArgs& g) {
     auto ok = [](const float* p, long long z, long long pitch, int cols) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ((z | pitch | cols) & 3) == 0; };
-    return ok(g.A, g.sAz, KIND == DW ? g.sAk : g.sAm, KIND == DW ? g.M : g.K) && ok(g.B, g.sBz, KIND == FORWARD ? g.sBn : g.sBk, KIND == FORWARD ? g.K : g.N);
+    return ok(g.A, g.sAz, KIND == DW ? g.sAk : g.sAm, KIND == DW ? g.M : g.K) && ok(g.B, g.sBz, g.sBk, g.N);
 }
 
 // The MMAs of k step s of a tile by a converged warp; `tiles`, `half`: where its operands lie.  The pieces of the 64-row operand lie
@@ -242,17 +243,17 @@ __host__ __device__ inline bool aligned(const GemmArgs& g) {
 // which leaves the sums of h h in the first or the last 64 columns and those of the smaller products in the two between.
 template <int KIND>
 __device__ __forceinline__ void issue_step(uint32_t tmem, uint32_t tiles, int s, int half, uint64_t* done) {
-    constexpr bool AK = KIND != DW, BK = KIND == FORWARD;
+    constexpr bool AK = KIND != DW;
     constexpr int BS = block_steps(KIND);
     const bool odd = (s / BS) & 1;
     const uint32_t sn = tiles, sm = tiles + 3 * kPieceA;
-    const uint64_t dn0 = BK ? kmajor_sw128_desc(sn) : mnmajor_sw128_desc(sn, 8192), dm0 = AK ? kmajor_sw128_desc(sm) : mnmajor_sw128_desc(sm, kPieceB);
-    constexpr uint32_t i1 = idesc(kN, !BK, !AK), i2 = idesc(2 * kN, !BK, !AK), i3 = idesc(3 * kN, !BK, !AK);
+    const uint64_t dn0 = mnmajor_sw128_desc(sn, 8192), dm0 = AK ? kmajor_sw128_desc(sm) : mnmajor_sw128_desc(sm, kPieceB);
+    constexpr uint32_t i1 = idesc(kN, true, !AK), i2 = idesc(2 * kN, true, !AK), i3 = idesc(3 * kN, true, !AK);
     const uint32_t d_h = tmem + (odd ? kN : 0), d_m = tmem + kN, d_l = tmem + (odd ? kN : 2 * kN);
     const uint32_t m_at = (odd ? kPieceB : 0) >> 4, l_at = (odd ? 2 * kPieceB : 0) >> 4;
 #pragma unroll
     for (int j = 0; j < kStep / 16; ++j) {
-        const uint64_t dn = dn0 + ((BK ? half * 64 + j * 32 : (half * 32 + j * 16) * 128) >> 4), dm = dm0 + ((AK ? half * 64 + j * 32 : (half * 32 + j * 16) * 128) >> 4);
+        const uint64_t dn = dn0 + (((half * 32 + j * 16) * 128) >> 4), dm = dm0 + ((AK ? half * 64 + j * 32 : (half * 32 + j * 16) * 128) >> 4);
         if (j == 0 && (BS == 1 || half == 0)) {  // the block's sum of h h begins anew; those of the smaller products run on
             mma(odd ? tmem + 3 * kN : tmem, dn, dm + (odd ? 2 * kPieceB >> 4 : 0), i1, 0u);
             mma(tmem + kN, dn, dm + (odd ? 0 : kPieceB >> 4), i2, s > 0);
@@ -289,12 +290,11 @@ __device__ __forceinline__ void add_smaller(uint32_t taddr, float (&v)[COLS]) {
     }
 }
 
-// Stores outputs (m1 .. m1 + COLS - 1, n) of a thread: bias and ReLU (FORWARD), the mask (DA).
+// Stores outputs (m1 .. m1 + COLS - 1, n) of a thread: the mask (DA).
 template <int KIND, bool NC, int COLS>
 __device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, const float (&v)[COLS]) {
     if (n >= g.N) return;
     const int count = min(COLS, g.M - m1);
-    const float bias = KIND == FORWARD ? load_g<NC>(g.bias + (size_t)z * g.sBiasz + n) : 0.f;
     float* C = g.C + (size_t)z * g.sCz + (size_t)m1 * g.sCm + n;
     const float* mask = KIND == DA ? g.mask + (size_t)z * g.sMz + (size_t)m1 * g.sMm + n : nullptr;
     float none = 0.f;  // NaN as soon as one of the outputs is not finite
@@ -302,8 +302,7 @@ __device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, 
     for (int j = 0; j < COLS; ++j) {
         if (j < count) {
             none = fmaf(v[j], 0.f, none);
-            float x = v[j] + bias;
-            if (KIND == FORWARD && g.relu) x = fmaxf(x, 0.f);
+            float x = v[j];
             if (KIND == DA && !(load_g<NC>(mask) > 0.f)) x = 0.f;
             *C = x;
             C += g.sCm;
@@ -313,8 +312,7 @@ __device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, 
     if (none != 0.f) {
 #pragma unroll 1
         for (int j = 0; j < count; ++j) {
-            float x = sum_directly<NC>(g, z, m1 + j, n) + bias;
-            if (KIND == FORWARD && g.relu) x = fmaxf(x, 0.f);
+            float x = sum_directly<NC>(g, z, m1 + j, n);
             if (KIND == DA && !(load_g<NC>(g.mask + (size_t)z * g.sMz + (size_t)(m1 + j) * g.sMm + n) > 0.f)) x = 0.f;
             g.C[(size_t)z * g.sCz + (size_t)(m1 + j) * g.sCm + n] = x;
         }
@@ -355,15 +353,15 @@ __device__ __forceinline__ void for_steps(int steps, F step) {
     }
 }
 
-// Tile `tile` of the products C[z][m][n] = epilogue(sum_k A(m, k) B(k, n)) by the eight warps of a block.  FORWARD: both operands along k, bias
-// and ReLU; DW: both along the outputs, with the sums of A over k if wanted; DA: A along k, B along n, masked.  AHEAD: steps whose loads
+// Tile `tile` of the products C[z][m][n] = epilogue(sum_k A(m, k) B(k, n)) by the eight warps of a block.  DW: both operands along the
+// outputs, with the sums of A over k if wanted; DA: A along k, B along n, masked.  AHEAD: steps whose loads
 // are on their way.  `ready` (block_begin) is called with the first loads on their way.  MMA_WARP: a ninth warp issues the MMAs
 // (issue_tile).
 template <int KIND, bool VEC, bool NC, int RING, int AHEAD, bool MMA_WARP, class Ready>
 __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const Tiles& tiles, int tile, Ready ready) {
-    constexpr bool AK = KIND != DW, BK = KIND == FORWARD;
+    constexpr bool AK = KIND != DW;
     constexpr int BS = block_steps(KIND);
-    typedef Operand<kM, BK, VEC, NC> OpN;  // the operand with C's contiguous index
+    typedef Operand<kM, false, VEC, NC> OpN;  // the operand with C's contiguous index
     typedef Operand<kN, AK, VEC, NC> OpM;
     const int steps = (g.K + kStep - 1) / kStep, tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31, q = warp & 3, mh = warp >> 2;  // a warp finishes 32 outputs along n (its lanes of tensor memory) x 32 along m
@@ -371,7 +369,7 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
     tiles.at(tile, z, m0, n0);
     OpN on;
     OpM om;
-    on.begin(g.B + (size_t)z * g.sBz, BK ? g.sBn : g.sBk, n0, g.N, g.K);
+    on.begin(g.B + (size_t)z * g.sBz, g.sBk, n0, g.N, g.K);
     om.begin(g.A + (size_t)z * g.sAz, AK ? g.sAm : g.sAk, m0, g.M, g.K);
     typename OpN::Runs fn[AHEAD];
     typename OpM::Runs fm[AHEAD];

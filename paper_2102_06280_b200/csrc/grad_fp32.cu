@@ -547,8 +547,8 @@ enum GemmStep { GEMM_FORWARD, GEMM_DW, GEMM_DA };
 int run_gemm(dbw_handle* h, GemmArgs& g, GemmStep step, int batch, cudaStream_t s) {
     const int sm_count = h->sm_count;
     g.status = h->d_status;
-    if (fp32_gemm_split(g.M, g.N, g.K, batch, step == GEMM_DW))
-        return step == GEMM_FORWARD ? launch_split<split::FORWARD>(h, g, batch, s) : step == GEMM_DW ? launch_split<split::DW>(h, g, batch, s) : launch_split<split::DA>(h, g, batch, s);
+    if (step != GEMM_FORWARD && fp32_gemm_split(g.M, g.N, g.K, batch, step == GEMM_DW))
+        return step == GEMM_DW ? launch_split<split::DW>(h, g, batch, s) : launch_split<split::DA>(h, g, batch, s);
     g.slice = step == GEMM_FORWARD ? g.K : fp32_gemm_slice(g.M, g.N, g.K, batch, step == GEMM_DW, sm_count);
     if (gemm_vec_ok(g) && g.slice < g.K) {
         launch_gemm_slice(g, batch, s);
@@ -598,13 +598,12 @@ int run_gemm(dbw_handle* h, GemmArgs& g, GemmStep step, int batch, cudaStream_t 
 
 }  // namespace
 
-// Which GEMMs run on the tensor cores: those of many multiply-adds; fewer where operand rows are not whole 16-byte groups and the CUDA-core
-// kernel is the scalar one.  Measured on 900 GEMMs of 4 - 64 workers (us, CUDA cores / tensor cores): 10 workers, M x N x K =
-// 1024 x 256 x 256 42 / 22.6, 32, 64 x 200 x 784 30.6 / 20.7; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4, 36, 168 x 256 x
-// 45 (40 million) 8.3 / 10.4; unaligned 14, 124 x 52 x 578 (52 million) 16.5 / 20.6 and 37, 57 x 157 x 128 (42 million) 12.4 / 8.9.  What it
-// costs is a launch's chain: operands to bf16 pieces, MMAs and a barrier between them for every 32 k, about 0.5 us whatever the
-// size; a k of one such step does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5), nor does a long one of few multiply-adds (5, 49 x
-// 240 x 563, 33 million: a gradient call 48 / 52).
+// Which backward GEMMs run on the tensor cores: those of many multiply-adds; fewer where operand rows are not whole 16-byte groups and
+// the CUDA-core kernel is the scalar one.  Measured on 900 GEMMs of 4 - 64 workers (us, CUDA cores / tensor cores): 10 workers, M x
+// N x K = 1024 x 256 x 256 42 / 23.5, 32, 200 x 784 x 64 26.6 / 19.6; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4 and 12, 32 x
+// 256 x 307 (30 million) 10.4 / 13.9; unaligned 7, 58 x 276 x 457 (51 million) 12.4 / 16.5.  What it costs is a launch's chain:
+// operands to bf16 pieces, MMAs and a barrier between them for every 32 k, about 0.5 us whatever the size; a k of one such step
+// does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5), nor does a long one of few multiply-adds.
 bool fp32_gemm_split(int M, int N, int K, int batch, bool is_dw) {
     const bool rows_aligned = N % 4 == 0 && (is_dw ? M : K) % 4 == 0;
     return (long long)M * N * K * batch >= (rows_aligned || K > 512 ? 60000000 : 30000000) && (K > split::kStep || !rows_aligned);

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
         g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in; g.status = a.status;
-        gemm_any<split::FORWARD, GENERAL>(a.fwd_var[l], g, N, smem, blk);
+        gemm_any<split::DA, false>(a.fwd_var[l], g, N, smem, blk);
         grid.sync();
     }
 
@@ -405,15 +405,16 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     widest = std::max<long long>(widest, (long long)N * (((m.dims[m.n_layers - 1] + 3) / 4 + head_chunk4(a.head_slices) - 1) / head_chunk4(a.head_slices)));
     const int grid = (int)std::min<long long>(h->fused->max_blocks, std::max<long long>(widest + 1, 2));
     for (int l = 0; l < m.n_layers; ++l) {
-        auto variant = [&](int M, int Nn, int K, bool is_dw) {
+        enum { FORWARD, DW, DA };
+        auto variant = [&](int M, int Nn, int K, int kind) {
             if (l >= (a.head ? m.n_layers - 1 : m.n_layers)) return 0;  // not a GEMM
-            const bool on_tensor_cores = fp32_gemm_split(M, Nn, K, N, is_dw);
+            const bool on_tensor_cores = kind != FORWARD && fp32_gemm_split(M, Nn, K, N, kind == DW);
             a.any_split |= on_tensor_cores;
             return on_tensor_cores ? (int)V_SPLIT : pick_variant(M, Nn, K, N, grid);
         };
-        a.fwd_var[l] = (signed char)variant(B, m.dims[l + 1], m.dims[l], false);
-        a.dw_var[l] = (signed char)variant(m.dims[l + 1], m.dims[l], B, true);
-        a.da_var[l] = (signed char)variant(B, m.dims[l], m.dims[l + 1], false);
+        a.fwd_var[l] = (signed char)variant(B, m.dims[l + 1], m.dims[l], FORWARD);
+        a.dw_var[l] = (signed char)variant(m.dims[l + 1], m.dims[l], B, DW);
+        a.da_var[l] = (signed char)variant(B, m.dims[l], m.dims[l + 1], DA);
     }
     for (int l = 0; l < m.n_layers; ++l) {
         a.dw_slice[l] = fp32_gemm_slice(m.dims[l + 1], m.dims[l], B, N, true, h->sm_count);
