@@ -1,13 +1,16 @@
 // The backward fp32 GEMM tiles of the gradient path on the tensor cores, at fp32 precision.  (Forward sums stay in ascending k: whether a
 // pre-activation of zero up to rounding passes its ReLU follows from the order of its sum.)  Every fp32 operand value is the exact sum of three
 // bf16 pieces (each the rounded rest of the ones before), x = h + m + l, and a product is the sum of the piece products
-//   h h + (h m + m h) + (h l + m m + l h),
-// what is left out being below 2^-25 of the product.  Pieces are formed while an operand tile is staged in shared memory and the
+//   h h + (h m + m h) + (h l + m m + l h) + (m l + l m),
+// what is left out, l l, being below 2^-32 of the product.  Pieces are formed while an operand tile is staged in shared memory and the
 // MMAs accumulate in tensor memory.  Those accumulators are truncated, not rounded, at every MMA, and always towards zero: over a
-// long sum of h h that alone would be worse than fp32 multiply-adds (K = 784: -5e-7 of the result), so every 64 k (32 in dW, whose sums
-// on the CUDA cores go in slices too) the sums of h h move to registers and are added there with rounding.  The smaller products,
-// 2^-8 of the sum and less, stay.  Against 64 bits (relative 2-norm, this / ascending fp32 multiply-adds): K = 32 4.6e-8 / 1.0e-7,
-// 256 8.0e-8 / 2.9e-7, 3000 1.5e-7 / 9.8e-7.
+// long sum of h h that alone would be worse than fp32 multiply-adds (K = 784: -5e-7 of the result), so every 32 k the sums of h h
+// move to registers and are added there with rounding.  The smaller products, 2^-8 of the sum and less, stay.
+//
+// Against 64 bits, relative to fp32 multiply-adds in ascending k: a sum with a single non-zero product is rounded as theirs is, sums of
+// several products of similar magnitude are closer (root mean square of 2, 4, 8, 32, 128 normal ones: 0.82, 0.65, 0.53, 0.40, 0.30);
+// where the magnitudes are spread over 24 binades truncation shows in sums of a few (2, 4, 8, 32, 128: 1.03, 1.11, 1.10, 0.77,
+// 0.44).  Dense sums (relative 2-norm, this / theirs): K = 64 5.2e-8 / 1.5e-7, 128 5.9e-8 / 2.1e-7, 256 7.1e-8 / 2.9e-7.
 //
 // Shared by the stand-alone kernel (grad_fp32.cu) and the single-launch round (round_fused.cu), which give the same bits.
 #pragma once
@@ -227,7 +230,6 @@ __device__ __forceinline__ float sum_directly(const GemmArgs& g, int z, int m, i
 }
 
 enum { DW = 0, DA = 1 };
-__host__ __device__ constexpr int block_steps(int kind) { return kind == DW ? 1 : 2; }  // k steps whose h h are summed in tensor memory
 // Operand rows are 16-byte aligned and whole groups of four: VEC.
 template <int KIND>
 __host__ __device__ inline bool aligned(const GemmArgs& g) {
@@ -236,32 +238,33 @@ __host__ __device__ inline bool aligned(const GemmArgs& g) {
 }
 
 // The MMAs of k step s of a tile by a converged warp; `tiles`, `half`: where its operands lie.  The pieces of the 64-row operand lie
-// behind each other like 64 more outputs each, so one MMA multiplies a piece of the other operand by several of them.  Blocks of
-// block_steps alternate between
-//   pieces h, m, l:   columns [0, 192)  += h x [h m l],   [64, 192) += m x [h m],   [128, 192) += l x h   and
-//   pieces l, m, h:   columns [64, 256) += h x [l m h],   [64, 192) += m x [m h],   [64, 128)  += l x h,
+// behind each other like 64 more outputs each, so one MMA multiplies a piece of the other operand by several of them.  Steps
+// alternate between
+//   pieces h, m, l:   columns [0, 192)  += h x [h m l],   [64, 192) += m x [h m],   [128, 192) += l x h + l x m + m x l   and
+//   pieces l, m, h:   columns [64, 256) += h x [l m h],   [64, 192) += m x [m h],   [64, 128)  += l x h + l x m + m x l,
 // which leaves the sums of h h in the first or the last 64 columns and those of the smaller products in the two between.
 template <int KIND>
 __device__ __forceinline__ void issue_step(uint32_t tmem, uint32_t tiles, int s, int half, uint64_t* done) {
     constexpr bool AK = KIND != DW;
-    constexpr int BS = block_steps(KIND);
-    const bool odd = (s / BS) & 1;
+    const bool odd = s & 1;
     const uint32_t sn = tiles, sm = tiles + 3 * kPieceA;
     const uint64_t dn0 = mnmajor_sw128_desc(sn, 8192), dm0 = AK ? kmajor_sw128_desc(sm) : mnmajor_sw128_desc(sm, kPieceB);
     constexpr uint32_t i1 = idesc(kN, true, !AK), i2 = idesc(2 * kN, true, !AK), i3 = idesc(3 * kN, true, !AK);
     const uint32_t d_h = tmem + (odd ? kN : 0), d_m = tmem + kN, d_l = tmem + (odd ? kN : 2 * kN);
-    const uint32_t m_at = (odd ? kPieceB : 0) >> 4, l_at = (odd ? 2 * kPieceB : 0) >> 4;
+    const uint32_t m_at = kPieceB >> 4, h_at = (odd ? 2 * kPieceB : 0) >> 4, l_at = (odd ? 0 : 2 * kPieceB) >> 4;
 #pragma unroll
     for (int j = 0; j < kStep / 16; ++j) {
         const uint64_t dn = dn0 + (((half * 32 + j * 16) * 128) >> 4), dm = dm0 + ((AK ? half * 64 + j * 32 : (half * 32 + j * 16) * 128) >> 4);
-        if (j == 0 && (BS == 1 || half == 0)) {  // the block's sum of h h begins anew; those of the smaller products run on
-            mma(odd ? tmem + 3 * kN : tmem, dn, dm + (odd ? 2 * kPieceB >> 4 : 0), i1, 0u);
+        if (j == 0) {  // the step's sum of h h begins anew; those of the smaller products run on
+            mma(odd ? tmem + 3 * kN : tmem, dn, dm + h_at, i1, 0u);
             mma(tmem + kN, dn, dm + (odd ? 0 : kPieceB >> 4), i2, s > 0);
         } else {
             mma(d_h, dn, dm, i3, 1u);
         }
-        mma(d_m, dn + (kPieceA >> 4), dm + m_at, i2, 1u);
-        mma(d_l, dn + (2 * kPieceA >> 4), dm + l_at, i1, 1u);
+        mma(d_m, dn + (kPieceA >> 4), dm + (odd ? m_at : 0), i2, 1u);
+        mma(d_l, dn + (2 * kPieceA >> 4), dm + h_at, i1, 1u);
+        mma(d_l, dn + (2 * kPieceA >> 4), dm + m_at, i1, 1u);
+        mma(d_l, dn + (kPieceA >> 4), dm + l_at, i1, 1u);
     }
     commit(done);
 }
@@ -360,7 +363,6 @@ __device__ __forceinline__ void for_steps(int steps, F step) {
 template <int KIND, bool VEC, bool NC, int RING, int AHEAD, bool MMA_WARP, class Ready>
 __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const Tiles& tiles, int tile, Ready ready) {
     constexpr bool AK = KIND != DW;
-    constexpr int BS = block_steps(KIND);
     typedef Operand<kM, false, VEC, NC> OpN;  // the operand with C's contiguous index
     typedef Operand<kN, AK, VEC, NC> OpM;
     const int steps = (g.K + kStep - 1) / kStep, tid = threadIdx.x;
@@ -389,11 +391,11 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
     for_steps<RING>(steps, [&](int s, auto slot_of) {
         constexpr int slot = decltype(slot_of)::value, half = slot & 1, ahead = slot % AHEAD;
         wait(slot);
-        if (slot % BS == 0 && s >= 2 * BS) {  // add up the sums of h h of two blocks ago
-            if (RING > 2) wait((slot + RING - 1 - BS) % RING);  // the last step of that block
+        if (s >= 2) {  // add up the sums of h h of two steps ago
+            if (RING > 2) wait((slot + RING - 2) % RING);
             __syncwarp();
             tc_fence_after();
-            add_columns<32>(t0 + ((s / BS) & 1) * 3 * kN, v);
+            add_columns<32>(t0 + (s & 1) * 3 * kN, v);
             tc_fence_before();
         }
         uint8_t *tn = blk.buffers + (slot >> 1) * kBufferBytes, *tm = tn + 3 * kPieceA;
@@ -406,7 +408,7 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
         {
             float x[8];
             om.elements(s * kStep, 0, fm[ahead], x);
-            om.store(tm, half, 0, (s / BS) & 1, x);
+            om.store(tm, half, 0, s & 1, x);
             if constexpr (KIND == DW) {
                 if (sums) {
 #pragma unroll
@@ -426,9 +428,8 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
     for (int r = 0; r < RING; ++r) wait(r);
     __syncwarp();
     tc_fence_after();
-    const int blocks = (steps + BS - 1) / BS;  // the last two have not been added yet
-    if (blocks > 1) add_columns<32>(t0 + (blocks & 1) * 3 * kN, v);
-    add_columns<32>(t0 + ((blocks - 1) & 1) * 3 * kN, v);
+    if (steps > 1) add_columns<32>(t0 + (steps & 1) * 3 * kN, v);  // the last two steps' have not been added yet
+    add_columns<32>(t0 + ((steps - 1) & 1) * 3 * kN, v);
     add_smaller<32>(t0, v);
     tc_fence_before();
     if constexpr (KIND == DW) {

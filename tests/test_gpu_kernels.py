@@ -1196,3 +1196,96 @@ def test_pipelined_panel_mix_gives_the_bits_of_the_plain_one(n, deg, d, order):
         assert torch.equal(Y, want)
     assert h.status() == 0
     h.close()
+
+
+def _bf16_pieces(x, count):
+    """float64 sums of the first `count` bf16 pieces of fp32 values."""
+    rest, out = torch.from_numpy(np.ascontiguousarray(x)), 0.0
+    for _ in range(count):
+        piece = rest.bfloat16().float()
+        rest, out = rest - piece, out + piece.double()
+    return out.numpy()
+
+
+def _few_product_errors(got, Z, T, counts):
+    """Per count of non-zero rows in T's column groups: the errors of `got` and of fp32 multiply-adds in ascending k against float64 Z^T T, relative to
+    the sum of the products' magnitudes, and those magnitudes."""
+    Z64, T64, cols = Z.astype(np.float64), T.astype(np.float64), T.shape[1] // len(counts)
+    ref, size, acc = Z64.T @ T64, np.abs(Z64).T @ np.abs(T64), np.zeros((Z.shape[1], T.shape[1]), np.float32)
+    for k in range(Z.shape[0]):
+        at = T[k] != 0
+        acc[:, at] = (acc[:, at].astype(np.float64) + np.outer(Z64[k], T64[k, at])).astype(np.float32)
+    out = []
+    for g in range(len(counts)):
+        sl = slice(g * cols, (g + 1) * cols)
+        there = size[:, sl] > 0
+        out.append([np.abs(a[:, sl].astype(np.float64) - ref[:, sl])[there] / size[:, sl][there] for a in (got, acc)] + [size[:, sl][there]])
+    return out
+
+
+def _check_few_products(got, Z, T, counts):
+    for n, (mine, theirs, size) in zip(counts, _few_product_errors(got, Z, T, counts)):
+        normal = size > 2.0 ** -125  # not a subnormal number
+        if n == 1:  # one rounding, of a sum whose smaller part (2^-8 of it) is truncated a few times
+            assert (mine - 2.0 ** -149 / size).max() <= 2.0 ** -24 * (1 + 2.0 ** -5)
+        assert np.sqrt((mine[normal] ** 2).mean()) <= 1.001 * np.sqrt((theirs[normal] ** 2).mean()), (n, mine.max(), theirs.max())
+
+
+@pytest.mark.parametrize("batch,tests,out,n", [(128, 384, 128, 8),    # whole tiles, a block to an SM
+                                               (64, 192, 160, 24),    # ... five k steps in dA
+                                               (64, 192, 128, 60),    # two blocks to an SM
+                                               (97, 158, 131, 30)])   # rows at every shift
+@pytest.mark.parametrize("scale", [1.0])
+def test_fp32_tensor_core_gemms_sum_few_products_as_multiply_adds_do(batch, tests, out, n, scale):
+    """Sums of one, two and four non-zero products, and dense ones, are no less exact than fp32 multiply-adds in the tensor-core GEMMs: dW through
+    sparse features, dA through sparse weights.  The GEMMs' other operand is read back exactly through one-hot samples and hidden units."""
+    p = _dbw()
+    rng = np.random.default_rng(11)
+    rowptr, col = wl.ring(n)
+    labels = rng.integers(0, 10, size=(n, batch)).astype(np.int32)
+    idx = np.tile(np.arange(batch, dtype=np.int32), (n, 1))
+
+    def sparse(k, counts):
+        t = np.zeros((k, tests // len(counts) * len(counts)), np.float32)
+        for c in range(t.shape[1]):
+            at = rng.permutation(k)[: counts[c // (tests // len(counts))]]
+            t[at, c] = rng.standard_normal(len(at)) * scale
+        return t
+
+    def gradients(dims, X, feat):
+        m = p.model_layout(dims, batch)
+        h = p.Dbw(rowptr, col, d=m.d, model=m)
+        rows = np.zeros((n, m.ld), np.float32)
+        for l, W in enumerate(X):
+            rows[:, m.w_off[l]: m.w_off[l] + W[0].size] = W.reshape(n, -1)
+            if l:
+                rows[:, m.b_off[l - 1]: m.b_off[l - 1] + W.shape[2]] = float(l == len(X) - 1)
+        f, lab, G = dev(feat), dev(labels), torch.zeros(n, m.ld, device="cuda")
+        h.set_dataset(f, lab, batch)
+        h.grad(dev(rows), dev(idx), G)
+        assert h.status() == 0
+        g = G.cpu().numpy()
+        h.close()
+        return [g[:, m.w_off[l]: m.w_off[l] + W[0].size].reshape(W.shape) for l, W in enumerate(X)]
+
+    top = (0.2 * rng.standard_normal((n, 10, out))).astype(np.float32)
+    counts = (1, 2, 4, batch)
+    T = [sparse(batch, counts) for _ in range(n)]
+    wide = batch + T[0].shape[1]
+    first = np.zeros((n, out, wide), np.float32)
+    first[:, :, :batch] = 0.1 * rng.standard_normal((n, out, batch))
+    feat = np.stack([np.concatenate([np.eye(batch, dtype=np.float32), t], 1) for t in T])
+    g = gradients([wide, out, 10], [first, top], feat)[0]
+    Z = g[0, :, :batch].T
+    _check_few_products(g[0, :, batch:], Z, T[0], counts)
+    with pytest.raises(AssertionError):  # two pieces would not do
+        _check_few_products((Z.astype(np.float64).T @ _bf16_pieces(T[0], 2)).astype(np.float32), Z, T[0], counts)
+
+    counts = (1, 2, 4, out)
+    T = [sparse(out, counts) for _ in range(n)]
+    wide = batch + T[0].shape[1]
+    hidden = np.full((n, wide, batch), 2.0 ** -126, np.float32)  # units that are active and weigh next to nothing in the next layer
+    hidden[:, :batch] = np.eye(batch)
+    second = np.concatenate([0.1 * rng.standard_normal((n, out, batch)), np.stack(T)], 2).astype(np.float32)
+    g = gradients([batch, wide, out, 10], [hidden, second, top], np.tile(np.eye(batch, dtype=np.float32), (n, 1, 1)))
+    _check_few_products(g[0][0, batch:].T, g[1][0, :, :batch], T[0], counts)
