@@ -37,6 +37,10 @@ constexpr int kTmemCols = 4 * kN;                      // two sums of h h, used 
 constexpr int kBufferBytes = 3 * (kPieceA + kPieceB);  // three pieces of the 128-row operand, then of the 64-row operand
 __host__ __device__ constexpr size_t smem_bytes(int ring) { return (size_t)(ring / 2) * kBufferBytes + 1024 /*align slack*/; }
 constexpr uint32_t kWaitLimit = 1u << 24;
+// Pieces are formed of 2^24 times the value.  A bf16 number has the exponents of a float, so the last piece of a value below 2^-110 would
+// be less than the smallest of them; scaled, the pieces of every float, subnormal ones included, are normal numbers.  Values and sums
+// beyond the other end (2^104 and 2^80) come out infinite or NaN and are summed again (finish).
+constexpr float kScale = 16777216.f, kUnscale = 1.f / kScale / kScale;
 
 // Barriers and tensor memory of a block, set up once and used for any number of tiles.
 struct Block {
@@ -118,8 +122,10 @@ __device__ __forceinline__ void ld16(uint32_t taddr, float (&v)[16]) {
     tc_ld_wait();
 }
 
-// Two neighbouring elements: their bf16 pieces, packed.
+// Two neighbouring elements: the bf16 pieces of kScale times them, packed.
 __device__ __forceinline__ void split2(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+    x *= kScale;
+    y *= kScale;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(y), "f"(x));
     x -= __uint_as_float(h << 16);
     y -= __uint_as_float(h & 0xffff0000u);
@@ -305,7 +311,7 @@ __device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, 
     for (int j = 0; j < COLS; ++j) {
         if (j < count) {
             none = fmaf(v[j], 0.f, none);
-            float x = v[j];
+            float x = v[j] * kUnscale;
             if (KIND == DA && !(load_g<NC>(mask) > 0.f)) x = 0.f;
             *C = x;
             C += g.sCm;

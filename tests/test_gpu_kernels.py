@@ -1235,7 +1235,7 @@ def _check_few_products(got, Z, T, counts):
                                                (64, 192, 160, 24),    # ... five k steps in dA
                                                (64, 192, 128, 60),    # two blocks to an SM
                                                (97, 158, 131, 30)])   # rows at every shift
-@pytest.mark.parametrize("scale", [1.0])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -112, 2.0 ** 118])  # ... whose last pieces are below the smallest bf16 number; whose sums overflow when scaled
 def test_fp32_tensor_core_gemms_sum_few_products_as_multiply_adds_do(batch, tests, out, n, scale):
     """Sums of one, two and four non-zero products, and dense ones, are no less exact than fp32 multiply-adds in the tensor-core GEMMs: dW through
     sparse features, dA through sparse weights.  The GEMMs' other operand is read back exactly through one-hot samples and hidden units."""
