@@ -223,18 +223,6 @@ struct Operand {
     }
 };
 
-// An output whose pieces do not add up to a finite number: an operand or the result is infinite or NaN (an infinite operand has no
-// finite rest).  Summed again as the CUDA-core kernels do.
-template <bool NC>
-__device__ __forceinline__ float sum_directly(const GemmArgs& g, int z, int m, int n) {
-    const float* a = g.A + (size_t)z * g.sAz + (size_t)m * g.sAm;
-    const float* b = g.B + (size_t)z * g.sBz + (size_t)n * g.sBn;
-    float t = 0.f;
-#pragma unroll 1
-    for (int k = 0; k < g.K; ++k) t = fmaf(load_g<NC>(a + (size_t)k * g.sAk), load_g<NC>(b + (size_t)k * g.sBk), t);
-    return t;
-}
-
 enum { DW = 0, DA = 1 };
 // Operand rows are 16-byte aligned and whole groups of four: VEC.
 template <int KIND>
@@ -299,10 +287,10 @@ __device__ __forceinline__ void add_smaller(uint32_t taddr, float (&v)[COLS]) {
     }
 }
 
-// Stores outputs (m1 .. m1 + COLS - 1, n) of a thread: the mask (DA).
+// Stores outputs (m1 .. m1 + COLS - 1, n) of a thread: the mask (DA).  Returns whether they are finite.
 template <int KIND, bool NC, int COLS>
-__device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, const float (&v)[COLS]) {
-    if (n >= g.N) return;
+__device__ __forceinline__ bool finish(const GemmArgs& g, int z, int m1, int n, const float (&v)[COLS]) {
+    if (n >= g.N) return true;
     const int count = min(COLS, g.M - m1);
     float* C = g.C + (size_t)z * g.sCz + (size_t)m1 * g.sCm + n;
     const float* mask = KIND == DA ? g.mask + (size_t)z * g.sMz + (size_t)m1 * g.sMm + n : nullptr;
@@ -318,14 +306,20 @@ __device__ __forceinline__ void finish(const GemmArgs& g, int z, int m1, int n, 
             if (KIND == DA) mask += g.sMm;
         }
     }
-    if (none != 0.f) {
-#pragma unroll 1
-        for (int j = 0; j < count; ++j) {
-            float x = sum_directly<NC>(g, z, m1 + j, n);
-            if (KIND == DA && !(load_g<NC>(g.mask + (size_t)z * g.sMz + (size_t)(m1 + j) * g.sMm + n) > 0.f)) x = 0.f;
-            g.C[(size_t)z * g.sCz + (size_t)(m1 + j) * g.sCm + n] = x;
-        }
-    }
+    return none == 0.f;
+}
+// Whether `p` holds in any of the eight filling warps; what they have stored is visible to all of them afterwards.
+__device__ __forceinline__ bool any_of_fill(bool p) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)p), "n"(kFillThreads)
+        : "memory");
+    return any != 0;
 }
 
 struct Tiles {
@@ -360,6 +354,17 @@ __device__ __forceinline__ void for_steps(int steps, F step) {
             if (s + 3 < steps) step(s + 3, std::integral_constant<int, 3>{});
         }
     }
+}
+
+// A tile with an output that is not finite: an operand or the result is infinite or NaN, or so large that the scaled one is.  Its
+// outputs are summed again as the CUDA-core kernels do, by the eight filling warps with the buffer (which no MMA reads any more) as
+// staging.
+template <bool NC>
+__device__ __forceinline__ void sum_on_cuda_cores(const GemmArgs& g, int z, int m0, int n0, float* smem) {
+    float(*As)[68] = reinterpret_cast<float(*)[68]>(smem);
+    float(*Bs)[68] = reinterpret_cast<float(*)[68]>(smem + 16 * 68);
+#pragma unroll 1
+    for (int n1 = n0; n1 < min(n0 + kM, g.N); n1 += 64) dev::gemm_tile<4, 16, NC, false, kFillThreads>(g, z, m0, n1, As, Bs);
 }
 
 // Tile `tile` of the products C[z][m][n] = epilogue(sum_k A(m, k) B(k, n)) by the eight warps of a block.  DW: both operands along the
@@ -455,7 +460,9 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
             asm volatile("bar.sync 1, %0;" ::"n"(kFillThreads) : "memory");  // before the next tile is filled
         }
     }
-    finish<KIND, NC, 32>(g, z, m0 + 32 * mh, n0 + 32 * q + lane, v);
+    const bool finite = finish<KIND, NC, 32>(g, z, m0 + 32 * mh, n0 + 32 * q + lane, v);
+    __syncwarp();
+    if (any_of_fill(!finite)) sum_on_cuda_cores<NC>(g, z, m0, n0, reinterpret_cast<float*>(blk.buffers));
 }
 
 // The ninth warp's part of a tile.

@@ -76,8 +76,15 @@ __device__ __forceinline__ T load_g(const T* p) {
     else return *p;
 }
 
-// SLICED: g.slice may be less than K.
-template <int R, int TK, bool NC = true, bool SLICED = false>
+// A barrier of all threads of the block, or (THREADS > 0) of the first so many, which are the ones that share its work.
+template <int THREADS>
+__device__ __forceinline__ void block_barrier() {
+    if constexpr (THREADS == 0) __syncthreads();
+    else asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory");
+}
+
+// SLICED: g.slice may be less than K.  THREADS: of block_barrier.
+template <int R, int TK, bool NC = true, bool SLICED = false, int THREADS = 0>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int n0, float (*As)[16 * R + 4], float (*Bs)[16 * R + 4]) {
     constexpr int T = 16 * R;        // tile edge
     constexpr int PER = T * TK / 256;  // elements of each operand tile a thread stages
@@ -110,7 +117,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
             As[a_k_fast ? (e % TK) : (e / T)][a_k_fast ? (e / TK) : (e % T)] = pa[r];
             Bs[b_k_fast ? (e % TK) : (e / T)][b_k_fast ? (e / TK) : (e % T)] = pb[r];
         }
-        __syncthreads();
+        block_barrier<THREADS>();
         fetch(next);  // all zero past the end
 #pragma unroll
         for (int kk = 0; kk < TK; ++kk) {
@@ -131,7 +138,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int z, int m0, int 
 #pragma unroll
                 for (int j = 0; j < R; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
         }
-        __syncthreads();
+        block_barrier<THREADS>();
     };
     if constexpr (!SLICED) {
         for (int k0 = 0; k0 < g.K; k0 += TK) step(k0 + TK);

@@ -1289,3 +1289,72 @@ def test_fp32_tensor_core_gemms_sum_few_products_as_multiply_adds_do(batch, test
     second = np.concatenate([0.1 * rng.standard_normal((n, out, batch)), np.stack(T)], 2).astype(np.float32)
     g = gradients([batch, wide, out, 10], [hidden, second, top], np.tile(np.eye(batch, dtype=np.float32), (n, 1, 1)))
     _check_few_products(g[0][0, batch:].T, g[1][0, :, :batch], T[0], counts)
+
+
+def test_fp32_tensor_core_gemms_with_outputs_that_are_not_finite():
+    """A NaN, an infinity and values that overflow make the outputs they reach what multiply-adds make of them, leave the others alone, and do not
+    take many times as long (a network that has diverged)."""
+    p = _dbw()
+    n, batch, dims = 12, 128, [300, 256, 200, 10]
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    rng = np.random.default_rng(21)
+    h = p.Dbw(rowptr, col, d=m.d, model=m)
+    feat, labels = rng.random((n, batch, dims[0]), dtype=np.float32) + 0.1, rng.integers(0, 10, size=(n, batch)).astype(np.int32)
+    X = m.pack((0.05 * rng.standard_normal((n, m.d))).astype(np.float32))
+    for l in range(2):  # every unit active
+        X[:, m.b_off[l]: m.b_off[l] + dims[l + 1]] = 9.0
+    idx = np.tile(np.arange(batch, dtype=np.int32), (n, 1))
+
+    def gradients(feat, X):
+        f, lab, G, loss = dev(feat), dev(labels), torch.zeros(n, m.ld, device="cuda"), torch.zeros(n, device="cuda")
+        h.set_dataset(f, lab, batch)
+        x, ix = dev(X), dev(idx)
+        h.grad(x, ix, G, loss)
+        best = 1e9
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(5):
+                h.grad(x, ix, G, loss)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        g = G.cpu().numpy()
+        return [g[:, m.w_off[l]: m.w_off[l] + dims[l] * dims[l + 1]].reshape(n, dims[l + 1], dims[l]) for l in range(3)], best
+
+    plain, usual = gradients(feat, X)
+    # a feature of one sample: the column of dW that it is multiplied into (its weights are zero, so nothing else is reached)
+    X0, bad = X.copy(), feat.copy()
+    X0[:, m.w_off[0]: m.w_off[0] + dims[0] * dims[1]].reshape(n, dims[1], dims[0])[:, :, 7] = 0.0
+    want, _ = gradients(feat, X0)
+    for value in (3e38, -1e35):  # above the largest bf16; scaled, infinite
+        bad[2, 5, 7] = value
+        got, _ = gradients(bad, X0)
+        z = got[0][2, :, 7].astype(np.float64)
+        ref = want[0][2, :, 7].astype(np.float64)
+        assert np.isfinite(z).all() and np.abs(z - ref).max() > 1e30
+        assert np.array_equal(got[0][[i for i in range(n) if i != 2]], want[0][[i for i in range(n) if i != 2]])
+        others = np.arange(dims[0]) != 7
+        assert np.abs(got[0][2][:, others] - want[0][2][:, others]).max() <= 1e-6 * np.abs(want[0][2]).max()
+        dz = z / value  # dZ of that sample, up to the rounding of one product and the other samples' share
+        bad[2, 5, 7] = value / 4
+        again, _ = gradients(bad, X0)
+        assert np.abs(again[0][2, :, 7] / (value / 4) - dz).max() <= 2.0 ** -22 * np.abs(dz).max()
+    # a weight of the second layer, in dA (times every dZ) and, through NaN logits, in every dZ
+    for value in (np.nan, np.inf):
+        X1 = X.copy()
+        X1[3, m.w_off[1] + 4] = value
+        got, _ = gradients(feat, X1)
+        if np.isinf(value):
+            assert not np.isfinite(got[0][3]).any()
+        else:  # a NaN is no activation, so it is in that one unit's dZ alone
+            assert np.isnan(got[0][3][4]).all() and np.isfinite(np.delete(got[0][3], 4, 0)).all()
+        assert all(np.array_equal(got[l][i], plain[l][i]) for l in range(3) for i in range(n) if i != 3)
+    X1 = X.copy()
+    X1[:, m.w_off[2]] = np.nan
+    got, time = gradients(feat, X1)
+    assert all(np.isnan(g[g0 != 0]).all() for g, g0 in zip(got, plain))
+    assert time <= 4 * usual, (time, usual)
+    assert h.status() == 0
+    h.close()
