@@ -420,14 +420,15 @@ __device__ __forceinline__ void head_forward_samples(int i, int s, int B, int in
         }
     }
     // the sums over the lanes; with U = 4 a lane keeps the samples 2 (lane / 16) .. of a pair first, then sample lane / 8
-    float z[CP];
+    float mx = -INFINITY;
+    float(&z)[CP] = acc[0];  // in their place
     int y = label[0];
     if (U == 4) y = lane & 16 ? (lane & 8 ? label[U - 1] : label[U / 2]) : (lane & 8 ? label[U > 1] : label[0]);
 #pragma unroll
     for (int c = 0; c < CP; ++c) {
         if (c < C) {
             if (U == 1) {
-                z[c] = warp_sum(acc[0][c]);
+                z[c] = warp_sum(z[c]);
             } else {
                 auto halve = [](bool upper, float lo, float hi, int o) { return (upper ? hi : lo) + __shfl_xor_sync(0xffffffffu, upper ? lo : hi, o); };
                 const float lo = halve(lane & 16, acc[0][c], acc[U / 2][c], 16), hi = halve(lane & 16, acc[U > 1][c], acc[U - 1][c], 16);
@@ -436,12 +437,9 @@ __device__ __forceinline__ void head_forward_samples(int i, int s, int B, int in
                 for (int o = 4; o > 0; o >>= 1) z[c] += __shfl_xor_sync(0xffffffffu, z[c], o);
             }
             z[c] += load_g<NC>(bias + c);
+            mx = fmaxf(mx, z[c]);
         }
     }
-    float mx = -INFINITY;
-#pragma unroll
-    for (int c = 0; c < CP; ++c)
-        if (c < C) mx = fmaxf(mx, z[c]);
     float sum = 0.f, zy = 0.f;
 #pragma unroll
     for (int c = 0; c < CP; ++c) {

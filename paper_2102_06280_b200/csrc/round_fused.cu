@@ -154,19 +154,21 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         rows.feat = a.feat; rows.labels = a.labels; rows.batch_idx = a.batch_idx; rows.S = a.S;
     }
     float* loss_s = a.act[L];
-    auto head_variant = [&](auto f) {  // by the number of classes, and whether rows are aligned
-        if (a.C <= 16) !GENERAL || a.head_aligned ? f(std::integral_constant<int, 16>{}, std::true_type{}) : f(std::integral_constant<int, 16>{}, std::bool_constant<!GENERAL>{});
-        else !GENERAL || a.head_aligned ? f(std::integral_constant<int, 32>{}, std::true_type{}) : f(std::integral_constant<int, 32>{}, std::bool_constant<!GENERAL>{});
-    };
     auto head_forward = [&](int first, int step) {
         for (int item = first * (kThreads / 32) + warp; item < N * B; item += step * (kThreads / 32)) {
             const int i = item / B;
             const float* Xi = a.X + (size_t)i * a.ld;
-            auto sample = [&](auto cp, auto vec) {
-                head_forward_samples<decltype(cp)::value, 1, decltype(vec)::value, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1],
-                                                                                        Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
-            };
-            head_variant(sample);
+            if (!GENERAL || a.head_aligned) {
+                if (a.C <= 16)
+                    head_forward_samples<16, 1, true, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+                else
+                    head_forward_samples<32, 1, true, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+            } else {
+                if (a.C <= 16)
+                    head_forward_samples<16, 1, !GENERAL, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+                else
+                    head_forward_samples<32, 1, !GENERAL, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+            }
         }
     };
 
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.B = a.X + a.w_off[l]; g.sBz = a.ld; g.sBn = in; g.sBk = 1;
         g.C = a.act[l + 1]; g.sCz = (long long)B * out; g.sCm = out;
         g.bias = a.X + a.b_off[l]; g.sBiasz = a.ld;
-        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in; g.status = a.status;
+        g.M = B; g.N = out; g.K = in; g.relu = l < L - 1; g.slice = in;
         gemm_any<split::DA, false>(a.fwd_var[l], g, N, smem, blk);
         grid.sync();
     }
@@ -231,16 +233,26 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
                 scale = 1.f;
             }
             float* dz_prev = L > 1 ? a.dz[L - 1] : nullptr;
-            auto part_of = [&](auto cp, auto vec) {
-                constexpr int CP = decltype(cp)::value;
-                constexpr bool VEC = decltype(vec)::value;
-                const float* W = Xi + a.w_off[L - 1];
-                if (GENERAL && a.head_slices == 16)
-                    head_backward_part<CP, 16, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+            const float* W = Xi + a.w_off[L - 1];
+            if constexpr (!GENERAL) {
+                if (a.C <= 16)
+                    head_backward_part<16, 8, true, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
                 else
-                    head_backward_part<CP, 8, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
-            };
-            head_variant(part_of);
+                    head_backward_part<32, 8, true, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+            } else {  // by the number of classes, whether rows are aligned, and the lanes to a feature group
+                auto part_of = [&](auto cp, auto vec) {
+                    constexpr int CP = decltype(cp)::value;
+                    constexpr bool VEC = decltype(vec)::value;
+                    if (a.head_slices == 16)
+                        head_backward_part<CP, 16, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+                    else
+                        head_backward_part<CP, 8, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+                };
+                if (a.C <= 16)
+                    a.head_aligned ? part_of(std::integral_constant<int, 16>{}, std::true_type{}) : part_of(std::integral_constant<int, 16>{}, std::false_type{});
+                else
+                    a.head_aligned ? part_of(std::integral_constant<int, 32>{}, std::true_type{}) : part_of(std::integral_constant<int, 32>{}, std::false_type{});
+            }
         }
         if (parts > 1) {
             grid.sync();
@@ -269,7 +281,8 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         g.A = a.dz[l + 1]; g.sAz = (long long)B * out; g.sAm = 1; g.sAk = out;
         g.B = a.act[l]; g.sBz = (long long)B * in; g.sBn = 1; g.sBk = in;
         g.C = a.G + a.w_off[l]; g.sCz = a.ld; g.sCm = in;
-        g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l]; g.status = a.status;
+        g.M = out; g.N = in; g.K = B; g.slice = a.dw_slice[l];
+        if constexpr (GENERAL) g.status = a.status;
         const bool needs_db = l < L - 1 && !(a.head && l == L - 2);  // the last layer's bias gradient came out of the loss step, the one before's out of the last layer's backward step
         if (GENERAL && needs_db && a.dw_var[l] == V_SPLIT) {  // the sums of dZ's columns come with the GEMM
             g.rowsum = a.G + a.b_off[l];
@@ -285,7 +298,8 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
             d.B = a.X + a.w_off[l]; d.sBz = a.ld; d.sBn = 1; d.sBk = in;
             d.C = a.dz[l]; d.sCz = (long long)B * in; d.sCm = in;
             d.mask = a.act[l]; d.sMz = (long long)B * in; d.sMm = in;
-            d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l]; d.status = a.status;
+            d.M = B; d.N = in; d.K = out; d.slice = a.da_slice[l];
+            if constexpr (GENERAL) d.status = a.status;
             gemm_any<split::DA, GENERAL>(a.da_var[l], d, N, smem, blk);
         }
         grid.sync();
