@@ -315,6 +315,9 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
     if (GENERAL && a.any_split) split::block_end(blk);
 }
 
+// Layers that run as GEMMs.
+int gemm_layers(const dbw_handle* h) { return fp32_head_usable(h) ? h->model.n_layers - 1 : h->model.n_layers; }
+
 // Which tile variant a GEMM of `workers` problems M x N x K should take on a grid of `grid` blocks: the
 // one with the fewest waves x k-steps, a k-step costing a global-memory round trip plus its multiply-adds.
 int pick_variant(int M, int Nn, int K, int workers, int grid) {
@@ -340,6 +343,7 @@ int pick_variant(int M, int Nn, int K, int workers, int grid) {
 struct FusedState {
     bool usable = false;
     bool auto_on = false;
+    bool any_split = false;  // some GEMM of the network runs on the tensor cores
     int max_blocks = 0;
 };
 
@@ -357,11 +361,14 @@ void round_fused_prepare(dbw_handle* h) {
     h->fused = st;
     int coop = 0, per_sm = 0;
     if (!cuda_ok(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device)) || !coop) return;
-    for (auto kernel : {round_fused_kernel<false>, round_fused_kernel<true>})
-        if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, kSmemBytes)) || per_sm < 1) return;
-    if (!cuda_ok(cudaFuncSetAttribute(round_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
-    st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     const dbw_model_desc& m = h->model;
+    for (int l = 0; l < gemm_layers(h); ++l)  // layer 0 has no dA
+        st->any_split |= fp32_gemm_split(m.dims[l + 1], m.dims[l], m.batch, h->N, true) || (l > 0 && fp32_gemm_split(m.batch, m.dims[l], m.dims[l + 1], h->N, false));
+    const bool general = st->any_split || (fp32_head_usable(h) && (!fp32_head_aligned(h) || fp32_head_slices(h) == 16));
+    if (st->any_split && !cuda_ok(cudaFuncSetAttribute(round_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
+    if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, general ? round_fused_kernel<true> : round_fused_kernel<false>, kThreads,
+                                                               st->any_split ? kSplitSmemBytes : kSmemBytes)) || per_sm < 1) return;
+    st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     const long long samples = (long long)h->N * m.batch;
     long long macs = 0, tiles = 0;
     for (int l = 0; l < m.n_layers; ++l) {
@@ -418,17 +425,12 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
     widest = std::max<long long>(widest, ((long long)N * B + kThreads / 32 - 1) / (kThreads / 32));  // last layer: a warp per sample
     widest = std::max<long long>(widest, (long long)N * (((m.dims[m.n_layers - 1] + 3) / 4 + head_chunk4(a.head_slices) - 1) / head_chunk4(a.head_slices)));
     const int grid = (int)std::min<long long>(h->fused->max_blocks, std::max<long long>(widest + 1, 2));
-    for (int l = 0; l < m.n_layers; ++l) {
-        enum { FORWARD, DW, DA };
-        auto variant = [&](int M, int Nn, int K, int kind) {
-            if (l >= (a.head ? m.n_layers - 1 : m.n_layers)) return 0;  // not a GEMM
-            const bool on_tensor_cores = kind != FORWARD && fp32_gemm_split(M, Nn, K, N, kind == DW);
-            a.any_split |= on_tensor_cores;
-            return on_tensor_cores ? (int)V_SPLIT : pick_variant(M, Nn, K, N, grid);
-        };
-        a.fwd_var[l] = (signed char)variant(B, m.dims[l + 1], m.dims[l], FORWARD);
-        a.dw_var[l] = (signed char)variant(m.dims[l + 1], m.dims[l], B, DW);
-        a.da_var[l] = (signed char)variant(B, m.dims[l], m.dims[l + 1], DA);
+    a.any_split = h->fused->any_split;
+    for (int l = 0; l < gemm_layers(h); ++l) {
+        auto variant = [&](int M, int Nn, int K, bool is_dw) { return fp32_gemm_split(M, Nn, K, N, is_dw) ? (int)V_SPLIT : pick_variant(M, Nn, K, N, grid); };
+        a.fwd_var[l] = (signed char)pick_variant(B, m.dims[l + 1], m.dims[l], N, grid);
+        a.dw_var[l] = (signed char)variant(m.dims[l + 1], m.dims[l], B, true);
+        if (l > 0) a.da_var[l] = (signed char)variant(B, m.dims[l], m.dims[l + 1], false);
     }
     for (int l = 0; l < m.n_layers; ++l) {
         a.dw_slice[l] = fp32_gemm_slice(m.dims[l + 1], m.dims[l], B, N, true, h->sm_count);
