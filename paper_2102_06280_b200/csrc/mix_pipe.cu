@@ -214,7 +214,8 @@ int launch_pipe(dbw_handle* h, const Shape& sh, const CUtensorMap& mx, const CUt
 
 }  // namespace
 
-bool mix_pipe_usable(const dbw_handle* h, bool gradient) { return shape_of(h, gradient).gs != 0; }
+// Not without the driver's tensor maps, which the plain kernel has no need of.
+bool mix_pipe_usable(const dbw_handle* h, bool gradient) { return shape_of(h, gradient).gs != 0 && encode_tiled_fn(); }
 
 int launch_mix_pipe(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
                     const int* active_count) {

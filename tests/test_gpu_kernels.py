@@ -1166,10 +1166,15 @@ def test_fp32_last_layer_of_any_width(dims, batch, n):
     h.close()
 
 
-@pytest.mark.parametrize("n,deg,d", [(5, 2, 3_000_001), (17, 4, 900_000), (33, 4, 450_003),   # panels of 256, 128 and 64 columns
-                                     (70, 32, 210_000),                                        # a long plan
-                                     (129, 8, 120_001), (200, 6, 40_002), (257, 8, 20_000),    # 32 columns, two blocks an SM and one; two boxes of rows
-                                     (439, 6, 19_000), (750, 4, 20_000)])                      # without gradients alone
+# Workers, degree, columns; columns of a panel and blocks to an SM with gradients and without (tests/test_mix_pipe_cpu.py), 0: the plain kernel.
+PIPE_SHAPES = [(5, 2, 4_200_001, (256, 2, 256, 2)), (17, 4, 1_250_000, (128, 2, 128, 2)), (33, 4, 640_003, (64, 2, 64, 2)),
+               (70, 32, 300_000, (64, 2, 64, 2)),                              # a long plan
+               (129, 8, 165_001, (32, 2, 64, 2)), (200, 6, 110_002, (32, 2, 64, 2)),
+               (257, 8, 85_000, (32, 1, 32, 2)),                               # two boxes of rows
+               (400, 6, 53_000, (32, 1, 64, 1)), (439, 6, 19_000, (0, 0, 32, 1)), (750, 4, 20_000, (0, 0, 32, 1))]
+
+
+@pytest.mark.parametrize("n,deg,d", [c[:3] for c in PIPE_SHAPES])
 @pytest.mark.parametrize("order", ["local_then_mix", "mix_then_correct"])
 def test_pipelined_panel_mix_gives_the_bits_of_the_plain_one(n, deg, d, order):
     """The panel mix with its next panels on their way, at the edges of its panel widths: with and without gradients, with a learning rate per
