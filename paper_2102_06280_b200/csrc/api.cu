@@ -235,7 +235,7 @@ int dbw_init(dbw_handle** out, int32_t N, int64_t d, int64_t ld, const int32_t* 
     if ((rc = dev_alloc(&h->d_rowptr, N + 1)) || (rc = dev_alloc(&h->d_col, h->nnz)) ||
         (rc = dev_alloc(&h->d_links, 2 * D)) || (rc = dev_alloc(&h->d_covered, D)) ||
         (rc = dev_alloc(&h->d_epoch, 2)) || (rc = dev_alloc(&h->d_status, 1)) ||
-        (rc = dev_alloc(&h->d_waited, N)) || (rc = dev_alloc(&h->d_ticket, 1)) ||
+        (rc = dev_alloc(&h->d_waited, N)) || (rc = dev_alloc(&h->d_ticket, 2)) ||
         (rc = dev_alloc(&h->d_Tnbr_ws, N)) || (rc = dev_alloc(&h->plan.idx, (size_t)N * h->plan.stride)) ||
         (rc = dev_alloc(&h->plan.w, (size_t)N * h->plan.stride)) || (rc = dev_alloc(&h->plan.w_self, N)) ||
         (rc = dev_alloc(&h->plan.cnt, N)))
@@ -250,6 +250,7 @@ int dbw_init(dbw_handle** out, int32_t N, int64_t d, int64_t ld, const int32_t* 
               cuda_ok(cudaMemset(h->d_ticket, 0, sizeof(uint32_t)));
     if (!ok) return fail(DBW_ERR_CUDA);
     h->plan.status = h->d_status;
+    h->d_panel_rows = reinterpret_cast<int*>(h->d_ticket + 1);
     if (!cuda_ok(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking)) ||
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming)) ||
         !cuda_ok(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming)) ||

@@ -144,6 +144,7 @@ struct dbw_handle {
     uint32_t* d_status = nullptr;    // [1]
     uint32_t* d_waited = nullptr;    // [N] scratch flags of the selection kernel (kept zero between calls)
     uint32_t* d_ticket = nullptr;    // [1] block ticket of the selection kernel (kept zero between calls)
+    int* d_panel_rows = nullptr;     // [1] behind the ticket: rows that mix_pipe_kernel leaves to mix_panel_kernel in this round, all or none
     double* d_Tnbr_ws = nullptr;     // [N]
     dbw::ActiveRows active;          // participants of the round (tensor-core rounds only, allocated with that path)
 
@@ -231,8 +232,9 @@ int mix_kernel_kind(const dbw_handle* h);
 
 // mix_pipe.cu: the panel mix as a pipeline, where that is the faster one
 bool mix_pipe_usable(const dbw_handle* h, bool gradient);
+long long mix_pipe_kept_limit(const dbw_handle* h, bool gradient);  // 0, or the neighbours kept in all below which the plain one is faster
 int launch_mix_pipe(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
-                    const int* active_count = nullptr);
+                    const int* active_count = nullptr, long long kept_limit = 0);
 
 // mix_staged.cu
 bool mix_staged_usable(const dbw_handle* h);

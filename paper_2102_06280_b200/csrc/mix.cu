@@ -29,7 +29,7 @@ mix_panel_kernel(int N, long long ld, const float* X, const float* __restrict__ 
                  int mix_then_correct, int n_panels, const int* active_count) {
     dependent_begin();
     extern __shared__ float4 sm[];  // [N][GS]
-    if (active_count && *active_count <= active_limit(N)) return;  // mix_active_kernel's round
+    if (active_count && *active_count <= active_limit(N)) return;  // mix_active_kernel's round (mix_pipe_kernel's: no rows left)
     for (int panel = blockIdx.x; panel < n_panels; panel += gridDim.x) {
         mix_panel_body<GS, kMixThreads, true, LOCAL>(panel, sm, N, ld, X, G, lr, lr_pw, Xout, shadow, plan, mix_then_correct);
         __syncthreads();
@@ -248,7 +248,8 @@ int launch_panel_of(dbw_handle* h, const float* X, const float* G, float lr, con
     // neighbours: 75 us early, 51 in order; 1032 x 1196: 141 / 62; up to 256 workers early is the better one, by 1 - 2 us), and so
     // do the blocks with a second panel of two, which counts where rows are many neighbours long (1091 x 10,761, 48 neighbours:
     // 242 early, 209 in order).
-    if (n_panels >= (h->nnz > 12 * h->N ? 2 : 1) * slots || h->N <= 256)
+    // Not behind mix_pipe_kernel either: the SMs would keep its split between shared memory and L1.
+    if (active_count != h->d_panel_rows && (n_panels >= (h->nnz > 12 * h->N ? 2 : 1) * slots || h->N <= 256))
         launch(mix_panel_kernel<GS, LOCAL>, std::min(n_panels, slots), kMixThreads, smem, s, h->N, h->ld, X, G, lr, lr_pw, X_out, shadow, h->plan, mtc, n_panels,
                active_count);
     else
@@ -424,7 +425,13 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
         if (rc || kept_limit == 0) return rc;
     }
     int gs = auto_group_size(h);
-    if (gs >= 8 && h->mix_panel_cols == 0 && mix_pipe_usable(h, G != nullptr)) return launch_mix_pipe(h, X, G, lr, lr_pw, X_out, shadow, s);
+    const int* left = nullptr;  // mix_pipe_kernel's word on whether it has left the round to the panel kernel
+    if (gs >= 8 && h->mix_panel_cols == 0 && mix_pipe_usable(h, G != nullptr)) {
+        const long long limit = mix_pipe_kept_limit(h, G != nullptr);
+        const int rc = launch_mix_pipe(h, X, G, lr, lr_pw, X_out, shadow, s, nullptr, limit);
+        if (rc || limit == 0) return rc;
+        left = h->d_panel_rows;
+    }
     if (gs == 32 && h->mix_panel_cols == 0 && h->N >= 64) {
         bool narrower = false;
         const int rc = panel_local(h) ? narrower_panel<true>(h, &narrower) : narrower_panel<false>(h, &narrower);
@@ -432,11 +439,11 @@ int launch_mix(dbw_handle* h, const float* X, const float* G, float lr, const fl
         if (narrower) gs = 16;
     }
     switch (gs) {
-        case 64: return launch_panel<64>(h, X, G, lr, lr_pw, X_out, shadow, s);
-        case 32: return launch_panel<32>(h, X, G, lr, lr_pw, X_out, shadow, s);
-        case 16: return launch_panel<16>(h, X, G, lr, lr_pw, X_out, shadow, s);
-        case 8: return launch_panel<8>(h, X, G, lr, lr_pw, X_out, shadow, s);
-        case 4: return launch_panel<4>(h, X, G, lr, lr_pw, X_out, shadow, s);
+        case 64: return launch_panel<64>(h, X, G, lr, lr_pw, X_out, shadow, s, left);
+        case 32: return launch_panel<32>(h, X, G, lr, lr_pw, X_out, shadow, s, left);
+        case 16: return launch_panel<16>(h, X, G, lr, lr_pw, X_out, shadow, s, left);
+        case 8: return launch_panel<8>(h, X, G, lr, lr_pw, X_out, shadow, s, left);
+        case 4: return launch_panel<4>(h, X, G, lr, lr_pw, X_out, shadow, s, left);
         default: break;
     }
     if (X_out == X) return DBW_ERR_BAD_SHAPE;

@@ -39,6 +39,8 @@ struct PipeArgs {
     uint16_t* shadow;
     MixPlan plan;
     const int* active_count;  // nullable: with at most active_limit(N) participants the round is mix_active_kernel's
+    long long kept_limit;     // with fewer neighbours kept in all it is mix_panel_kernel's, which is told by the number of rows left to it
+    int* panel_rows;
 };
 
 __device__ __forceinline__ void load_box(void* dst, const CUtensorMap* map, int c, int row, uint64_t* bar) {
@@ -61,6 +63,11 @@ __global__ void __launch_bounds__(kThreads, 2) mix_pipe_kernel(const __grid_cons
     volatile uint32_t* abort = &abort_word;
     const int N = a.N, tid = threadIdx.x, stride = a.plan.stride;
     if (a.active_count && *a.active_count <= active_limit(N)) return;
+    if (a.kept_limit > 0) {
+        const bool mine = keeps_at_least(a.plan, N, a.kept_limit);
+        if (blockIdx.x == 0 && tid == 0) *a.panel_rows = mine ? 0 : N;
+        if (!mine) return;
+    }
     const int matrix = a.boxes * a.box_rows * GS * 16, stage = matrix * (MODE == NO_GRADIENT ? 1 : 2);
     uint8_t* panels = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pipe_smem) + 127) & ~(uintptr_t)127);
     float* w = reinterpret_cast<float*>(panels + (size_t)a.stages * stage);
@@ -171,8 +178,8 @@ struct Shape {
 // panels of 64 columns where they fit, then of 32; wider ones only where a panel would have fewer pieces than a block has threads.
 // Measured (us, plain / here, other widths in brackets): 96 workers x 300,007 columns, 6 neighbours 98 / 72 (32 columns 80); 128 x
 // 1,000,000, 8 407 / 314 (64 columns, one block 342); 192 x 400,000, 6 244 / 181; 192, 24 neighbours 487 / 370 (32 columns 417); 320 x
-// 300,000, 8 386 / 248; 400, 6 482 / 286; 750 x 200,000, 4, no gradient 463 / 235; where few are kept the plain one is as
-// fast (256 x 400,000 233 / 239, 94 x 2,504,265 539 / 561; 33 x 7,844,177 637 / 613).
+// 300,000, 8 386 / 248; 400, 6 482 / 286; 750 x 200,000, 4, no gradient 463 / 235; where
+// few are kept see mix_pipe_kept_limit.
 // The plain kernel stays where the matrices lie in L2 or the blocks have a turn or two each: filling the ring then costs more than
 // it hides (15 x 60,000: 8.0 / 10.6, 96 x 20,000: 11.1 / 12.7, 128 x 50,000: 22.5 / 22.8; 256 x 30,000: 31.8 / 29.1, 400 x 20,000:
 // 38.6 / 31.1).
@@ -217,11 +224,22 @@ int launch_pipe(dbw_handle* h, const Shape& sh, const CUtensorMap& mx, const CUt
 // Not without the driver's tensor maps, which the plain kernel has no need of.
 bool mix_pipe_usable(const dbw_handle* h, bool gradient) { return shape_of(h, gradient).gs != 0 && encode_tiled_fn(); }
 
+// Workers that keep hardly a neighbour leave the plain kernel next to nothing to sum, and its panels are up to four times as wide.  How
+// many are kept only the device knows: both kernels are launched then, and the one whose round it is not leaves after a look at the
+// plan's counts (5 us in all, so not where a mix is short).  Measured with 0 / 0.25 / 0.5 / 1 kept a worker (us; plain, here alone, both): 94
+// workers x 2,504,265 columns 531 530 552 619, 585 585 594 602, 535 533 599 602; 64 x 3,000,000 403 407 428 502, 425 434 432 375, 411
+// 420 387 399; 200 x 900,000 423 429 454 494, 454 450 447 446, 427 431 450 446; 128 x 1,000,000 280 281 294 337, 296 297 296 306, 289
+// 289 307 310.  With more workers the plain kernel's panels are narrow too (256 x 400,000 231 231 242 274, 234 203 209 231; 320 x
+// 600,000 507 525 561 627, 403 424 416 435), and without gradients this kernel is always the faster.
+long long mix_pipe_kept_limit(const dbw_handle* h, bool gradient) {
+    return gradient && h->N <= 224 && (long long)h->N * h->ld * 12 >= (1ll << 30) ? (h->N + 1) / 2 : 0;
+}
+
 int launch_mix_pipe(dbw_handle* h, const float* X, const float* G, float lr, const float* lr_pw, float* X_out, uint16_t* shadow, cudaStream_t s,
-                    const int* active_count) {
+                    const int* active_count, long long kept_limit) {
     const Shape sh = shape_of(h, G != nullptr);
     PipeArgs a{};
-    a.N = h->N; a.ld = h->ld; a.lr = lr; a.lr_pw = lr_pw; a.Xout = X_out; a.shadow = shadow; a.plan = h->plan; a.active_count = active_count;
+    a.N = h->N; a.ld = h->ld; a.lr = lr; a.lr_pw = lr_pw; a.Xout = X_out; a.shadow = shadow; a.plan = h->plan; a.active_count = active_count; a.kept_limit = kept_limit; a.panel_rows = h->d_panel_rows;
     a.n_panels = (int)((h->ld + 4 * sh.gs - 1) / (4 * sh.gs));
     a.stages = sh.stages; a.boxes = sh.boxes; a.box_rows = sh.box_rows;
     CUtensorMap mx{}, mg{};

@@ -1363,3 +1363,38 @@ def test_fp32_tensor_core_gemms_with_outputs_that_are_not_finite():
     assert time <= 4 * usual, (time, usual)
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("n,deg,d,order", [(24, 4, 3_800_000, "local_then_mix"), (65, 6, 1_500_003, "mix_then_correct"), (224, 4, 420_000, "local_then_mix")])
+def test_pipelined_panel_mix_leaves_rounds_with_few_kept_neighbours_to_the_plain_one(n, deg, d, order):
+    """Matrices large enough for both kernels to be launched: nothing kept, one neighbour less than the line, the line, everything; in place and
+    out of place, against the plain panel kernel bit for bit."""
+    p = _dbw()
+    rowptr, col = wl.random_regular(n, deg, 3)
+    h = p.Dbw(rowptr, col, d=d, flags=p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    assert n * h.ld * 12 >= 1 << 30
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X, G = (torch.randn(n, h.ld, device="cuda", generator=gen) for _ in range(2))
+    want, got = torch.empty_like(X), torch.empty_like(X)
+    kept = torch.zeros(len(col), dtype=torch.uint8, device="cuda")
+    t = torch.rand(n, device="cuda", generator=gen, dtype=torch.float64)
+    line = (n + 1) // 2
+    for total in (0, line - 1, line, n * deg):
+        b = torch.full((n,), deg, dtype=torch.int32, device="cuda")
+        if total == n * deg:
+            b.zero_()
+        else:
+            b[torch.randperm(n, device="cuda", generator=gen)[:total]] -= 1
+        h.select(t, b, kept)
+        assert int(kept.sum()) == total
+        h.set_mix_panel(16)
+        h.mix(X, G, kept, b, 0.05, want)
+        h.set_mix_panel(0)
+        got.zero_()
+        h.mix(X, G, kept, b, 0.05, got)
+        assert torch.equal(got, want), total
+        got.copy_(X)
+        h.mix(got, G, kept, b, 0.05, got)
+        assert torch.equal(got, want), total
+    assert h.status() == 0
+    h.close()
