@@ -1076,10 +1076,10 @@ def test_round_host_on_two_streams_gives_the_bits_of_dbw_round(kind, dynamic):
 
 
 @pytest.mark.parametrize("dims,batch,n", [([129, 127, 65, 10], 97, 40),   # nothing a multiple of four: rows at every shift, partial tiles one short and one over
-                                          ([132, 128, 64, 10], 128, 64),  # whole tiles, a last step of a few k, more tiles than SMs
-                                          ([784, 64, 10], 64, 20),        # one tile a worker: the deep ring, an odd number of steps
-                                          ([36, 256, 10], 128, 60),       # a step and four k
-                                          ([31, 301, 10], 100, 40),       # less than a step
+                                          ([132, 128, 64, 10], 128, 64),  # whole tiles, more of them than SMs, and dW with four columns over
+                                          ([784, 64, 10], 64, 20),        # dW alone, two steps, no more tiles than SMs: the deep ring
+                                          ([36, 256, 10], 128, 60),       # dW of 36 columns
+                                          ([31, 301, 10], 100, 40),       # dW of three steps and four samples
                                           ([300, 201, 10], 33, 20),       # dW of a step and one sample
                                           ([65, 500, 130, 10], 250, 12)])
 def test_fp32_gemms_on_the_tensor_cores(dims, batch, n):
@@ -1129,6 +1129,8 @@ def test_fp32_gemms_on_the_tensor_cores(dims, batch, n):
                                           ([64, 132, 12], 301, 30),      # ... aligned, two parts, four samples to a warp and one left over
                                           ([64, 35, 16], 258, 41),       # ... unaligned
                                           ([64, 130, 32], 50, 30),       # the most classes
+                                          ([64, 132, 30], 90, 30),       # ... with sixteen lanes to a feature group, aligned
+                                          ([64, 131, 20], 72, 35),       # ... and not
                                           ([20, 1, 3], 9, 4)])           # a single feature
 def test_fp32_last_layer_of_any_width(dims, batch, n):
     """The last layer's two steps with rows that are not 16-byte aligned, and their variants by size: gradients and losses against the
@@ -1239,7 +1241,9 @@ def _check_few_products(got, Z, T, counts):
 @pytest.mark.parametrize("batch,tests,out,n", [(128, 384, 128, 8),    # whole tiles, a block to an SM
                                                (64, 192, 160, 24),    # ... five k steps in dA
                                                (64, 192, 128, 60),    # two blocks to an SM
-                                               (97, 158, 131, 30)])   # rows at every shift
+                                               (97, 158, 131, 30),    # rows at every shift
+                                               (27, 302, 131, 40),    # ... and dW of less than a step
+                                               (130, 300, 27, 40)])   # ... and dA
 @pytest.mark.parametrize("scale", [1.0, 2.0 ** -112, 2.0 ** 118])  # ... whose last pieces are below the smallest bf16 number; whose sums overflow when scaled
 def test_fp32_tensor_core_gemms_sum_few_products_as_multiply_adds_do(batch, tests, out, n, scale):
     """Sums of one, two and four non-zero products, and dense ones, are no less exact than fp32 multiply-adds in the tensor-core GEMMs: dW through
@@ -1398,3 +1402,44 @@ def test_pipelined_panel_mix_leaves_rounds_with_few_kept_neighbours_to_the_plain
         assert torch.equal(got, want), total
     assert h.status() == 0
     h.close()
+
+
+@pytest.mark.parametrize("order", ["local_then_mix", "mix_then_correct"])
+@pytest.mark.parametrize("n,dims", [(20, [3072, 304, 10]), (96, [3072, 64, 10]), (210, [1024, 120, 10])])  # panels of 128, 64 and 32 columns
+def test_pipelined_panel_mix_in_tensor_core_rounds(n, dims, order):
+    """Rounds whose mix is the pipeline's where more than half of the workers take part and another kernel's where fewer do, with the bf16 copy of
+    the parameters that the next round reads: against rounds on the plain panel kernel bit for bit, in place and out of place."""
+    p = _dbw()
+    batch = 8
+    rowptr, col = wl.ring(n)
+    m = p.model_layout(dims, batch)
+    flags = p.GEMM_BF16 | (p.ORDER_MIX_THEN_CORRECT if order == "mix_then_correct" else 0)
+    assert 12 * n * m.ld >= 160 << 20
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    feat = torch.rand(n, batch, dims[0], device="cuda", generator=gen)
+    labels = torch.randint(0, 10, (n, batch), device="cuda", generator=gen, dtype=torch.int32)
+    idx = torch.arange(batch, device="cuda", dtype=torch.int32).repeat(n, 1)
+    t = 1.0 + torch.rand(n, device="cuda", generator=gen, dtype=torch.float64)
+    everyone = torch.zeros(n, dtype=torch.int32, device="cuda")
+    few = torch.where(torch.arange(n, device="cuda") < n // 6, 1, 2).int()
+    X0 = torch.zeros(n, m.ld, device="cuda")
+    for l in range(2):
+        X0[:, m.w_off[l]: m.w_off[l] + dims[l] * dims[l + 1]].normal_(0.0, 0.03, generator=gen)
+    outs = []
+    for panel in (0, 16):
+        h = p.Dbw(rowptr, col, d=m.d, model=m, flags=flags)
+        h.set_dataset(feat, labels, batch)
+        h.set_mix_panel(panel)
+        h.set_param_tracking(True)
+        kept, loss = torch.zeros(len(col), dtype=torch.uint8, device="cuda"), torch.zeros(n, device="cuda")
+        X, Y, got = X0.clone(), torch.zeros_like(X0), []
+        for b in (everyone, few, everyone, everyone):
+            out = X if len(got) == 2 else Y
+            h.round(X, t, b, 0.05, out, kept, batch_idx=idx, loss=loss)
+            got.append((out.clone(), loss.clone()))
+            X, Y = out, (Y if out is X else X)
+        assert h.status() == 0
+        h.close()
+        outs.append(got)
+    for (x, l), (y, k) in zip(*outs):
+        assert torch.equal(x, y) and torch.equal(l, k)
