@@ -290,6 +290,9 @@ inline bool fp32_head_aligned(const dbw_handle* h) {
     const int L = m.n_layers;
     return (m.dims[L - 1] & 3) == 0 && (m.w_off[L - 1] & 3) == 0 && (h->ld & 3) == 0 && ((uintptr_t)h->feat & 15) == 0;
 }
+// Networks that the single launch takes unasked, with a last layer in its two steps (round_fused.cu): samples of all workers in networks of
+// one layer (fewer in deeper ones), workers in deeper ones.
+constexpr int kSingleLaunchSamples = 2560, kSingleLaunchWorkers = 20;
 // Lanes that share a feature group's samples in the last layer's backward step, and the feature groups of a block.  Sixteen instead of
 // eight make twice the blocks, each half as long, which pays where the blocks are few and their samples many (us, 8 / 16: 10 workers
 // x batch 1024, 256 features 46 / 32, 32 x 64, 200 features 13.4 / 10.3), not where a lane is left with a few samples for as many
@@ -299,7 +302,7 @@ __host__ __device__ constexpr int head_chunk4(int slices) { return 8 * 32 / slic
 inline int fp32_head_slices(const dbw_handle* h) {
     const int B = h->model.batch, in4 = (h->model.dims[h->model.n_layers - 1] + 3) / 4;
     const long long blocks = (long long)h->N * ((in4 + head_chunk4(8) - 1) / head_chunk4(8)) * fp32_head_parts(B);
-    const bool large = (long long)h->N * B > 2560 || (h->model.n_layers > 1 && h->N > 20);
+    const bool large = (long long)h->N * B > kSingleLaunchSamples || (h->model.n_layers > 1 && h->N > kSingleLaunchWorkers);
     return large && B >= 64 && 2 * blocks <= h->sm_count + h->sm_count / 4 ? 16 : 8;
 }
 // Slices over k of an fp32 backward GEMM of `batch` problems M x N x K (GemmArgs::slice), the same for the per-step kernels and

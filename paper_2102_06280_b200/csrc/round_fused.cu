@@ -42,17 +42,22 @@ constexpr int kBlocksPerSM = 1;                  // registers are spent on deep 
 // the slowest block.  Where the lines lie was measured on 1700 networks of 3 - 64 workers (single launch / step by step, us):
 //  - one layer, whose last layer's two steps read the data set themselves: up to 2560 samples over all workers (8 workers x batch 32,
 //    784-10: 19 / 33, 16 x 64, 784-10: 24 / 36, 41 x 52, 784-10: 39 / 40, 23 x 372, 256-10: 60 / 49);
-//  - one layer whose rows are not aligned (features no multiple of four): 64 samples (12 x 6, 281-10: 29 / 26, 25 x 265, 121-10: 92 / 62);
+//  - one layer whose rows are not aligned (features no multiple of four), or of more than 32 classes: 64 samples;
 //  - more layers, the last one in those two steps: 2048 samples of at most 20 workers (8 x 128, 256-64-10: 50 / 59, 8 x 268, 64-96-10:
 //    74 / 79; 40 x 17, 16-108-10: 45 / 36);
-//  - more layers, the last one's rows not aligned: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16 million multiply-adds.
+//  - more layers, the last one's rows not aligned or of more than 32 classes: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16
+//    million multiply-adds.
+// The lines for rows that are not aligned were drawn when such a last layer ran as GEMMs in both forms (one layer 12 x 6, 281-10: 29 / 26,
+// 25 x 265, 121-10: 92 / 62).  In its two steps the single launch would pay up to 1024 samples of 24 workers with one layer (10 x 62,
+// 686-10: 28 / 32; 8 x 150, 870-10: 44 / 37; 59 x 4, 245-10: 34 / 28), and with more it is the slower one in 93 of 100 networks inside its
+// lines, by a seventh in the mean (8 x 4, 256-65-10: 39 / 34; 3 x 105, 784-41-10: 68 / 62).
 // Never above 64 million multiply-adds of the forward pass.
 struct AutoLimits {
     long long samples, tiles, workers, macs;
 };
 constexpr long long kAny = 1ll << 40;
-constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {2560, kAny, kAny, 64 << 20}},   // one layer: rows not aligned / aligned
-                                    {{512, 148, kAny, 16 << 20}, {2048, kAny, 20, 64 << 20}}};    // more
+constexpr AutoLimits kAuto[2][2] = {{{64, kAny, kAny, 64 << 20}, {kSingleLaunchSamples, kAny, kAny, 64 << 20}},           // one layer: rows not aligned / aligned
+                                    {{512, 148, kAny, 16 << 20}, {2048, kAny, kSingleLaunchWorkers, 64 << 20}}};    // more
 
 // GEMM tile variants (R, TK) the kernel instantiates; which one a GEMM uses is chosen on the host.
 enum { V_2_16 = 0, V_2_64 = 1, V_4_16 = 2, V_4_64 = 3, V_2_128 = 4, kVariants = 5, V_SPLIT = 5 };
