@@ -39,7 +39,7 @@ __host__ __device__ constexpr size_t smem_bytes(int ring) { return (size_t)(ring
 constexpr uint32_t kWaitLimit = 1u << 24;
 // Pieces are formed of 2^24 times the value.  A bf16 number has the exponents of a float, so the last piece of a value below 2^-110 would
 // be less than the smallest of them; scaled, the pieces of every float, subnormal ones included, are normal numbers.  Values and sums
-// beyond the other end (2^104 and 2^80) come out infinite or NaN and are summed again (finish).
+// beyond the other end (2^104 and 2^80) come out infinite or NaN and are summed again (sum_on_cuda_cores).
 constexpr float kScale = 16777216.f, kUnscale = 1.f / kScale / kScale;
 
 // Barriers and tensor memory of a block, set up once and used for any number of tiles.
@@ -80,13 +80,15 @@ __device__ __forceinline__ void block_begin(Block& b, uint8_t* smem, BlockSmem& 
     tc_fence_after();
     b.tmem = __shfl_sync(0xffffffffu, fixed.tmem, 0);
 }
-__device__ __forceinline__ void block_end(const Block& b) {
+// Returns whether `p` holds in any thread of the block.
+__device__ __forceinline__ bool block_end(const Block& b, bool p = false) {
     tc_fence_before();
-    __syncthreads();
+    p = __syncthreads_or(p);
     if (threadIdx.x < 32) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(b.tmem), "r"(kTmemCols) : "memory");
     }
+    return p;
 }
 
 // By a converged warp, one lane of which issues.
@@ -308,20 +310,6 @@ __device__ __forceinline__ bool finish(const GemmArgs& g, int z, int m1, int n, 
     }
     return none == 0.f;
 }
-// Whether `p` holds in any of the eight filling warps; what they have stored is visible to all of them afterwards.
-__device__ __forceinline__ bool any_of_fill(bool p) {
-    uint32_t any;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(any)
-        : "r"((uint32_t)p), "n"(kFillThreads)
-        : "memory");
-    return any != 0;
-}
-
 struct Tiles {
     int n, m, total;  // along n (walked first), along m, in all
     __host__ __device__ Tiles(int M, int N, int batch) : n((N + kM - 1) / kM), m((M + kN - 1) / kN), total(n * m * batch) {}
@@ -360,19 +348,21 @@ __device__ __forceinline__ void for_steps(int steps, F step) {
 // outputs are summed again as the CUDA-core kernels do, by the eight filling warps with the buffer (which no MMA reads any more) as
 // staging.
 template <bool NC>
-__device__ __forceinline__ void sum_on_cuda_cores(const GemmArgs& g, int z, int m0, int n0, float* smem) {
-    float(*As)[68] = reinterpret_cast<float(*)[68]>(smem);
-    float(*Bs)[68] = reinterpret_cast<float(*)[68]>(smem + 16 * 68);
+__device__ __forceinline__ void sum_on_cuda_cores(const Block& blk, const GemmArgs& g, const Tiles& tiles, int tile) {
+    float(*As)[68] = reinterpret_cast<float(*)[68]>(blk.buffers);
+    int z, m0, n0;
+    tiles.at(tile, z, m0, n0);
 #pragma unroll 1
-    for (int n1 = n0; n1 < min(n0 + kM, g.N); n1 += 64) dev::gemm_tile<4, 16, NC, false, kFillThreads>(g, z, m0, n1, As, Bs);
+    for (int n1 = n0; n1 < min(n0 + kM, g.N); n1 += 64) dev::gemm_tile<4, 16, NC, false, kFillThreads>(g, z, m0, n1, As, As + 16);
 }
 
 // Tile `tile` of the products C[z][m][n] = epilogue(sum_k A(m, k) B(k, n)) by the eight warps of a block.  DW: both operands along the
 // outputs, with the sums of A over k if wanted; DA: A along k, B along n, masked.  AHEAD: steps whose loads
 // are on their way.  `ready` (block_begin) is called with the first loads on their way.  MMA_WARP: a ninth warp issues the MMAs
-// (issue_tile).
+// (issue_tile).  Returns whether the thread's outputs are finite; where one's are not the tile is for sum_on_cuda_cores, once every
+// thread is here.
 template <int KIND, bool VEC, bool NC, int RING, int AHEAD, bool MMA_WARP, class Ready>
-__device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const Tiles& tiles, int tile, Ready ready) {
+__device__ __forceinline__ bool gemm_tile(Block& blk, const GemmArgs& g, const Tiles& tiles, int tile, Ready ready) {
     constexpr bool AK = KIND != DW;
     typedef Operand<kM, false, VEC, NC> OpN;  // the operand with C's contiguous index
     typedef Operand<kN, AK, VEC, NC> OpM;
@@ -460,9 +450,7 @@ __device__ __forceinline__ void gemm_tile(Block& blk, const GemmArgs& g, const T
             asm volatile("bar.sync 1, %0;" ::"n"(kFillThreads) : "memory");  // before the next tile is filled
         }
     }
-    const bool finite = finish<KIND, NC, 32>(g, z, m0 + 32 * mh, n0 + 32 * q + lane, v);
-    __syncwarp();
-    if (any_of_fill(!finite)) sum_on_cuda_cores<NC>(g, z, m0, n0, reinterpret_cast<float*>(blk.buffers));
+    return finish<KIND, NC, 32>(g, z, m0 + 32 * mh, n0 + 32 * q + lane, v);
 }
 
 // The ninth warp's part of a tile.

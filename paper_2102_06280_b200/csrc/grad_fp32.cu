@@ -437,13 +437,15 @@ __global__ void __launch_bounds__(split::kFillThreads + 32, DEEP ? 1 : 2) gemm_s
     extern __shared__ uint8_t split_smem[];
     __shared__ split::BlockSmem fixed;
     split::Block blk;
+    bool finite = true;
     if (threadIdx.x < split::kFillThreads) {
-        split::gemm_tile<KIND, VEC, true, RING, AHEAD, true>(blk, g, tiles, blockIdx.x, [&] { split::block_begin(blk, split_smem, fixed); });
+        finite = split::gemm_tile<KIND, VEC, true, RING, AHEAD, true>(blk, g, tiles, blockIdx.x, [&] { split::block_begin(blk, split_smem, fixed); });
     } else {
         split::block_begin(blk, split_smem, fixed);
         split::issue_tile<KIND, RING>(blk, g);
     }
-    split::block_end(blk);
+    const bool again = split::block_end(blk, !finite);
+    if (again && threadIdx.x < split::kFillThreads) split::sum_on_cuda_cores<true>(blk, g, tiles, blockIdx.x);
 }
 
 template <int KIND, bool VEC, bool DEEP>

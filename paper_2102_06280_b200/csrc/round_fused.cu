@@ -117,7 +117,10 @@ template <int KIND, bool GENERAL>
 __device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int workers, float* smem, split::Block& blk) {
     if (GENERAL && variant == V_SPLIT) {
         const split::Tiles tiles(g.M, g.N, workers);
-        for (int tile = blockIdx.x; tile < tiles.total; tile += gridDim.x) split::gemm_tile<KIND, false, false, 2, 1, false>(blk, g, tiles, tile, [] {});
+        for (int tile = blockIdx.x; tile < tiles.total; tile += gridDim.x) {
+            const bool finite = split::gemm_tile<KIND, false, false, 2, 1, false>(blk, g, tiles, tile, [] {});
+            if (__syncthreads_or(!finite)) split::sum_on_cuda_cores<false>(blk, g, tiles, tile);
+        }
         __syncthreads();
         return;
     }
