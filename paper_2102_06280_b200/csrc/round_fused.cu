@@ -48,9 +48,9 @@ constexpr int kBlocksPerSM = 1;                  // registers are spent on deep 
 //  - more layers, the last one's rows not aligned or of more than 32 classes: 512 samples, no more 32 x 32 tiles than SMs in a layer, 16
 //    million multiply-adds.
 // The lines for rows that are not aligned were drawn when such a last layer ran as GEMMs in both forms (one layer 12 x 6, 281-10: 29 / 26,
-// 25 x 265, 121-10: 92 / 62).  In its two steps the single launch would pay up to 1024 samples of 24 workers with one layer (10 x 62,
-// 686-10: 28 / 32; 8 x 150, 870-10: 44 / 37; 59 x 4, 245-10: 34 / 28), and with more it is the slower one in 93 of 100 networks inside its
-// lines, by a seventh in the mean (8 x 4, 256-65-10: 39 / 34; 3 x 105, 784-41-10: 68 / 62).
+// 25 x 265, 121-10: 92 / 62).  In its two steps the single launch would pay up to 1200 samples of 40 workers with one layer (10 x 62,
+// 686-10: 27 / 32; 8 x 150, 870-10: 41 / 38; 59 x 4, 245-10: 33 / 26), and with more it is the slower one in 91 of 100 networks inside its
+// lines, by a tenth in the mean (10 x 36, 256-17-10: 44 / 38; 4 x 41, 768-73-10: 57 / 52).
 // Never above 64 million multiply-adds of the forward pass.
 struct AutoLimits {
     long long samples, tiles, workers, macs;
@@ -137,11 +137,13 @@ __device__ __forceinline__ void gemm_any(int variant, const GemmArgs& g, int wor
     }
 }
 
-// GENERAL = false leaves out what most rounds of this size have no use for: GEMMs on the tensor cores, last layers whose rows are not
-// aligned or whose backward step has sixteen lanes to a feature group.  The launch is short enough for code that is not run to show
-// (21 workers, 784-10, batch 57: 33.0 us a round with it, 30.0 without).
-template <bool GENERAL>
+// Three instances: last layers whose rows are aligned, those whose rows are not, and the general one, with GEMMs on the tensor cores and
+// backward steps of sixteen lanes to a feature group.  The launch is short enough for code that is not run to show (21 workers, 784-10, batch
+// 57: 33.0 us a round with all of it, 30.0 without).
+enum { ALIGNED = 0, UNALIGNED = 1, ANY = 2 };
+template <int KIND>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(FusedArgs a) {
+    constexpr bool GENERAL = KIND == ANY;
     extern __shared__ __align__(16) float smem[];
     __shared__ float sl[8];
     __shared__ double red[kThreads / 32];
@@ -166,16 +168,17 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
         for (int item = first * (kThreads / 32) + warp; item < N * B; item += step * (kThreads / 32)) {
             const int i = item / B;
             const float* Xi = a.X + (size_t)i * a.ld;
-            if (!GENERAL || a.head_aligned) {
+            if (KIND == ALIGNED || (GENERAL && a.head_aligned)) {
                 if (a.C <= 16)
                     head_forward_samples<16, 1, true, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
                 else
                     head_forward_samples<32, 1, true, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
             } else {
+                constexpr bool VEC = KIND == ALIGNED;  // never reached then
                 if (a.C <= 16)
-                    head_forward_samples<16, 1, !GENERAL, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+                    head_forward_samples<16, 1, VEC, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
                 else
-                    head_forward_samples<32, 1, !GENERAL, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
+                    head_forward_samples<32, 1, VEC, false>(i, item % B, B, a.dims[L - 1], a.C, rows, Xi + a.w_off[L - 1], Xi + a.b_off[L - 1], a.dz[L], loss_s, a.status);
             }
         }
     };
@@ -243,10 +246,11 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
             float* dz_prev = L > 1 ? a.dz[L - 1] : nullptr;
             const float* W = Xi + a.w_off[L - 1];
             if constexpr (!GENERAL) {
+                constexpr bool VEC = KIND == ALIGNED;
                 if (a.C <= 16)
-                    head_backward_part<16, 8, true, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+                    head_backward_part<16, 8, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
                 else
-                    head_backward_part<32, 8, true, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
+                    head_backward_part<32, 8, VEC, false>(i, s_lo, s_hi, scale, k_lo, k_hi, B, in, a.C, rows, a.dz[L], loss_s, W, Gw, Gb, li, dz_prev, Gp, smem, a.status);
             } else {  // by the number of classes, whether rows are aligned, and the lanes to a feature group
                 auto part_of = [&](auto cp, auto vec) {
                     constexpr int CP = decltype(cp)::value;
@@ -326,6 +330,12 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM) round_fused_kernel(Fus
 // Layers that run as GEMMs.
 int gemm_layers(const dbw_handle* h) { return fp32_head_usable(h) ? h->model.n_layers - 1 : h->model.n_layers; }
 
+// The instance that runs a network.
+auto kernel_of(const dbw_handle* h, bool any_split, bool aligned) {
+    if (any_split || (fp32_head_usable(h) && fp32_head_slices(h) == 16)) return round_fused_kernel<ANY>;
+    return aligned || !fp32_head_usable(h) ? round_fused_kernel<ALIGNED> : round_fused_kernel<UNALIGNED>;
+}
+
 // Which tile variant a GEMM of `workers` problems M x N x K should take on a grid of `grid` blocks: the
 // one with the fewest waves x k-steps, a k-step costing a global-memory round trip plus its multiply-adds.
 int pick_variant(int M, int Nn, int K, int workers, int grid) {
@@ -372,9 +382,8 @@ void round_fused_prepare(dbw_handle* h) {
     const dbw_model_desc& m = h->model;
     for (int l = 0; l < gemm_layers(h); ++l)  // layer 0 has no dA
         st->any_split |= fp32_gemm_split(m.dims[l + 1], m.dims[l], m.batch, h->N, true) || (l > 0 && fp32_gemm_split(m.batch, m.dims[l], m.dims[l + 1], h->N, false));
-    const bool general = st->any_split || (fp32_head_usable(h) && (!fp32_head_aligned(h) || fp32_head_slices(h) == 16));
-    if (st->any_split && !cuda_ok(cudaFuncSetAttribute(round_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
-    if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, general ? round_fused_kernel<true> : round_fused_kernel<false>, kThreads,
+    if (st->any_split && !cuda_ok(cudaFuncSetAttribute(round_fused_kernel<ANY>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemBytes))) return;
+    if (!cuda_ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_of(h, st->any_split, fp32_head_aligned(h)), kThreads,
                                                                st->any_split ? kSplitSmemBytes : kSmemBytes)) || per_sm < 1) return;
     st->max_blocks = h->sm_count * std::min(per_sm, kBlocksPerSM);
     const long long samples = (long long)h->N * m.batch;
@@ -445,8 +454,7 @@ int launch_round_fused(dbw_handle* h, const float* X, const double* t, const int
         a.da_slice[l] = fp32_gemm_slice(B, m.dims[l], m.dims[l + 1], N, false, h->sm_count);
     }
     void* params[] = {&a};
-    const bool general = a.any_split || (a.head && (!a.head_aligned || a.head_slices == 16));
-    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(general ? round_fused_kernel<true> : round_fused_kernel<false>), dim3(grid), dim3(kThreads), params, a.any_split ? kSplitSmemBytes : kSmemBytes, s));
+    DBW_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(kernel_of(h, a.any_split, a.head_aligned)), dim3(grid), dim3(kThreads), params, a.any_split ? kSplitSmemBytes : kSmemBytes, s));
     DBW_LAUNCHED();
     return DBW_OK;
 }
