@@ -1,6 +1,7 @@
-// Mini-batch stochastic gradient (Eq. 2) of the ReLU MLP with softmax cross-entropy, fp32 on the
-// CUDA cores, for all workers at once: every kernel is batched over workers (blockIdx.z), whose
-// weights are slices of their rows of X.
+// Mini-batch stochastic gradient (Eq. 2) of the ReLU MLP with softmax cross-entropy in fp32, for all
+// workers at once: every kernel is batched over workers (blockIdx.z), whose weights are slices of their
+// rows of X.  On the CUDA cores, but for backward GEMMs of many multiply-adds, which run on the tensor
+// cores at fp32 precision (gemm_split.cuh).
 #include "common.cuh"
 #include "gemm_split.cuh"
 #include "round_dev.cuh"
@@ -428,6 +429,9 @@ __global__ void __launch_bounds__(32, 8) gemm_warp_kernel(const __grid_constant_
     }
 }
 
+// A call of its own: inlined, dA's kernel with two blocks to an SM spills 132 bytes for 68 (10 workers, 1024 x 256 x 256: 2 us a round).
+__device__ __noinline__ void sum_again(const split::Block& blk, const GemmArgs& g, const split::Tiles& tiles) { split::sum_on_cuda_cores<true>(blk, g, tiles, blockIdx.x); }
+
 // On the tensor cores (gemm_split.cuh), a block to a tile.  DEEP: a block to an SM with loads two steps ahead and a ring of four, for
 // launches of no more tiles than SMs, which wait for their chain of k steps; else two blocks to an SM with half of that each.
 template <int KIND, bool VEC, bool DEEP>
@@ -445,7 +449,10 @@ __global__ void __launch_bounds__(split::kFillThreads + 32, DEEP ? 1 : 2) gemm_s
         split::issue_tile<KIND, RING>(blk, g);
     }
     const bool again = split::block_end(blk, !finite);
-    if (again && threadIdx.x < split::kFillThreads) split::sum_on_cuda_cores<true>(blk, g, tiles, blockIdx.x);
+    if (again && threadIdx.x < split::kFillThreads) {
+        if constexpr (KIND == split::DA) sum_again(blk, g, tiles);
+        else split::sum_on_cuda_cores<true>(blk, g, tiles, blockIdx.x);
+    }
 }
 
 template <int KIND, bool VEC, bool DEEP>
@@ -602,7 +609,7 @@ int run_gemm(dbw_handle* h, GemmArgs& g, GemmStep step, int batch, cudaStream_t 
 
 // Which backward GEMMs run on the tensor cores: those of many multiply-adds; fewer where operand rows are not whole 16-byte groups and
 // the CUDA-core kernel is the scalar one.  Measured on 900 GEMMs of 4 - 64 workers (us, CUDA cores / tensor cores): 10 workers, M x
-// N x K = 1024 x 256 x 256 42 / 23.5, 32, 200 x 784 x 64 26.6 / 19.6; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4 and 12, 32 x
+// N x K = 1024 x 256 x 256 42 / 24.8, 32, 200 x 784 x 64 26.6 / 20.1; at the lines 49, 92 x 168 x 92 (70 million) 10.4 / 10.4 and 12, 32 x
 // 256 x 307 (30 million) 10.4 / 13.9; unaligned 7, 58 x 276 x 457 (51 million) 12.4 / 16.5.  What it costs is a launch's chain:
 // operands to bf16 pieces, MMAs and a barrier between them for every 32 k, about 0.5 us whatever the size; a k of one such step
 // does not pay for it (38, 252 x 784 x 28: 24.7 / 26.5), nor does a long one of few multiply-adds.
