@@ -52,7 +52,7 @@ enum {
 #define DBW_WEIGHT_UNIFORM 1u    /* w_ii = w_ij = 1/(1+p_i) over self and the kept neighbours */
 #define DBW_ORDER_LOCAL_THEN_MIX 0u   /* Algorithm 1, Eqs. 4-5 */
 #define DBW_ORDER_MIX_THEN_CORRECT 2u /* Eq. 3 restricted to the kept set */
-#define DBW_GEMM_FP32 0u /* dense layers in fp32 on the CUDA cores */
+#define DBW_GEMM_FP32 0u /* dense layers in fp32 (large backward products as sums of exact bf16 pieces on the tensor cores, accumulated in fp32) */
 #define DBW_GEMM_BF16 4u /* dense layers with BF16 operands on tcgen05 tensor cores, fp32 accumulate */
 
 /* bits of the device status word */

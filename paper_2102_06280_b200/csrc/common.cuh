@@ -273,8 +273,8 @@ int launch_update_backups(dbw_handle* h, const double* t, int32_t* b_out, double
 // fp32 gradient path: the last layer's backward step works on parts of at most kHeadPart samples (a worker's dZ of a part,
 // its row offsets and losses lie in shared memory); more than one part leave partial sums that are added in a fixed order.
 // Bound by the latency of a block's serial passes, so the part length sets the time: 256 samples give ten workers x batch 1024
-// x 256 features 80 blocks and 45 us (with the whole batch in one block the layer fell back to GEMMs, a loss kernel of a block
-// per worker and a column sum: 230 us).
+// x 256 features 80 blocks and 45 us, or with sixteen lanes to a feature group (fp32_head_slices) 160 and 32 (with the whole batch
+// in one block the layer fell back to GEMMs, a loss kernel of a block per worker and a column sum: 230 us).
 constexpr int kHeadPart = 256;
 __host__ __device__ inline int fp32_head_parts(int B) { return (B + kHeadPart - 1) / kHeadPart; }
 inline size_t fp32_head_smem_bytes(int B, int C) {

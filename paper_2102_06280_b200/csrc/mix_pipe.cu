@@ -3,7 +3,7 @@
 //
 // The plain panel kernel (mix.cu) loads a panel through registers, then sums its rows, then loads the next: between the two the memory
 // system has only what the SM's other blocks ask for (96 workers x 300,007 columns, 6 neighbours: 98 us, 0.54 of the copy
-// bandwidth; here 72, 0.73).  Here a ring of panels lies in shared memory, a copy of a whole panel is a few instructions of one
+// bandwidth; here 76, 0.70).  Here a ring of panels lies in shared memory, a copy of a whole panel is a few instructions of one
 // thread, and the loads in flight need neither registers nor L1.  The mixing plan, which L1 then has no room for, is copied to
 // shared memory once per block.  A panel is complete before any of it is written and panels are disjoint, so X' may overwrite X.
 // Every output is summed as in the plain kernel: the same bits.  What bounds it is HBM, then the blocks' gather.
@@ -176,7 +176,7 @@ struct Shape {
 
 // Panel width (columns / 4), blocks to an SM and depth of the ring; gs = 0: the plain kernel is the faster one.  Two blocks to an SM with
 // panels of 64 columns where they fit, then of 32; wider ones only where a panel would have fewer pieces than a block has threads.
-// Measured (us, plain / here, other widths in brackets): 96 workers x 300,007 columns, 6 neighbours 98 / 72 (32 columns 80); 128 x
+// Measured (us, plain / here, other widths in brackets): 96 workers x 300,007 columns, 6 neighbours 98 / 76 (32 columns 80); 128 x
 // 1,000,000, 8 407 / 314 (64 columns, one block 342); 192 x 400,000, 6 244 / 181; 192, 24 neighbours 487 / 370 (32 columns 417); 320 x
 // 300,000, 8 386 / 248; 400, 6 482 / 286; 750 x 200,000, 4, no gradient 463 / 235; where
 // few are kept see mix_pipe_kept_limit.
